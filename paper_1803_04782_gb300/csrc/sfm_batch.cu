@@ -29,7 +29,6 @@ struct BatchScene {
   long long ct_off;    // first float of the lattice's class tables
   unsigned long long seed;
   int bin_off;  // first bin
-  int grp_off;  // first bin group (4 bins x 32 rows)
   int ped_off;  // first pedestrian
   int n;        // pedestrians
   int sp;       // class-table row stride
@@ -46,7 +45,7 @@ struct BatchChunk {
 
 struct BatchArgs {
   const BatchScene* scenes;
-  const uint16_t* grp_scene;
+  const uint16_t* bin_scene;  // lattice of each bin
   const BatchChunk* chunks;
   const uint16_t* ped_scene;
   const uint8_t* cell;
@@ -73,7 +72,6 @@ struct BatchArgs {
   unsigned int* bar;
   int* work;
   int n;             // pedestrians (all lattices)
-  int total_groups;  // bin groups (all lattices)
   int total_bins;
   int total_chunks;
   int expect_blocks;  // CTAs the grid barrier waits for
@@ -85,11 +83,11 @@ struct BatchState {
   int nscenes = 0;
   std::vector<BatchScene> hs;
   BatchScene* scenes = nullptr;
-  uint16_t* grp_scene = nullptr;
+  uint16_t* bin_scene = nullptr;
   uint16_t* ped_scene = nullptr;
   BatchChunk* chunks = nullptr;
   int total_chunks = 0, chunk_cap = 0;
-  int total_groups = 0, total_bins = 0;
+  int total_bins = 0;
   long long total_ocls = 0;
   float *own = nullptr, *dirdot = nullptr, *CT = nullptr;
   unsigned int* bar = nullptr;
@@ -245,10 +243,11 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_tick_batch(BatchArgs a) {
     }
   if (gtid == 0) *a.work = 0;
   // S1: bins -- counts, exclusive scan over all lattices' bins, fill
-  for (int w = gwarp; w < a.total_groups; w += nwarps) {
-    const BatchScene& sc = a.scenes[a.grp_scene[w]];
-    const int lg = w - sc.grp_off, ngx = (sc.g.nbx + 3) >> 2;
-    bin_count_group(sc.g, a.ocls + sc.ocls_off, a.bin_count + sc.bin_off, lg % ngx, lg / ngx, lane);
+  for (int w = gwarp; w < a.total_bins; w += nwarps) {
+    const BatchScene& sc = a.scenes[a.bin_scene[w]];
+    const int b = w - sc.bin_off;
+    const int c = bin_count_one(sc.g, a.ocls + sc.ocls_off, b % sc.g.nbx, b / sc.g.nbx, lane);
+    if (lane == 0) a.bin_count[w] = c;
   }
   if (!grid_sync(a.bar, a.expect_blocks, a.ctr)) return;
   const int nsc = (a.total_bins + kScanChunk - 1) / kScanChunk;
@@ -293,11 +292,11 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_tick_batch(BatchArgs a) {
     if (c == nsc - 1 && tid == kBatchThreads - 1) a.bin_start[a.total_bins] = e;
   }
   if (!grid_sync(a.bar, a.expect_blocks, a.ctr)) return;
-  for (int w = gwarp; w < a.total_groups; w += nwarps) {
-    const BatchScene& sc = a.scenes[a.grp_scene[w]];
-    const int lg = w - sc.grp_off, ngx = (sc.g.nbx + 3) >> 2;
-    bin_fill_group(sc.g, a.ocls + sc.ocls_off, a.occ + sc.su_off, a.bin_start + sc.bin_off, a.rec,
-                   a.rec_id, lg % ngx, lg / ngx, lane);
+  for (int w = gwarp; w < a.total_bins; w += nwarps) {
+    const BatchScene& sc = a.scenes[a.bin_scene[w]];
+    const int b = w - sc.bin_off;
+    bin_fill_one(sc.g, a.ocls + sc.ocls_off, a.occ + sc.su_off, a.bin_start[w], a.rec, a.rec_id,
+                 b % sc.g.nbx, b / sc.g.nbx, lane);
   }
   if (!grid_sync(a.bar, a.expect_blocks, a.ctr)) return;
 
@@ -471,7 +470,7 @@ BatchArgs make_args(sfm_ctx* ctx, int field_only) {
   BatchState* B = ctx->batch;
   BatchArgs a{};
   a.scenes = B->scenes;
-  a.grp_scene = B->grp_scene;
+  a.bin_scene = B->bin_scene;
   a.chunks = B->chunks;
   a.ped_scene = B->ped_scene;
   a.cell = ctx->cell;
@@ -498,7 +497,6 @@ BatchArgs make_args(sfm_ctx* ctx, int field_only) {
   a.bar = B->bar;
   a.work = B->work;
   a.n = ctx->n;
-  a.total_groups = B->total_groups;
   a.total_bins = B->total_bins;
   a.total_chunks = B->total_chunks;
   a.expect_blocks = B->grid + B->missing;
@@ -646,7 +644,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
   };
   // offsets
   long long su = 0, oc = 0, ct = 0;
-  int bins = 0, grps = 0;
+  int bins = 0;
   B->hs.resize(nscenes);
   for (int s = 0; s < nscenes; ++s) {
     BatchScene& sc = B->hs[s];
@@ -663,7 +661,6 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     sc.su_off = su;
     sc.ocls_off = oc;
     sc.bin_off = bins;
-    sc.grp_off = grps;
     sc.sp = class_table_stride(g.r);
     sc.ts = (int)(class_table_floats(g.r) / 4);
     sc.ct_off = ct;
@@ -673,7 +670,6 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     oc += (long long)g.opitch * g.H;
     ct += 4LL * sc.ts;
     bins += g.nbx * g.nby;
-    grps += ((g.nbx + 3) / 4) * g.nby;
     B->max_ts = std::max(B->max_ts, sc.ts);
   }
   if (su > ((long long)1 << 31) || bins > (1 << 30)) {
@@ -681,7 +677,6 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     return bail(SFM_EINVAL);
   }
   B->total_bins = bins;
-  B->total_groups = grps;
   B->total_ocls = oc;
   sfm_status st;
 #define BALLOC(p, n)                               \
@@ -700,7 +695,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
   BALLOC(ctx->bin_start, (size_t)bins + 1);
   BALLOC(ctx->scan_tmp, (size_t)bins / kScanChunk + 64);
   BALLOC(B->scenes, (size_t)nscenes);
-  BALLOC(B->grp_scene, (size_t)grps);
+  BALLOC(B->bin_scene, (size_t)bins);
   BALLOC(B->bar, 1);
   BALLOC(B->work, 1);
   BALLOC(ctx->ctr, 1);
@@ -725,7 +720,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
       (st = balloc(ctx, &KO, (size_t)maxS * maxS)) != SFM_OK ||
       (st = balloc(ctx, &KE, (size_t)maxS * maxS)) != SFM_OK || (st = balloc(ctx, &hvec, 9)) != SFM_OK)
     return bail(st);
-  std::vector<uint16_t> gs(grps);
+  std::vector<uint16_t> bs(bins);
   for (int sidx = 0; sidx < nscenes; ++sidx) {
     const BatchScene& sc = B->hs[sidx];
     const size_t nsu = (size_t)sc.g.W * sc.g.H;
@@ -743,14 +738,13 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     launch_static_field(sc.g, ctx->cell + sc.su_off, tb, ctx->Fs + sc.su_off, s);
     st = compute_guidance(sc.g, ctx->cell + sc.su_off, ctx->D + sc.su_off, s, &ctx->err);
     if (st != SFM_OK) return bail(st);
-    const int ng = ((sc.g.nbx + 3) / 4) * sc.g.nby;
-    for (int k = 0; k < ng; ++k) gs[sc.grp_off + k] = (uint16_t)sidx;
+    std::fill_n(bs.begin() + sc.bin_off, sc.g.nbx * sc.g.nby, (uint16_t)sidx);
   }
   cudaMemsetAsync(ctx->occ, 0xff, (size_t)su * sizeof(int32_t), s);
   cudaMemsetAsync(ctx->ocls, 0, (size_t)oc, s);
   cudaMemsetAsync(ctx->ctr, 0, sizeof(Counters), s);
   cudaMemsetAsync(B->bar, 0, sizeof(unsigned int), s);
-  cudaMemcpyAsync(B->grp_scene, gs.data(), gs.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(B->bin_scene, bs.data(), bs.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(B->scenes, B->hs.data(), B->hs.size() * sizeof(BatchScene), cudaMemcpyHostToDevice,
                   s);
   // persistent grid: one 1024-thread CTA per SM, if the shared memory allows

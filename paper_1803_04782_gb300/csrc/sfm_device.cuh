@@ -96,10 +96,6 @@ __device__ __forceinline__ int floor_div(int a, int b) {
   return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
 }
 
-__device__ __forceinline__ int nonzero_bytes(uint32_t v) {
-  return __popc((((v & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v) & 0x80808080u);
-}
-
 // Counter-based election priority: SplitMix64 (Steele, Lea, Flood 2014).
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
@@ -111,61 +107,78 @@ __device__ __forceinline__ uint64_t splitmix_nth(uint64_t s, uint64_t i) {
 }
 
 // ---------------------------------------------------------------- S1 bins
-// One warp covers bins 4*gx .. 4*gx+3 of bin row by (32 rows of the
-// 128-byte-pitched class grid, 4 bytes per lane); lanes 8b..8b+7 cover bin b.
-__device__ __forceinline__ void bin_count_group(const Geo& g, const uint8_t* __restrict__ ocls,
-                                                int32_t* __restrict__ count, int gx, int by,
-                                                int lane) {
-  const uint8_t* base = ocls + (size_t)by * kBin * g.opitch + gx * 128 + 4 * lane;
-  const int rows = min(kBin, g.H - by * kBin);
-  int c = 0;
-  for (int row = 0; row < rows; ++row)
-    c += nonzero_bytes(*reinterpret_cast<const uint32_t*>(base + (size_t)row * g.opitch));
-  c += __shfl_xor_sync(0xffffffffu, c, 1);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  c += __shfl_xor_sync(0xffffffffu, c, 4);
-  const int bx = gx * 4 + (lane >> 3);
-  if ((lane & 7) == 0 && bx < g.nbx) count[by * g.nbx + bx] = c;
+// One warp a bin, lane = row of the bin's 32 rows: the 32-byte row of the
+// 128-byte-pitched class grid in two 16-byte loads, all rows in flight at
+// once, as a 32-bit mask of its occupied columns (0 below the lattice).
+__device__ __forceinline__ uint32_t bin_row_mask(const Geo& g, const uint8_t* __restrict__ ocls, int bx,
+                                                 int by, int lane) {
+  const int y = by * kBin + lane;
+  if (y >= g.H) return 0u;
+  const uint4* row = reinterpret_cast<const uint4*>(ocls + (size_t)y * g.opitch + bx * kBin);
+  const uint4 a = row[0], b = row[1];
+  const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  uint32_t m = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    // bit 7 of each byte that is not 0, then the four bits side by side
+    const uint32_t t = ((((w[i] & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w[i]) & 0x80808080u) >> 7;
+    m |= ((t * 0x01020408u) >> 24 & 0xfu) << (4 * i);
+  }
+  return m;
 }
 
-// Records of the group's bins in row-major su order, with the pedestrian
-// index (the occupancy value) of each record.
-__device__ __forceinline__ void bin_fill_group(const Geo& g, const uint8_t* __restrict__ ocls,
-                                               const int32_t* __restrict__ occ,
-                                               const int32_t* __restrict__ start,
-                                               uint32_t* __restrict__ rec,
-                                               int32_t* __restrict__ rec_id, int gx, int by,
-                                               int lane) {
-  const int sub = lane & 7;
-  const int bx = gx * 4 + (lane >> 3);
-  const int x = gx * 128 + 4 * lane;
-  const uint8_t* base = ocls + (size_t)by * kBin * g.opitch + x;
-  const int rows = min(kBin, g.H - by * kBin);
-  int off = bx < g.nbx ? start[by * g.nbx + bx] : 0;
-  for (int row = 0; row < rows; ++row) {
-    const uint32_t v = *reinterpret_cast<const uint32_t*>(base + (size_t)row * g.opitch);
-    const int nz = nonzero_bytes(v);
-    int inc = nz;
+__device__ __forceinline__ int bin_count_one(const Geo& g, const uint8_t* __restrict__ ocls, int bx,
+                                             int by, int lane) {
+  return __reduce_add_sync(0xffffffffu, __popc(bin_row_mask(g, ocls, bx, by, lane)));
+}
+
+// Records of bin (bx, by) from slot `first` on, in row-major su order, with
+// the pedestrian index (the occupancy value) of each.  The rows' offsets come
+// from one warp scan, so a row's loads wait for no other row's; a row is
+// written by the whole warp, lane = column (coalesced).  Latency bounds it: a
+// row loop in which each row's offset followed the last row's took 34 us for
+// the 16 bins of a 100 x 100 lattice (one-pass ncu, cold) against 6.5 us here (a
+// 1000 x 1000 lattice half full: 37.7 us, now 7.9).
+__device__ __forceinline__ void bin_fill_one(const Geo& g, const uint8_t* __restrict__ ocls,
+                                             const int32_t* __restrict__ occ, int first,
+                                             uint32_t* __restrict__ rec,
+                                             int32_t* __restrict__ rec_id, int bx, int by,
+                                             int lane) {
+  const uint32_t mine = bin_row_mask(g, ocls, bx, by, lane);
+  int inc = __popc(mine);
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, inc, o, 8);
-      if (sub >= o) inc += t;
-    }
-    const int grp = __shfl_sync(0xffffffffu, inc, 7, 8);
-    if (nz) {
-      int k = off + inc - nz;
-      const int y = by * kBin + row;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  const int off = first + inc - __popc(mine);
+  const int x = bx * kBin + lane;
+  const uint32_t lt = (1u << lane) - 1u;
+  constexpr int kRows = 16;  // rows whose reads are in flight together
+#pragma unroll 1
+  for (int r0 = 0; r0 < kBin; r0 += kRows) {
+    uint32_t cls[kRows];
+    int32_t id[kRows];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const uint32_t cls = (v >> (8 * b)) & 0xffu;
-        if (cls) {
-          rec[k] = (uint32_t)(4 * sub + b) | ((uint32_t)row << 8) | ((cls - 1u) << 16);
-          rec_id[k] = occ[(size_t)y * g.W + x + b];
-          ++k;
-        }
+    for (int j = 0; j < kRows; ++j) {
+      const uint32_t m = __shfl_sync(0xffffffffu, mine, r0 + j);
+      const size_t y = (size_t)(by * kBin + r0 + j);
+      cls[j] = 0u;
+      id[j] = 0;
+      if ((m >> lane) & 1u) {
+        cls[j] = ocls[y * g.opitch + x];
+        id[j] = occ[y * g.W + x];
       }
     }
-    off += grp;
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      const uint32_t m = __shfl_sync(0xffffffffu, mine, r0 + j);
+      const int k = __shfl_sync(0xffffffffu, off, r0 + j) + __popc(m & lt);
+      if (cls[j]) {
+        rec[k] = (uint32_t)lane | ((uint32_t)(r0 + j) << 8) | ((cls[j] - 1u) << 16);
+        rec_id[k] = id[j];
+      }
+    }
   }
 }
 

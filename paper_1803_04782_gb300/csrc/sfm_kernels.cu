@@ -485,34 +485,31 @@ void launch_place_scatter(int n, const int2* xy, const uint8_t* heading, const u
 // --------------------------------------------------------- S1: binning
 // Counting sort of the live pedestrians into 32 x 32-su bins, read off the
 // per-su occupancy-class grid so that the order inside a bin is row-major
-// and therefore deterministic.  One warp covers 4 bins side by side (128
-// columns of a 128-byte-pitched grid, 4 bytes per lane) for 32 rows; lanes
-// 8b..8b+7 cover bin b.
+// and therefore deterministic; one warp a bin.
+constexpr int kBinWarps = 4;  // bins a block: small blocks spread a small lattice's bins over the SMs
+
 __global__ void k_bin_count(Geo g, const uint8_t* __restrict__ ocls, int32_t* __restrict__ count) {
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int ngx = (g.nbx + 3) >> 2;
-  if (wid >= ngx * g.nby) return;
-  bin_count_group(g, ocls, count, wid % ngx, wid / ngx, threadIdx.x & 31);
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (b >= g.nbx * g.nby) return;
+  const int c = bin_count_one(g, ocls, b % g.nbx, b / g.nbx, lane);
+  if (lane == 0) count[b] = c;
 }
 
 __global__ void k_bin_fill(Geo g, const uint8_t* __restrict__ ocls, const int32_t* __restrict__ occ,
                            const int32_t* __restrict__ start, uint32_t* __restrict__ rec,
                            int32_t* __restrict__ rec_id) {
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int ngx = (g.nbx + 3) >> 2;
-  if (wid >= ngx * g.nby) return;
-  bin_fill_group(g, ocls, occ, start, rec, rec_id, wid % ngx, wid / ngx, threadIdx.x & 31);
+  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (b >= g.nbx * g.nby) return;
+  bin_fill_one(g, ocls, occ, start[b], rec, rec_id, b % g.nbx, b / g.nbx, threadIdx.x & 31);
 }
 
 void launch_bin_count(const Geo& g, const uint8_t* ocls, int32_t* count, cudaStream_t s) {
-  const int nw = ((g.nbx + 3) >> 2) * g.nby;
-  k_bin_count<<<cdiv(nw * 32, 256), 256, 0, s>>>(g, ocls, count);
+  k_bin_count<<<cdiv(g.nbx * g.nby, kBinWarps), 32 * kBinWarps, 0, s>>>(g, ocls, count);
 }
 
 void launch_bin_fill(const Geo& g, const uint8_t* ocls, const int32_t* occ, const int32_t* start,
                      uint32_t* rec, int32_t* rec_id, cudaStream_t s) {
-  const int nw = ((g.nbx + 3) >> 2) * g.nby;
-  k_bin_fill<<<cdiv(nw * 32, 256), 256, 0, s>>>(g, ocls, occ, start, rec, rec_id);
+  k_bin_fill<<<cdiv(g.nbx * g.nby, kBinWarps), 32 * kBinWarps, 0, s>>>(g, ocls, occ, start, rec, rec_id);
 }
 
 // The same records driven by the pedestrian list, for sparse crowds where
