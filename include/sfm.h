@@ -272,6 +272,17 @@ sfm_status sfm_set_binning(sfm_ctx* ctx, int32_t mode);
  * the class-table gather (r > 50). */
 sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);
 
+/* How the field of a crowded lattice is summed.  0 (the default): by the
+ * context's own crowd -- from 9 pedestrians of the last placement on 20 su
+ * the field is a matrix product whose sums are exact (radius 1..44; laws
+ * whose range over the window fits its fixed-point tables), rounded once;
+ * below that, a gather of FP32 sums.  Both lie within the field's error
+ * bound, the product closer, so they may differ in the last bits.  1: always
+ * the gather, 2: the product at any density where it can serve the radius.
+ * For a context that is one band of a larger lattice and has to round as the
+ * whole does.  Kept across placements.  Anything else is SFM_EINVAL. */
+sfm_status sfm_set_field_rule(sfm_ctx* ctx, int32_t mode);
+
 /* Wait for the context's stream and report device-side errors. */
 sfm_status sfm_sync(sfm_ctx* ctx);
 

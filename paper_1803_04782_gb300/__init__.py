@@ -33,7 +33,7 @@ EXPORTS = [
     "sfm_set_time", "sfm_step", "sfm_compute_field", "sfm_sync", "sfm_read_field",
     "sfm_compute_field_into", "sfm_read_static_field", "sfm_read_guidance", "sfm_read_peds",
     "sfm_read_decisions", "sfm_stats", "sfm_set_timing", "sfm_stage_times",
-    "sfm_autotune", "sfm_set_field_footprint", "sfm_set_binning", "sfm_set_walk_periods",
+    "sfm_autotune", "sfm_set_field_footprint", "sfm_set_field_rule", "sfm_set_binning", "sfm_set_walk_periods",
     "sfm_place_sized", "sfm_snapshot", "sfm_restore", "sfm_set_ids", "sfm_set_guidance", "sfm_field_noalloc", "sfm_batch_create", "sfm_batch_place", "sfm_batch_offsets",
     "sfm_batch_autotune", "sfm_batch_test_missing_ctas", "sfm_surrogate_nparams",
     "sfm_surrogate_create", "sfm_surrogate_destroy", "sfm_surrogate_last_error",
@@ -118,6 +118,7 @@ def lib():
             "sfm_set_timing": (C.c_int, [P, I32]),
             "sfm_autotune": (C.c_int, [P, P]),
             "sfm_set_field_footprint": (C.c_int, [P, I32]),
+            "sfm_set_field_rule": (C.c_int, [P, I32]),
             "sfm_set_binning": (C.c_int, [P, I32]),
             "sfm_set_walk_periods": (C.c_int, [P, P, P, I32]),
             "sfm_set_ids": (C.c_int, [P, P, I32]),
@@ -569,6 +570,10 @@ class Sim:
 
     def set_footprint(self, shape: str):
         _check(self.ctx, lib().sfm_set_field_footprint(self.ctx, FOOTPRINTS.index(shape)))
+
+    def set_field_rule(self, rule: str):
+        """"auto" (by the crowd's density), "gather" or "product" (sfm_set_field_rule)."""
+        _check(self.ctx, lib().sfm_set_field_rule(self.ctx, ("auto", "gather", "product").index(rule)))
 
     def set_timing(self, every=True):
         """Stage events on every ``every``-th tick (True: every tick; False: off)."""

@@ -89,6 +89,7 @@ class BandLayout:
             raise ValueError(f"a periodic lattice is split only when its height is a multiple of {BIN}")
         self.H, self.py, self.r, self.nranks = int(H), int(periodic_y), int(r), int(nranks)
         self.h = self.r + HALO_EXTRA
+        self.crowd = None  # pedestrians of the whole lattice, as own_of last saw them
         units = -(-self.H // BIN)
         if units < nranks:
             raise ValueError(f"{H} rows give fewer than {nranks} bands of {BIN} rows")
@@ -150,7 +151,10 @@ class BandLayout:
 
 
 def own_of(layout: BandLayout, k: int, peds: Peds) -> Peds:
-    """The pedestrians of a whole-lattice set that rank k owns."""
+    """The pedestrians of a whole-lattice set that rank k owns.  The layout
+    keeps the set's size: it decides how the whole lattice's field is summed
+    (sfm_set_field_rule), and the bands must round alike."""
+    layout.crowd = peds.n
     return peds.take(layout.owner(peds.xy[:, 1]) == k)
 
 
@@ -231,6 +235,8 @@ def sim_stepper(layout: BandLayout, k: int, W: int, periodic_x: int, cell: np.nd
     sim.set_guidance(np.ascontiguousarray(D[rows], np.int32))
 
     def step(xy, heading, goal, ids, t):
+        crowded = layout.crowd is not None and 20 * layout.crowd >= 9 * W * layout.H
+        sim.set_field_rule("product" if crowded else "gather")
         sim.place(xy, heading, goal)
         sim.set_ids(ids)
         sim.set_time(t)

@@ -118,33 +118,37 @@ sfm_status check_flags(sfm_ctx* ctx) {
 // Field of the current pedestrian state for lattice rows [ya, yb) stored in
 // out with row ya at out row `main_off`; optionally the single halo rows
 // ya-1 and yb (wrapped in periodic y) at out rows 0 and yb-ya+1.  Uses whole
-// tiles so every su is summed in the same order in every mode.
+// tiles so every su is summed in the same order in every mode.  A crowded
+// lattice's rows come from the product, whose sums are exact.
+void launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int ring = 0) {
+  if (c->use_product()) {
+    ProductArgs a = c->prod;
+    a.out = out;
+    a.out_row0 = out_row0;
+    a.store_lo = lo;
+    a.store_hi = hi;
+    a.ring = ring;
+    launch_product(a, c->stream);
+  } else {
+    launch_field(c->geo, c->bin_start, c->rec, c->tables(), c->Fs, out, out_row0, lo, hi, c->ctr,
+                 c->stream, FarPart(), ring);
+  }
+  ++c->launches;
+}
+
 void field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos) {
   const Geo& g = c->geo;
-  const Tables tb = c->tables();
   if (!halos) {
-    launch_field(g, c->bin_start, c->rec, tb, c->Fs, out, ya - main_off, ya, yb, c->ctr,
-                 c->stream);
-    ++c->launches;
+    launch_field_of(c, out, ya - main_off, ya, yb);
     return;
   }
   // one launch for the band and its in-lattice halo rows ya-1 and yb (out rows
   // 0 and yb-ya+1 follow from the same row mapping, main_off == 1)
   const int lo = ya - 1 >= 0 ? ya - 1 : 0, hi = yb + 1 <= g.H ? yb + 1 : g.H;
-  launch_field(g, c->bin_start, c->rec, tb, c->Fs, out, ya - main_off, lo, hi, c->ctr,
-               c->stream);
-  ++c->launches;
+  launch_field_of(c, out, ya - main_off, lo, hi);
   // halo rows that wrap around a periodic y boundary
-  if (g.py && ya == 0) {
-    launch_field(g, c->bin_start, c->rec, tb, c->Fs, out, g.H - 1, g.H - 1, g.H, c->ctr,
-                 c->stream);
-    ++c->launches;
-  }
-  if (g.py && yb == g.H) {
-    launch_field(g, c->bin_start, c->rec, tb, c->Fs, out, -(yb - ya + 1), 0, 1, c->ctr,
-                 c->stream);
-    ++c->launches;
-  }
+  if (g.py && ya == 0) launch_field_of(c, out, g.H - 1, g.H - 1, g.H);
+  if (g.py && yb == g.H) launch_field_of(c, out, -(yb - ya + 1), 0, 1);
 }
 
 // Pedestrian-list binning when the crowd is sparse: its cost follows the
@@ -209,9 +213,7 @@ void run_tick(sfm_ctx* c) {
       const int s_hi = yb + kTile < g.H ? yb + kTile : g.H;
       if (s_hi > s_lo) {
         StageScope sc(c, SFM_STAGE_FIELD);
-        launch_field(g, c->bin_start, c->rec, tb, c->Fs, c->band_buf, s_lo - s_lo % R, s_lo, s_hi,
-                     c->ctr, c->stream, FarPart(), R);
-        ++c->launches;
+        launch_field_of(c, c->band_buf, s_lo - s_lo % R, s_lo, s_hi, R);
       }
       const int y_lo = ya > 0 ? ya - 1 : 0, y_hi = yb + 1 < g.H ? yb + 1 : g.H;
       StageScope sc(c, SFM_STAGE_DECIDE);
@@ -417,6 +419,49 @@ void* device_view(const void* p, int on_device) {
     return nullptr;
   }
   return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+}
+
+// Limb tables and split-tile sums of the product, made when a crowd first
+// asks for it.  Where the law's range does not fit the fixed-point form, or
+// the workspace cannot be had, the gathers go on serving the lattice.
+void ensure_product(sfm_ctx* c) {
+  const Geo& g = c->geo;
+  if (c->product_tried || !c->wants_product()) return;
+  c->product_tried = true;
+  ProductScales sc;
+  if (!product_crowd_scales(g.r, c->prm, &sc)) return;
+  ProductArgs a;
+  // tiles of one launch that may be split: fewer than CTAs
+  const size_t split = (size_t)std::min(product_tiles_x(g.W) * product_tiles_y(g.H), device_sm_count());
+  uint8_t* tab = nullptr;
+  const std::string err = c->err;
+  if (dalloc(c, &tab, product_table_bytes(g.r, 5)) != SFM_OK || dalloc(c, &a.tick, split) != SFM_OK ||
+      dalloc(c, &a.scratch, product_scratch_floats() * split) != SFM_OK) {
+    cudaGetLastError();
+    c->err = err;
+    dfree(c, tab);
+    dfree(c, a.tick);
+    return;
+  }
+  cudaMemsetAsync(a.tick, 0, split * sizeof(int), c->stream);
+  cudaMemsetAsync(a.scratch, 0, product_scratch_floats() * split * sizeof(float), c->stream);
+  launch_limb_tables(g.r, c->prm, sc, 5, tab, c->stream);
+  ++c->launches;
+  a.ctr = c->ctr;
+  a.one.src = c->ocls;
+  a.one.spitch = g.opitch;
+  a.one.Fs = c->Fs;
+  a.one.tab = tab;
+  a.one.W = g.W;
+  a.one.H = g.H;
+  a.one.px = g.px;
+  a.one.py = g.py;
+  a.one.r = g.r;
+  a.one.ntx = product_tiles_x(g.W);
+  a.one.c0 = (float)(1.0 / sc.s0);
+  a.one.c1 = (float)(1.0 / (sc.s0 * sc.s1));
+  product_layout(g.r, &a);
+  c->prod = a;
 }
 
 sfm_status copy_out(sfm_ctx* ctx, void* dst, const void* src, size_t bytes, int on_device) {
@@ -769,6 +814,7 @@ static sfm_status place_impl(sfm_ctx* ctx, int32_t n, const int32_t* xy, const u
   ctx->walk_periods = false;  // a placement starts with every pedestrian active
   ctx->has_ids = false;       // and numbers its pedestrians by index
   ctx->n = n;
+  ensure_product(ctx);
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (n > 0 && !direct) {
     CU(cudaMemcpyAsync(ctx->xy, xy, (size_t)n * sizeof(int2), kind, s));
@@ -1071,6 +1117,18 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape) {
     return fail(ctx, SFM_EINVAL, "footprint must be 0, 1 or 2");
   if (ctx->field_shape != shape) {
     ctx->field_shape = shape;
+    drop_graph(ctx);
+  }
+  return SFM_OK;
+}
+
+sfm_status sfm_set_field_rule(sfm_ctx* ctx, int32_t mode) {
+  if (!ctx) return SFM_EINVAL;
+  if (ctx->batch) return fail(ctx, SFM_EINVAL, "a batch judges each lattice by its own crowd");
+  if (mode < 0 || mode > 2) return fail(ctx, SFM_EINVAL, "field rule must be 0, 1 or 2");
+  if (ctx->field_rule != mode) {
+    ctx->field_rule = mode;
+    ensure_product(ctx);
     drop_graph(ctx);
   }
   return SFM_OK;

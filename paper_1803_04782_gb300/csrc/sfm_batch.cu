@@ -97,6 +97,15 @@ struct BatchState {
   int missing = 0;  // test hook: CTAs the barrier expects beyond those launched
   int grid = 0;
   std::vector<int> order;  // lattices by decreasing field cost
+  // lattices whose crowd of the last placement is summed by the product, in a
+  // launch ahead of the tick's (they have no chunks then); their limb tables
+  std::vector<uint8_t> crowded;
+  std::vector<uint8_t*> tabs;
+  std::vector<sfm_params> prms;
+  ProductLattice* plat = nullptr;
+  int2* tiles = nullptr;
+  int tiles_cap = 0;
+  ProductArgs prod;
   cudaGraphExec_t graph = nullptr;
   int graph_field_only = -1;
 };
@@ -295,7 +304,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_tick_batch(BatchArgs a) {
   for (int w = gwarp; w < a.total_bins; w += nwarps) {
     const BatchScene& sc = a.scenes[a.bin_scene[w]];
     const int b = w - sc.bin_off;
-    bin_fill_one(sc.g, a.ocls + sc.ocls_off, a.occ + sc.su_off, a.bin_start[w], a.rec, a.rec_id,
+    bin_fill_one<8>(sc.g, a.ocls + sc.ocls_off, a.occ + sc.su_off, a.bin_start[w], a.rec, a.rec_id,
                  b % sc.g.nbx, b / sc.g.nbx, lane);
   }
   if (!grid_sync(a.bar, a.expect_blocks, a.ctr)) return;
@@ -446,7 +455,7 @@ void build_chunks(BatchState* B, std::vector<BatchChunk>& out, int only_sp) {
   out.clear();
   for (int s : B->order) {
     const BatchScene& sc = B->hs[s];
-    if (only_sp > 0 && sc.sp != only_sp) continue;
+    if ((only_sp > 0 && sc.sp != only_sp) || B->crowded[s]) continue;
     const int shape = B->shape_of_sp[class_of_stride(sc.sp)];
     const int nf = shape_nf(sc.g, shape);
     for (int f0 = 0; f0 < nf; f0 += 32) out.push_back(BatchChunk{s, f0, shape, 0});
@@ -510,8 +519,100 @@ size_t batch_smem(const BatchState* B) {
          (size_t)kBatchThreads / 32 * 32 * sizeof(int2);
 }
 
+// The product's share of the batch for the crowds just placed (as
+// ensure_product in sfm_api.cu does for one context): limb tables, one for
+// each radius and law in use, the lattices' descriptions and the tile list.
+// A lattice that cannot be served stays with the gathers.
+sfm_status setup_product(sfm_ctx* ctx) {
+  BatchState* B = ctx->batch;
+  cudaStream_t s = ctx->stream;
+  const int ns = B->nscenes;
+  B->crowded.assign(ns, 0);
+  B->prod.ntiles = 0;
+  std::vector<ProductLattice> pl(ns);
+  std::vector<int> who;
+  int rmax = 0, tiles = 0;
+  for (int i = 0; i < ns; ++i) {
+    const BatchScene& sc = B->hs[i];
+    const Geo& g = sc.g;
+    const sfm_params& p = B->prms[i];
+    ProductScales w;
+    if (!lattice_crowded(g.W, g.H, sc.n) || !product_crowd_scales(g.r, p, &w)) continue;
+    for (int k = 0; k < ns && !B->tabs[i]; ++k) {
+      const sfm_params& q = B->prms[k];
+      if (B->tabs[k] && q.r == p.r && q.kP == p.kP && q.aP == p.aP && q.gamma == p.gamma) B->tabs[i] = B->tabs[k];
+    }
+    if (!B->tabs[i]) {
+      uint8_t* t = nullptr;
+      if (balloc(ctx, &t, product_table_bytes(g.r, 5)) != SFM_OK) {
+        cudaGetLastError();
+        continue;
+      }
+      launch_limb_tables(g.r, p, w, 5, t, s);
+      ctx->launches += 1;
+      B->tabs[i] = t;
+    }
+    ProductLattice& l = pl[i];
+    l.src = ctx->ocls + sc.ocls_off;
+    l.spitch = g.opitch;
+    l.Fs = ctx->Fs + sc.su_off;
+    l.out = ctx->F + sc.su_off;
+    l.tab = B->tabs[i];
+    l.W = g.W;
+    l.H = g.H;
+    l.px = g.px;
+    l.py = g.py;
+    l.r = g.r;
+    l.ntx = product_tiles_x(g.W);
+    l.c0 = (float)(1.0 / w.s0);
+    l.c1 = (float)(1.0 / (w.s0 * w.s1));
+    who.push_back(i);
+    rmax = std::max(rmax, g.r);
+    tiles += l.ntx * product_tiles_y(g.H);
+  }
+  if (!tiles) return SFM_OK;
+  if (!B->prod.scratch) {
+    const size_t split = (size_t)device_sm_count();
+    ProductArgs a;
+    if (balloc(ctx, &B->plat, (size_t)ns) != SFM_OK || balloc(ctx, &a.tick, split) != SFM_OK ||
+        balloc(ctx, &a.scratch, product_scratch_floats() * split) != SFM_OK) {
+      cudaGetLastError();
+      return SFM_OK;
+    }
+    BCU(cudaMemsetAsync(a.tick, 0, split * sizeof(int), s));
+    BCU(cudaMemsetAsync(a.scratch, 0, product_scratch_floats() * split * sizeof(float), s));
+    B->prod = a;
+  }
+  if (tiles > B->tiles_cap) {
+    if (balloc(ctx, &B->tiles, (size_t)tiles) != SFM_OK) {
+      cudaGetLastError();
+      return SFM_OK;
+    }
+    B->tiles_cap = tiles;
+  }
+  std::stable_sort(who.begin(), who.end(), [&](int a, int b) { return B->hs[a].g.r > B->hs[b].g.r; });
+  std::vector<int2> list;
+  for (int i : who) {
+    B->crowded[i] = 1;
+    for (int t = 0; t < pl[i].ntx * product_tiles_y(pl[i].H); ++t) list.push_back(make_int2(i, t));
+  }
+  BCU(cudaMemcpyAsync(B->plat, pl.data(), pl.size() * sizeof(ProductLattice), cudaMemcpyHostToDevice, s));
+  BCU(cudaMemcpyAsync(B->tiles, list.data(), list.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  BCU(cudaStreamSynchronize(s));  // the host arrays are gone after this
+  ProductArgs& a = B->prod;
+  product_layout(rmax, &a);
+  a.lattices = B->plat;
+  a.tiles = B->tiles;
+  a.ntiles = tiles;
+  a.store_lo = 0;
+  a.store_hi = INT32_MAX;
+  a.ctr = ctx->ctr;
+  return SFM_OK;
+}
+
 cudaError_t launch_tick(sfm_ctx* ctx, int field_only, cudaStream_t s) {
   BatchState* B = ctx->batch;
+  if (B->prod.ntiles) launch_product(B->prod, s);
   BatchArgs a = make_args(ctx, field_only);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(B->grid);
@@ -597,7 +698,7 @@ sfm_status batch_tick(sfm_ctx* ctx, int nsteps, int field_only) {
     } else {
       BCU(cudaGraphLaunch(B->graph, ctx->stream));
     }
-    ctx->launches += 1;
+    ctx->launches += B->prod.ntiles ? 2 : 1;
     if (!field_only) ++ctx->t;
   }
   if (ctx->timing && !field_only) ctx->timed_ticks += nsteps;
@@ -633,6 +734,9 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
   ctx->batch = new BatchState;
   BatchState* B = ctx->batch;
   B->nscenes = nscenes;
+  B->prms.assign(prms, prms + nscenes);
+  B->tabs.assign(nscenes, nullptr);
+  B->crowded.assign(nscenes, 0);
   ctx->stream = static_cast<cudaStream_t>(stream);
   ctx->lat = lats[0];
   ctx->prm = prms[0];
@@ -888,6 +992,7 @@ sfm_status sfm_batch_place(sfm_ctx* ctx, const int32_t* counts, const int32_t* x
     }
     std::stable_sort(B->order.begin(), B->order.end(),
                      [&](int a, int b) { return cost[a] > cost[b]; });
+    BTRY(setup_product(ctx));
     std::vector<BatchChunk> v;
     build_chunks(B, v, 0);
     BTRY(upload_chunks(ctx, v));

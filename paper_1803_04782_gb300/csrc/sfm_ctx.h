@@ -57,6 +57,11 @@ struct sfm_ctx {
   uint32_t* bin_key = nullptr;  // pedestrian-list binning: su keys in slot order
   int binning = 0;              // 0 automatic, 1 class grid, 2 pedestrian list
   sfm::Counters* ctr = nullptr;
+  // the tensor-core product of a crowded lattice (made by the first placement
+  // that needs it; smem_bytes == 0: not there) and sfm_set_field_rule's mode
+  sfm::ProductArgs prod;
+  bool product_tried = false;
+  int field_rule = 0;
   // pedestrians
   int n = 0, cap = 0;
   int2* xy = nullptr;
@@ -133,6 +138,10 @@ struct sfm_ctx {
     }
     return sz;
   }
+  bool wants_product() const {
+    return field_rule == 2 || (field_rule == 0 && sfm::lattice_crowded(geo.W, geo.H, n));
+  }
+  bool use_product() const { return prod.smem_bytes && wants_product(); }
   const int32_t* ids() const { return has_ids ? gid : nullptr; }
   sfm::WalkPeriods walk() const {
     sfm::WalkPeriods wp;

@@ -139,6 +139,9 @@ __device__ __forceinline__ int bin_count_one(const Geo& g, const uint8_t* __rest
 // row loop in which each row's offset followed the last row's took 34 us for
 // the 16 bins of a 100 x 100 lattice (one-pass ncu, cold) against 6.5 us here (a
 // 1000 x 1000 lattice half full: 37.7 us, now 7.9).
+// ROWS rows' reads are in flight together (the batched tick, which has few
+// registers to spare, takes 8).
+template <int ROWS = 16>
 __device__ __forceinline__ void bin_fill_one(const Geo& g, const uint8_t* __restrict__ ocls,
                                              const int32_t* __restrict__ occ, int first,
                                              uint32_t* __restrict__ rec,
@@ -154,13 +157,12 @@ __device__ __forceinline__ void bin_fill_one(const Geo& g, const uint8_t* __rest
   const int off = first + inc - __popc(mine);
   const int x = bx * kBin + lane;
   const uint32_t lt = (1u << lane) - 1u;
-  constexpr int kRows = 16;  // rows whose reads are in flight together
 #pragma unroll 1
-  for (int r0 = 0; r0 < kBin; r0 += kRows) {
-    uint32_t cls[kRows];
-    int32_t id[kRows];
+  for (int r0 = 0; r0 < kBin; r0 += ROWS) {
+    uint32_t cls[ROWS];
+    int32_t id[ROWS];
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) {
+    for (int j = 0; j < ROWS; ++j) {
       const uint32_t m = __shfl_sync(0xffffffffu, mine, r0 + j);
       const size_t y = (size_t)(by * kBin + r0 + j);
       cls[j] = 0u;
@@ -171,7 +173,7 @@ __device__ __forceinline__ void bin_fill_one(const Geo& g, const uint8_t* __rest
       }
     }
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) {
+    for (int j = 0; j < ROWS; ++j) {
       const uint32_t m = __shfl_sync(0xffffffffu, mine, r0 + j);
       const int k = __shfl_sync(0xffffffffu, off, r0 + j) + __popc(m & lt);
       if (cls[j]) {

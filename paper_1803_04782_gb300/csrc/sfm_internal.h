@@ -173,6 +173,61 @@ inline int default_field_shape(int r) {
   return r > 30 ? (field3_stride(r) ? kShape32x32 : kShape32x16) : kShape16x16;
 }
 
+// ---- crowded lattices (sfm_product.cu) ----
+// Largest radius of the tensor-core product: with 11-bit limbs the sums over
+// a full window of (2r + 1)^2 - 1 su stay below 2^24, and a plane and two
+// table stages fit in shared memory.
+constexpr int kProductMaxRadius = 44;
+// A lattice is crowded, and its field summed by the product and not by a
+// gather, from 9 pedestrians on 20 su.  The product is the faster way from
+// far fewer (its time does not depend on the crowd: at radius 38 a 1000 x
+// 1000 lattice half full takes 1298 us by the gather, 168 by the product, and
+// at radius 3 70 and 30, one-pass ncu), but the two round differently,
+// and in a run of many ticks one decision in 10^5 that falls the other way
+// moves its neighbours: the line lies above the room, corridor and batch
+// workloads (at most 2 su in 5), whose runs stay bit for bit what they were.
+inline bool lattice_crowded(int W, int H, int64_t n) { return 20 * n >= 9 * (int64_t)W * H; }
+
+// One lattice of a product launch: the source bytes (class grid or cell
+// grid), the limb tables of its radius, and where the sums go.
+struct ProductLattice {
+  const uint8_t* src = nullptr;
+  const float* Fs = nullptr;   // added to the sum (NULL: nothing)
+  float* out = nullptr;        // W x H field (a launch may give its own)
+  const uint8_t* tab = nullptr;
+  int W = 0, H = 0, px = 0, py = 0, r = 0;
+  int spitch = 0;  // bytes of a source row
+  int ntx = 0;     // tiles a row
+  float c0 = 0.f, c1 = 0.f;  // weights of the two limbs' sums
+};
+struct ProductArgs {
+  ProductLattice one;                        // the lattice, when `lattices` is NULL
+  const ProductLattice* lattices = nullptr;  // a batch's
+  const int2* tiles = nullptr;               // a batch's tiles (lattice, tile), costly ones first
+  int tile0 = 0, ntiles = 0;  // of `one`: set by launch_product from the rows to store
+  int nch = 5;                // planes: 5 of a crowd, 2 of a cell grid
+  float* scratch = nullptr;   // sums of split tiles, product_scratch_floats() a tile, zero between launches
+  int* tick = nullptr;        // arrivals of each split tile, zero between launches
+  float* out = nullptr;       // overrides the lattice's own
+  int out_row0 = 0, store_lo = 0, store_hi = 0, ring = 0;  // as launch_field's
+  int plane_bytes = 0, stage_bytes = 0, nplanes = 0, nstages = 0, smem_bytes = 0;
+  Counters* ctr = nullptr;
+};
+// Fixed-point scales of the limb tables: T = L0 / s0 + L1 / (s0 s1).  false:
+// the law's range over the window is too wide for them.
+struct ProductScales {
+  double s0 = 0.0, s1 = 0.0;
+};
+bool product_crowd_scales(int r, const sfm_params& p, ProductScales* out);
+size_t product_table_bytes(int r, int nch);
+void launch_limb_tables(int r, const sfm_params& p, const ProductScales& sc, int nch, uint8_t* tab,
+                        cudaStream_t s);
+void product_layout(int rmax, ProductArgs* a);  // shared-memory split for radii up to rmax
+int product_tiles_x(int W);
+int product_tiles_y(int H);
+size_t product_scratch_floats();
+void launch_product(ProductArgs a, cudaStream_t s);
+
 // ---- launchers (sfm_kernels.cu) ----
 void launch_tables(int r, const sfm_params& p, float* T0, float* TX, float* TY, float* KO,
                    float* KE, float* own, float* dirdot, float2* hvec, cudaStream_t s);

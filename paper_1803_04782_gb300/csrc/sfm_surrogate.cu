@@ -1172,12 +1172,13 @@ __global__ void __launch_bounds__(kFbThreads, 1)
                    const uint32_t* __restrict__ rec, const float* __restrict__ CT, int TS,
                    const float* __restrict__ Fs, const int32_t* __restrict__ fb_dd,
                    const uint32_t* __restrict__ fb_info, float beta, const float* __restrict__ own,
-                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice) {
+                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
+                   const float* __restrict__ Fx) {
   extern __shared__ __align__(16) float sm[];
   float* sT = sm + kTableGuard;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int2* scr = reinterpret_cast<int2*>(sT + 4 * TS) + w * 32;
-  copy_to_shared<8>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
+  if (!Fx) copy_to_shared<8>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
   __syncthreads();
   const int nrec = bin_start[nbins], r = g.r;
   const int nchunks = (nrec + 31) / 32;
@@ -1186,6 +1187,7 @@ __global__ void __launch_bounds__(kFbThreads, 1)
     const bool fl = i < nrec && fb_flag[i] != 0;
     unsigned todo = __ballot_sync(0xffffffffu, fl);
     if (!todo) continue;
+    if (Fx) todo = 0;  // the exact lattice field is at hand: nothing to sum
     const int2 q = fl ? xy[rec_id[i]] : make_int2(0, 0);
     const int brow = q.y / kBin, bcol = q.x / kBin;
     float acc[9];
@@ -1256,7 +1258,8 @@ __global__ void __launch_bounds__(kFbThreads, 1)
         int tx, ty;
         const bool ok = wrap_coord(q.x + move_dx(k), g.W, g.px, tx) &
                         wrap_coord(q.y + move_dy(k), g.H, g.py, ty);
-        f[k] = ok ? Fs[(size_t)ty * g.W + tx] + acc[k] : 0.f;
+        const size_t c = (size_t)ty * g.W + tx;
+        f[k] = ok ? (Fx ? Fx[c] : Fs[c] + acc[k]) : 0.f;
         dd[k] = fb_dd[(size_t)i * 9 + k];
         oc[k] = (info >> k) & 1u ? 0 : 1;  // admissible iff its mask bit is set
       }
@@ -1823,7 +1826,7 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
                       (size_t)kFbThreads / 32 * 32 * sizeof(int2);
   void (*fb)(const uint8_t*, const int32_t*, int, Geo, const int2*, const int32_t*, const uint32_t*,
              const float*, int, const float*, const int32_t*, const uint32_t*, float, const float*,
-             const float*, uint8_t*);
+             const float*, uint8_t*, const float*);
   switch (SP) {
     case 34: fb = k_sur_fallback<34>; break;
     case 50: fb = k_sur_fallback<50>; break;
@@ -1834,12 +1837,19 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
     default: fb = k_sur_fallback<kNarrowStride>; break;
   }
   cudaFuncSetAttribute(fb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // a crowded lattice's exact field is the product's, on the whole lattice
+  // (Fnear is free outside training)
+  const float* Fx = nullptr;
+  if (ctx->use_product()) {
+    ctx_field_rows(ctx, S->Fnear, 0, g.H, 0, false);
+    Fx = S->Fnear;
+  }
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   fb<<<nsm > 0 ? nsm : 1, kFbThreads, smem, st>>>(
       S->fb_flag, ctx->rec_id, nbins, g, ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs,
-      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice);
+      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice, Fx);
 }
 
 void round_params(sfm_surrogate* S) {

@@ -1,0 +1,129 @@
+"""Crowded lattices (9 pedestrians on 20 su and more), whose field the
+tensor-core product sums: against the FP64 oracle at the edges of its tiles,
+radii and alignments, closed and periodic; closer to it than the gather; and
+bit for bit the same in bands, in a batch and at the candidates only."""
+import numpy as np
+import pytest
+
+import paper_1803_04782_gb300 as sfm
+import scenegen as SG
+from paper_1803_04782_gb300 import build as B
+from parity import OracleRun, assert_field
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+    sfm.lib()
+
+
+def _crowd(W, H, r, px=1, py=1, rho=0.5, seed=0, **kw):
+    free = (W - (0 if px else 2)) * (H - (0 if py else 2))
+    return SG.random_scene(W, H, int(rho * free), r=r, seed=300 + seed + r, periodic_x=px, periodic_y=py,
+                           ring=not (px and py), exits=() if (px and py) else ("east",),
+                           goal_mode="fixed" if (px and py) else "mixed", heading_mode="random", **kw)
+
+
+@pytest.mark.parametrize("W,H,r,px,py", [(64, 256, 3, 1, 1), (65, 257, 3, 0, 0), (127, 255, 9, 1, 0),
+                                         (130, 300, 20, 0, 1), (7, 300, 3, 1, 0), (89, 89, 44, 1, 1),
+                                         (200, 130, 38, 0, 0), (33, 40, 1, 1, 1)])
+def test_product_field_against_the_oracle_and_the_gather(W, H, r, px, py):
+    sc = _crowd(W, H, r, px, py, rho=0.6)
+    assert 20 * sc.n >= 9 * W * H
+    orc = OracleRun(sc)
+    Fo, So = orc.field()
+    with sfm.Sim(sc) as a, sfm.Sim(sc) as b:
+        b.set_field_rule("gather")
+        for s in (a, b):
+            s.compute_field()
+        Fa, Fb = a.field(), b.field()
+        assert_field(Fa, Fo, So)
+        # the product's sums are exact (its entries are off by 2^-24 of the
+        # law's largest, its result by one rounding): no further off than FP32 sums
+        err = [np.linalg.norm(F - Fo) / np.linalg.norm(Fo) for F in (Fa, Fb)]
+        assert err[0] <= max(err[1], 6e-8) and not np.array_equal(Fa, Fb)
+        a.compute_field()
+        np.testing.assert_array_equal(a.field(), Fa)  # the split tiles' sums are zero again
+        # the rule holds for any crowd when it is asked for
+        b.set_field_rule("product")
+        b.place(sc.xy[:40], sc.heading[:40], sc.goal[:40])
+        b.compute_field()
+        assert_field(b.field(), *_field_of(sc, 40))
+        with pytest.raises(sfm.SfmError) as e:
+            sfm._check(a.ctx, sfm.lib().sfm_set_field_rule(a.ctx, 3))
+        assert e.value.status == sfm.SFM_EINVAL
+
+
+def _field_of(sc, n):
+    part = sc.copy()
+    part.xy, part.heading, part.goal = sc.xy[:n].copy(), sc.heading[:n].copy(), sc.goal[:n].copy()
+    return OracleRun(part).field()
+
+
+@pytest.mark.parametrize("px,py,r,rows", [(0, 0, 36, 64), (1, 1, 36, 96), (1, 0, 5, 32)])
+def test_bands_batch_and_candidates_round_as_one_launch(px, py, r, rows):
+    sc = _crowd(150, 256, r, px, py, rho=0.55, seed=7)
+    budget = sfm.band_budget(sc.W, sc.H, rows, px, py)
+    init = np.zeros(int(sfm.lib().sfm_surrogate_nparams()), np.float32)
+    even = _crowd(144, 256, r, px, py, rho=0.55, seed=8)  # the candidates want a multiple of their cells
+    with sfm.Sim(sc) as a, sfm.Sim(sc, hbm_budget_bytes=budget) as b, sfm.Batch([sc, even]) as c, \
+            sfm.Sim(even) as d, sfm.Sim(even) as e, sfm.Surrogate(coarsen=4, params=init) as sur:
+        assert b.stats()["bands"] > 1
+        if r == 36:
+            b.set_footprint("32x32r")  # with closed y: the ring of rows
+        a.compute_field()
+        np.testing.assert_array_equal(a.field(), b.field_banded())
+        c.compute_field()
+        np.testing.assert_array_equal(a.field(), c.fields()[0])
+        for _ in range(4):
+            for s in (a, b, c, d):
+                s.step(1)
+            sur.step(e, 1)
+            for x, y, z in zip(a.peds(), b.peds(), c.peds()):
+                np.testing.assert_array_equal(x, y)
+                np.testing.assert_array_equal(x, z[0])
+            for x, y, z in zip(d.peds(), e.peds(), c.peds()):
+                np.testing.assert_array_equal(x, y)
+                np.testing.assert_array_equal(x, z[1])
+            np.testing.assert_array_equal(d.decisions()[0], e.decisions()[0])
+        for s in (a, b, c, d, e):
+            assert s.stats()["error_flags"] == 0
+
+
+def test_two_row_bands_round_as_the_whole_lattice():
+    """The stepper of a row-band decomposition sums its field as the whole
+    lattice does, whatever its own rows hold."""
+    from paper_1803_04782_gb300 import bands as BD
+    sc = _crowd(96, 320, 12, 1, 0, rho=0.5, seed=9)
+    sc.xy = sc.xy[np.argsort(sc.xy[:, 1], kind="stable")]  # then thin the upper half out
+    keep = np.flatnonzero((sc.xy[:, 1] < 160) | (np.arange(sc.n) % 10 != 0))
+    sc.xy, sc.heading, sc.goal = sc.xy[keep], sc.heading[keep], sc.goal[keep]
+    assert 20 * sc.n >= 9 * sc.W * sc.H
+    L = BD.BandLayout(sc.H, 0, 12, 2)
+    peds = BD.Peds(np.arange(sc.n, dtype=np.int32), sc.xy, sc.heading, sc.goal)
+    with sfm.Sim(sc) as whole:
+        D = whole.guidance()
+        owned = [BD.own_of(L, k, peds) for k in range(2)]
+        steps = [BD.sim_stepper(L, k, sc.W, 1, sc.cell, D, sc.params) for k in range(2)]
+        for t in range(3):
+            sends = [BD.sends_of(L, k, owned[k]) for k in range(2)]
+
+            class Comm:
+                def __init__(self, k):
+                    self.k = k
+
+                def exchange(self, mine):
+                    return {j: sends[j][self.k].pack() for j in mine}
+            owned = [BD.band_tick(L, k, Comm(k), steps[k][0], owned[k], t)[0] for k in range(2)]
+        whole.step(3)
+        xy, hd, al = whole.peds()
+        for _, sim in steps:
+            sim.close()
+    ids = np.concatenate([o.ids for o in owned])
+    order = np.argsort(ids)
+    live = np.flatnonzero(al)
+    np.testing.assert_array_equal(ids[order], live)
+    np.testing.assert_array_equal(np.concatenate([o.xy for o in owned])[order], xy[live])
+    np.testing.assert_array_equal(np.concatenate([o.heading for o in owned])[order], hd[live])
