@@ -597,7 +597,7 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
   ALLOC(ctx->cell, nsu);
   ALLOC(ctx->Fs, nsu);
   ALLOC(ctx->D, nsu);
-  ALLOC(ctx->occ, nsu);
+  ALLOC(ctx->occ, std::max(nsu, static_tmp_bytes(g.r, ctx->prm) / sizeof(int32_t)));
   ALLOC(ctx->ocls, (size_t)g.opitch * g.H);
   if (ctx->bands <= 1) {
     ALLOC(ctx->F, nsu);
@@ -628,13 +628,14 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
     return bail(SFM_ECUDA);
   }
   cudaMemsetAsync(ctx->ctr, 0, sizeof(Counters), s);
-  cudaMemsetAsync(ctx->occ, 0xff, nsu * sizeof(int32_t), s);
   cudaMemsetAsync(ctx->ocls, 0, (size_t)g.opitch * g.H, s);
   launch_tables(g.r, ctx->prm, ctx->T0, ctx->TX, ctx->TY, ctx->KO, ctx->KE, ctx->own, ctx->dirdot,
                 ctx->hvec, s);
   if (ctx->CT) launch_class_tables(g.r, ctx->prm, ctx->CT, s);
   if (ctx->CT3) launch_class_tables3(g.r, ctx->prm, ctx->CT3, s);
-  launch_static_field(g, ctx->cell, ctx->tables(), ctx->Fs, s);
+  // the occupancy grid is scratch until it is cleared
+  launch_static_field(g, ctx->cell, ctx->tables(), ctx->prm, ctx->Fs, ctx->occ, ctx->ctr, s);
+  cudaMemsetAsync(ctx->occ, 0xff, nsu * sizeof(int32_t), s);
 
   {
     const sfm_status gst = compute_guidance(g, ctx->cell, ctx->D, s, &ctx->err);
@@ -646,6 +647,8 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
     fail(ctx, SFM_ECUDA, "scene set-up: %s", cudaGetErrorString(e));
     return bail(SFM_ECUDA);
   }
+  st = check_flags(ctx);
+  if (st != SFM_OK) return bail(st);
   *out = ctx;
   return SFM_OK;
 }

@@ -790,7 +790,12 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
   BALLOC(ctx->Fs, (size_t)su);
   BALLOC(ctx->F, (size_t)su);
   BALLOC(ctx->D, (size_t)su);
-  BALLOC(ctx->occ, (size_t)su);
+  {
+    // the occupancy grids are the static fields' scratch until they are cleared
+    size_t tmp = 0;
+    for (int i = 0; i < nscenes; ++i) tmp = std::max(tmp, static_tmp_bytes(B->hs[i].g.r, prms[i]));
+    BALLOC(ctx->occ, std::max((size_t)su, tmp / sizeof(int32_t)));
+  }
   BALLOC(ctx->ocls, (size_t)oc);
   BALLOC(B->own, (size_t)81 * nscenes);
   BALLOC(B->dirdot, (size_t)81 * nscenes);
@@ -813,6 +818,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
 #undef BALLOC
   ctx->nsu_total = su;
   cudaStream_t s = ctx->stream;
+  cudaMemsetAsync(ctx->ctr, 0, sizeof(Counters), s);
   // per-lattice tables, static field and guidance (set-up, lattice by lattice)
   int maxS = 1;
   for (const BatchScene& sc : B->hs) maxS = std::max(maxS, 2 * sc.g.r + 1);
@@ -839,14 +845,14 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     Tables tb{};
     tb.KO = KO;
     tb.KE = KE;
-    launch_static_field(sc.g, ctx->cell + sc.su_off, tb, ctx->Fs + sc.su_off, s);
+    launch_static_field(sc.g, ctx->cell + sc.su_off, tb, prms[sidx], ctx->Fs + sc.su_off,
+                        ctx->occ, ctx->ctr, s);
     st = compute_guidance(sc.g, ctx->cell + sc.su_off, ctx->D + sc.su_off, s, &ctx->err);
     if (st != SFM_OK) return bail(st);
     std::fill_n(bs.begin() + sc.bin_off, sc.g.nbx * sc.g.nby, (uint16_t)sidx);
   }
   cudaMemsetAsync(ctx->occ, 0xff, (size_t)su * sizeof(int32_t), s);
   cudaMemsetAsync(ctx->ocls, 0, (size_t)oc, s);
-  cudaMemsetAsync(ctx->ctr, 0, sizeof(Counters), s);
   cudaMemsetAsync(B->bar, 0, sizeof(unsigned int), s);
   cudaMemcpyAsync(B->bin_scene, bs.data(), bs.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(B->scenes, B->hs.data(), B->hs.size() * sizeof(BatchScene), cudaMemcpyHostToDevice,
@@ -873,6 +879,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     ctx->err = std::string("batch set-up: ") + cudaGetErrorString(e);
     return bail(SFM_ECUDA);
   }
+  if ((st = check_batch(ctx)) != SFM_OK) return bail(st);
   *out = ctx;
   return SFM_OK;
 }

@@ -174,9 +174,9 @@ inline int default_field_shape(int r) {
 }
 
 // ---- crowded lattices (sfm_product.cu) ----
-// Largest radius of the tensor-core product: with 11-bit limbs the sums over
-// a full window of (2r + 1)^2 - 1 su stay below 2^24, and a plane and two
-// table stages fit in shared memory.
+// Largest radius of the tensor-core product: the sums over a full window of
+// (2r + 1)^2 - 1 su stay below 2^24 with 23 bits and more to a table entry,
+// and a plane and two table stages fit in shared memory.
 constexpr int kProductMaxRadius = 44;
 // A lattice is crowded, and its field summed by the product and not by a
 // gather, from 9 pedestrians on 20 su.  The product is the faster way from
@@ -206,7 +206,9 @@ struct ProductArgs {
   const int2* tiles = nullptr;               // a batch's tiles (lattice, tile), costly ones first
   int tile0 = 0, ntiles = 0;  // of `one`: set by launch_product from the rows to store
   int nch = 5;                // planes: 5 of a crowd, 2 of a cell grid
-  float* scratch = nullptr;   // sums of split tiles, product_scratch_floats() a tile, zero between launches
+  // sums of split tiles, product_scratch_floats() a tile, zero between
+  // launches (NULL: no tile is split)
+  float* scratch = nullptr;
   int* tick = nullptr;        // arrivals of each split tile, zero between launches
   float* out = nullptr;       // overrides the lattice's own
   int out_row0 = 0, store_lo = 0, store_hi = 0, ring = 0;  // as launch_field's
@@ -219,6 +221,7 @@ struct ProductScales {
   double s0 = 0.0, s1 = 0.0;
 };
 bool product_crowd_scales(int r, const sfm_params& p, ProductScales* out);
+bool product_cell_scales(int r, const sfm_params& p, ProductScales* out);
 size_t product_table_bytes(int r, int nch);
 void launch_limb_tables(int r, const sfm_params& p, const ProductScales& sc, int nch, uint8_t* tab,
                         cudaStream_t s);
@@ -231,8 +234,11 @@ void launch_product(ProductArgs a, cudaStream_t s);
 // ---- launchers (sfm_kernels.cu) ----
 void launch_tables(int r, const sfm_params& p, float* T0, float* TX, float* TY, float* KO,
                    float* KE, float* own, float* dirdot, float2* hvec, cudaStream_t s);
-void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, float* Fs,
-                         cudaStream_t s);
+// tmp: static_tmp_bytes() of device memory, 16-byte aligned, overwritten (limb
+// tables).  ctr: error flags of a bounded wait.
+size_t static_tmp_bytes(int r, const sfm_params& prm);
+void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, const sfm_params& prm,
+                         float* Fs, void* tmp, Counters* ctr, cudaStream_t s);
 // One relaxation round of the guidance distances; returns via *changed.
 void launch_guidance_init(const Geo& g, const uint8_t* cell, int32_t* D, cudaStream_t s);
 void launch_guidance_export(int32_t* D, size_t n, cudaStream_t s);

@@ -117,8 +117,49 @@ __global__ void __launch_bounds__(kFieldThreads)
   }
 }
 
-void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, float* Fs,
-                         cudaStream_t s) {
+// From radius 12 on, the product of the wall and exit planes with the two
+// laws' tables (sfm_product.cu; rounded once, like the compensated sum above).
+// The dense gather reads (2r + 1)^2 cells a su: a 2048 x 2048 floor's field at
+// radius 40 took 7719 us, the product 162 and its tables 32 (one-pass ncu),
+// the whole set-up 10.5 ms against 2.9.  A 100 x 100 lattice is set up in the
+// same time either way at radius 12 (360 us; 372 against 347 at radius 8,
+// where a tile's start costs more than the gather), a 4096 x 4096 one in 6.3
+// ms against 9.2.  The rule looks at the radius and the laws alone, so a
+// lattice, its row bands and a batch round alike.
+static bool static_product(int r, const sfm_params& prm, ProductScales* sc) {
+  return r >= 12 && product_cell_scales(r, prm, sc);
+}
+
+size_t static_tmp_bytes(int r, const sfm_params& prm) {
+  ProductScales sc;
+  return static_product(r, prm, &sc) ? product_table_bytes(r, 2) : 0;
+}
+
+void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, const sfm_params& prm,
+                         float* Fs, void* tmp, Counters* ctr, cudaStream_t s) {
+  ProductScales sc;
+  if (static_product(g.r, prm, &sc)) {
+    launch_limb_tables(g.r, prm, sc, 2, static_cast<uint8_t*>(tmp), s);
+    ProductArgs a;
+    product_layout(g.r, &a);
+    a.nch = 2;
+    a.ctr = ctr;
+    a.store_hi = g.H;
+    a.one.src = cell;
+    a.one.spitch = g.W;
+    a.one.out = Fs;
+    a.one.tab = static_cast<const uint8_t*>(tmp);
+    a.one.W = g.W;
+    a.one.H = g.H;
+    a.one.px = g.px;
+    a.one.py = g.py;
+    a.one.r = g.r;
+    a.one.ntx = product_tiles_x(g.W);
+    a.one.c0 = (float)(1.0 / sc.s0);
+    a.one.c1 = (float)(1.0 / (sc.s0 * sc.s1));
+    launch_product(a, s);
+    return;
+  }
   const int S = 2 * g.r + 1, HW = kTile + 2 * g.r;
   const size_t smem = (size_t)2 * S * S * sizeof(float) + (size_t)HW * HW;
   cudaFuncSetAttribute(k_static_field, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

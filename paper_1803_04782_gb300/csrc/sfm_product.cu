@@ -7,7 +7,7 @@
 // Arithmetic.  A crowd is five planes of {-1, 0, +1}: occupancy and the four
 // heading axes (E-W, N-S, NE-SW, NW-SE), and K_P is the sum of five window
 // tables, one a plane.  Each table entry is held in fixed point as two
-// integers of FP16 ("limbs"): T = L0 / s0 + L1 / (s0 s1), |L0|, |L1| <= 2048.
+// integers of FP16 ("limbs"): T = L0 / s0 + L1 / (s0 s1), |L0|, |L1| <= 4096.
 // Products with {-1, 0, +1} and every partial sum are integers below 2^24 in
 // magnitude (product_scales), so the FP32 accumulators hold them exactly: a
 // sum is the same whatever the order, the tile or the split, and is rounded
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
   int S;
   {
     const int r = a.lattices ? a.lattices[a.tiles[T - 1].x].r : a.one.r;
-    S = slices_of(rest, nch, G, (2 * r + 16) * chunks_of(r) * 128 + 2000);
+    S = a.scratch ? slices_of(rest, nch, G, (2 * r + 16) * chunks_of(r) * 128 + 2000) : 1;
   }
   const int units = whole + (rest * S) / G + (me < rest * S % G ? 1 : 0);
   struct Unit {
@@ -589,45 +589,65 @@ __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, d
       if (ch == 4) v *= gamma * q * (dy - dx) / d;
     }
   }
-  const double hi = rint(v * s0), lo = rint((v * s0 - hi) * s1);
+  // an integer of FP16: any up to 2048, the nearest even one above
+  const __half hi = __double2half(fabs(v * s0) > 2048.0 ? v * s0 : rint(v * s0));
+  const __half lo = __double2half(rint((v * s0 - (double)__half2float(hi)) * s1));
   __half* o = tab + ((size_t)(ch * C + c) * J + j) * 256 + h * 64 + nx * 8 + kx;
-  o[0] = __double2half(hi);
-  o[128] = __double2half(lo);
+  o[0] = hi;
+  o[128] = lo;
 }
 
-// Largest power of two for the first limb and the second that keep every
-// entry within 2048 (exact in FP16) and every sum over a full window below
-// 2^24 (exact in FP32): `big` bounds an entry, `per` what one su adds to a
-// sum (over `entries` entries), `least` is the smallest magnitude of the law
-// in the window, which the rounding of the second limbs must stay 5e-6 below.
-bool product_scales(int r, double big, double per, int entries, double least, ProductScales* out) {
-  if (r < 1 || r > kProductMaxRadius || !(big > 0.0) || !isfinite(big) || !isfinite(per)) return false;
-  const double n = (2.0 * r + 1) * (2.0 * r + 1) - 1.0, top = 16777215.0;
-  double s0 = ldexp(1.0, (int)floor(log2(2048.0 / big)));
-  while (n * (per * s0 + 0.5 * entries) > top) s0 *= 0.5;
-  double s1 = 4096.0;  // |L1| <= s1 / 2
+// A law k d^a over the window of radius r: largest and smallest magnitude and
+// the sum of the magnitudes.
+struct LawRange {
+  double big = 0.0, least = 0.0, sum = 0.0;
+};
+LawRange law_range(int r, double k, double a) {
+  LawRange l;
+  const double u = fabs(k), v = fabs(k) * pow(r * sqrt(2.0), a);
+  l.big = u > v ? u : v;
+  l.least = u > v ? v : u;
+  for (int x = 1; x <= r; ++x)  // an octant: (x, 0) and (x, x) stand for 4 su, the others for 8
+    for (int y = 0; y <= x; ++y)
+      l.sum += (y == 0 || y == x ? 4.0 : 8.0) * fabs(k) * pow((double)(x * x + y * y), 0.5 * a);
+  return l;
+}
+
+// Largest powers of two whose limbs are FP16 integers (up to 2048 any, up to
+// 4096 even ones) and whose sums over a full window stay below 2^24 (exact in
+// FP32).  `big` bounds an entry, `sum` what a full window adds to a first
+// limb, `entries` the tables a su is in; the second limbs are at most s1 / 2,
+// but for the few entries above half of `big`.  What their rounding leaves
+// must stay 5e-6 below `least`, the law's smallest magnitude in the window.
+bool product_scales(int r, double big, double sum, int entries, double least, ProductScales* out) {
+  if (r < 1 || r > kProductMaxRadius || !(big > 0.0) || !isfinite(big) || !isfinite(sum)) return false;
+  const double n = (2.0 * r + 1) * (2.0 * r + 1) + 60.0, top = 16777215.0;
+  double s0 = ldexp(1.0, (int)floor(log2(4096.0 / big)));
+  while (sum * s0 + n * entries > top) s0 *= 0.5;
+  double s1 = 4096.0;
   while (n * entries * s1 * 0.5 > top) s1 *= 0.5;
-  if (!(entries * 0.5 / (s0 * s1) <= 5e-6 * least)) return false;
+  if (!(entries * 1.0 / (s0 * s1) <= 5e-6 * least)) return false;
   if (!(s0 > 1e-30 && s0 * s1 < 1e30)) return false;  // the limbs' weights are FP32
   out->s0 = s0;
   out->s1 = s1;
   return true;
 }
 
-// largest and smallest |k d^a| of a window of radius r
-void law_range(int r, double k, double a, double* big, double* least) {
-  const double u = fabs(k), v = fabs(k) * pow(r * sqrt(2.0), a);
-  *big = u > v ? u : v;
-  *least = u > v ? v : u;
-}
-
 }  // namespace
 
 bool product_crowd_scales(int r, const sfm_params& p, ProductScales* out) {
-  double big, least;
-  law_range(r, p.kP, p.aP, &big, &least);
+  const LawRange l = law_range(r, p.kP, p.aP);
   const double g = fabs((double)p.gamma);
-  return product_scales(r, g > 1.0 ? big * g : big, big * (1.0 + g) * (1.0 + 1e-9), 2, least, out);
+  return product_scales(r, g > 1.0 ? l.big * g : l.big, l.sum * (1.0 + g), 2, l.least, out);
+}
+
+// a su is a wall, an exit or neither, so it adds one entry
+bool product_cell_scales(int r, const sfm_params& p, ProductScales* out) {
+  LawRange o = law_range(r, p.kO, p.aO), e = law_range(r, p.kE, p.aE);
+  if (p.kO == 0.f) o.least = e.least;
+  if (p.kE == 0.f) e.least = o.least;
+  return product_scales(r, o.big > e.big ? o.big : e.big, o.sum + e.sum, 1,
+                        o.least < e.least ? o.least : e.least, out);
 }
 
 size_t product_table_bytes(int r, int nch) { return (size_t)nch * chunks_of(r) * stage_bytes_of(r); }
