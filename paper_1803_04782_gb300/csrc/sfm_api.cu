@@ -478,45 +478,6 @@ void sfm::ctx_field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, b
   field_rows(c, out, ya, yb, main_off, halos);
 }
 
-// Guidance distances of one lattice: relaxation rounds until no tile changes
-// (at most 4 * tiles + 256 rounds, then SFM_ETIMEOUT).
-sfm_status sfm::compute_guidance(const Geo& g, const uint8_t* cell, int32_t* D, cudaStream_t s,
-                                 std::string* err) {
-  const int ntiles = ((g.W + kTile - 1) / kTile) * ((g.H + kTile - 1) / kTile);
-  uint8_t *a0 = nullptr, *a1 = nullptr;
-  int* changed = nullptr;
-  if (cudaMalloc(&a0, ntiles) != cudaSuccess || cudaMalloc(&a1, ntiles) != cudaSuccess ||
-      cudaMalloc(&changed, sizeof(int)) != cudaSuccess) {
-    cudaFree(a0);
-    cudaFree(a1);
-    if (err) *err = "guidance scratch allocation failed";
-    return SFM_ENOMEM;
-  }
-  launch_guidance_init(g, cell, D, s);
-  cudaMemsetAsync(a0, 1, ntiles, s);
-  int h_changed = 1, rounds = 0;
-  const int max_rounds = 4 * ntiles + 256;
-  while (h_changed && rounds < max_rounds) {
-    cudaMemsetAsync(a1, 0, ntiles, s);
-    cudaMemsetAsync(changed, 0, sizeof(int), s);
-    launch_guidance_round(g, cell, D, a0, a1, changed, s);
-    cudaMemcpyAsync(&h_changed, changed, sizeof(int), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    uint8_t* tmp = a0;
-    a0 = a1;
-    a1 = tmp;
-    ++rounds;
-  }
-  cudaFree(a0);
-  cudaFree(a1);
-  cudaFree(changed);
-  if (h_changed) {
-    if (err) *err = "guidance relaxation did not converge";
-    return SFM_ETIMEOUT;
-  }
-  return SFM_OK;
-}
-
 extern "C" {
 
 int32_t sfm_abi_version(void) { return SFM_ABI_VERSION; }
@@ -597,7 +558,7 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
   ALLOC(ctx->cell, nsu);
   ALLOC(ctx->Fs, nsu);
   ALLOC(ctx->D, nsu);
-  ALLOC(ctx->occ, std::max(nsu, static_tmp_bytes(g.r, ctx->prm) / sizeof(int32_t)));
+  ALLOC(ctx->occ, std::max({nsu, static_tmp_bytes(g.r, ctx->prm) / sizeof(int32_t), guidance_scratch_ints(g)}));
   ALLOC(ctx->ocls, (size_t)g.opitch * g.H);
   if (ctx->bands <= 1) {
     ALLOC(ctx->F, nsu);
@@ -635,12 +596,9 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
   if (ctx->CT3) launch_class_tables3(g.r, ctx->prm, ctx->CT3, s);
   // the occupancy grid is scratch until it is cleared
   launch_static_field(g, ctx->cell, ctx->tables(), ctx->prm, ctx->Fs, ctx->occ, ctx->ctr, s);
+  launch_guidance(g, ctx->cell, ctx->D, ctx->occ, ctx->ctr, s);
   cudaMemsetAsync(ctx->occ, 0xff, nsu * sizeof(int32_t), s);
 
-  {
-    const sfm_status gst = compute_guidance(g, ctx->cell, ctx->D, s, &ctx->err);
-    if (gst != SFM_OK) return bail(gst);
-  }
   e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {

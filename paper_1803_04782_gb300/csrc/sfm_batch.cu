@@ -793,7 +793,9 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
   {
     // the occupancy grids are the static fields' scratch until they are cleared
     size_t tmp = 0;
-    for (int i = 0; i < nscenes; ++i) tmp = std::max(tmp, static_tmp_bytes(B->hs[i].g.r, prms[i]));
+    for (int i = 0; i < nscenes; ++i)
+      tmp = std::max({tmp, static_tmp_bytes(B->hs[i].g.r, prms[i]),
+                      guidance_scratch_ints(B->hs[i].g) * sizeof(int32_t)});
     BALLOC(ctx->occ, std::max((size_t)su, tmp / sizeof(int32_t)));
   }
   BALLOC(ctx->ocls, (size_t)oc);
@@ -847,8 +849,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     tb.KE = KE;
     launch_static_field(sc.g, ctx->cell + sc.su_off, tb, prms[sidx], ctx->Fs + sc.su_off,
                         ctx->occ, ctx->ctr, s);
-    st = compute_guidance(sc.g, ctx->cell + sc.su_off, ctx->D + sc.su_off, s, &ctx->err);
-    if (st != SFM_OK) return bail(st);
+    launch_guidance(sc.g, ctx->cell + sc.su_off, ctx->D + sc.su_off, ctx->occ, ctx->ctr, s);
     std::fill_n(bs.begin() + sc.bin_off, sc.g.nbx * sc.g.nby, (uint16_t)sidx);
   }
   cudaMemsetAsync(ctx->occ, 0xff, (size_t)su * sizeof(int32_t), s);

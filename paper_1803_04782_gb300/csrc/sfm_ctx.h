@@ -11,8 +11,6 @@
 struct sfm_ctx;
 namespace sfm {
 struct BatchState;  // sfm_batch.cu
-sfm_status compute_guidance(const Geo& g, const uint8_t* cell, int32_t* D, cudaStream_t s,
-                            std::string* err);
 // message returned by sfm_last_error(NULL) on this thread
 void set_create_error(const std::string& msg);
 // bins of the context's current state (S1), field rows (S2) into `out`

@@ -239,12 +239,13 @@ void launch_tables(int r, const sfm_params& p, float* T0, float* TX, float* TY, 
 size_t static_tmp_bytes(int r, const sfm_params& prm);
 void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, const sfm_params& prm,
                          float* Fs, void* tmp, Counters* ctr, cudaStream_t s);
-// One relaxation round of the guidance distances; returns via *changed.
-void launch_guidance_init(const Geo& g, const uint8_t* cell, int32_t* D, cudaStream_t s);
+// Guidance distances; scratch: guidance_scratch_ints() ints of device memory,
+// overwritten.  A bounded wait that runs out sets kErrTimeout in ctr.
+size_t guidance_scratch_ints(const Geo& g);
+void launch_guidance(const Geo& g, const uint8_t* cell, int32_t* D, int* scratch, Counters* ctr,
+                     cudaStream_t s);
 void launch_guidance_export(int32_t* D, size_t n, cudaStream_t s);
 void launch_guidance_import(const uint8_t* cell, int32_t* D, size_t n, cudaStream_t s);
-void launch_guidance_round(const Geo& g, const uint8_t* cell, int32_t* D, const uint8_t* act_in,
-                           uint8_t* act_out, int* changed, cudaStream_t s);
 
 void launch_place_clear(int n, const int2* xy, const uint8_t* alive, const Geo& g, int32_t* occ,
                         uint8_t* ocls, cudaStream_t s, const Sizes& sz = Sizes());

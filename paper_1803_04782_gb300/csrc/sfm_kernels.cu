@@ -169,16 +169,98 @@ void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, co
 
 // --------------------------------------------------------------- guidance
 // Chamfer (5, 7) geodesic distance to the nearest EXIT through non-WALL su
-// (kDInf where none is reachable, kDWall on WALL su),
-// solved as the fixed point of D(c) = min_k D(c + Delta_k) + w_k by tile-local
-// relaxation in shared memory; a tile is revisited only when it or a
-// neighbour changed in the previous round.  The fixed point is unique, so the
-// result is exact and independent of the visiting order.
-__global__ void k_guidance_init(Geo g, const uint8_t* __restrict__ cell, int32_t* __restrict__ D) {
-  const size_t n = (size_t)g.W * g.H;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    D[i] = cell[i] == kExit ? 0 : (cell[i] == kWall ? kDWall : kDInf);
+// (kDInf where none is reachable, kDWall on WALL su), the fixed point of
+// D(c) = min_k D(c + Delta_k) + w_k.  The fixed point is unique and every
+// update only lowers values towards it, so the result is exact whatever the
+// order of the updates.
+//
+// Tiles of 32 x 32 su are relaxed in shared memory by persistent CTAs that
+// take them from a queue, without rounds: a tile whose border a CTA lowers
+// puts the neighbours that see it into the queue.  The time is the chain of
+// tiles from an exit to the farthest su, so what matters is one tile's
+// latency: a thread a su, a row looked at again only after it or the row
+// above or below changed, and distances carried along a whole row or column
+// by one scan, so a front crosses a tile in a few steps.  A 2048 x 2048 floor
+// takes 563 us (one-pass ncu); a launch a round, with the host asking for the
+// outcome of each, took 35 rounds of 36 us and their round trips: 1.9 ms
+// (scene set-up 2.90 against 1.61 ms).  256 threads a tile, eight CTAs an SM:
+// 878 us; without the scan down the columns 642.
+constexpr int kGuideThreads = kTile * kTile;
+constexpr int kGuideSpins = 1 << 23;  // naps of an idle CTA, each 100 ns and more: about a second
+
+// Queue of tiles: entry pos of the run sits in ring[pos mod ntiles] with its
+// position, so nothing is cleared.  A tile is in it at most once (`queued`), so
+// an entry is never overwritten before it is taken.  `work` holds the entries
+// made so far (low half) and the tiles queued or being relaxed (high half), so
+// that one atomic makes an entry's place and keeps the run alive.
+struct GuideQueue {
+  unsigned long long work;
+  int head, pad;
+};
+struct GuideTiles {
+  GuideQueue* q;
+  unsigned long long* ring;  // (pos + 1) << 32 | tile
+  int* queued;
+};
+__host__ __device__ __forceinline__ GuideTiles guide_tiles(int* scratch, int ntiles) {
+  GuideTiles t;
+  t.q = reinterpret_cast<GuideQueue*>(scratch);
+  t.ring = reinterpret_cast<unsigned long long*>(t.q + 1);
+  t.queued = reinterpret_cast<int*>(t.ring + ntiles);
+  return t;
+}
+
+__device__ __forceinline__ void guide_push(const GuideTiles& gt, int ntiles, int t) {
+  if (atomicExch(&gt.queued[t], 1) != 0) return;
+  const unsigned pos = (unsigned)atomicAdd(&gt.q->work, (1ull << 32) + 1ull);
+  *reinterpret_cast<volatile unsigned long long*>(&gt.ring[pos % (unsigned)ntiles]) =
+      (unsigned long long)(pos + 1u) << 32 | (unsigned)t;
+}
+
+// the next tile of the queue, -1 when no tile is left (or the wait ran out)
+__device__ int guide_pop(const GuideTiles& gt, int ntiles, Counters* ctr) {
+  const unsigned pos = (unsigned)atomicAdd(&gt.q->head, 1);
+  volatile unsigned long long* slot = &gt.ring[pos % (unsigned)ntiles];
+  for (int i = 0; i < kGuideSpins; ++i) {
+    const unsigned long long v = *slot;
+    if ((unsigned)(v >> 32) == pos + 1u) {
+      const int t = (int)(unsigned)v;
+      atomicExch(&gt.queued[t], 0);  // from here on a neighbour may queue it again
+      __threadfence();               // and its values are read after that
+      return t;
+    }
+    if ((*reinterpret_cast<volatile unsigned long long*>(&gt.q->work) >> 32) == 0) return -1;
+    __nanosleep(100);
+  }
+  atomicOr(&ctr->err, kErrTimeout);
+  return -1;
+}
+
+// neighbour (dx, dy) of tile (tx, ty), wrapped in periodic dimensions; -1: none
+__device__ __forceinline__ int guide_neighbour(const Geo& g, int ntx, int nty, int tx, int ty, int dx, int dy) {
+  int nx = tx + dx, ny = ty + dy;
+  if (g.px) nx = (nx + ntx) % ntx;
+  if (g.py) ny = (ny + nty) % nty;
+  return nx >= 0 && nx < ntx && ny >= 0 && ny < nty ? ny * ntx + nx : -1;
+}
+
+// start values, and the tiles that see an exit into the queue
+__global__ void __launch_bounds__(1024)
+    k_guidance_init(Geo g, const uint8_t* __restrict__ cell, int32_t* __restrict__ D, GuideTiles gt) {
+  const int ntx = (g.W + kTile - 1) / kTile, nty = (g.H + kTile - 1) / kTile;
+  const int tx = blockIdx.x % ntx, ty = blockIdx.x / ntx;
+  const int x = tx * kTile + (threadIdx.x & 31), y = ty * kTile + (threadIdx.x >> 5);
+  bool source = false;
+  if (x < g.W && y < g.H) {
+    const size_t c = (size_t)y * g.W + x;
+    const uint8_t v = cell[c];
+    source = v == kExit;
+    D[c] = source ? 0 : (v == kWall ? kDWall : kDInf);
+  }
+  if (__syncthreads_or(source) && threadIdx.x < 9) {
+    const int t = guide_neighbour(g, ntx, nty, tx, ty, (int)threadIdx.x % 3 - 1, (int)threadIdx.x / 3 - 1);
+    if (t >= 0) guide_push(gt, ntx * nty, t);
+  }
 }
 
 // the exported form: WALL su read kDInf, like unreachable ones
@@ -195,62 +277,136 @@ __global__ void k_guidance_import(const uint8_t* __restrict__ cell, int32_t* __r
     if (cell[i] == kWall) D[i] = kDWall;
 }
 
-__global__ void __launch_bounds__(1024)
-    k_guidance_round(Geo g, const uint8_t* __restrict__ cell, int32_t* __restrict__ D,
-                     const uint8_t* __restrict__ act_in, uint8_t* __restrict__ act_out,
-                     int* __restrict__ changed) {
-  __shared__ int32_t sD[kTile + 2][kTile + 2];
-  const int ntx = (g.W + kTile - 1) / kTile, nty = (g.H + kTile - 1) / kTile;
-  const int tile = blockIdx.x;
-  if (!act_in[tile]) return;
-  const int tx = tile % ntx, ty = tile / ntx;
-  const int x0 = tx * kTile, y0 = ty * kTile;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < (kTile + 2) * (kTile + 2); i += blockDim.x) {
-    const int hx = i % (kTile + 2), hy = i / (kTile + 2);
-    int gx, gy;
-    int32_t v = kDInf;
-    if (wrap_coord(x0 - 1 + hx, g.W, g.px, gx) && wrap_coord(y0 - 1 + hy, g.H, g.py, gy))
-      v = D[(size_t)gy * g.W + gx];
-    sD[hy][hx] = v;
-  }
-  const int lx = tid % kTile, ly = tid / kTile;
-  const int gx = x0 + lx, gy = y0 + ly;
-  const bool valid = gx < g.W && gy < g.H;
-  uint8_t cv = kWall;
-  if (valid) cv = cell[(size_t)gy * g.W + gx];
-  const bool relax = valid && cv == kFree;
-  __syncthreads();
-  bool mine = false;
-  for (int it = 0; it < 4 * kTile * kTile; ++it) {
-    bool ch = false;
-    if (relax) {
-      const int32_t cur = sD[ly + 1][lx + 1];
-      int32_t best = cur;
+// Distances carried along a line of 32 su (a lane a su), 5 a step, to the
+// walls on either side (`open`: the line's su without walls), where some su
+// lies more than a step above its neighbour.
+__device__ __forceinline__ int guide_scan(int v, uint32_t open, int lane) {
+  const bool mine = (open >> lane) & 1u;
+  const int l1 = __shfl_up_sync(0xffffffffu, v, 1), r1 = __shfl_down_sync(0xffffffffu, v, 1);
+  if (!__any_sync(0xffffffffu, mine && ((lane > 0 && v > l1 + 5) || (lane < 31 && v > r1 + 5)))) return v;
+  // open su next to this one on either side
+  const uint32_t below = ~open & ((1u << lane) - 1u), above = lane == 31 ? 0u : ~open >> (lane + 1);
+  const int runl = mine ? (below ? lane - 32 + __clz(below) : lane) : 0;
+  const int runr = mine ? (above ? __ffs(above) - 1 : 31 - lane) : 0;
 #pragma unroll
-      for (int k = 1; k <= 8; ++k) {
-        const int32_t v = sD[ly + 1 + c_dy[k]][lx + 1 + c_dx[k]];
-        const int32_t wk = (c_dx[k] != 0 && c_dy[k] != 0) ? 7 : 5;
-        if (v < kDInf && v + wk < best) best = v + wk;
-      }
-      if (best < cur) {
-        sD[ly + 1][lx + 1] = best;
-        ch = true;
-      }
-    }
-    mine |= ch;
-    if (!__syncthreads_or(ch)) break;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, v, o);
+    if (runl >= o) v = min(v, u + 5 * o);
   }
-  if (mine) D[(size_t)gy * g.W + gx] = sD[ly + 1][lx + 1];
-  if (__syncthreads_or(mine) && tid == 0) {
-    *changed = 1;
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx) {
-        int nx = tx + dx, ny = ty + dy;
-        if (g.px) nx = (nx + ntx) % ntx;
-        if (g.py) ny = (ny + nty) % nty;
-        if (nx >= 0 && nx < ntx && ny >= 0 && ny < nty) act_out[ny * ntx + nx] = 1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_down_sync(0xffffffffu, v, o);
+    if (runr >= o) v = min(v, u + 5 * o);
+  }
+  return v;
+}
+
+__global__ void __launch_bounds__(kGuideThreads, 2)
+    k_guidance(Geo g, int32_t* __restrict__ D, GuideTiles gt, Counters* ctr) {
+  // odd pitch: columns are read without bank conflicts too
+  __shared__ int sD[kTile + 2][kTile + 3];
+  __shared__ uint32_t s_open[kTile];               // su of a row that are inside and no walls
+  __shared__ int s_row[kTile + 2], s_col[kTile];   // last step that changed a row, a column
+  __shared__ int s_tile;
+  __shared__ uint32_t s_edge;
+  const int ntx = (g.W + kTile - 1) / kTile, nty = (g.H + kTile - 1) / kTile;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;  // lane: column, w: row (and column w of a scan)
+  for (;;) {
+    if (tid == 0) {
+      s_tile = guide_pop(gt, ntx * nty, ctr);
+      s_edge = 0u;
+    }
+    __syncthreads();
+    const int tile = s_tile;
+    if (tile < 0) break;
+    const int tx = tile % ntx, ty = tile / ntx, x0 = tx * kTile, y0 = ty * kTile;
+    const int gx = x0 + lane, gy = y0 + w;
+    // other CTAs lower these values meanwhile: read past L1.  Where a last
+    // tile is cut short by a periodic lattice's end, the su just beyond it is
+    // the one on the other side.
+    int wx, wy;
+    int32_t first = kDWall;
+    if (gx <= g.W && gy <= g.H && wrap_coord(gx, g.W, g.px, wx) && wrap_coord(gy, g.H, g.py, wy))
+      first = __ldcg(&D[(size_t)wy * g.W + wx]);
+    sD[w + 1][lane + 1] = first;
+    const uint32_t open = __ballot_sync(0xffffffffu, gx < g.W && gy < g.H && first != kDWall);
+    if (lane == 0) s_open[w] = open;
+    if (tid < kTile + 2) s_row[tid] = -1;
+    if (tid < kTile) s_col[tid] = -1;
+    if (tid < 4 * kTile + 4) {
+      // the ring of su around the tile: two rows of 34, then two columns of 32
+      int hx, hy;
+      if (tid < 2 * (kTile + 2)) {
+        hy = tid < kTile + 2 ? 0 : kTile + 1;
+        hx = tid % (kTile + 2);
+      } else {
+        const int k = tid - 2 * (kTile + 2);
+        hx = k < kTile ? 0 : kTile + 1;
+        hy = 1 + k % kTile;
       }
+      sD[hy][hx] = wrap_coord(x0 - 1 + hx, g.W, g.px, wx) && wrap_coord(y0 - 1 + hy, g.H, g.py, wy)
+                       ? __ldcg(&D[(size_t)wy * g.W + wx])
+                       : kDInf;
+    }
+    __syncthreads();
+    const uint32_t copen = __ballot_sync(0xffffffffu, (s_open[lane] >> w) & 1u);  // column w
+    volatile int(*vD)[kTile + 3] = sD;
+    volatile int *vrow = s_row, *vcol = s_col;
+    for (int step = 0; step < 4 * kTile * kTile; ++step) {
+      bool changed = false;
+      // rows: the eight neighbours, then along the row
+      if (step == 0 || vrow[w] >= step - 1 || vrow[w + 1] >= step - 1 || vrow[w + 2] >= step - 1) {
+        const int cur = vD[w + 1][lane + 1];
+        int best = cur;
+        if ((open >> lane) & 1u) {
+          best = min(best, min(vD[w][lane + 1], vD[w + 2][lane + 1]) + 5);
+          best = min(best, min(vD[w + 1][lane], vD[w + 1][lane + 2]) + 5);
+          best = min(best, min(vD[w][lane], vD[w][lane + 2]) + 7);
+          best = min(best, min(vD[w + 2][lane], vD[w + 2][lane + 2]) + 7);
+        }
+        best = guide_scan(best, open, lane);
+        if (best < cur) {
+          vD[w + 1][lane + 1] = best;
+          vrow[w + 1] = step;
+          vcol[lane] = step;
+          changed = true;
+        }
+      }
+      __syncthreads();
+      // columns that changed: along the column
+      if (vcol[w] == step) {
+        const int cur = vD[lane + 1][w + 1], best = guide_scan(cur, copen, lane);
+        if (best < cur) {
+          vD[lane + 1][w + 1] = best;
+          vrow[lane + 1] = step;
+        }
+      }
+      if (!__syncthreads_or(changed)) break;
+    }
+    // what this CTA lowered (another one may be at the same tile: the smaller
+    // value stays), and which neighbours see it: bit (dy + 1) * 3 + (dx + 1)
+    uint32_t edge = 0u;
+    const int v = vD[w + 1][lane + 1];
+    if (v < first && gx < g.W && gy < g.H) {
+      atomicMin(&D[(size_t)gy * g.W + gx], v);
+      const bool l = lane == 0, r = lane == kTile - 1 || gx == g.W - 1;
+      const bool t = w == 0, b = w == kTile - 1 || gy == g.H - 1;
+      edge = (l ? 1u << 3 : 0u) | (r ? 1u << 5 : 0u) | (t ? 1u << 1 : 0u) | (b ? 1u << 7 : 0u) |
+             (l && t ? 1u : 0u) | (r && t ? 1u << 2 : 0u) | (l && b ? 1u << 6 : 0u) | (r && b ? 1u << 8 : 0u);
+    }
+    edge = __reduce_or_sync(0xffffffffu, edge);
+    if (lane == 0 && edge) atomicOr(&s_edge, edge);
+    __threadfence();
+    __syncthreads();
+    if (tid < 32) {
+      if (tid < 9 && ((s_edge >> tid) & 1u)) {
+        const int t = guide_neighbour(g, ntx, nty, tx, ty, tid % 3 - 1, tid / 3 - 1);
+        if (t >= 0) guide_push(gt, ntx * nty, t);
+      }
+      __syncwarp();
+      if (tid == 0) atomicAdd(&gt.q->work, ~0ull << 32);  // one open tile less
+    }
+    __syncthreads();
   }
 }
 
@@ -266,12 +422,21 @@ int device_sm_count() {
   return cached[dev];
 }
 
-void launch_guidance_init(const Geo& g, const uint8_t* cell, int32_t* D, cudaStream_t s) {
-  const size_t n = (size_t)g.W * g.H;
-  int blocks = (int)((n + 255) / 256);
-  // grid-stride: at most 64 blocks of 256 per SM
-  if (blocks > device_sm_count() * 64) blocks = device_sm_count() * 64;
-  k_guidance_init<<<blocks, 256, 0, s>>>(g, cell, D);
+size_t guidance_scratch_ints(const Geo& g) {
+  const size_t ntiles = (size_t)cdiv(g.W, kTile) * cdiv(g.H, kTile);
+  return sizeof(GuideQueue) / sizeof(int) + 3 * ntiles;
+}
+
+void launch_guidance(const Geo& g, const uint8_t* cell, int32_t* D, int* scratch, Counters* ctr,
+                     cudaStream_t s) {
+  const int ntiles = cdiv(g.W, kTile) * cdiv(g.H, kTile);
+  const GuideTiles gt = guide_tiles(scratch, ntiles);
+  cudaMemsetAsync(scratch, 0, guidance_scratch_ints(g) * sizeof(int), s);
+  k_guidance_init<<<ntiles, 1024, 0, s>>>(g, cell, D, gt);
+  // idle CTAs wait for work that running ones make, never for one another
+  const int fit = 2 * device_sm_count();
+  const int blocks = ntiles < fit ? ntiles : fit;
+  k_guidance<<<blocks, kGuideThreads, 0, s>>>(g, D, gt, ctr);
 }
 
 void launch_guidance_export(int32_t* D, size_t n, cudaStream_t s) {
@@ -286,12 +451,6 @@ void launch_guidance_import(const uint8_t* cell, int32_t* D, size_t n, cudaStrea
   int blocks = (int)((n + 255) / 256);
   if (blocks > device_sm_count() * 64) blocks = device_sm_count() * 64;
   k_guidance_import<<<blocks, 256, 0, s>>>(cell, D, n);
-}
-
-void launch_guidance_round(const Geo& g, const uint8_t* cell, int32_t* D, const uint8_t* act_in,
-                           uint8_t* act_out, int* changed, cudaStream_t s) {
-  const int ntiles = cdiv(g.W, kTile) * cdiv(g.H, kTile);
-  k_guidance_round<<<ntiles, kTile * kTile, 0, s>>>(g, cell, D, act_in, act_out, changed);
 }
 
 // ------------------------------------------------------------- placement

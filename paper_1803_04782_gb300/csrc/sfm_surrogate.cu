@@ -1163,6 +1163,32 @@ __device__ __forceinline__ void add_candidates(const float* __restrict__ p, floa
   for (int k = 0; k < 9; ++k) acc[k] += p[SY * (move_dy(k) + 1) * SP + SX * (move_dx(k) + 1)];
 }
 
+// The decision of listed slot i (pedestrian at q) on the exact field, at(k, su)
+// at candidate k: the exact path's energy (pick_move) from what k_sur_decide
+// or k_list_all stored for the slot.
+template <class At>
+__device__ __forceinline__ uint8_t decide_listed(int i, int2 q, const Geo& g,
+                                                 const int32_t* __restrict__ fb_dd,
+                                                 const uint32_t* __restrict__ fb_info, float beta,
+                                                 const float* __restrict__ own,
+                                                 const float* __restrict__ dirdot, At at) {
+  const uint32_t info = fb_info[i];
+  float f[9];
+  int32_t dd[9];
+  uint8_t oc[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    int tx, ty;
+    const bool ok = wrap_coord(q.x + move_dx(k), g.W, g.px, tx) & wrap_coord(q.y + move_dy(k), g.H, g.py, ty);
+    f[k] = ok ? at(k, (size_t)ty * g.W + tx) : 0.f;
+    dd[k] = fb_dd[(size_t)i * 9 + k];
+    oc[k] = (info >> k) & 1u ? 0 : 1;  // admissible iff its mask bit is set
+  }
+  const bool ok3[3] = {true, true, true};
+  return (uint8_t)pick_move<false>(f, dd, oc, ok3, ok3, (int)((info >> 9) & 15u), (int)((info >> 16) & 255u),
+                                   beta, own, dirdot, nullptr);
+}
+
 constexpr int kFbRunBins = 8;  // widest run of bins whose pedestrians share one walk
 
 template <int SP>
@@ -1172,13 +1198,12 @@ __global__ void __launch_bounds__(kFbThreads, 1)
                    const uint32_t* __restrict__ rec, const float* __restrict__ CT, int TS,
                    const float* __restrict__ Fs, const int32_t* __restrict__ fb_dd,
                    const uint32_t* __restrict__ fb_info, float beta, const float* __restrict__ own,
-                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
-                   const float* __restrict__ Fx) {
+                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice) {
   extern __shared__ __align__(16) float sm[];
   float* sT = sm + kTableGuard;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int2* scr = reinterpret_cast<int2*>(sT + 4 * TS) + w * 32;
-  if (!Fx) copy_to_shared<8>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
+  copy_to_shared<8>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
   __syncthreads();
   const int nrec = bin_start[nbins], r = g.r;
   const int nchunks = (nrec + 31) / 32;
@@ -1187,7 +1212,6 @@ __global__ void __launch_bounds__(kFbThreads, 1)
     const bool fl = i < nrec && fb_flag[i] != 0;
     unsigned todo = __ballot_sync(0xffffffffu, fl);
     if (!todo) continue;
-    if (Fx) todo = 0;  // the exact lattice field is at hand: nothing to sum
     const int2 q = fl ? xy[rec_id[i]] : make_int2(0, 0);
     const int brow = q.y / kBin, bcol = q.x / kBin;
     float acc[9];
@@ -1246,29 +1270,23 @@ __global__ void __launch_bounds__(kFbThreads, 1)
             }
           });
     }
-    if (fl) {
-      // the decision again on the exact candidate field, by the exact path's
-      // energy (pick_move) from what k_sur_decide stored for this slot
-      const uint32_t info = fb_info[i];
-      float f[9];
-      int32_t dd[9];
-      uint8_t oc[9];
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        int tx, ty;
-        const bool ok = wrap_coord(q.x + move_dx(k), g.W, g.px, tx) &
-                        wrap_coord(q.y + move_dy(k), g.H, g.py, ty);
-        const size_t c = (size_t)ty * g.W + tx;
-        f[k] = ok ? (Fx ? Fx[c] : Fs[c] + acc[k]) : 0.f;
-        dd[k] = fb_dd[(size_t)i * 9 + k];
-        oc[k] = (info >> k) & 1u ? 0 : 1;  // admissible iff its mask bit is set
-      }
-      const bool ok3[3] = {true, true, true};
-      choice[rec_id[i]] = (uint8_t)pick_move<false>(f, dd, oc, ok3, ok3, (int)((info >> 9) & 15u),
-                                                    (int)((info >> 16) & 255u), beta, own, dirdot,
-                                                    nullptr);
-    }
+    if (fl)
+      choice[rec_id[i]] = decide_listed(i, q, g, fb_dd, fb_info, beta, own, dirdot,
+                                        [&](int k, size_t c) { return Fs[c] + acc[k]; });
   }
+}
+
+// The listed pedestrians decided on an exact lattice field F.
+__global__ void k_sur_listed(const uint8_t* __restrict__ fb_flag, const int32_t* __restrict__ rec_id,
+                             const int32_t* __restrict__ bin_start, int nbins, Geo g,
+                             const int2* __restrict__ xy, const float* __restrict__ F,
+                             const int32_t* __restrict__ fb_dd, const uint32_t* __restrict__ fb_info,
+                             float beta, const float* __restrict__ own, const float* __restrict__ dirdot,
+                             uint8_t* __restrict__ choice) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= bin_start[nbins] || !fb_flag[i]) return;
+  const int p = rec_id[i];
+  choice[p] = decide_listed(i, xy[p], g, fb_dd, fb_info, beta, own, dirdot, [&](int, size_t c) { return F[c]; });
 }
 
 // Every pedestrian listed for the exact candidate field (delta = +inf): per
@@ -1820,13 +1838,22 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
   const Tables tb = ctx->tables();
   const int nbins = g.nbx * g.nby;
   cudaStream_t st = ctx->stream;
+  if (ctx->use_product()) {
+    // a crowded lattice's exact field is the product's, on the whole lattice
+    // (Fnear is free outside training)
+    ctx_field_rows(ctx, S->Fnear, 0, g.H, 0, false);
+    k_sur_listed<<<cdiv(ctx->n, 256), 256, 0, st>>>(S->fb_flag, ctx->rec_id, ctx->bin_start, nbins, g, ctx->xy,
+                                                    S->Fnear, S->fb_dd, S->fb_info, ctx->prm.beta, tb.own,
+                                                    tb.dirdot, choice);
+    return;
+  }
   const int SP = class_table_stride(g.r);
   const int TS = (2 * g.r + 1 + 2 * kFieldPadRows) * SP;
   const size_t smem = (kTableGuard + 4 * (size_t)TS) * sizeof(float) +
                       (size_t)kFbThreads / 32 * 32 * sizeof(int2);
   void (*fb)(const uint8_t*, const int32_t*, int, Geo, const int2*, const int32_t*, const uint32_t*,
              const float*, int, const float*, const int32_t*, const uint32_t*, float, const float*,
-             const float*, uint8_t*, const float*);
+             const float*, uint8_t*);
   switch (SP) {
     case 34: fb = k_sur_fallback<34>; break;
     case 50: fb = k_sur_fallback<50>; break;
@@ -1837,19 +1864,12 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
     default: fb = k_sur_fallback<kNarrowStride>; break;
   }
   cudaFuncSetAttribute(fb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  // a crowded lattice's exact field is the product's, on the whole lattice
-  // (Fnear is free outside training)
-  const float* Fx = nullptr;
-  if (ctx->use_product()) {
-    ctx_field_rows(ctx, S->Fnear, 0, g.H, 0, false);
-    Fx = S->Fnear;
-  }
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   fb<<<nsm > 0 ? nsm : 1, kFbThreads, smem, st>>>(
       S->fb_flag, ctx->rec_id, nbins, g, ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs,
-      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice, Fx);
+      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice);
 }
 
 void round_params(sfm_surrogate* S) {
