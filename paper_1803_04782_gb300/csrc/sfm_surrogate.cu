@@ -40,7 +40,6 @@ constexpr int kOffW[4] = {0, kNW1 + kL1o, kNW1 + kL1o + kNW2 + kLh,
                           kNW1 + kL1o + 2 * (kNW2 + kLh)};
 constexpr int kOffB[4] = {kNW1, kNW1 + kL1o + kNW2, kNW1 + kL1o + 2 * kNW2 + kLh,
                           kNW1 + kL1o + 2 * (kNW2 + kLh) + kNW4};
-constexpr int kTile = 16;  // output pixels per CTA side
 static_assert(kNParams == 3 * 32 * 25 + 32 + 2 * (32 * 32 * 9 + 32) + 32 * 9 + 1, "params");
 
 // ------------------------------------------- tensor-core 3x3 (mma.sync)
@@ -531,6 +530,14 @@ __global__ void k_pack_w3(const float* __restrict__ w, bf16* __restrict__ wt) {
   wt[i] = __float2bfloat16(w[(kk * 32 + c) * 32 + o]);
 }
 
+// a channel-planar FP32 image of n pixels as channel-last BF16
+__global__ void k_pack_x(const float* __restrict__ X, int n, bf16* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[(size_t)i * 3 + c] = __float2bfloat16(X[(size_t)c * n + i]);
+}
+
 // BF16 weights of layer 4 (3x3, 32 -> 1) as one n8 tile: [ky][kx][8][in],
 // row 0 the output's weights, rows 1-7 zero.
 __global__ void k_pack_w4(const float* __restrict__ w, bf16* __restrict__ wt) {
@@ -675,103 +682,388 @@ __global__ void k_pack_w1(const float* __restrict__ w, bf16* __restrict__ wt) {
 }
 
 // -------------------------------------------------------------- backward
-// dZ of a layer output: the incoming gradient, masked by the ReLU (A > 0).
-__device__ __forceinline__ float dz_at(const float* dA, const bf16* A, size_t i, bool relu) {
-  return relu ? (__bfloat162float(A[i]) > 0.f ? dA[i] : 0.f) : dA[i];
+// FP32 throughout, on the FMA pipes: dZ is FP32, and splitting it over
+// tensor-core passes would round its sums otherwise.  Each data gradient is
+// written already masked by the ReLU of the activation it belongs to (dZ of
+// the layer before), so nothing else reads the activations for their sign.
+// Weight gradients are summed per CTA over a fixed share of the image and the
+// CTAs' sums in CTA order: the result does not depend on the timing.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// Data gradient of a 3x3 32 -> 32 layer, masked:
+//   dZin[y][x][c] = (Ain[y][x][c] > 0) sum_{ky,kx,o} W[ky][kx][c][o] dZ[y-ky][x-kx][o]
+// FMA-bound: 9216 a pixel, 2.4e9 for a 512 x 512 image, 125 000 clocks of
+// 152 x 128 lanes.  A CTA takes 8 rows x 64 pixels: warp = row, lane = 8
+// pixels x 8 inputs, so 34 16-byte shared reads feed 768 packed FMAs (even
+// and odd outputs o side by side).  Shared 16-byte groups are swizzled by the
+// pixel's eight (dZ) and the input's eight (weights): no bank conflicts.
+// 131 us a layer on a 512 x 512 image (695 with a thread a pixel, which
+// read a scalar weight from shared memory per FMA).
+constexpr int kDxW = 64, kDxH = 8, kDxThreads = 32 * kDxH;
+constexpr int kDxPx = (kDxH + 2) * (kDxW + 2);
+constexpr size_t kDxSmem = (size_t)(kDxPx * 32 + 9 * 32 * 32) * sizeof(float);
+
+__global__ void __launch_bounds__(kDxThreads, 1)
+    k_conv3_dx(const float* __restrict__ dZ, int Hout, int Wout, const float* __restrict__ Wt,
+               const bf16* __restrict__ Ain, float* __restrict__ dZin) {
+  extern __shared__ __align__(16) float smf[];
+  float4* sD = reinterpret_cast<float4*>(smf);
+  float4* sW = sD + kDxPx * 8;
+  const int Hin = Hout + 2, Win = Wout + 2;
+  const int ntx = (Win + kDxW - 1) / kDxW, ntiles = ntx * ((Hin + kDxH - 1) / kDxH);
+  const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
+  for (int i = tid; i < 9 * 32 * 8; i += kDxThreads) {
+    const int q = i & 7, c = (i >> 3) & 31;
+    sW[(i & ~7) | (q ^ (c >> 3))] = reinterpret_cast<const float4*>(Wt)[i];
+  }
+  const int cg = lane & 3, pg = lane >> 2;  // inputs 8 cg .., pixels 8 pg ..
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int x0 = t % ntx * kDxW, y0 = t / ntx * kDxH;
+    __syncthreads();
+    for (int i = tid; i < kDxPx * 8; i += kDxThreads) {
+      const int q = i & 7, p = i >> 3, px = p % (kDxW + 2), py = p / (kDxW + 2);
+      const int gy = y0 - 2 + py, gx = x0 - 2 + px;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (gy >= 0 && gy < Hout && gx >= 0 && gx < Wout)
+        v = __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q);
+      sD[p * 8 + (q ^ ((px >> 3) & 7))] = v;
+    }
+    __syncthreads();
+    float2 acc[8][8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) acc[p][c] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int kq = 0; kq < 24; ++kq) {
+      const int ky = kq >> 3, q = kq & 7;
+      const float4* dr = sD + (row + 2 - ky) * (kDxW + 2) * 8;
+      float4 d[10];
+#pragma unroll
+      for (int i = 0; i < 10; ++i) {
+        const int px = 8 * pg + i;
+        d[i] = dr[px * 8 + (q ^ ((px >> 3) & 7))];
+      }
+#pragma unroll
+      for (int kx = 0; kx < 3; ++kx) {
+        const float4* wr = sW + ((ky * 3 + kx) * 32 + 8 * cg) * 8 + (q ^ cg);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float4 w = wr[c * 8];
+#pragma unroll
+          for (int p = 0; p < 8; ++p) {
+            const float4 v = d[p + 2 - kx];
+            acc[p][c] = fma2(make_float2(v.x, v.y), make_float2(w.x, w.y), acc[p][c]);
+            acc[p][c] = fma2(make_float2(v.z, v.w), make_float2(w.z, w.w), acc[p][c]);
+          }
+        }
+      }
+    }
+    const int y = y0 + row;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      const int x = x0 + 8 * pg + p;
+      if (y >= Hin || x >= Win) continue;
+      const size_t at = ((size_t)y * Win + x) * 32 + 8 * cg;
+      const uint4 m = __ldg(reinterpret_cast<const uint4*>(Ain + at));
+      const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
+      float o[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        // BF16 activation > 0: its sign bit clear and not zero
+        const uint32_t h = (mw[c >> 1] >> (16 * (c & 1))) & 0xffffu;
+        o[c] = (h - 1u < 0x7fffu) ? acc[p][c].x + acc[p][c].y : 0.f;
+      }
+      float4* dst = reinterpret_cast<float4*>(dZin + at);
+      dst[0] = make_float4(o[0], o[1], o[2], o[3]);
+      dst[1] = make_float4(o[4], o[5], o[6], o[7]);
+    }
+  }
 }
 
-// dIn[y][x][c] = sum_{ky,kx,o} W[ky][kx][c][o] * dZ[y-ky][x-kx][o]
-template <int CIN, int COUT, int K, bool RELU>
-__global__ void __launch_bounds__(kTile* kTile)
-    k_conv_dx(const float* __restrict__ dA, const bf16* __restrict__ A, int Hout, int Wout,
-              const float* __restrict__ Wt, float* __restrict__ dIn) {
-  constexpr int TI = kTile + K - 1;
-  extern __shared__ __align__(16) float sm[];
-  float* sW = sm;
-  float* sD = sm + K * K * CIN * COUT;  // dZ tile: output rows y0-K+1 .. y0+kTile-1
-  const int Hin = Hout + K - 1, Win = Wout + K - 1;
-  const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < K * K * CIN * COUT; i += blockDim.x) sW[i] = Wt[i];
-  for (int i = tid; i < TI * TI * COUT; i += blockDim.x) {
-    const int o = i % COUT, p = i / COUT, px = p % TI, py = p / TI;
-    const int gy = y0 - (K - 1) + py, gx = x0 - (K - 1) + px;
+// Data gradient of the last layer (32 -> 1), masked: as above with one output.
+// Bound by the write of 128 bytes a pixel; a thread has 4 inputs of a pixel.
+__global__ void __launch_bounds__(256)
+    k_conv4_dx(const float* __restrict__ dY, int Hout, int Wout, const float* __restrict__ Wt,
+               const bf16* __restrict__ Ain, float* __restrict__ dZin) {
+  const int Hin = Hout + 2, Win = Wout + 2;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, q = i & 7, p = i >> 3;
+  if (p >= Hin * Win) return;
+  const int y = p / Win, x = p % Win;
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+    for (int kx = 0; kx < 3; ++kx) {
+      const int gy = y - ky, gx = x - kx;
+      const float v = gy >= 0 && gy < Hout && gx >= 0 && gx < Wout ? __ldg(dY + (size_t)gy * Wout + gx) : 0.f;
+      const float4 w = __ldg(reinterpret_cast<const float4*>(Wt) + (ky * 3 + kx) * 8 + q);
+      acc[0] = fmaf(v, w.x, acc[0]);
+      acc[1] = fmaf(v, w.y, acc[1]);
+      acc[2] = fmaf(v, w.z, acc[2]);
+      acc[3] = fmaf(v, w.w, acc[3]);
+    }
+  const uint2 m = __ldg(reinterpret_cast<const uint2*>(Ain + (size_t)i * 4));
+  const uint32_t h[4] = {m.x & 0xffffu, m.x >> 16, m.y & 0xffffu, m.y >> 16};
+  reinterpret_cast<float4*>(dZin)[i] =
+      make_float4(h[0] - 1u < 0x7fffu ? acc[0] : 0.f, h[1] - 1u < 0x7fffu ? acc[1] : 0.f,
+                  h[2] - 1u < 0x7fffu ? acc[2] : 0.f, h[3] - 1u < 0x7fffu ? acc[3] : 0.f);
+}
+
+// Weight and bias gradients of a 3x3 32 -> 32 layer, per CTA over its tiles of
+// 4 rows x 64 pixels: part[cta][e], e over W (9216) then b (32).  FMA-bound
+// like the data gradient.  Twelve warps: a kernel row ky and a tile row each;
+// lane = 4 inputs x 8 outputs of the three kx, whose inputs slide along the
+// row, so a pixel is 48 packed FMAs on three 16-byte shared reads:
+// 130 us a layer on a 512 x 512 image (620 with a thread a weight, two
+// scalar shared reads per FMA and a partial sum for every 16 x 16 tile).
+constexpr int kDwW = 64, kDwH = 4, kDwThreads = 32 * 3 * kDwH;
+constexpr int kDwIn = (kDwH + 2) * (kDwW + 2) * 32, kDwD = kDwH * kDwW * 32;  // floats
+constexpr int kDwE = kNW2 + kLh;
+constexpr size_t kDwSmem = (size_t)std::max(kDwIn + kDwD, kDwH * kNW2) * sizeof(float);
+
+__global__ void __launch_bounds__(kDwThreads, 1)
+    k_conv3_dw(const bf16* __restrict__ in, const float* __restrict__ dZ, int Hout, int Wout,
+               float* __restrict__ part) {
+  extern __shared__ __align__(16) float smf[];
+  __shared__ float sB[kDwThreads];
+  float *sI = smf, *sD = smf + kDwIn;
+  const int Hin = Hout + 2, Win = Wout + 2;
+  const int ntx = (Wout + kDwW - 1) / kDwW, ntiles = ntx * ((Hout + kDwH - 1) / kDwH);
+  const int tid = threadIdx.x, lane = tid & 31, ky = (tid >> 5) % 3, row = (tid >> 5) / 3;
+  const int c4 = (lane >> 2) * 4, o8 = (lane & 3) * 8;
+  float2 acc[3][4][4];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) acc[k][c][o] = make_float2(0.f, 0.f);
+  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);  // outputs 4 (tid mod 8) .. of the pixels this thread loads
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int x0 = t % ntx * kDwW, y0 = t / ntx * kDwH;
+    __syncthreads();
+    for (int i = tid; i < kDwIn / 8; i += kDwThreads) {
+      const int q = i & 3, p = i >> 2, px = p % (kDwW + 2), py = p / (kDwW + 2);
+      const int gy = y0 + py, gx = x0 + px;
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (gy < Hin && gx < Win) v = __ldg(reinterpret_cast<const uint4*>(in) + ((size_t)gy * Win + gx) * 4 + q);
+      // BF16 to FP32: the upper half of the word
+      float4* dst = reinterpret_cast<float4*>(sI) + i * 2;
+      dst[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                           __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+      dst[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
+                           __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
+    }
+    for (int i = tid; i < kDwD / 4; i += kDwThreads) {
+      const int q = i & 7, p = i >> 3, px = p % kDwW, py = p / kDwW;
+      const int gy = y0 + py, gx = x0 + px;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (gy < Hout && gx < Wout)
+        v = __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q);
+      reinterpret_cast<float4*>(sD)[i] = v;
+      bias.x += v.x;
+      bias.y += v.y;
+      bias.z += v.z;
+      bias.w += v.w;
+    }
+    __syncthreads();
+    const float4* ir = reinterpret_cast<const float4*>(sI + (row + ky) * (kDwW + 2) * 32 + c4);
+    const float4* dr = reinterpret_cast<const float4*>(sD + row * kDwW * 32 + o8);
+    float4 w0 = ir[0], w1 = ir[8];
+#pragma unroll 2
+    for (int x = 0; x < kDwW; ++x) {
+      const float4 w2 = ir[(x + 2) * 8];
+      const float4 da = dr[x * 8], db = dr[x * 8 + 1];
+      const float2 d[4] = {make_float2(da.x, da.y), make_float2(da.z, da.w), make_float2(db.x, db.y),
+                           make_float2(db.z, db.w)};
+      const float v[3][4] = {{w0.x, w0.y, w0.z, w0.w}, {w1.x, w1.y, w1.z, w1.w}, {w2.x, w2.y, w2.z, w2.w}};
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int o = 0; o < 4; ++o) acc[k][c][o] = fma2(make_float2(v[k][c], v[k][c]), d[o], acc[k][c][o]);
+      w0 = w1;
+      w1 = w2;
+    }
+  }
+  __syncthreads();
+  // the four tile rows' sums, then the bias
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int o = 0; o < 4; ++o)
+        *reinterpret_cast<float2*>(smf + row * kNW2 + ((ky * 3 + k) * 32 + c4 + c) * 32 + o8 + 2 * o) = acc[k][c][o];
+  __syncthreads();
+  float* dst = part + (size_t)blockIdx.x * kDwE;
+  for (int e = tid; e < kNW2; e += kDwThreads)
+    dst[e] = (smf[e] + smf[kNW2 + e]) + (smf[2 * kNW2 + e] + smf[3 * kNW2 + e]);
+  const float bv[4] = {bias.x, bias.y, bias.z, bias.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    __syncthreads();
+    sB[tid] = bv[k];
+    __syncthreads();
+    if (tid < 8) {
+      float b = 0.f;
+      for (int i = tid; i < kDwThreads; i += 8) b += sB[i];
+      dst[kNW2 + tid * 4 + k] = b;
+    }
+  }
+}
+
+// Weight and bias gradients of the last layer (32 -> 1), per CTA: part[cta][289].
+// Bound by the read of the activations, each once: a warp takes an input row's
+// 64 pixels, lane = input, and adds a pixel to the 9 taps with the dY that
+// see it (staged in shared memory with their border).
+constexpr int kDw4W = 64, kDw4H = 8, kDw4E = kNW4 + 1;
+__global__ void __launch_bounds__(32 * kDw4H)
+    k_conv4_dw(const bf16* __restrict__ in, const float* __restrict__ dY, int Hout, int Wout,
+               float* __restrict__ part) {
+  __shared__ float sY[kDw4H + 2][kDw4W + 2];
+  __shared__ float sP[kDw4H][kNW4], sB[kDw4H];
+  const int Hin = Hout + 2, Win = Wout + 2;
+  const int ntx = (Win + kDw4W - 1) / kDw4W, ntiles = ntx * ((Hin + kDw4H - 1) / kDw4H);
+  const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
+  float acc[9], bias = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) acc[k] = 0.f;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int x0 = t % ntx * kDw4W, y0 = t / ntx * kDw4H;
+    __syncthreads();
+    for (int i = tid; i < (kDw4H + 2) * (kDw4W + 2); i += blockDim.x) {
+      const int px = i % (kDw4W + 2), py = i / (kDw4W + 2), gy = y0 - 2 + py, gx = x0 - 2 + px;
+      const float v = gy >= 0 && gy < Hout && gx >= 0 && gx < Wout ? __ldg(dY + (size_t)gy * Wout + gx) : 0.f;
+      sY[py][px] = v;
+      if (py >= 2 && px >= 2) bias += v;  // each dY in one tile
+    }
+    __syncthreads();
+    const int y = y0 + row;
+    if (y < Hin) {
+      const bf16* src = in + ((size_t)y * Win + x0) * 32 + lane;
+      const int n = min(kDw4W, Win - x0);
+#pragma unroll 8
+      for (int x = 0; x < n; ++x) {
+        const float v = __bfloat162float(src[(size_t)x * 32]);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] = fmaf(v, sY[row + 2 - k / 3][x + 2 - k % 3], acc[k]);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) sP[row][k * 32 + lane] = acc[k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) bias += __shfl_xor_sync(0xffffffffu, bias, o);
+  if (lane == 0) sB[row] = bias;
+  __syncthreads();
+  for (int e = tid; e < kDw4E; e += blockDim.x) {
     float v = 0.f;
-    if (gy >= 0 && gy < Hout && gx >= 0 && gx < Wout)
-      v = dz_at(dA, A, ((size_t)gy * Wout + gx) * COUT + o, RELU);
-    sD[i] = v;
-  }
-  __syncthreads();
-  const int tx = tid % kTile, ty = tid / kTile;
-  const int y = y0 + ty, x = x0 + tx;
-  float acc[CIN];
-#pragma unroll
-  for (int c = 0; c < CIN; ++c) acc[c] = 0.f;
-  for (int ky = 0; ky < K; ++ky)
-    for (int kx = 0; kx < K; ++kx) {
-      const float* d = sD + ((ty - ky + K - 1) * TI + (tx - kx + K - 1)) * COUT;
-      const float* w = sW + (ky * K + kx) * CIN * COUT;
-      for (int o = 0; o < COUT; ++o) {
-        const float v = d[o];
-#pragma unroll
-        for (int c = 0; c < CIN; ++c) acc[c] = fmaf(v, w[c * COUT + o], acc[c]);
-      }
-    }
-  if (y >= Hin || x >= Win) return;
-#pragma unroll
-  for (int c = 0; c < CIN; ++c) dIn[((size_t)y * Win + x) * CIN + c] = acc[c];
-}
-
-// Per-CTA partial weight and bias gradients over a 16 x 16 tile of output
-// pixels: part[cta][e] for e over W (K*K*CIN*COUT entries) then b (COUT).
-template <int CIN, int COUT, int K, bool RELU>
-__global__ void __launch_bounds__(kTile* kTile)
-    k_conv_dw(const bf16* __restrict__ in, const float* __restrict__ dA, const bf16* __restrict__ A,
-              int Hout, int Wout, float* __restrict__ part) {
-  constexpr int TI = kTile + K - 1;
-  constexpr int NE = K * K * CIN * COUT + COUT;
-  extern __shared__ __align__(16) float sm[];
-  float* sIn = sm;                   // TI*TI*CIN
-  float* sD = sm + TI * TI * CIN;    // kTile*kTile*COUT
-  const int Win = Wout + K - 1, Hin = Hout + K - 1;
-  const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < TI * TI * CIN; i += blockDim.x) {
-    const int c = i % CIN, p = i / CIN, px = p % TI, py = p / TI;
-    const int gy = y0 + py, gx = x0 + px;
-    sIn[i] = (gy < Hin && gx < Win) ? __bfloat162float(in[((size_t)gy * Win + gx) * CIN + c]) : 0.f;
-  }
-  for (int i = tid; i < kTile * kTile * COUT; i += blockDim.x) {
-    const int o = i % COUT, p = i / COUT, px = p % kTile, py = p / kTile;
-    const int gy = y0 + py, gx = x0 + px;
-    sD[i] = (gy < Hout && gx < Wout) ? dz_at(dA, A, ((size_t)gy * Wout + gx) * COUT + o, RELU) : 0.f;
-  }
-  __syncthreads();
-  float* dst = part + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * NE;
-  for (int e = tid; e < NE; e += blockDim.x) {
-    float s = 0.f;
-    if (e < K * K * CIN * COUT) {
-      const int o = e % COUT, c = (e / COUT) % CIN, kk = e / (COUT * CIN), kx = kk % K, ky = kk / K;
-      for (int p = 0; p < kTile * kTile; ++p) {
-        const int px = p % kTile, py = p / kTile;
-        s = fmaf(sIn[((py + ky) * TI + (px + kx)) * CIN + c], sD[p * COUT + o], s);
-      }
-    } else {
-      const int o = e - K * K * CIN * COUT;
-      for (int p = 0; p < kTile * kTile; ++p) s += sD[p * COUT + o];
-    }
-    dst[e] = s;
+    for (int r = 0; r < kDw4H; ++r) v += e < kNW4 ? sP[r][e] : sB[r];
+    part[(size_t)blockIdx.x * kDw4E + e] = v;
   }
 }
 
-// g[e] = sum over CTAs (fixed order) of part[cta][e]
-__global__ void k_reduce_parts(const float* __restrict__ part, int nparts, int ne,
-                               float* __restrict__ g) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= ne) return;
-  float s = 0.f;
-  for (int k = 0; k < nparts; ++k) s += part[(size_t)k * ne + e];
-  g[e] = s;
+// Weight and bias gradients of layer 1 (3 -> 32, 5x5), per CTA: part[cta][2432].
+// Fifteen warps: a kernel row ky and a tile row each, lane = output, one sum
+// for each of the row's 15 (kx, c), which are 15 consecutive elements of the
+// channel-last input; four pixels share the 24 elements they see.
+constexpr int kDw1W = 64, kDw1H = 3, kDw1Threads = 32 * 5 * kDw1H, kDw1E = kNW1 + kL1o;
+constexpr int kDw1Row = (kDw1W + 4) * 3 + 12;  // floats of an input row, a multiple of 4, room for the last window
+__global__ void __launch_bounds__(kDw1Threads)
+    k_conv1_dw(const bf16* __restrict__ in, const float* __restrict__ dZ, int Hout, int Wout,
+               float* __restrict__ part) {
+  __shared__ __align__(16) float sX[kDw1H + 4][kDw1Row];
+  __shared__ __align__(16) float sD[kDw1H * kDw1W * 32];
+  const int Hin = Hout + 4, Win = Wout + 4;
+  const int ntx = (Wout + kDw1W - 1) / kDw1W, ntiles = ntx * ((Hout + kDw1H - 1) / kDw1H);
+  const int tid = threadIdx.x, lane = tid & 31, ky = (tid >> 5) % 5, row = (tid >> 5) / 5;
+  float acc[15], bias = 0.f;
+#pragma unroll
+  for (int k = 0; k < 15; ++k) acc[k] = 0.f;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int x0 = t % ntx * kDw1W, y0 = t / ntx * kDw1H;
+    __syncthreads();
+    for (int i = tid; i < (kDw1H + 4) * kDw1Row; i += kDw1Threads) {
+      const int e = i % kDw1Row, py = i / kDw1Row, gy = y0 + py;
+      sX[py][e] = gy < Hin && x0 * 3 + e < Win * 3 ? __bfloat162float(in[((size_t)gy * Win + x0) * 3 + e]) : 0.f;
+    }
+    for (int i = tid; i < kDw1H * kDw1W * 8; i += kDw1Threads) {
+      const int q = i & 7, p = i >> 3, gy = y0 + p / kDw1W, gx = x0 + p % kDw1W;
+      reinterpret_cast<float4*>(sD)[i] =
+          gy < Hout && gx < Wout ? __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q)
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    const float4* xr = reinterpret_cast<const float4*>(sX[row + ky]);
+    const float* dr = sD + row * kDw1W * 32 + lane;
+    float w[24];
+    auto load = [&](int q, int k) {
+      const float4 v = xr[q];
+      w[4 * k] = v.x;
+      w[4 * k + 1] = v.y;
+      w[4 * k + 2] = v.z;
+      w[4 * k + 3] = v.w;
+    };
+    load(0, 0);
+    load(1, 1);
+    load(2, 2);
+#pragma unroll 1
+    for (int x = 0; x < kDw1W; x += 4) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) load(3 * (x / 4) + 3 + k, 3 + k);
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const float d = dr[(x + p) * 32];
+        if (ky == 0) bias += d;
+#pragma unroll
+        for (int k = 0; k < 15; ++k) acc[k] = fmaf(w[3 * p + k], d, acc[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < 12; ++k) w[k] = w[12 + k];
+    }
+  }
+  // the tile rows' sums in row order
+  float* sum = sD;
+  for (int r = 0; r < kDw1H; ++r) {
+    __syncthreads();
+    if (row == r) {
+#pragma unroll
+      for (int k = 0; k < 15; ++k) {
+        float* s = sum + (ky * 15 + k) * 32 + lane;
+        *s = r ? *s + acc[k] : acc[k];
+      }
+      if (ky == 0) {
+        float* s = sum + kNW1 + lane;
+        *s = r ? *s + bias : bias;
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < kDw1E; e += kDw1Threads) part[(size_t)blockIdx.x * kDw1E + e] = sum[e];
+}
+static_assert(kDw1E <= kDw1H * kDw1W * 32 && kDw1Row % 4 == 0, "the sums reuse the tile's memory");
+
+// g[e] = the sum over CTAs of part[cta][e]: eight interleaved runs of CTAs in
+// parallel, joined in order
+__global__ void __launch_bounds__(256)
+    k_reduce_parts(const float* __restrict__ part, int nparts, int ne, float* __restrict__ g) {
+  __shared__ float s[8][32];
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  float v = 0.f;
+  if (e < ne) {
+#pragma unroll 4
+    for (int k = r; k < nparts; k += 8) v += __ldg(part + (size_t)k * ne + e);
+  }
+  s[r][lane] = v;
+  __syncthreads();
+  if (r == 0 && e < ne) {
+#pragma unroll
+    for (int k = 1; k < 8; ++k) v += s[k][lane];
+    g[e] = v;
+  }
 }
 
 // ------------------------------------------------------------------ loss
@@ -1384,9 +1676,12 @@ struct sfm_surrogate {
   // activations for an image of (Hc + 2 kHalo) x (Wc + 2 kHalo) coarse cells
   int Hc = 0, Wc = 0;
   bf16 *X = nullptr, *A1 = nullptr, *A2 = nullptr, *A3 = nullptr;
+  // dA3, dA2, dA1: gradients of the layers' outputs before their ReLU
+  float* Xf = nullptr;  // an image as the caller gave it
   float *Y = nullptr, *T = nullptr, *dY = nullptr, *dA3 = nullptr, *dA2 = nullptr,
-        *dA1 = nullptr, *part = nullptr;
+        *dA1 = nullptr, *part = nullptr, *mse = nullptr;
   size_t part_cap = 0;
+  int mse_cap = 0;  // CTAs' squared errors
   // lattice-sized buffers
   size_t nsu = 0;
   float *Fnear = nullptr, *Fsur = nullptr;
@@ -1455,12 +1750,13 @@ void sfree(sfm_surrogate* S, void* p) {
 sfm_status ensure_image(sfm_surrogate* S, int Hc, int Wc) {
   if (S->Hc == Hc && S->Wc == Wc && S->X) return SFM_OK;
   for (void* q : {(void*)S->X, (void*)S->A1, (void*)S->A2, (void*)S->A3, (void*)S->Y, (void*)S->T,
-                  (void*)S->dY, (void*)S->dA3, (void*)S->dA2, (void*)S->dA1})
+                  (void*)S->dY, (void*)S->dA3, (void*)S->dA2, (void*)S->dA1, (void*)S->Xf})
     sfree(S, q);
   const size_t p0 = (size_t)(Hc + 2 * kHalo) * (Wc + 2 * kHalo);
   const size_t p1 = (size_t)(Hc + 6) * (Wc + 6), p2 = (size_t)(Hc + 4) * (Wc + 4),
                p3 = (size_t)(Hc + 2) * (Wc + 2), p4 = (size_t)Hc * Wc;
   STRY(salloc(S, &S->X, p0 * 3));
+  STRY(salloc(S, &S->Xf, p0 * 3));
   STRY(salloc(S, &S->A1, p1 * 32));
   STRY(salloc(S, &S->A2, p2 * 32));
   STRY(salloc(S, &S->A3, p3 * 32));
@@ -1475,43 +1771,58 @@ sfm_status ensure_image(sfm_surrogate* S, int Hc, int Wc) {
   return SFM_OK;
 }
 
-template <int CIN, int COUT, int K>
-size_t dx_smem() {
-  return ((size_t)K * K * CIN * COUT + (size_t)(kTile + K - 1) * (kTile + K - 1) * COUT) * 4;
-}
-template <int CIN, int COUT, int K>
-size_t dw_smem() {
-  return ((size_t)(kTile + K - 1) * (kTile + K - 1) * CIN + (size_t)kTile * kTile * COUT) * 4;
-}
+int sm_count() { return device_sm_count(); }
 
-template <int CIN, int COUT, int K, bool RELU>
-void conv_dx(const float* dA, const bf16* A, int Hout, int Wout, const float* W, float* dIn,
-             cudaStream_t s) {
-  const size_t sm = dx_smem<CIN, COUT, K>();
-  cudaFuncSetAttribute(k_conv_dx<CIN, COUT, K, RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sm);
-  dim3 grid(cdiv(Wout + K - 1, kTile), cdiv(Hout + K - 1, kTile));
-  k_conv_dx<CIN, COUT, K, RELU><<<grid, kTile * kTile, sm, s>>>(dA, A, Hout, Wout, W, dIn);
-}
-
-template <int CIN, int COUT, int K, bool RELU>
-sfm_status conv_dw(sfm_surrogate* S, const bf16* in, const float* dA, const bf16* A, int Hout,
-                   int Wout, float* gW, cudaStream_t s) {
-  constexpr int NE = K * K * CIN * COUT + COUT;
-  dim3 grid(cdiv(Wout, kTile), cdiv(Hout, kTile));
-  const size_t nparts = (size_t)grid.x * grid.y;
-  if (nparts * NE > S->part_cap) {
-    sfree(S, S->part);
-    STRY(salloc(S, &S->part, nparts * NE));
-    S->part_cap = nparts * NE;
-  }
-  const size_t sm = dw_smem<CIN, COUT, K>();
-  cudaFuncSetAttribute(k_conv_dw<CIN, COUT, K, RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sm);
-  k_conv_dw<CIN, COUT, K, RELU><<<grid, kTile * kTile, sm, s>>>(in, dA, A, Hout, Wout, S->part);
-  // W block then b block are adjacent in the flat gradient (W at kOffW, b right after)
-  k_reduce_parts<<<cdiv(NE, 256), 256, 0, s>>>(S->part, (int)nparts, NE, gW);
+// CTAs' partial sums of a weight gradient of ne entries
+sfm_status ensure_part(sfm_surrogate* S, size_t floats) {
+  if (floats <= S->part_cap) return SFM_OK;
+  sfree(S, S->part);
+  S->part = nullptr;
+  S->part_cap = 0;
+  STRY(salloc(S, &S->part, floats));
+  S->part_cap = floats;
   return SFM_OK;
+}
+
+void reduce_parts(sfm_surrogate* S, int nparts, int ne, float* g, cudaStream_t s) {
+  k_reduce_parts<<<cdiv(ne, 32), 256, 0, s>>>(S->part, nparts, ne, g);
+}
+
+// weight (and bias, next to them) gradients of the layers
+sfm_status conv3_dw(sfm_surrogate* S, const bf16* in, const float* dZ, int Hout, int Wout, float* g,
+                    cudaStream_t s) {
+  const int grid = std::min(cdiv(Wout, kDwW) * cdiv(Hout, kDwH), sm_count());
+  STRY(ensure_part(S, (size_t)grid * kDwE));
+  cudaFuncSetAttribute(k_conv3_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwSmem);
+  k_conv3_dw<<<grid, kDwThreads, kDwSmem, s>>>(in, dZ, Hout, Wout, S->part);
+  reduce_parts(S, grid, kDwE, g, s);
+  return SFM_OK;
+}
+
+sfm_status conv4_dw(sfm_surrogate* S, const bf16* in, const float* dY, int Hout, int Wout, float* g,
+                    cudaStream_t s) {
+  const int grid = std::min(cdiv(Wout + 2, kDw4W) * cdiv(Hout + 2, kDw4H), 6 * sm_count());
+  STRY(ensure_part(S, (size_t)grid * kDw4E));
+  k_conv4_dw<<<grid, 32 * kDw4H, 0, s>>>(in, dY, Hout, Wout, S->part);
+  reduce_parts(S, grid, kDw4E, g, s);
+  return SFM_OK;
+}
+
+sfm_status conv1_dw(sfm_surrogate* S, const bf16* in, const float* dZ, int Hout, int Wout, float* g,
+                    cudaStream_t s) {
+  const int grid = std::min(cdiv(Wout, kDw1W) * cdiv(Hout, kDw1H), 4 * sm_count());
+  STRY(ensure_part(S, (size_t)grid * kDw1E));
+  k_conv1_dw<<<grid, kDw1Threads, 0, s>>>(in, dZ, Hout, Wout, S->part);
+  reduce_parts(S, grid, kDw1E, g, s);
+  return SFM_OK;
+}
+
+// masked data gradient of a 3x3 32 -> 32 layer
+void conv3_dx(const float* dZ, int Hout, int Wout, const float* W, const bf16* Ain, float* dZin,
+              cudaStream_t s) {
+  const int grid = std::min(cdiv(Wout + 2, kDxW) * cdiv(Hout + 2, kDxH), sm_count());
+  cudaFuncSetAttribute(k_conv3_dx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDxSmem);
+  k_conv3_dx<<<grid, kDxThreads, kDxSmem, s>>>(dZ, Hout, Wout, W, Ain, dZin);
 }
 
 // 3x3 layer on the tensor cores: 32 -> 32 into out (BF16), or with yout
@@ -1621,28 +1932,31 @@ void forward(sfm_surrogate* S, cudaStream_t s) {
 sfm_status backward(sfm_surrogate* S, float* loss_out, cudaStream_t s) {
   const int Hc = S->Hc, Wc = S->Wc, n = Hc * Wc;
   const int nb = cdiv(n, 256);
-  if ((size_t)nb > S->part_cap) {
-    sfree(S, S->part);
-    STRY(salloc(S, &S->part, (size_t)nb));
-    S->part_cap = nb;
+  if (nb > S->mse_cap) {
+    sfree(S, S->mse);
+    S->mse = nullptr;
+    S->mse_cap = 0;
+    STRY(salloc(S, &S->mse, (size_t)nb));
+    S->mse_cap = nb;
   }
-  k_mse<<<nb, 256, 0, s>>>(S->Y, S->T, n, S->dY, S->part);
+  k_mse<<<nb, 256, 0, s>>>(S->Y, S->T, n, S->dY, S->mse);
+  const float* q = S->pq;
+  // layer 4 (linear), 3, 2, 1
+  STRY(conv4_dw(S, S->A3, S->dY, Hc, Wc, S->g + kOffW[3], s));
+  k_conv4_dx<<<cdiv((Hc + 2) * (Wc + 2) * 8, 256), 256, 0, s>>>(S->dY, Hc, Wc, q + kOffW[3], S->A3, S->dA3);
+  STRY(conv3_dw(S, S->A2, S->dA3, Hc + 2, Wc + 2, S->g + kOffW[2], s));
+  conv3_dx(S->dA3, Hc + 2, Wc + 2, q + kOffW[2], S->A2, S->dA2, s);
+  STRY(conv3_dw(S, S->A1, S->dA2, Hc + 4, Wc + 4, S->g + kOffW[1], s));
+  conv3_dx(S->dA2, Hc + 4, Wc + 4, q + kOffW[1], S->A1, S->dA1, s);
+  STRY(conv1_dw(S, S->X, S->dA1, Hc + 6, Wc + 6, S->g + kOffW[0], s));
+  SCU(cudaGetLastError());
+  // the loss last: the host waits for it once the gradients are under way
   std::vector<float> hp(nb);
-  SCU(cudaMemcpyAsync(hp.data(), S->part, nb * sizeof(float), cudaMemcpyDeviceToHost, s));
+  SCU(cudaMemcpyAsync(hp.data(), S->mse, nb * sizeof(float), cudaMemcpyDeviceToHost, s));
   SCU(cudaStreamSynchronize(s));
   double L = 0.0;
   for (float x : hp) L += x;
   if (loss_out) *loss_out = (float)(0.5 * L / n);
-  const float* q = S->pq;
-  // layer 4 (linear), 3, 2, 1
-  STRY((conv_dw<32, 1, 3, false>(S, S->A3, S->dY, nullptr, Hc, Wc, S->g + kOffW[3], s)));
-  conv_dx<32, 1, 3, false>(S->dY, nullptr, Hc, Wc, q + kOffW[3], S->dA3, s);
-  STRY((conv_dw<32, 32, 3, true>(S, S->A2, S->dA3, S->A3, Hc + 2, Wc + 2, S->g + kOffW[2], s)));
-  conv_dx<32, 32, 3, true>(S->dA3, S->A3, Hc + 2, Wc + 2, q + kOffW[2], S->dA2, s);
-  STRY((conv_dw<32, 32, 3, true>(S, S->A1, S->dA2, S->A2, Hc + 4, Wc + 4, S->g + kOffW[1], s)));
-  conv_dx<32, 32, 3, true>(S->dA2, S->A2, Hc + 4, Wc + 4, q + kOffW[1], S->dA1, s);
-  STRY((conv_dw<3, 32, 5, true>(S, S->X, S->dA1, S->A1, Hc + 6, Wc + 6, S->g + kOffW[0], s)));
-  SCU(cudaGetLastError());
   return SFM_OK;
 }
 
@@ -1896,13 +2210,12 @@ sfm_status umma_check(sfm_surrogate* S) {
   return SFM_OK;
 }
 
-// channel-planar FP32 image [3][Hin][Win] (host) into S->X (channel-last BF16)
+// channel-planar FP32 image [3][Hin][Win] (host) into S->X (channel-last
+// BF16), rounded on the device
 sfm_status upload_image(sfm_surrogate* S, int Hin, int Win, const float* X) {
-  std::vector<bf16> hx((size_t)Hin * Win * 3);
-  for (int c = 0; c < 3; ++c)
-    for (int i = 0; i < Hin * Win; ++i) hx[(size_t)i * 3 + c] = __float2bfloat16(X[(size_t)c * Hin * Win + i]);
-  SCU(cudaMemcpyAsync(S->X, hx.data(), hx.size() * sizeof(bf16), cudaMemcpyHostToDevice, S->stream));
-  SCU(cudaStreamSynchronize(S->stream));
+  const int n = Hin * Win;
+  SCU(cudaMemcpyAsync(S->Xf, X, (size_t)n * 3 * sizeof(float), cudaMemcpyHostToDevice, S->stream));
+  k_pack_x<<<cdiv(n, 256), 256, 0, S->stream>>>(S->Xf, n, S->X);
   return SFM_OK;
 }
 

@@ -103,6 +103,29 @@ def test_gradients_match_the_oracle_within_bf16_bound():
             assert cos >= 0.999, (li, cos)
 
 
+# Output sizes at the edges of the gradient kernels' tiles (8 x 64 and 4 x 64,
+# 3 and 4 rows or pixels of halo), one pixel, and more tiles than CTAs.  The
+# target is the network's own output but for the last row and column, which are
+# off by one: the gradients come from the edge alone.  Same BF16 bound as above,
+# doubled: the other pixels' BF16 noise (Y to 2e-2 of its scale) adds to the
+# edge's gradient of 1 a pixel.
+@pytest.mark.parametrize("hc,wc", [(1, 1), (1, 64), (4, 61), (9, 3), (8, 65), (3, 129), (613, 67)])
+def test_gradients_at_the_edges_of_the_tiles(hc, wc):
+    rng = np.random.default_rng(hc * 1000 + wc)
+    params = [(W, bf16(rng.normal(0, 0.05, b.shape))) for W, b in _rounded_params(3)]
+    X = bf16(rng.random((3, hc + 2 * OS.HALO, wc + 2 * OS.HALO)) * 0.3)
+    T = np.array(OS.forward(params, X)[0])
+    T[-1] -= 1.0
+    T[:, -1] -= 1.0
+    L_o, g_o = OS.loss_and_grad(params, X, T)
+    with sfm.Surrogate(params=sfm.flatten_params(params)) as s:
+        L_g, g_flat = s.grad(X, T)
+    assert L_g == pytest.approx(L_o, rel=4e-2)
+    for (gw_o, gb_o), (gw_g, gb_g) in zip(g_o, sfm.unflatten_params(g_flat)):
+        for a, b in ((gw_o, gw_g), (gb_o, gb_g)):
+            assert np.linalg.norm(a.ravel() - b.ravel()) <= 4e-2 * np.linalg.norm(a.ravel())
+
+
 @pytest.mark.parametrize("rn,taper", [(2, None), (6, 2.5)])
 def test_surrogate_field_matches_the_oracle_composition(rn, taper):
     """F_sur = F_static + (tapered) near part + scale * bilinear(network
