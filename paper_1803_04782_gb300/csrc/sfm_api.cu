@@ -120,7 +120,8 @@ sfm_status check_flags(sfm_ctx* ctx) {
 // ya-1 and yb (wrapped in periodic y) at out rows 0 and yb-ya+1.  Uses whole
 // tiles so every su is summed in the same order in every mode.  A crowded
 // lattice's rows come from the product, whose sums are exact.
-void launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int ring = 0) {
+void launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int ring = 0,
+                     bool early = false) {
   if (c->use_product()) {
     ProductArgs a = c->prod;
     a.out = out;
@@ -131,15 +132,16 @@ void launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int r
     launch_product(a, c->stream);
   } else {
     launch_field(c->geo, c->bin_start, c->rec, c->tables(), c->Fs, out, out_row0, lo, hi, c->ctr,
-                 c->stream, FarPart(), ring);
+                 c->stream, FarPart(), ring, early);
   }
   ++c->launches;
 }
 
-void field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos) {
+void field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos,
+                bool early = false) {
   const Geo& g = c->geo;
   if (!halos) {
-    launch_field_of(c, out, ya - main_off, ya, yb);
+    launch_field_of(c, out, ya - main_off, ya, yb, 0, early);
     return;
   }
   // one launch for the band and its in-lattice halo rows ya-1 and yb (out rows
@@ -153,43 +155,51 @@ void field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos
 
 // Pedestrian-list binning when the crowd is sparse: its cost follows the
 // pedestrians (tens of bytes each), the grid scan's the area (2 bytes per su).
+// A lattice of up to kBinsPrefix bins always takes the grid's two launches
+// (the list has five): a tick of 512 x 512 with a pedestrian on every 268th su
+// takes 33 us against 41 with the list, of 2048 x 2048 44.8 against 45.9; of
+// 4096 x 4096 134 against 114.
 bool bins_from_peds(const sfm_ctx* c) {
   if (c->binning) return c->binning == 2;
+  if (c->geo.nbx * c->geo.nby <= kBinsPrefix) return false;
   return (int64_t)c->n * 64 < (int64_t)c->geo.W * c->geo.H;
 }
 
-void run_bins(sfm_ctx* c) {
+void run_bins(sfm_ctx* c, bool early = false) {
   StageScope sc(c, SFM_STAGE_BIN);
   const Geo& g = c->geo;
-  // the bin scan: three passes, or one when a block covers every bin
-  const int scan_launches = scan_tmp_elems(g.nbx * g.nby) == 1 ? 1 : 3;
-  if (bins_from_peds(c)) {
-    launch_bins_from_peds(g, c->n, c->xy, c->alive, c->heading, c->bin_count, c->bin_start,
-                          c->scan_tmp, c->bin_slot, c->bin_key, c->rec, c->rec_id, c->stream);
-    c->launches += (c->n > 0 ? 3 : 0) + scan_launches;  // count, scan, scatter, rank
-    return;
-  }
-  launch_bin_count(g, c->ocls, c->bin_count, c->stream);
-  launch_scan(c->bin_count, c->bin_start, g.nbx * g.nby, c->scan_tmp, c->stream);
-  launch_bin_fill(g, c->ocls, c->occ, c->bin_start, c->rec, c->rec_id, c->stream);
-  c->launches += 2 + scan_launches;  // count, scan, fill
+  c->launches +=
+      bins_from_peds(c)
+          ? launch_bins_from_peds(g, c->n, c->xy, c->alive, c->heading, c->bin_count, c->bin_start,
+                                  c->scan_tmp, c->bin_slot, c->bin_key, c->rec, c->rec_id, c->stream)
+          : launch_bins_from_grid(g, c->ocls, c->occ, c->bin_count, c->bin_start, c->scan_tmp, c->rec,
+                                  c->rec_id, c->stream, early);
 }
 
+// One tick.  The kernels of the grid's binning, the gather and k_move start
+// while their predecessor ends (`early`): their launch, and the gather's table
+// copy, hide behind it; 26.8 -> 24.7 us a tick of a 100 x 100 lattice, 67.7 ->
+// 65.5 of 1000 x 200.  Decide, vote and commit, and the list's binning, do not:
+// blocks that start early pile up on the SMs that are free first (163 -> 186
+// us a tick of 4096 x 4096 at r = 40 with all of them early).
 void run_tick(sfm_ctx* c) {
   StageScope whole(c, SFM_STAGE_STEP);
   const Geo& g = c->geo;
   const Tables tb = c->tables();
   const int nbins = g.nbx * g.nby;
-  {
-    StageScope sc(c, SFM_STAGE_BIN);
-    launch_clear_dead(c->n, c->alive, c->choice, c->won, c->stream);
-    if (c->n > 0) ++c->launches;
-  }
-  run_bins(c);
+  const bool early = !c->timing && nbins <= kBinsPrefix && !bins_from_peds(c);
+  run_bins(c, early);
   if (c->bands <= 1) {
     {
       StageScope sc(c, SFM_STAGE_FIELD);
-      field_rows(c, c->F, 0, g.H, 0, false);
+      field_rows(c, c->F, 0, g.H, 0, false, early);
+    }
+    if (!c->timing && c->n > 0 && c->n <= kMoveMaxPeds) {
+      launch_move(c->n, c->rec_id, c->bin_start, c->xy, c->alive, c->heading, c->goal, c->cell, c->occ,
+                  c->ocls, c->D, c->F, g, c->prm.beta, c->prm.seed, tb, c->choice, c->won, c->ctr,
+                  c->stream, c->walk(), c->sizes(), c->ids(), early);
+      ++c->launches;
+      return;
     }
     StageScope sc(c, SFM_STAGE_DECIDE);
     launch_decide(c->n, c->rec_id, c->bin_start, 0, nbins, c->xy, c->heading, c->goal, c->cell,
@@ -244,8 +254,8 @@ void run_tick(sfm_ctx* c) {
   }
   {
     StageScope sc(c, SFM_STAGE_VOTE);
-    launch_vote(c->n, c->rec_id, c->bin_start, c->xy, c->choice, c->occ, g, c->prm.seed, c->ctr,
-                c->won, c->stream, c->sizes(), c->ids());
+    launch_vote(c->n, c->rec_id, c->bin_start, c->xy, c->alive, c->choice, c->occ, g, c->prm.seed,
+                c->ctr, c->won, c->stream, c->sizes(), c->ids());
     if (c->n > 0) ++c->launches;
   }
   StageScope sc(c, SFM_STAGE_COMMIT);

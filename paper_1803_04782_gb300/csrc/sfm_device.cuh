@@ -11,6 +11,15 @@
 
 namespace sfm {
 
+// Head of a kernel launched by launch_tick_kernel: the kernel after it may
+// start, and everything before this one is complete and visible.  Arrays that
+// change from tick to tick are no `const __restrict__` parameters of such
+// kernels, so that they are not read through the non-coherent path.
+__device__ __forceinline__ void tick_kernel_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // move offsets of the direction classes 0..8 and the class of the opposite move
 static __constant__ int c_dx[9] = {0, 1, 1, 0, -1, -1, -1, 0, 1};
 static __constant__ int c_dy[9] = {0, 0, 1, 1, 1, 0, -1, -1, -1};

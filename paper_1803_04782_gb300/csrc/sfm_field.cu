@@ -110,10 +110,9 @@ __device__ __forceinline__ void far_epilogue(const Geo& g, const FarPart& far, c
 
 template <int SP, int SHAPE, int FAR>
 __global__ void __launch_bounds__(kV2Threads, 1)
-    k_field_v2(Geo g, const int32_t* __restrict__ bin_start, const uint32_t* __restrict__ rec,
-               const float* __restrict__ CT, const float* __restrict__ Fs,
-               float* __restrict__ out, int out_row0, int fy0, int fy1, int store_lo,
-               int store_hi, FarPart far, unsigned int* __restrict__ tickets) {
+    k_field_v2(Geo g, const int32_t* bin_start, const uint32_t* rec, const float* __restrict__ CT,
+               const float* __restrict__ Fs, float* out, int out_row0, int fy0, int fy1,
+               int store_lo, int store_hi, FarPart far, unsigned int* tickets) {
   extern __shared__ __align__(16) float sm[];
   constexpr int FW = SHAPE ? 32 : 16, FH = 16, NJ = SHAPE ? 16 : 8;
   const int r = g.r;
@@ -128,6 +127,7 @@ __global__ void __launch_bounds__(kV2Threads, 1)
     copy_to_shared<12>(dst, src, 2 * TS);  // 4*TS floats
     if (threadIdx.x < kTableGuard) sm[threadIdx.x] = 0.f;
   }
+  tick_kernel_begin();  // the tables never change: copied while the binning still runs
   __syncthreads();
   const int wpb = blockDim.x >> 5;
   const int tw = gridDim.x * wpb;
@@ -228,7 +228,7 @@ static int g_num_sms = 0;
 template <int SP, int SHAPE, int FAR>
 static void launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const float* CT,
                       const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-                      cudaStream_t s, const FarPart& far, unsigned int* tickets) {
+                      cudaStream_t s, const FarPart& far, unsigned int* tickets, bool early) {
   constexpr int FW = SHAPE ? 32 : 16, FH = 16;
   const size_t smem = (kTableGuard + class_table_floats(g.r)) * sizeof(float) +
                       kV2Threads / 32 * 32 * sizeof(int2);
@@ -251,32 +251,31 @@ static void launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* re
   // warp or more); a small lattice keeps the static deal, without the
   // counter's atomics at the start and end of the launch
   if (nf < 4 * wpb * blocks) tickets = nullptr;
-  k_field_v2<SP, SHAPE, FAR><<<blocks, kV2Threads, smem, s>>>(g, bin_start, rec, CT, Fs, out, out_row0,
-                                                         fy0, fy1, store_lo, store_hi, far,
-                                                         tickets);
+  launch_tick_kernel(k_field_v2<SP, SHAPE, FAR>, blocks, kV2Threads, smem, s, early, g, bin_start, rec,
+                     CT, Fs, out, out_row0, fy0, fy1, store_lo, store_hi, far, tickets);
 }
 
 template <int SP>
 static void launch_v2_shape(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                             const Tables& tb, const float* Fs, float* out, int out_row0,
                             int store_lo, int store_hi, cudaStream_t s, const FarPart& far,
-                            unsigned int* tickets) {
+                            unsigned int* tickets, bool early) {
   // the far part (surrogate) has its own instantiations, 32 x 16 footprint
   // only (one for coarsening 8, one for any), so the exact gather carries no
   // code for it
   if (far.Y && far.s == 8)
-    launch_v2<SP, 1, 8>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets);
+    launch_v2<SP, 1, 8>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
   else if (far.Y)
-    launch_v2<SP, 1, 1>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets);
+    launch_v2<SP, 1, 1>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
   else if (tb.shape != kShape16x16)  // the row-trimmed shape where that gather is off
-    launch_v2<SP, 1, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets);
+    launch_v2<SP, 1, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
   else
-    launch_v2<SP, 0, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets);
+    launch_v2<SP, 0, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
 }
 
 void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
                   const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-                  Counters* ctr, cudaStream_t s, const FarPart& far, int ring) {
+                  Counters* ctr, cudaStream_t s, const FarPart& far, int ring, bool early) {
   if (store_hi <= store_lo) return;
   const int sp = tb.CT ? class_table_stride(g.r) : 0;
   if (!sp) {
@@ -290,17 +289,17 @@ void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, c
   // footprints per warp (launch_v2).
   unsigned int* tickets = ctr && !far.Y ? ctr->field_tickets : nullptr;
   if (!far.Y && launch_field_v3(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi,
-                                tickets, s, ring))
+                                tickets, s, ring, early))
     return;
   if (ring) return;  // the caller checked that the row-trimmed gather is in use
   switch (sp) {
-    case 34: launch_v2_shape<34>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
-    case 50: launch_v2_shape<50>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
-    case 66: launch_v2_shape<66>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
-    case 82: launch_v2_shape<82>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
-    case 98: launch_v2_shape<98>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
-    case 114: launch_v2_shape<114>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
-    default: launch_v2_shape<kNarrowStride>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets); break;
+    case 34: launch_v2_shape<34>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    case 50: launch_v2_shape<50>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    case 66: launch_v2_shape<66>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    case 82: launch_v2_shape<82>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    case 98: launch_v2_shape<98>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    case 114: launch_v2_shape<114>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    default: launch_v2_shape<kNarrowStride>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
   }
 }
 

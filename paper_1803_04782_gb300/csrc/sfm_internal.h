@@ -267,20 +267,24 @@ void launch_place_diff(int n, const int2* xy_prev, const uint8_t* alive_prev,
                        const uint8_t* goal, const uint8_t* alive, const uint8_t* cell, const Geo& g,
                        int32_t* occ, uint8_t* ocls, Counters* ctr, cudaStream_t s);
 
-void launch_bin_count(const Geo& g, const uint8_t* ocls, int32_t* count, cudaStream_t s);
+// `early`: launched while the kernel before it in the stream still runs
+// (programmatic dependent launch; launch_tick_kernel below).
 void launch_scan(const int32_t* in, int32_t* out, int n, int32_t* block_tmp, cudaStream_t s);
 int scan_tmp_elems(int n);
 // Records of each bin in row-major su order, and the pedestrian id of each
-// record (the per-pedestrian stages walk pedestrians in this spatial order).
-void launch_bin_fill(const Geo& g, const uint8_t* ocls, const int32_t* occ, const int32_t* start,
-                     uint32_t* rec, int32_t* rec_id, cudaStream_t s);
-// choice = won = 0 for pedestrians that are not alive.
-void launch_bins_from_peds(const Geo& g, int n, const int2* xy, const uint8_t* alive,
-                           const uint8_t* heading, int32_t* count, int32_t* start,
-                           int32_t* scan_tmp, int32_t* slot, uint32_t* key, uint32_t* rec,
-                           int32_t* rec_id, cudaStream_t s);
+// record (the per-pedestrian stages walk pedestrians in this spatial order),
+// from the class grid or from the pedestrian list.  Returns the kernels launched.
+int launch_bins_from_grid(const Geo& g, const uint8_t* ocls, const int32_t* occ, int32_t* count,
+                          int32_t* start, int32_t* scan_tmp, uint32_t* rec, int32_t* rec_id,
+                          cudaStream_t s, bool early = false);
+int launch_bins_from_peds(const Geo& g, int n, const int2* xy, const uint8_t* alive,
+                          const uint8_t* heading, int32_t* count, int32_t* start,
+                          int32_t* scan_tmp, int32_t* slot, uint32_t* key, uint32_t* rec,
+                          int32_t* rec_id, cudaStream_t s);
+// lattices of at most this many bins: binned from the class grid by two
+// launches instead of a count, a scan and a fill
+constexpr int kBinsPrefix = 4096;
 void launch_reset_counters(Counters* ctr, cudaStream_t s);
-void launch_clear_dead(int n, const uint8_t* alive, uint8_t* choice, uint8_t* won, cudaStream_t s);
 
 // Field gather; stores lattice rows y in [store_lo, store_hi) at
 // out[(y - out_row0) * W + x].  Every su is summed in the same order whatever
@@ -294,7 +298,8 @@ void launch_field_v1(const Geo& g, const int32_t* bin_start, const uint32_t* rec
 // (launch_field_v3 returns false otherwise)
 void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
                   const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-                  Counters* ctr, cudaStream_t s, const FarPart& far = FarPart(), int ring = 0);
+                  Counters* ctr, cudaStream_t s, const FarPart& far = FarPart(), int ring = 0,
+                  bool early = false);
 int class_table_stride(int r);
 size_t class_table_floats(int r);
 // taper_in < r: entries weighted by 1 up to Euclidean distance taper_in and
@@ -305,7 +310,8 @@ void launch_class_tables(int r, const sfm_params& p, float* T, cudaStream_t s,
 // radius, the tables or the footprint do not select it
 bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                      const Tables& tb, const float* Fs, float* out, int out_row0, int store_lo,
-                     int store_hi, unsigned int* tickets, cudaStream_t s, int ring = 0);
+                     int store_hi, unsigned int* tickets, cudaStream_t s, int ring = 0,
+                     bool early = false);
 void launch_class_tables3(int r, const sfm_params& p, float* T, cudaStream_t s);
 
 // The per-pedestrian stages visit the live pedestrians of bins [b_lo, b_hi)
@@ -330,13 +336,45 @@ void launch_decide(int n, const int32_t* rec_id, const int32_t* bin_start, int b
                    const Geo& g, float beta, const Tables& tb, uint8_t* choice, cudaStream_t s,
                    const WalkPeriods& wp = WalkPeriods(), const Sizes& sz = Sizes(),
                    const int32_t* occ = nullptr, Counters* ctr = nullptr, int ring = 0);
+// The vote also sets choice = won = 0 for pedestrians that are not alive.
 void launch_vote(int n, const int32_t* rec_id, const int32_t* bin_start, const int2* xy,
-                 const uint8_t* choice, const int32_t* occ, const Geo& g, uint64_t seed,
-                 Counters* ctr, uint8_t* won, cudaStream_t s, const Sizes& sz = Sizes(),
-                 const int32_t* gid = nullptr);
+                 const uint8_t* alive, uint8_t* choice, const int32_t* occ, const Geo& g,
+                 uint64_t seed, Counters* ctr, uint8_t* won, cudaStream_t s,
+                 const Sizes& sz = Sizes(), const int32_t* gid = nullptr);
 void launch_commit(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy,
                    uint8_t* alive, uint8_t* heading, const uint8_t* choice, const uint8_t* won,
                    const uint8_t* cell, int32_t* occ, uint8_t* ocls, const Geo& g, Counters* ctr,
                    cudaStream_t s, const Sizes& sz = Sizes());
+// Decide, vote and commit of a whole lattice (F: its rows) of n <=
+// kMoveMaxPeds pedestrian slots in one launch.
+constexpr int kMoveMaxPeds = 1024;
+void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy, uint8_t* alive,
+                 uint8_t* heading, const uint8_t* goal, const uint8_t* cell, int32_t* occ,
+                 uint8_t* ocls, const int32_t* D, const float* F, const Geo& g, float beta,
+                 uint64_t seed, const Tables& tb, uint8_t* choice, uint8_t* won, Counters* ctr,
+                 cudaStream_t s, const WalkPeriods& wp, const Sizes& sz, const int32_t* gid,
+                 bool early);
+
+// k<<<grid, block, smem, s>>>(args...), with `early` as a programmatic
+// dependent launch: its blocks start once every block of the kernel before it
+// has called tick_kernel_begin() (or ended), and its own tick_kernel_begin()
+// waits for that kernel's completion.  Every thread of a kernel launched so
+// calls it before it reads or writes anything that changes from tick to tick,
+// so a kernel that has passed it has all the work before it behind it.
+template <class... P, class... A>
+inline cudaError_t launch_tick_kernel(void (*k)(P...), int grid, int block, size_t smem,
+                                      cudaStream_t s, bool early, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
 
 }  // namespace sfm

@@ -688,28 +688,73 @@ void launch_place_scatter(int n, const int2* xy, const uint8_t* heading, const u
 // and therefore deterministic; one warp a bin.
 constexpr int kBinWarps = 4;  // bins a block: small blocks spread a small lattice's bins over the SMs
 
-__global__ void k_bin_count(Geo g, const uint8_t* __restrict__ ocls, int32_t* __restrict__ count) {
+__global__ void k_bin_count(Geo g, const uint8_t* ocls, int32_t* count) {
+  tick_kernel_begin();
   const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (b >= g.nbx * g.nby) return;
   const int c = bin_count_one(g, ocls, b % g.nbx, b / g.nbx, lane);
   if (lane == 0) count[b] = c;
 }
 
-__global__ void k_bin_fill(Geo g, const uint8_t* __restrict__ ocls, const int32_t* __restrict__ occ,
-                           const int32_t* __restrict__ start, uint32_t* __restrict__ rec,
-                           int32_t* __restrict__ rec_id) {
-  const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (b >= g.nbx * g.nby) return;
-  bin_fill_one(g, ocls, occ, start[b], rec, rec_id, b % g.nbx, b / g.nbx, threadIdx.x & 31);
+// launches of launch_scan: three passes, or one when a block covers all n
+static int scan_launches(int n) { return scan_tmp_elems(n) == 1 ? 1 : 3; }
+
+// SCANNED: a scan has put the bins' first slots into `start`; else a block adds
+// up the counts of the bins before its own and writes its part of `start`.
+template <bool SCANNED>
+__global__ void __launch_bounds__(32 * kBinWarps)
+    k_bin_fill(Geo g, const uint8_t* ocls, const int32_t* occ, const int32_t* count, int32_t* start,
+               uint32_t* rec, int32_t* rec_id) {
+  tick_kernel_begin();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nbins = g.nbx * g.nby, b0 = blockIdx.x * kBinWarps, b = b0 + warp;
+  int first = 0;
+  if (SCANNED) {
+    if (b < nbins) first = start[b];
+  } else {
+    __shared__ int sBefore[kBinWarps], sMine[kBinWarps];
+    int before = 0;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < b0; i += 32 * kBinWarps) before += count[i];
+    const int mine = b < nbins ? count[b] : 0;
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) {
+      sBefore[warp] = before;
+      sMine[warp] = mine;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kBinWarps; ++w) first += sBefore[w] + (w < warp ? sMine[w] : 0);
+    if (lane == 0 && b < nbins) {
+      start[b] = first;
+      if (b == nbins - 1) start[nbins] = first + mine;
+    }
+  }
+  if (b >= nbins) return;
+  bin_fill_one(g, ocls, occ, first, rec, rec_id, b % g.nbx, b / g.nbx, lane);
 }
 
-void launch_bin_count(const Geo& g, const uint8_t* ocls, int32_t* count, cudaStream_t s) {
-  k_bin_count<<<cdiv(g.nbx * g.nby, kBinWarps), 32 * kBinWarps, 0, s>>>(g, ocls, count);
-}
-
-void launch_bin_fill(const Geo& g, const uint8_t* ocls, const int32_t* occ, const int32_t* start,
-                     uint32_t* rec, int32_t* rec_id, cudaStream_t s) {
-  k_bin_fill<<<cdiv(g.nbx * g.nby, kBinWarps), 32 * kBinWarps, 0, s>>>(g, ocls, occ, start, rec, rec_id);
+// Launches, not work, are what binning a small lattice costs, so its scan is
+// part of the fill: a tick of a 100 x 100 lattice took 24.3 us with a scan of
+// its own and 21.4 without, one of 512 x 512 34.6 and 32.3, one of 2048 x 2048
+// (4096 bins, as many as the one-launch scan takes; a block then adds up 16 KB
+// of counts at most) 112.3 and 110.4.  Counting in the fill as well, each
+// block the bins before its own, gained nothing (21.5 us with 16 bins, 35.8
+// against 29.7 with 64).
+int launch_bins_from_grid(const Geo& g, const uint8_t* ocls, const int32_t* occ, int32_t* count,
+                          int32_t* start, int32_t* scan_tmp, uint32_t* rec, int32_t* rec_id,
+                          cudaStream_t s, bool early) {
+  const int nbins = g.nbx * g.nby, blocks = cdiv(nbins, kBinWarps), threads = 32 * kBinWarps;
+  launch_tick_kernel(k_bin_count, blocks, threads, 0, s, early, g, ocls, count);
+  if (nbins <= kBinsPrefix) {
+    launch_tick_kernel(k_bin_fill<false>, blocks, threads, 0, s, early, g, ocls, occ,
+                       count, start, rec, rec_id);
+    return 2;
+  }
+  launch_scan(count, start, nbins, scan_tmp, s);
+  launch_tick_kernel(k_bin_fill<true>, blocks, threads, 0, s, early, g, ocls, occ, count,
+                     start, rec, rec_id);
+  return 2 + scan_launches(nbins);
 }
 
 // The same records driven by the pedestrian list, for sparse crowds where
@@ -758,32 +803,18 @@ __global__ void k_binp_rank(int n, Geo g, const int2* __restrict__ xy,
   rec_id[s + rank] = p;
 }
 
-void launch_bins_from_peds(const Geo& g, int n, const int2* xy, const uint8_t* alive,
-                           const uint8_t* heading, int32_t* count, int32_t* start,
-                           int32_t* scan_tmp, int32_t* slot, uint32_t* key, uint32_t* rec,
-                           int32_t* rec_id, cudaStream_t s) {
+int launch_bins_from_peds(const Geo& g, int n, const int2* xy, const uint8_t* alive,
+                          const uint8_t* heading, int32_t* count, int32_t* start,
+                          int32_t* scan_tmp, int32_t* slot, uint32_t* key, uint32_t* rec,
+                          int32_t* rec_id, cudaStream_t s) {
   const int nbins = g.nbx * g.nby;
   cudaMemsetAsync(count, 0, (size_t)nbins * sizeof(int32_t), s);
   if (n > 0) k_binp_count<<<cdiv(n, 256), 256, 0, s>>>(n, g, xy, alive, count, slot);
   launch_scan(count, start, nbins, scan_tmp, s);
-  if (n > 0) {
-    k_binp_scatter<<<cdiv(n, 256), 256, 0, s>>>(n, g, xy, alive, slot, start, key);
-    k_binp_rank<<<cdiv(n, 256), 256, 0, s>>>(n, g, xy, alive, heading, start, key, rec, rec_id);
-  }
-}
-
-__global__ void k_clear_dead(int n, const uint8_t* __restrict__ alive, uint8_t* __restrict__ choice,
-                             uint8_t* __restrict__ won) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n && !alive[p]) {
-    choice[p] = 0;
-    won[p] = 0;
-  }
-}
-
-void launch_clear_dead(int n, const uint8_t* alive, uint8_t* choice, uint8_t* won, cudaStream_t s) {
-  if (n <= 0) return;
-  k_clear_dead<<<cdiv(n, 256), 256, 0, s>>>(n, alive, choice, won);
+  if (n <= 0) return scan_launches(nbins);
+  k_binp_scatter<<<cdiv(n, 256), 256, 0, s>>>(n, g, xy, alive, slot, start, key);
+  k_binp_rank<<<cdiv(n, 256), 256, 0, s>>>(n, g, xy, alive, heading, start, key, rec, rec_id);
+  return 3 + scan_launches(nbins);
 }
 
 // ------------------------------------------------------------------ scan
@@ -1153,12 +1184,21 @@ void launch_decide(int n, const int32_t* rec_id, const int32_t* bin_start, int b
 }
 
 // ------------------------------------------------------------ S4: vote
-// The election of sub-job k-3 (vote_one), over the live pedestrians in bin order.
-__global__ void k_vote(const int32_t* __restrict__ rec_id, const int32_t* __restrict__ bin_start,
-                       int nbins, const int2* __restrict__ xy, const uint8_t* __restrict__ choice,
-                       const int32_t* __restrict__ occ, Geo g, uint64_t seed, Counters* ctr,
-                       uint8_t* __restrict__ won, Sizes sz, const int32_t* __restrict__ gid) {
+// The election of sub-job k-3 (vote_one), over the live pedestrians in bin
+// order; and choice = won = 0 for the pedestrians that are not alive, which
+// nothing else here reads or writes (a launch of its own for them, before the
+// binning, took 2-3 us a tick).
+__global__ void k_vote(int n, const int32_t* __restrict__ rec_id,
+                       const int32_t* __restrict__ bin_start, int nbins,
+                       const int2* __restrict__ xy, const uint8_t* __restrict__ alive,
+                       uint8_t* __restrict__ choice, const int32_t* __restrict__ occ, Geo g,
+                       uint64_t seed, Counters* ctr, uint8_t* __restrict__ won, Sizes sz,
+                       const int32_t* __restrict__ gid) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n && !alive[i]) {
+    choice[i] = 0;
+    won[i] = 0;
+  }
   if (i >= bin_start[nbins]) return;
   const int regs = sz.w ? vote_one_sized(rec_id[i], g, xy, choice, occ, sz.w, sz.h, seed, ctr->t, won)
                         : vote_one(rec_id[i], 0, g, xy, choice, occ, seed, ctr->t, won, gid);
@@ -1167,12 +1207,12 @@ __global__ void k_vote(const int32_t* __restrict__ rec_id, const int32_t* __rest
 }
 
 void launch_vote(int n, const int32_t* rec_id, const int32_t* bin_start, const int2* xy,
-                 const uint8_t* choice, const int32_t* occ, const Geo& g, uint64_t seed,
-                 Counters* ctr, uint8_t* won, cudaStream_t s, const Sizes& sz,
+                 const uint8_t* alive, uint8_t* choice, const int32_t* occ, const Geo& g,
+                 uint64_t seed, Counters* ctr, uint8_t* won, cudaStream_t s, const Sizes& sz,
                  const int32_t* gid) {
   if (n <= 0) return;
-  k_vote<<<cdiv(n, 256), 256, 0, s>>>(rec_id, bin_start, g.nbx * g.nby, xy, choice, occ, g, seed,
-                                      ctr, won, sz, gid);
+  k_vote<<<cdiv(n, 256), 256, 0, s>>>(n, rec_id, bin_start, g.nbx * g.nby, xy, alive, choice, occ, g,
+                                      seed, ctr, won, sz, gid);
 }
 
 // ---------------------------------------------------------- S5: commit
@@ -1207,6 +1247,75 @@ void launch_commit(int n, const int32_t* rec_id, const int32_t* bin_start, int2*
   const int blocks = n > 0 ? cdiv(n, 256) : 1;
   k_commit<<<blocks, 256, 0, s>>>(rec_id, bin_start, g.nbx * g.nby, xy, alive, heading, choice,
                                   won, cell, occ, ocls, g, ctr, sz);
+}
+
+// ------------------------------------------------- S3 - S5 in one block
+// Decide, vote and commit of up to 1024 pedestrian slots, a thread each, with
+// a block barrier where the single stages have a launch.  Bound by the chain of
+// dependent reads (record, position, neighbourhood, rivals), which the stages
+// have as well; with two launches less, the shorter binning and the early
+// starts a tick of the 100 x 100 room with 200 pedestrians went from 32 to 25 us.
+__global__ void __launch_bounds__(kMoveMaxPeds)
+    k_move(int n, const int32_t* rec_id, const int32_t* bin_start, int nbins, int2* xy,
+           uint8_t* alive, uint8_t* heading, const uint8_t* __restrict__ goal,
+           const uint8_t* __restrict__ cell, int32_t* occ, uint8_t* ocls,
+           const int32_t* __restrict__ D, const float* F, Geo g, float beta, uint64_t seed,
+           const float* __restrict__ own, const float* __restrict__ dirdot, uint8_t* choice,
+           uint8_t* won, Counters* ctr, WalkPeriods wp, Sizes sz,
+           const int32_t* __restrict__ gid) {
+  tick_kernel_begin();
+  const int i = threadIdx.x;
+  const long long t = ctr->t;
+  const int p = i < bin_start[nbins] ? rec_id[i] : -1;
+  if (i < n && !alive[i]) {
+    choice[i] = 0;
+    won[i] = 0;
+  }
+  bool decided = false, tie = false;
+  if (p >= 0) {
+    decided = !(wp.period && t % wp.period[p] != wp.phase[p]);
+    choice[p] = decided ? decide_one<true>(p, g, xy, heading, goal, cell, ocls, D, F, 0, -1, -1, 0, 0,
+                                           g.H, beta, own, dirdot, sz.w, sz.h, occ, &tie)
+                        : (uint8_t)0;
+  }
+  __syncthreads();
+  int regs = 0;
+  if (p >= 0)
+    regs = sz.w ? vote_one_sized(p, g, xy, choice, occ, sz.w, sz.h, seed, t, won)
+                : vote_one(p, 0, g, xy, choice, occ, seed, t, won, gid);
+  __syncthreads();
+  bool moved = false, left = false;
+  if (p >= 0) {
+    if (sz.w)
+      commit_one_sized(p, g, xy, alive, heading, choice, won, cell, occ, ocls, sz.w, sz.h, moved, left);
+    else
+      commit_one(p, g, xy, alive, heading, choice, won, cell, occ, ocls, moved, left);
+  }
+  const unsigned nd = __popc(__ballot_sync(0xffffffffu, decided));
+  const unsigned nt = __popc(__ballot_sync(0xffffffffu, tie));
+  const unsigned nm = __popc(__ballot_sync(0xffffffffu, moved));
+  const unsigned nl = __popc(__ballot_sync(0xffffffffu, left));
+  regs = __reduce_max_sync(0xffffffffu, regs);
+  if ((i & 31) == 0) {
+    if (nd) atomicAdd(&ctr->decided, (unsigned long long)nd);
+    if (nt) atomicAdd(&ctr->near_ties, (unsigned long long)nt);
+    if (nm) atomicAdd(&ctr->moved, (unsigned long long)nm);
+    if (nl) atomicAdd(&ctr->exited, (unsigned long long)nl);
+    if (regs > 2) atomicMax(&ctr->max_registrants, regs);
+    if (regs > 8) atomicOr(&ctr->err, kErrEnroll);
+  }
+  if (i == 0) ctr->t = t + 1;
+}
+
+void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy, uint8_t* alive,
+                 uint8_t* heading, const uint8_t* goal, const uint8_t* cell, int32_t* occ,
+                 uint8_t* ocls, const int32_t* D, const float* F, const Geo& g, float beta,
+                 uint64_t seed, const Tables& tb, uint8_t* choice, uint8_t* won, Counters* ctr,
+                 cudaStream_t s, const WalkPeriods& wp, const Sizes& sz, const int32_t* gid,
+                 bool early) {
+  launch_tick_kernel(k_move, 1, 32 * cdiv(n, 32), 0, s, early, n, rec_id, bin_start, g.nbx * g.nby, xy,
+                     alive, heading, goal, cell, occ, ocls, D, F, g, beta, seed, tb.own, tb.dirdot,
+                     choice, won, ctr, wp, sz, gid);
 }
 
 }  // namespace sfm

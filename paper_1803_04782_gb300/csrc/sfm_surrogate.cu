@@ -2443,12 +2443,11 @@ sfm_status sfm_surrogate_step(sfm_surrogate* S, sfm_ctx* ctx, int32_t nsteps) {
   cudaStream_t st = ctx->stream;
   const Geo& g = ctx->geo;
   for (int i = 0; i < nsteps; ++i) {
-    launch_clear_dead(ctx->n, ctx->alive, ctx->choice, ctx->won, st);
     ctx_run_bins(ctx);
     if (!std::isinf(S->delta)) surrogate_far(S, ctx);  // delta = +inf: no network (exact tick)
     surrogate_decide(S, ctx, ctx->choice, nullptr, nullptr, true);
     k_count_fallbacks<<<1, 1, 0, st>>>(S->nflag, ctx->bin_start + g.nbx * g.nby, S->fb_dev);
-    launch_vote(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->choice, ctx->occ, g,
+    launch_vote(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->alive, ctx->choice, ctx->occ, g,
                 ctx->prm.seed, ctx->ctr, ctx->won, st, Sizes(), ctx->ids());
     launch_commit(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->alive, ctx->heading,
                   ctx->choice, ctx->won, ctx->cell, ctx->occ, ctx->ocls, g, ctx->ctr, st);

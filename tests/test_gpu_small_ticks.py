@@ -1,0 +1,59 @@
+"""The short launch sequences of small lattices against the long ones: bins
+from the class grid in one launch (64 bins), two (4096) or three and more, the
+pedestrian list's bins, and decide, vote and commit in one block (1024
+pedestrian slots) or three launches.  All leave the same bits."""
+import numpy as np
+import pytest
+
+import paper_1803_04782_gb300 as sfm
+from paper_1803_04782_gb300 import build as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+    sfm.lib()
+
+
+def _sim(W, H, n, periodic, walk):
+    rng = np.random.default_rng(W + H + n)
+    cell = np.zeros((H, W), np.uint8)
+    cell[:, W // 2] = 1
+    cell[H // 3:H // 2, W // 2] = 0
+    cell[0, W // 4:W // 2] = 2
+    s = sfm.Sim(W=W, H=H, cell=cell, periodic_x=periodic, periodic_y=periodic, r=5)
+    at = rng.choice(np.flatnonzero(cell.ravel() == 0), n, replace=False)
+    s.place(np.stack([at % W, at // W], 1).astype(np.int32), rng.integers(0, 9, n).astype(np.uint8),
+            rng.integers(0, 9, n).astype(np.uint8), (rng.random(n) < 0.9).astype(np.uint8))
+    if walk:
+        period = rng.integers(1, 4, n).astype(np.uint8)
+        s.set_walk_periods(period, (rng.integers(0, 4, n) % period).astype(np.uint8))
+    return s
+
+
+def _run(s, ticks=3):
+    s.step(ticks)
+    s.sync()
+    st = s.stats()
+    return [*s.peds(), *s.decisions(), s.field()], {
+        k: st[k] for k in ("t", "alive", "exited", "moved_total", "max_registrants", "decided", "near_ties")}
+
+
+@pytest.mark.parametrize("W,H,n,periodic,walk", [
+    (7, 5, 1, 0, False), (33, 31, 300, 1, False), (100, 100, 1024, 0, True), (100, 100, 1025, 1, True),
+    (256, 256, 1000, 0, False), (257, 256, 1023, 0, False), (2048, 2048, 70000, 1, False),
+    (2049, 2048, 70000, 0, False)])
+def test_short_and_long_launch_sequences_agree(W, H, n, periodic, walk):
+    got = []
+    for timing in (False, True):  # a timed tick runs stage by stage
+        for binning in ("grid", "peds", "auto"):
+            with _sim(W, H, n, periodic, walk) as s:
+                s.set_binning(binning)
+                s.set_timing(timing)
+                got.append(_run(s))
+    for arrays, stats in got[1:]:
+        assert stats == got[0][1]
+        for a, b in zip(arrays, got[0][0]):
+            np.testing.assert_array_equal(a, b)
