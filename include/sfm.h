@@ -261,13 +261,14 @@ sfm_status sfm_set_guidance(sfm_ctx* ctx, const int32_t* D, int32_t on_device);
  * every result are identical either way): 1 = by scanning the per-su class
  * grid (cost follows the lattice area), 2 = from the pedestrian list with
  * atomic counts and an in-bin rank (cost follows the crowd), 0 = automatic
- * (the default: the list when n * 64 < W * H).  Anything else is SFM_EINVAL. */
+ * (the default: the list when n * 64 < W * H and the lattice has more
+ * than 4096 bins).  Anything else is SFM_EINVAL. */
 sfm_status sfm_set_binning(sfm_ctx* ctx, int32_t mode);
 
 /* Sets the warp footprint of the field gather by hand: 0 = 16 x 16 su,
  * 1 = 32 x 16 su (every pedestrian visit reads all 16 rows), 2 = 32 x 32 su
- * on the row-trimmed gather (a visit reads only the 8-row blocks the window
- * reaches; radius 1..40, beyond which 2 runs as 1).  Anything else is
+ * on the row-trimmed gather (a visit reads only the blocks of 16 x 16 su the
+ * window reaches; radius 1..40, beyond which 2 runs as 1).  Anything else is
  * SFM_EINVAL.  Ignored (but accepted) when the interaction radius exceeds
  * the class-table gather (r > 50). */
 sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);

@@ -520,7 +520,7 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
   sfm_ctx* ctx = new sfm_ctx;
   ctx->lat = *lat;
   ctx->nsu_total = (int64_t)lat->W * lat->H;
-  ctx->field_shape = default_field_shape(prm->r);
+  ctx->field_shape = default_field_shape(prm->r, lat->W, lat->H);
   ctx->prm = *prm;
   ctx->prm.bin = kBin;
   ctx->stream = static_cast<cudaStream_t>(stream);

@@ -9,6 +9,9 @@
 
 namespace sfm {
 
+// streaming multiprocessors of the current device (its attribute, cached)
+int device_sm_count();
+
 constexpr int kFree = 0, kWall = 1, kExit = 2;
 constexpr int32_t kDInf = 1 << 23;  // guidance distance of unreachable su (and WALL su, as exported)
 // the guidance array's value on WALL su inside the library: it marks the su
@@ -70,17 +73,17 @@ static_assert((kTableGuard + max_class_table_floats(kMaxTableRadius)) * 4 +
               "class tables exceed shared memory");
 
 // Row-trimmed class-table gather (sfm_field3.cu): 32 x 32 su footprints,
-// lane = column, blocks of 8 rows.  Seven zero rows above
-// and below each window (a visit reads whole blocks) and at least 31 zero
-// columns after each row; the row stride is one of a few compile-time
-// classes.  Radius 1..40.
-constexpr int kField3PadRows = 7;
+// blocks of 16 columns x 16 rows.  Fifteen zero rows above and below each window
+// (a visit reads whole blocks) and at least 15 zero columns after each row; the
+// row stride is one of a few compile-time classes.  Radius 1..40.
+constexpr int kField3PadRows = 15;
+constexpr int kField3Threads = 896;
 constexpr int kShape16x16 = 0, kShape32x16 = 1, kShape32x32 = 2;
 constexpr int field3_stride(int r) {
-  // >= 2r + 32: zero columns for 32 lanes
+  // >= 2r + 16: zero columns for the 16 of a block
   if (r < 1 || r > 40) return 0;
   for (int sp = 48; sp <= 112; sp += 32)
-    if (sp >= 2 * r + 32) return sp;
+    if (sp >= 2 * r + 16) return sp;
   return 0;
 }
 constexpr size_t field3_table_floats(int r) {
@@ -92,7 +95,7 @@ constexpr size_t max_field3_table_floats() {
     m = field3_table_floats(r) > m ? field3_table_floats(r) : m;
   return m;
 }
-static_assert((kTableGuard + max_field3_table_floats()) * 4 + kV2Threads / 32 * 32 * 8 <=
+static_assert((kTableGuard + max_field3_table_floats()) * 4 + kField3Threads / 32 * 32 * 8 <=
                   227 * 1024,
               "row-trimmed gather tables exceed shared memory");
 // the row-trimmed footprint `shape` can run at radius r
@@ -168,9 +171,17 @@ struct Tables {
   int shape = 0;        // class-table gather footprint: kShape16x16 .. kShape32x32
 };
 
-// footprint of the class-table gather used when none has been tuned
-inline int default_field_shape(int r) {
-  return r > 30 ? (field3_stride(r) ? kShape32x32 : kShape32x16) : kShape16x16;
+// Footprint of the class-table gather used when none has been tuned: the
+// largest of which a lattice has enough to occupy the warps (18 of an SM's 28;
+// 2736 on 152 SMs).  32 x 32 against 16 x 16, bins and field, a pedestrian on
+// every 40th su: 2048^2 68 us against 81 at r = 20 and 146 against 169 at r =
+// 40, 1750^2 (3025 footprints) 59 and 66, 118 and 128; but 1500^2 (2209) 54 and
+// 50, 105 and 97, 1000^2 49 and 34, 92 and 55.  Beyond the 32 x 32's radii, 32 x
+// 16 at r = 45: 1250^2 (3160) 89 against 112, but 1000^2 (2016) 78 and 68.
+inline int default_field_shape(int r, int W, int H) {
+  const int64_t nx = (W + 31) / 32, enough = 18 * (int64_t)device_sm_count();
+  if (field3_stride(r)) return nx * ((H + 31) / 32) >= enough ? kShape32x32 : kShape16x16;
+  return r > 30 && nx * ((H + 15) / 16) >= enough ? kShape32x16 : kShape16x16;
 }
 
 // ---- crowded lattices (sfm_product.cu) ----
@@ -327,8 +338,6 @@ struct WalkPeriods {
   const Counters* ctr = nullptr;
 };
 
-// streaming multiprocessors of the current device (its attribute, cached)
-int device_sm_count();
 void launch_decide(int n, const int32_t* rec_id, const int32_t* bin_start, int b_lo, int b_hi,
                    const int2* xy, const uint8_t* heading, const uint8_t* goal,
                    const uint8_t* cell, const uint8_t* ocls, const int32_t* D, const float* F,

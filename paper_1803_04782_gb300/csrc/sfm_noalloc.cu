@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "sfm_internal.h"
@@ -32,7 +33,8 @@ constexpr size_t kNaScanTmp = kNaStart + kNaBins + 64;  // scan block totals
 constexpr size_t kNaErr = kNaScanTmp + 64;              // error word
 constexpr size_t kNaRec = kNaErr + 64;                  // bin records
 constexpr size_t kNaTables = kNaRec + kNaPeds;          // heading-class tables
-constexpr size_t kNaTableFloats = max_class_table_floats(SFM_NOALLOC_MAX_RADIUS);
+constexpr size_t kNaTableFloats =
+    std::max(max_class_table_floats(SFM_NOALLOC_MAX_RADIUS), max_field3_table_floats());
 constexpr size_t kNaWords = (kNaTables + kNaTableFloats + 63) / 64 * 64;
 
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNaWords];
@@ -138,10 +140,15 @@ extern "C" sfm_status sfm_field_noalloc(const sfm_lattice* lat, const sfm_params
   launch_scan(count, start, nbins, scan_tmp, s);
   if (n > 0)
     k_na_fill<<<(n + 255) / 256, 256, 0, s>>>(n, pxy, heading, alive, g, start, cursor, rec, err);
-  launch_class_tables(g.r, *prm, tables, s);
   Tables tb{};
   tb.CT = tables;
-  tb.shape = default_field_shape(g.r);
+  tb.shape = default_field_shape(g.r, g.W, g.H);
+  if (field3_shape_ok(tb.shape, g.r)) {  // in the layout of the gather that runs
+    tb.CT3 = tables;
+    launch_class_tables3(g.r, *prm, tables, s);
+  } else {
+    launch_class_tables(g.r, *prm, tables, s);
+  }
   launch_field(g, start, rec, tb, base, field, 0, 0, g.H, nullptr, s);
 
   uint32_t h_err = 0;
