@@ -201,6 +201,23 @@ void run_tick(sfm_ctx* c) {
       ++c->launches;
       return;
     }
+    if (c->n > 0 && !c->sized && move_by_bins(g.W, g.H, c->n)) {
+      {
+        StageScope sc(c, SFM_STAGE_DECIDE);
+        launch_decide_bins(g, c->bin_start, c->rec, c->rec_id, c->goal, c->ocls, c->D, c->F, c->prm.beta,
+                           tb, c->choice, c->stream, c->walk(), c->ctr);
+      }
+      {
+        StageScope sc(c, SFM_STAGE_VOTE);
+        launch_vote_bins(c->n, g, c->bin_start, c->rec, c->rec_id, c->alive, c->choice, c->occ,
+                         c->prm.seed, c->ctr, c->won, c->stream, c->ids());
+      }
+      StageScope sc(c, SFM_STAGE_COMMIT);
+      launch_commit_bins(g, c->bin_start, c->rec, c->rec_id, c->xy, c->alive, c->heading, c->cell, c->occ,
+                         c->ocls, c->ctr, c->stream);
+      c->launches += 3;
+      return;
+    }
     StageScope sc(c, SFM_STAGE_DECIDE);
     launch_decide(c->n, c->rec_id, c->bin_start, 0, nbins, c->xy, c->heading, c->goal, c->cell,
                   c->ocls, c->D, c->F, 0, -1, -1, 0, 0, g.H, g, c->prm.beta, tb, c->choice,

@@ -364,6 +364,24 @@ void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* x
                  cudaStream_t s, const WalkPeriods& wp, const Sizes& sz, const int32_t* gid,
                  bool early);
 
+// The same stages of a whole lattice of 1 x 1 pedestrians, a block a bin
+// (sfm_move.cu): the choice and the win are kept in the records as well.
+// From a pedestrian on every tenth su on: a tick at r = 3 of 2048 x 2048 takes
+// 142 us by bins against 150 by pedestrian at a density of 1/8, but 100 against
+// 93 at 1/16 (1000 x 1000: 52 and 54, 40 and 41).
+inline bool move_by_bins(int W, int H, int n) { return (int64_t)n * 10 >= (int64_t)W * H; }
+void launch_decide_bins(const Geo& g, const int32_t* bin_start, uint32_t* rec, const int32_t* rec_id,
+                        const uint8_t* goal, const uint8_t* ocls, const int32_t* D, const float* F,
+                        float beta, const Tables& tb, uint8_t* choice, cudaStream_t s,
+                        const WalkPeriods& wp, Counters* ctr);
+void launch_vote_bins(int n, const Geo& g, const int32_t* bin_start, uint32_t* rec,
+                      const int32_t* rec_id, const uint8_t* alive, uint8_t* choice, const int32_t* occ,
+                      uint64_t seed, Counters* ctr, uint8_t* won, cudaStream_t s, const int32_t* gid);
+void launch_commit_bins(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
+                        const int32_t* rec_id, int2* xy, uint8_t* alive, uint8_t* heading,
+                        const uint8_t* cell, int32_t* occ, uint8_t* ocls, Counters* ctr,
+                        cudaStream_t s);
+
 // k<<<grid, block, smem, s>>>(args...), with `early` as a programmatic
 // dependent launch: its blocks start once every block of the kernel before it
 // has called tick_kernel_begin() (or ended), and its own tick_kernel_begin()

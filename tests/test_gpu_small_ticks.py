@@ -1,7 +1,8 @@
 """The short launch sequences of small lattices against the long ones: bins
 from the class grid in one launch (64 bins), two (4096) or three and more, the
 pedestrian list's bins, and decide, vote and commit in one block (1024
-pedestrian slots) or three launches.  All leave the same bits."""
+pedestrian slots) or three launches; and those stages bin by bin against
+pedestrian by pedestrian.  All leave the same bits."""
 import numpy as np
 import pytest
 
@@ -57,3 +58,41 @@ def test_short_and_long_launch_sequences_agree(W, H, n, periodic, walk):
         assert stats == got[0][1]
         for a, b in zip(arrays, got[0][0]):
             np.testing.assert_array_equal(a, b)
+
+
+# Lattices whose last bins are ragged; 512 threads a bin up to twice the SMs in
+# bins, else 128.  The crowd is a dense clump across the (periodic) border.
+@pytest.mark.parametrize("W,H,periodic", [(121, 131, 0), (129, 127, 1), (40, 397, 1), (601, 581, 0),
+                                          (609, 577, 1)])
+@pytest.mark.parametrize("numbered", [False, True])
+def test_stages_by_bins_agree_with_stages_by_pedestrian(W, H, periodic, numbered):
+    """The per-bin stages run from a pedestrian slot per ten su on: the same
+    crowd without and with enough slots that are not alive."""
+    rng = np.random.default_rng(W * H)
+    n, slots = W * H // 12, W * H // 9
+    cell = np.zeros((H, W), np.uint8)
+    cell[H // 2, :] = 1
+    cell[:, 5] = 2
+    free = np.flatnonzero(cell.ravel() == 0)
+    x, y = free % W, free // W
+    edge = np.minimum(x, W - 1 - x) + np.minimum(y, H - 1 - y)
+    at = rng.permutation(free[np.argsort(edge, kind="stable")][:n * 5 // 4])[:n]
+    xy = np.stack([at % W, at // W], 1).astype(np.int32)
+    heading, goal = (rng.integers(0, 9, slots).astype(np.uint8) for _ in range(2))
+    period = rng.integers(1, 4, slots).astype(np.uint8)
+    phase = (rng.integers(0, 4, slots) % period).astype(np.uint8)
+    ids = rng.permutation(slots).astype(np.int32)
+    out = []
+    for m in (n, slots):
+        with sfm.Sim(W=W, H=H, cell=cell, periodic_x=periodic, periodic_y=periodic, r=4) as s:
+            pad = np.zeros((m - n, 2), np.int32)
+            s.place(np.concatenate([xy, pad]), heading[:m], goal[:m], (np.arange(m) < n).astype(np.uint8))
+            s.set_walk_periods(period[:m], phase[:m])
+            if numbered:
+                s.set_ids(ids[:m])
+            arrays, stats = _run(s, 4)
+            assert not np.any(arrays[2][n:]) and not np.any(arrays[3][n:]) and not np.any(arrays[4][n:])
+            out.append(([a if a.shape == (H, W) else a[:n] for a in arrays], stats))
+    assert out[0][1] == out[1][1] and out[0][1]["max_registrants"] > 2 and out[0][1]["exited"] > 0
+    for a, b in zip(*(o[0] for o in out)):
+        np.testing.assert_array_equal(a, b)
