@@ -187,7 +187,7 @@ __device__ __forceinline__ void batch_footprint(const BatchArgs& a, const BatchS
     float2 acc[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j] = make_float2(0.f, 0.f);
-    gather_footprint16<SP>(g, a.bin_start + sc.bin_off, a.rec, sT, sc.ts, scr, lane, x0, y0, acc);
+    gather_footprint16<SP>(g, a.bin_start + sc.bin_off, a.rec, sT, sc.ts, scr, lane, x0, y0, acc, true);
     const int x = x0 + (lane & 15), yl = y0 + (lane >> 4) * 8;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -201,7 +201,7 @@ __device__ __forceinline__ void batch_footprint(const BatchArgs& a, const BatchS
     float2 acc[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = make_float2(0.f, 0.f);
-    gather_footprint32<SP>(g, a.bin_start + sc.bin_off, a.rec, sT, sc.ts, scr, lane, x0, y0, acc);
+    gather_footprint32<SP>(g, a.bin_start + sc.bin_off, a.rec, sT, sc.ts, scr, lane, x0, y0, acc, true);
     const int x = x0 + lane;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {

@@ -112,7 +112,7 @@ template <int SP, int SHAPE, int FAR>
 __global__ void __launch_bounds__(kV2Threads, 1)
     k_field_v2(Geo g, const int32_t* bin_start, const uint32_t* rec, const float* __restrict__ CT,
                const float* __restrict__ Fs, float* out, int out_row0, int fy0, int fy1,
-               int store_lo, int store_hi, FarPart far, unsigned int* tickets) {
+               int store_lo, int store_hi, FarPart far, unsigned int* tickets, bool sorted) {
   extern __shared__ __align__(16) float sm[];
   constexpr int FW = SHAPE ? 32 : 16, FH = 16, NJ = SHAPE ? 16 : 8;
   const int r = g.r;
@@ -168,9 +168,9 @@ __global__ void __launch_bounds__(kV2Threads, 1)
 #pragma unroll
     for (int j = 0; j < NJ / 2; ++j) acc[j] = make_float2(0.f, 0.f);
     if constexpr (SHAPE)
-      gather_footprint32<SP>(g, bin_start, rec, sT, TS, scr, lane, x0, y0, acc);
+      gather_footprint32<SP>(g, bin_start, rec, sT, TS, scr, lane, x0, y0, acc, !FAR && sorted);
     else
-      gather_footprint16<SP>(g, bin_start, rec, sT, TS, scr, lane, x0, y0, acc);
+      gather_footprint16<SP>(g, bin_start, rec, sT, TS, scr, lane, x0, y0, acc, sorted);
     if constexpr (FAR) {
       far_epilogue<NJ, FAR>(g, far, fax, Fs, out, out_row0, store_lo, store_hi, x0 + x, y0, acc);
     } else {
@@ -223,12 +223,155 @@ __global__ void __launch_bounds__(kV2Threads, 1)
   }
 }
 
+// ------------------------------------ S2 (v2) with few footprints a warp
+// A lattice of few 16 x 16 footprints leaves the SMs' warps idle, and a warp's
+// own chain of dependent steps bounds the launch: bin starts, records, items,
+// then a table read and its adds a pedestrian.  Here half as many warps have
+// twice the registers: four pedestrians' reads are in flight at once (their
+// adds stay in record order: the same bits), and a batch's records are fetched
+// while the batch before it is added.  A mirrored pedestrian's rows are read in
+// ascending order like the others' and swapped in registers, so the reads of
+// the four need no branches.  Bins and field at r = 20, 16 x 16 footprints: 1000
+// x 200 with 60 000 pedestrians 132 -> 74 us, with 20 000 58 -> 39; 700 x 700
+// (1936 footprints) with 150 000 138 -> 105.  From 16 footprints an SM on
+// the 32 warps are faster: 800 x 800 (2500) 120 against 123 here, 1000 x 1000
+// at r = 12 97 against 109.  Sharing a footprint's rows between two or four
+// warps gained 2 % at most.
+constexpr int kFewThreads = 512, kFewPerSm = 16;
+
+template <int SP>
+__device__ __forceinline__ void few_load(const float* __restrict__ sT, int2 it, int col, int down, int up,
+                                         float (&v)[8]) {
+  const float* q = sT + it.x + ((it.y & 1024) ? -col : col) + ((it.y & 2048) ? up : down);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = q[k * SP];
+}
+
+__device__ __forceinline__ void few_add(const float (&v)[8], bool flip, float2 (&acc)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    acc[k] = __fadd2_rn(acc[k], make_float2(flip ? v[7 - 2 * k] : v[2 * k],
+                                            flip ? v[6 - 2 * k] : v[2 * k + 1]));
+}
+
+template <int SP>
+__global__ void __launch_bounds__(kFewThreads, 1)
+    k_field_few(Geo g, const int32_t* bin_start, const uint32_t* rec, const float* __restrict__ CT,
+                const float* __restrict__ Fs, float* out, int out_row0, int fy0, int fy1,
+                int store_lo, int store_hi, bool sorted) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int FW = 16, FH = 16, GROUP = 4;
+  const int r = g.r;
+  const int TS = (2 * r + 1 + 2 * kFieldPad) * SP;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* sT = sm + kTableGuard;
+  int2* scr = reinterpret_cast<int2*>(sT + 4 * TS) + warp * 32;
+  copy_to_shared<12>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
+  if (threadIdx.x < kTableGuard) sm[threadIdx.x] = 0.f;
+  tick_kernel_begin();  // the tables never change: copied while the binning still runs
+  __syncthreads();
+  const int nfx = (g.W + FW - 1) / FW, nf = nfx * (fy1 - fy0);
+  const int col = lane & 15, row0 = (lane >> 4) * 8, down = row0 * SP, up = -down - 7 * SP;
+  const unsigned lt = (1u << lane) - 1u;
+  // footprint f to CTA f % gridDim.x: one warp of every SM before a second
+  for (int f = blockIdx.x + gridDim.x * warp; f < nf; f += gridDim.x * (kFewThreads / 32)) {
+    const int x0 = (f % nfx) * FW, y0 = (fy0 + f / nfx) * FH;
+    float2 acc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = make_float2(0.f, 0.f);
+    const int xlo = x0 - r, xhi = x0 + FW - 1 + r, ylo = y0 - r, yhi = y0 + FH - 1 + r;
+    const int nxl = halo_count(xlo, xhi, g.W, g.px);
+    const int ne = nxl * halo_count(ylo, yhi, g.H, g.py);
+    for (int e0 = 0; e0 < ne; e0 += 32) {
+      // the walk of walk_records_box (sfm_gather.cuh), a batch ahead
+      const int e = e0 + lane;
+      int start = 0, cnt = 0, xoff = 0, yoff = 0;
+      if (e < ne) {
+        int bx, by;
+        halo_entry(e % nxl, xlo, xhi, g.W, g.px, x0, bx, xoff);
+        halo_entry(e / nxl, ylo, yhi, g.H, g.py, y0, by, yoff);
+        const int id = by * g.nbx + bx;
+        start = bin_start[id];
+        cnt = bin_start[id + 1] - start;
+        if (sorted) trim_rows(rec, start, cnt, -r - yoff, FH + r - yoff);
+      }
+      int inc = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      const int total = __shfl_sync(0xffffffffu, inc, 31), pre = inc - cnt;
+      uint32_t rc = 0;
+      int xo = 0, yo = 0;
+      auto fetch = [&](int q) {
+        int lo = 0;  // entry holding record q: the last lane whose prefix is <= q
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+          const int p = __shfl_sync(0xffffffffu, pre, lo + step);
+          if (p <= q) lo += step;
+        }
+        const int s_lo = __shfl_sync(0xffffffffu, start, lo);
+        const int p_lo = __shfl_sync(0xffffffffu, pre, lo);
+        xo = __shfl_sync(0xffffffffu, xoff, lo);
+        yo = __shfl_sync(0xffffffffu, yoff, lo);
+        if (q < total) rc = rec[s_lo + (q - p_lo)];
+      };
+      fetch(lane);
+      for (int q0 = 0; q0 < total; q0 += 32) {
+        bool keep = false;
+        int2 item = make_int2(0, 0);
+        if (q0 + lane < total) {
+          const int rx = xo + (int)(rc & 0xffu), ry = yo + (int)((rc >> 8) & 0xffu);
+          const int cls = (int)((rc >> 16) & 0xfu);
+          keep = ry >= -r && ry <= FH - 1 + r && rx >= -r && rx <= FW - 1 + r;
+          const int sx = class_sx(cls), sy = class_sy(cls);
+          item = make_int2(class_table(cls) * TS + (r + kFieldPad - sy * ry) * SP + r - sx * rx,
+                           (sx < 0 ? 1024 : 0) | (sy < 0 ? 2048 : 0));
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        const int m = __popc(bal);
+        if (keep) scr[__popc(bal & lt)] = item;
+        // up to whole groups with items that read the zero columns after a window
+        // (+ 0: no change)
+        if (lane < (-m & (GROUP - 1))) scr[m + lane] = make_int2(2 * r + 1, 0);
+        __syncwarp();
+        if (q0 + 32 < total) fetch(q0 + 32 + lane);
+        for (int j = 0; j < m; j += GROUP) {
+          int4 two[GROUP / 2];
+          float v[GROUP][8];
+#pragma unroll
+          for (int k = 0; k < GROUP / 2; ++k) two[k] = *reinterpret_cast<const int4*>(scr + j + 2 * k);
+#pragma unroll
+          for (int k = 0; k < GROUP / 2; ++k) {
+            few_load<SP>(sT, make_int2(two[k].x, two[k].y), col, down, up, v[2 * k]);
+            few_load<SP>(sT, make_int2(two[k].z, two[k].w), col, down, up, v[2 * k + 1]);
+          }
+#pragma unroll
+          for (int k = 0; k < GROUP / 2; ++k) {
+            few_add(v[2 * k], two[k].y & 2048, acc);
+            few_add(v[2 * k + 1], two[k].w & 2048, acc);
+          }
+        }
+        __syncwarp();
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int y = y0 + row0 + j, xx = x0 + col;
+      if (xx < g.W && y < g.H && y >= store_lo && y < store_hi)
+        out[(size_t)(y - out_row0) * g.W + xx] =
+            Fs[(size_t)y * g.W + xx] + ((j & 1) ? acc[j >> 1].y : acc[j >> 1].x);
+    }
+  }
+}
+
 static int g_num_sms = 0;
 
 template <int SP, int SHAPE, int FAR>
 static void launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const float* CT,
                       const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-                      cudaStream_t s, const FarPart& far, unsigned int* tickets, bool early) {
+                      cudaStream_t s, const FarPart& far, unsigned int* tickets, bool sorted, bool early) {
   constexpr int FW = SHAPE ? 32 : 16, FH = 16;
   const size_t smem = (kTableGuard + class_table_floats(g.r)) * sizeof(float) +
                       kV2Threads / 32 * 32 * sizeof(int2);
@@ -247,30 +390,39 @@ static void launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* re
   int blocks = nf < 4 * wpb * g_num_sms ? nf : (nf + wpb - 1) / wpb;
   if (blocks > g_num_sms) blocks = g_num_sms;
   if (blocks < 1) blocks = 1;
+  if constexpr (SHAPE == 0 && FAR == 0 && SP != kNarrowStride) {
+    if (nf <= kFewPerSm * g_num_sms) {
+      const size_t few = (kTableGuard + class_table_floats(g.r)) * sizeof(float) + kFewThreads * sizeof(int2);
+      cudaFuncSetAttribute(k_field_few<SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)few);
+      launch_tick_kernel(k_field_few<SP>, blocks, kFewThreads, few, s, early, g, bin_start, rec, CT, Fs, out,
+                         out_row0, fy0, fy1, store_lo, store_hi, sorted);
+      return;
+    }
+  }
   // tickets only where there are whole rounds to rebalance (4 footprints per
   // warp or more); a small lattice keeps the static deal, without the
   // counter's atomics at the start and end of the launch
   if (nf < 4 * wpb * blocks) tickets = nullptr;
   launch_tick_kernel(k_field_v2<SP, SHAPE, FAR>, blocks, kV2Threads, smem, s, early, g, bin_start, rec,
-                     CT, Fs, out, out_row0, fy0, fy1, store_lo, store_hi, far, tickets);
+                     CT, Fs, out, out_row0, fy0, fy1, store_lo, store_hi, far, tickets, sorted);
 }
 
 template <int SP>
 static void launch_v2_shape(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                             const Tables& tb, const float* Fs, float* out, int out_row0,
                             int store_lo, int store_hi, cudaStream_t s, const FarPart& far,
-                            unsigned int* tickets, bool early) {
+                            unsigned int* tickets, bool sorted, bool early) {
   // the far part (surrogate) has its own instantiations, 32 x 16 footprint
   // only (one for coarsening 8, one for any), so the exact gather carries no
   // code for it
   if (far.Y && far.s == 8)
-    launch_v2<SP, 1, 8>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
+    launch_v2<SP, 1, 8>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
   else if (far.Y)
-    launch_v2<SP, 1, 1>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
+    launch_v2<SP, 1, 1>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
   else if (tb.shape != kShape16x16)  // the row-trimmed shape where that gather is off
-    launch_v2<SP, 1, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
+    launch_v2<SP, 1, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
   else
-    launch_v2<SP, 0, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early);
+    launch_v2<SP, 0, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
 }
 
 void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
@@ -288,18 +440,21 @@ void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, c
   // that one ticket each would queue on the counter.  So do lattices under 4
   // footprints per warp (launch_v2).
   unsigned int* tickets = ctr && !far.Y ? ctr->field_tickets : nullptr;
+  // a context's bins are sorted by row; those of the allocation-free field,
+  // which has none, are in order of arrival
+  const bool sorted = ctr != nullptr;
   if (!far.Y && launch_field_v3(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi,
-                                tickets, s, ring, early))
+                                tickets, sorted, s, ring, early))
     return;
   if (ring) return;  // the caller checked that the row-trimmed gather is in use
   switch (sp) {
-    case 34: launch_v2_shape<34>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
-    case 50: launch_v2_shape<50>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
-    case 66: launch_v2_shape<66>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
-    case 82: launch_v2_shape<82>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
-    case 98: launch_v2_shape<98>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
-    case 114: launch_v2_shape<114>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
-    default: launch_v2_shape<kNarrowStride>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, early); break;
+    case 34: launch_v2_shape<34>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    case 50: launch_v2_shape<50>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    case 66: launch_v2_shape<66>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    case 82: launch_v2_shape<82>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    case 98: launch_v2_shape<98>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    case 114: launch_v2_shape<114>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    default: launch_v2_shape<kNarrowStride>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
   }
 }
 

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kField3Threads, 1)
     k_field_v3(Geo g, const int32_t* bin_start, const uint32_t* rec,
                const float* __restrict__ CT3, const float* __restrict__ Fs, float* out,
                int out_row0, int fy0, int fy1, int store_lo, int store_hi, unsigned int* tickets,
-               int ring) {
+               bool sorted, int ring) {
   static_assert(FH % kBlockRows == 0 && FH / kBlockRows <= 8, "footprint height: whole blocks, at most 8");
   static_assert(SP % 32 == 16, "a read's two rows on different banks");
   // launched only for radii whose row stride class SP >= 2r + 16 (launch_field_v3)
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kField3Threads, 1)
             add_blocks<SP, NB, NG>(p + odd * SP, u, left);
             add_blocks<SP, NB, NG>(q + odd * SP, u >> NB, right);
           }
-        });
+        }, sorted);
     // eight static-field reads in flight
 #pragma unroll
     for (int j0 = 0; j0 < FH; j0 += 8) {
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kField3Threads, 1)
 template <int SP, int FH>
 void launch_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const float* CT3,
                const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-               cudaStream_t s, unsigned int* tickets, int ring, bool early) {
+               cudaStream_t s, unsigned int* tickets, bool sorted, int ring, bool early) {
   constexpr int FW = 32;
   const size_t smem = (kTableGuard + field3_table_floats(g.r)) * sizeof(float) +
                       kField3Threads / 32 * 32 * sizeof(int2);
@@ -210,7 +210,7 @@ void launch_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec, cons
   if (blocks < 1) blocks = 1;
   if (nf < 4 * wpb * blocks) tickets = nullptr;
   launch_tick_kernel(k_field_v3<SP, FH>, blocks, kField3Threads, smem, s, early, g, bin_start, rec, CT3, Fs,
-                     out, out_row0, fy0, fy1, store_lo, store_hi, tickets, ring);
+                     out, out_row0, fy0, fy1, store_lo, store_hi, tickets, sorted, ring);
 }
 
 // the class tables in the layout of the row-trimmed gather: [4][2r+3][SP],
@@ -230,10 +230,10 @@ __global__ void k_class_tables3(int r, int SP, double kP, double aP, double gamm
 
 bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                      const Tables& tb, const float* Fs, float* out, int out_row0, int store_lo,
-                     int store_hi, unsigned int* tickets, cudaStream_t s, int ring, bool early) {
+                     int store_hi, unsigned int* tickets, bool sorted, cudaStream_t s, int ring, bool early) {
   if (!tb.CT3 || !field3_shape_ok(tb.shape, g.r)) return false;
 #define SFM_V3(SP) \
-  case SP: launch_v3<SP, 32>(g, bin_start, rec, tb.CT3, Fs, out, out_row0, store_lo, store_hi, s, tickets, ring, early); break;
+  case SP: launch_v3<SP, 32>(g, bin_start, rec, tb.CT3, Fs, out, out_row0, store_lo, store_hi, s, tickets, sorted, ring, early); break;
   // one footprint: 32 x 32 su (measured against 32 x 16 and 16 x 32 row-
   // trimmed footprints, it was the fastest on the 16384^2 floor at r = 40)
   switch (field3_stride(g.r)) {

@@ -91,6 +91,31 @@ __device__ __forceinline__ void add_row_pairs(const float* __restrict__ p, float
     acc[k] = __fadd2_rn(acc[k], make_float2(p[2 * k * S], p[(2 * k + 1) * S]));
 }
 
+// Records of rec[0, n), sorted by row, whose row is below `row`.
+__device__ __forceinline__ int rows_below(const uint32_t* rec, int n, int row) {
+  int lo = 0;
+  while (n > 0) {
+    const int h = n >> 1;
+    const bool below = (int)((rec[lo + h] >> 8) & 0xffu) < row;
+    lo = below ? lo + h + 1 : lo;
+    n = below ? n - h - 1 : h;
+  }
+  return lo;
+}
+
+// The records [start, start + cnt) of a bin, sorted by row, that lie in its
+// rows [row_lo, row_hi).  A window meets a third to a half of the rows of the
+// bins that it touches; a search costs two dependent reads for each doubling,
+// so a bin that a batch or two of 32 records covers is left whole.
+__device__ __forceinline__ void trim_rows(const uint32_t* rec, int& start, int& cnt, int row_lo,
+                                          int row_hi) {
+  if (cnt <= 32) return;
+  const int end = row_hi < kBin ? rows_below(rec + start, cnt, row_hi) : cnt;
+  const int skip = row_lo > 0 ? rows_below(rec + start, end, row_lo) : 0;
+  start += skip;
+  cnt = end - skip;
+}
+
 // Visits, in bin-walk order (halo bins row-major, records in bin order), the
 // records within reach (Chebyshev r) of some su of the FW x FH window at
 // (x0, y0): a batch of 32 records is fetched lane-parallel, each lane turns
@@ -102,7 +127,8 @@ __device__ __forceinline__ void add_row_pairs(const float* __restrict__ p, float
 template <class Make, class Visit>
 __device__ __forceinline__ void walk_records_box(const Geo& g, const int32_t* __restrict__ bin_start,
                                                  const uint32_t* __restrict__ rec, int2* scr, int lane,
-                                                 int x0, int y0, int FW, int FH, Make make, Visit visit) {
+                                                 int x0, int y0, int FW, int FH, Make make, Visit visit,
+                                                 bool sorted = false) {
   const int r = g.r;
   const unsigned lt = (1u << lane) - 1u;
   const int xlo = x0 - r, xhi = x0 + FW - 1 + r, ylo = y0 - r, yhi = y0 + FH - 1 + r;
@@ -118,6 +144,7 @@ __device__ __forceinline__ void walk_records_box(const Geo& g, const int32_t* __
       const int id = by * g.nbx + bx;
       start = bin_start[id];
       cnt = bin_start[id + 1] - start;
+      if (sorted) trim_rows(rec, start, cnt, -r - yoff, FH + r - yoff);
     }
     int inc = cnt;
 #pragma unroll
@@ -171,8 +198,9 @@ __device__ __forceinline__ void walk_records_box(const Geo& g, const int32_t* __
 template <int FW, int FH, class Make, class Visit>
 __device__ __forceinline__ void walk_records(const Geo& g, const int32_t* __restrict__ bin_start,
                                              const uint32_t* __restrict__ rec, int2* scr, int lane,
-                                             int x0, int y0, Make make, Visit visit) {
-  walk_records_box(g, bin_start, rec, scr, lane, x0, y0, FW, FH, make, visit);
+                                             int x0, int y0, Make make, Visit visit,
+                                             bool sorted = false) {
+  walk_records_box(g, bin_start, rec, scr, lane, x0, y0, FW, FH, make, visit, sorted);
 }
 
 // The footprint gather's walk: items carry the table offset of the
@@ -180,14 +208,14 @@ __device__ __forceinline__ void walk_records(const Geo& g, const int32_t* __rest
 template <int SP, int FW, int FH, class Visit>
 __device__ __forceinline__ void walk_footprint(const Geo& g, const int32_t* __restrict__ bin_start,
                                                const uint32_t* __restrict__ rec, int TS, int2* scr,
-                                               int lane, int x0, int y0, Visit visit) {
+                                               int lane, int x0, int y0, Visit visit, bool sorted) {
   const int r = g.r;
   walk_records<FW, FH>(g, bin_start, rec, scr, lane, x0, y0, [&](int rx, int ry, int cls) {
     const int sx = c_csx[cls], sy = c_csy[cls];
     const int llo = max(0, rx - r), lhi = min(FW - 1, rx + r);
     return make_int2(c_ctab[cls] * TS + (r + kFieldPad - sy * ry) * SP + r - sx * rx,
                      llo | (lhi << 5) | (sx < 0 ? 1024 : 0) | (sy < 0 ? 2048 : 0));
-  }, visit);
+  }, visit, sorted);
 }
 
 // Adds the pedestrian field of the 16 x 16 footprint at (x0, y0): lane l owns
@@ -204,7 +232,8 @@ template <int SP>
 __device__ __forceinline__ void gather_footprint16(const Geo& g, const int32_t* __restrict__ bin_start,
                                                    const uint32_t* __restrict__ rec,
                                                    const float* __restrict__ sT, int TS, int2* scr,
-                                                   int lane, int x0, int y0, float2 (&acc)[4]) {
+                                                   int lane, int x0, int y0, float2 (&acc)[4],
+                                                   bool sorted = false) {
   const int col = lane & 15, hoff = (lane >> 4) * 8 * SP;
   walk_footprint<SP, 16, 16>(g, bin_start, rec, TS, scr, lane, x0, y0, [&](const int2 it) {
     const int llo = it.y & 31, lhi = (it.y >> 5) & 31;
@@ -215,7 +244,7 @@ __device__ __forceinline__ void gather_footprint16(const Geo& g, const int32_t* 
       else
         add_row_pairs<SP, 4, false>(p + hoff, acc);
     }
-  });
+  }, sorted);
 }
 
 // The 32 x 16 footprint: lane l owns column x0 + l and rows y0 + j, j < 16,
@@ -224,7 +253,8 @@ template <int SP>
 __device__ __forceinline__ void gather_footprint32(const Geo& g, const int32_t* __restrict__ bin_start,
                                                    const uint32_t* __restrict__ rec,
                                                    const float* __restrict__ sT, int TS, int2* scr,
-                                                   int lane, int x0, int y0, float2 (&acc)[8]) {
+                                                   int lane, int x0, int y0, float2 (&acc)[8],
+                                                   bool sorted = false) {
   walk_footprint<SP, 32, 16>(g, bin_start, rec, TS, scr, lane, x0, y0, [&](const int2 it) {
     const int llo = it.y & 31, lhi = (it.y >> 5) & 31;
     if (SP != kNarrowStride || (lane >= llo && lane <= lhi)) {
@@ -234,7 +264,7 @@ __device__ __forceinline__ void gather_footprint32(const Geo& g, const int32_t* 
       else
         add_row_pairs<SP, 8, false>(p, acc);
     }
-  });
+  }, sorted);
 }
 
 // The far part (see FarPart), split into a column part (per lane, once per

@@ -321,7 +321,7 @@ void launch_class_tables(int r, const sfm_params& p, float* T, cudaStream_t s,
 // radius, the tables or the footprint do not select it
 bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                      const Tables& tb, const float* Fs, float* out, int out_row0, int store_lo,
-                     int store_hi, unsigned int* tickets, cudaStream_t s, int ring = 0,
+                     int store_hi, unsigned int* tickets, bool sorted, cudaStream_t s, int ring = 0,
                      bool early = false);
 void launch_class_tables3(int r, const sfm_params& p, float* T, cudaStream_t s);
 

@@ -2,7 +2,8 @@
 from the class grid in one launch (64 bins), two (4096) or three and more, the
 pedestrian list's bins, and decide, vote and commit in one block (1024
 pedestrian slots) or three launches; and those stages bin by bin against
-pedestrian by pedestrian.  All leave the same bits."""
+pedestrian by pedestrian; and the gather of few footprints against the
+others.  All leave the same bits."""
 import numpy as np
 import pytest
 
@@ -96,3 +97,26 @@ def test_stages_by_bins_agree_with_stages_by_pedestrian(W, H, periodic, numbered
     assert out[0][1] == out[1][1] and out[0][1]["max_registrants"] > 2 and out[0][1]["exited"] > 0
     for a, b in zip(*(o[0] for o in out)):
         np.testing.assert_array_equal(a, b)
+
+
+# 16 x 16 footprints: up to 16 an SM (2432 on 152 SMs; 784^2 has 2401, 800^2
+# 2500) four pedestrians are gathered at a time; full bins (over 32 records) are
+# cut to the rows in reach.  One radius of each table stride the gather has.
+@pytest.mark.parametrize("W,H,rho,r,periodic", [
+    (3, 3, 0.4, 1, 1), (31, 33, 0.4, 1, 0), (83, 85, 0.4, 41, 1), (50, 70, 0.03, 9, 0), (97, 130, 0.3, 17, 1),
+    (784, 784, 0.3, 25, 0), (800, 800, 0.3, 25, 1), (784, 784, 0.01, 33, 1), (300, 200, 0.2, 40, 0),
+    (300, 200, 0.2, 45, 0)])
+def test_footprints_agree_on_either_side_of_the_few(W, H, rho, r, periodic):
+    rng = np.random.default_rng(r)
+    n = max(1, int(rho * W * H))
+    at = rng.choice(W * H, n, replace=False)
+    fields = []
+    with sfm.Sim(W=W, H=H, cell=np.zeros((H, W), np.uint8), periodic_x=periodic, periodic_y=periodic, r=r) as s:
+        s.place(np.stack([at % W, at // W], 1).astype(np.int32), rng.integers(0, 9, n).astype(np.uint8),
+                np.zeros(n, np.uint8))
+        for shape in ("16x16", "32x16", "32x32r"):
+            s.set_footprint(shape)
+            s.compute_field()
+            fields.append(s.field())
+    for f in fields[1:]:
+        np.testing.assert_array_equal(f, fields[0])
