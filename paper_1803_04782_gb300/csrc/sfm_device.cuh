@@ -203,22 +203,41 @@ __device__ __forceinline__ bool rect_su(const Geo& g, int cx, int cy, int i, int
   return true;
 }
 
-// Every su that the rectangle of half sides (a, b) centred on (x, y) newly
-// enters when its centre moves by class k is inside, not WALL and not
-// covered by a pedestrian (occ < 0) at tick start.
-__device__ __forceinline__ bool strip_free(const Geo& g, const uint8_t* __restrict__ cell,
-                                           const int32_t* __restrict__ occ, int x, int y, int a,
-                                           int b, int k) {
-  const int dx = move_dx(k), dy = move_dy(k);
-  for (int j = -b; j <= b; ++j)
-    for (int i = -a; i <= a; ++i) {
-      const int ox = i + dx, oy = j + dy;  // offset from the old centre
-      if (ox >= -a && ox <= a && oy >= -b && oy <= b) continue;
-      size_t s;
-      if (!rect_su(g, x, y, ox, oy, s)) return false;
-      if (cell[s] == kWall || occ[s] >= 0) return false;
-    }
-  return true;
+// The moves that a rectangle of half sides (a, b) centred on (x, y) may not make
+// (bit k for class k): some su that it newly enters is outside, WALL or covered
+// by a pedestrian (occ < 0: none) at tick start.  Those su lie on the ring around
+// the rectangle, which is read once for all eight moves and with its reads in
+// flight together: a diagonal move enters a corner and the two sides next to it
+// but for their far ends.  `sub` of LANES lanes reads every LANES-th su; the
+// moves are the OR of the lanes'.
+template <int LANES>
+__device__ __forceinline__ uint32_t blocked_moves(const Geo& g, const uint8_t* __restrict__ cell,
+                                                  const int32_t* __restrict__ occ, int x, int y, int a,
+                                                  int b, int sub) {
+  auto blocked = [&](int ox, int oy) {
+    size_t s;
+    const bool in = rect_su(g, x, y, ox, oy, s);
+    return !in || cell[s] == kWall || occ[s] >= 0;
+  };
+  uint32_t m = 0;
+#pragma unroll LANES == 1 ? 3 : 1
+  for (int j = sub - b; j <= b; j += LANES) {
+    const uint32_t up = j > -b, down = j < b;
+    const bool e = blocked(a + 1, j), w = blocked(-a - 1, j);
+    m |= e ? 1u << 1 | up << 2 | down << 8 : 0u;
+    m |= w ? 1u << 5 | up << 4 | down << 6 : 0u;
+  }
+#pragma unroll LANES == 1 ? 3 : 1
+  for (int i = sub - a; i <= a; i += LANES) {
+    const uint32_t right = i > -a, left = i < a;
+    const bool n = blocked(i, b + 1), s = blocked(i, -b - 1);
+    m |= n ? 1u << 3 | right << 2 | left << 4 : 0u;
+    m |= s ? 1u << 7 | right << 8 | left << 6 : 0u;
+  }
+#pragma unroll
+  for (int k = 2; k <= 8; k += 2)  // the corners
+    if ((k / 2 - 1) % LANES == sub && blocked(move_dx(k) * (a + 1), move_dy(k) * (b + 1))) m |= 1u << k;
+  return m;
 }
 
 // Offset d along a dimension of n su: the minimum image when periodic.
@@ -328,15 +347,14 @@ __device__ __forceinline__ void candidate_loads(const Geo& g, const uint8_t* __r
   }
 }
 
-template <bool TIE = false>
+template <bool TIE = false, bool SIZED = false>
 __device__ __forceinline__ uint8_t decide_one(
     int p, const Geo& g, const int2* __restrict__ xy, const uint8_t* __restrict__ heading,
     const uint8_t* __restrict__ goal, const uint8_t* __restrict__ cell,
     const uint8_t* __restrict__ ocls, const int32_t* __restrict__ D, const float* __restrict__ F,
     int main_off, int lo_row, int hi_row, int hi_off, int y_lo, int y_hi, float beta,
     const float* __restrict__ own, const float* __restrict__ dirdot,
-    const uint8_t* __restrict__ pw = nullptr, const uint8_t* __restrict__ ph = nullptr,
-    const int32_t* __restrict__ occ = nullptr, bool* tie = nullptr, int ring = 0) {
+    bool* tie = nullptr, int ring = 0, uint32_t blocked = 0) {
   const int2 q = xy[p];
   const int h = heading[p], gl = goal[p];
   // the 3 x 3 neighbourhood (wrapped or clipped); every load is issued
@@ -362,14 +380,8 @@ __device__ __forceinline__ uint8_t decide_one(
     const int xi = move_dx(k) + 1, yi = move_dy(k) + 1;
     f[k] = F[(size_t)fr[yi] * g.W + cx[xi]];
     dd[k] = D[(size_t)ry[yi] * g.W + cx[xi]];  // kDWall on WALL su: no cell read
-    oc[k] = ocls[(size_t)ry[yi] * g.opitch + cx[xi]];
-  }
-  if (pw) {
-    // multi-su pedestrian: a move is admissible iff the su its rectangle
-    // newly enters are free (walls included in the test)
-    const int a = pw[p] >> 1, b = ph[p] >> 1;
-#pragma unroll
-    for (int k = 1; k < 9; ++k) oc[k] = strip_free(g, cell, occ, q.x, q.y, a, b, k) ? 0 : 1;
+    // a multi-su pedestrian's moves: blocked_moves() (walls included)
+    oc[k] = SIZED ? (uint8_t)(blocked >> k & 1u) : ocls[(size_t)ry[yi] * g.opitch + cx[xi]];
   }
   return (uint8_t)pick_move<false, TIE>(f, dd, oc, okx, oky, h, gl, beta, own, dirdot, nullptr,
                                        nullptr, tie);
@@ -460,49 +472,66 @@ __device__ __forceinline__ void commit_one(int p, const Geo& g, int2* __restrict
 // enters and wins iff its (priority, id) is smaller than that of every other
 // mover claiming one of them.  A rival claiming su s covers a su next to s,
 // so the 8 neighbours of each claimed su hold every rival's id.  Returns the
-// most claimants of one su.
+// most claimants of one su and whether it wins.  `sub` of LANES lanes looks at
+// every LANES-th su claimed: the pedestrian's result is the lanes' largest count
+// and whether it wins with all of them.
+template <int LANES>
 __device__ __forceinline__ int vote_one_sized(int p, const Geo& g, const int2* __restrict__ xy,
                                               const uint8_t* __restrict__ choice,
                                               const int32_t* __restrict__ occ,
                                               const uint8_t* __restrict__ pw,
                                               const uint8_t* __restrict__ ph, uint64_t seed,
-                                              long long t, uint8_t* __restrict__ won) {
+                                              long long t, int sub, bool& win) {
   const int k = choice[p];
-  if (k == 0) {
-    won[p] = 0;
-    return 0;
-  }
+  win = k != 0;
+  if (k == 0) return 0;
   const int2 q = xy[p];
   const int a = pw[p] >> 1, b = ph[p] >> 1, dx = move_dx(k), dy = move_dy(k);
   const uint64_t st = splitmix_nth(seed, (uint64_t)t + 1);
   const uint64_t mine = splitmix_nth(st, (uint64_t)p + 1);
-  bool win = true;
   int regs = 1;
-  for (int j = -b; j <= b; ++j)
-    for (int i = -a; i <= a; ++i) {
-      const int ox = i + dx, oy = j + dy;
-      if (ox >= -a && ox <= a && oy >= -b && oy <= b) continue;  // not newly entered
-      int sx, sy;
-      if (!(wrap_coord(q.x + ox, g.W, g.px, sx) & wrap_coord(q.y + oy, g.H, g.py, sy))) continue;
-      int seen[8], ns = 0;
-      for (int e = 1; e <= 8; ++e) {
-        int nx, ny;
-        if (!(wrap_coord(sx + move_dx(e), g.W, g.px, nx) & wrap_coord(sy + move_dy(e), g.H, g.py, ny)))
-          continue;
-        const int o = occ[(size_t)ny * g.W + nx];
-        if (o < 0 || o == p) continue;
-        bool dup = false;
-        for (int u = 0; u < ns; ++u) dup |= seen[u] == o;
-        if (dup || choice[o] == 0) continue;
-        const int2 qo = xy[o];
-        if (!in_entered(g, sx, sy, qo.x, qo.y, pw[o] >> 1, ph[o] >> 1, choice[o])) continue;
-        seen[ns++] = o;
-        const uint64_t po = splitmix_nth(st, (uint64_t)o + 1);
-        if (po < mine || (po == mine && o < p)) win = false;
-      }
-      regs = max(regs, ns + 1);
+  // the su newly entered: the column dx (a + 1) if dx, then the rest of the row
+  // dy (b + 1) if dy
+  const int ncol = dx ? 2 * b + 1 : 0, nrow = dy ? 2 * a + 1 - (dx != 0) : 0;
+  for (int e0 = sub; e0 < ncol + nrow; e0 += LANES) {
+    const bool incol = e0 < ncol;
+    const int ox = incol ? dx * (a + 1) : e0 - ncol - a + (dx > 0), oy = incol ? e0 - b + dy : dy * (b + 1);
+    int sx, sy;
+    if (!(wrap_coord(q.x + ox, g.W, g.px, sx) & wrap_coord(q.y + oy, g.H, g.py, sy))) continue;
+    // the eight neighbours at once, then the choices and the rectangles of the
+    // pedestrians there (a pedestrian met twice counts once)
+    int o[9], ko[9], ns = 0;
+#pragma unroll
+    for (int e = 1; e <= 8; ++e) {
+      int nx, ny;
+      const bool in = wrap_coord(sx + move_dx(e), g.W, g.px, nx) & wrap_coord(sy + move_dy(e), g.H, g.py, ny);
+      o[e] = in ? occ[(size_t)ny * g.W + nx] : -1;
     }
-  won[p] = win ? 1 : 0;
+#pragma unroll
+    for (int e = 1; e <= 8; ++e) {
+      bool other = o[e] >= 0 && o[e] != p;
+#pragma unroll
+      for (int u = 1; u < e; ++u) other = other && o[u] != o[e];
+      ko[e] = other ? choice[o[e]] : 0;
+    }
+    int2 qo[9];
+    int ao[9], bo[9];
+#pragma unroll
+    for (int e = 1; e <= 8; ++e)
+      if (ko[e]) {
+        qo[e] = xy[o[e]];
+        ao[e] = pw[o[e]] >> 1;
+        bo[e] = ph[o[e]] >> 1;
+      }
+#pragma unroll
+    for (int e = 1; e <= 8; ++e) {
+      if (!ko[e] || !in_entered(g, sx, sy, qo[e].x, qo[e].y, ao[e], bo[e], ko[e])) continue;
+      ++ns;
+      const uint64_t po = splitmix_nth(st, (uint64_t)o[e] + 1);
+      if (po < mine || (po == mine && o[e] < p)) win = false;
+    }
+    regs = max(regs, ns + 1);
+  }
   return regs;
 }
 

@@ -1129,8 +1129,7 @@ __global__ void __launch_bounds__(256, 4) k_decide(const int32_t* __restrict__ r
                          int lo_row, int hi_row, int hi_off, int y_lo, int y_hi, Geo g,
                          float beta, const float* __restrict__ own,
                          const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
-                         WalkPeriods wp, Sizes sz, const int32_t* __restrict__ occ,
-                         Counters* __restrict__ ctr, int ring) {
+                         WalkPeriods wp, Counters* __restrict__ ctr, int ring) {
   // grid-stride over the records of bins [b_lo, b_hi): a band's launch needs
   // no more blocks than the GPU holds, whatever its share of the crowd.  The
   // records are taken from the last backwards: the gather wrote the band's
@@ -1148,12 +1147,59 @@ __global__ void __launch_bounds__(256, 4) k_decide(const int32_t* __restrict__ r
     }
     bool tie = false;
     choice[p] = decide_one<true>(p, g, xy, heading, goal, cell, ocls, D, F, main_off, lo_row,
-                                 hi_row, hi_off, y_lo, y_hi, beta, own, dirdot, sz.w, sz.h, occ,
-                                 &tie, ring);
+                                 hi_row, hi_off, y_lo, y_hi, beta, own, dirdot, &tie, ring);
     ++decided;
     ties += tie ? 1u : 0u;
   }
   // decisions and near ties, one atomic per warp
+  decided = __reduce_add_sync(0xffffffffu, decided);
+  ties = __reduce_add_sync(0xffffffffu, ties);
+  if (ctr && (threadIdx.x & 31) == 0 && decided) {
+    atomicAdd(&ctr->decided, (unsigned long long)decided);
+    if (ties) atomicAdd(&ctr->near_ties, (unsigned long long)ties);
+  }
+}
+
+// Multi-su pedestrians, kQuad lanes each, which share the su that it may enter:
+// the chains of dependent reads bound these stages (55 000 pedestrians of 3 x 3
+// su on 1000 x 1000: decide 22 -> 18 us and vote 29 -> 19, against a thread a
+// pedestrian that tests the su of each move one after the other).
+constexpr int kQuad = 4;
+
+__global__ void __launch_bounds__(256, 4)
+    k_decide_sized(const int32_t* __restrict__ rec_id, const int32_t* __restrict__ bin_start, int b_lo,
+                   int b_hi, const int2* __restrict__ xy, const uint8_t* __restrict__ heading,
+                   const uint8_t* __restrict__ goal, const uint8_t* __restrict__ cell,
+                   const int32_t* __restrict__ D, const float* __restrict__ F, int main_off, int lo_row,
+                   int hi_row, int hi_off, int y_lo, int y_hi, Geo g, float beta,
+                   const float* __restrict__ own, const float* __restrict__ dirdot,
+                   uint8_t* __restrict__ choice, WalkPeriods wp, Sizes sz,
+                   const int32_t* __restrict__ occ, Counters* __restrict__ ctr, int ring) {
+  const int end = bin_start[b_hi], cnt = end - bin_start[b_lo];
+  const long long t = wp.period ? wp.ctr->t : 0;
+  const int sub = threadIdx.x % kQuad, step = gridDim.x * blockDim.x / kQuad;
+  unsigned decided = 0, ties = 0;
+  for (int k0 = blockIdx.x * blockDim.x / kQuad; k0 < cnt; k0 += step) {
+    const int k = k0 + threadIdx.x / kQuad;
+    const int p = k < cnt ? rec_id[end - 1 - k] : -1;
+    const bool walks = p >= 0 && !(wp.period && t % wp.period[p] != wp.phase[p]);
+    uint32_t blocked = 0;
+    if (walks) {
+      const int2 q = xy[p];
+      blocked = blocked_moves<kQuad>(g, cell, occ, q.x, q.y, sz.w[p] >> 1, sz.h[p] >> 1, sub);
+    }
+#pragma unroll
+    for (int o = 1; o < kQuad; o <<= 1) blocked |= __shfl_xor_sync(0xffffffffu, blocked, o);
+    if (p < 0 || sub) continue;
+    bool tie = false;
+    choice[p] = walks ? decide_one<true, true>(p, g, xy, heading, goal, cell, nullptr, D, F, main_off,
+                                               lo_row, hi_row, hi_off, y_lo, y_hi, beta, own, dirdot,
+                                               &tie, ring, blocked)
+                      : (uint8_t)0;
+    decided += walks;
+    ties += tie ? 1u : 0u;
+  }
+  __syncwarp();
   decided = __reduce_add_sync(0xffffffffu, decided);
   ties = __reduce_add_sync(0xffffffffu, ties);
   if (ctr && (threadIdx.x & 31) == 0 && decided) {
@@ -1177,10 +1223,17 @@ void launch_decide(int n, const int32_t* rec_id, const int32_t* bin_start, int b
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     max_blocks = (nsm > 0 ? nsm : 1) * 8;  // two rounds of the 4 blocks of 256 an SM holds (64 registers)
   }
+  if (sz.w) {
+    const int blocks = cdiv(n, 256 / kQuad) < max_blocks ? cdiv(n, 256 / kQuad) : max_blocks;
+    k_decide_sized<<<blocks, 256, 0, s>>>(rec_id, bin_start, b_lo, b_hi, xy, heading, goal, cell, D, F,
+                                          main_off, lo_row, hi_row, hi_off, y_lo, y_hi, g, beta, tb.own,
+                                          tb.dirdot, choice, wp, sz, occ, ctr, ring);
+    return;
+  }
   const int blocks = cdiv(n, 256) < max_blocks ? cdiv(n, 256) : max_blocks;
   k_decide<<<blocks, 256, 0, s>>>(rec_id, bin_start, b_lo, b_hi, xy, heading, goal, cell,
                                         ocls, D, F, main_off, lo_row, hi_row, hi_off, y_lo, y_hi,
-                                        g, beta, tb.own, tb.dirdot, choice, wp, sz, occ, ctr, ring);
+                                        g, beta, tb.own, tb.dirdot, choice, wp, ctr, ring);
 }
 
 // ------------------------------------------------------------ S4: vote
@@ -1192,7 +1245,7 @@ __global__ void k_vote(int n, const int32_t* __restrict__ rec_id,
                        const int32_t* __restrict__ bin_start, int nbins,
                        const int2* __restrict__ xy, const uint8_t* __restrict__ alive,
                        uint8_t* __restrict__ choice, const int32_t* __restrict__ occ, Geo g,
-                       uint64_t seed, Counters* ctr, uint8_t* __restrict__ won, Sizes sz,
+                       uint64_t seed, Counters* ctr, uint8_t* __restrict__ won,
                        const int32_t* __restrict__ gid) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n && !alive[i]) {
@@ -1200,8 +1253,33 @@ __global__ void k_vote(int n, const int32_t* __restrict__ rec_id,
     won[i] = 0;
   }
   if (i >= bin_start[nbins]) return;
-  const int regs = sz.w ? vote_one_sized(rec_id[i], g, xy, choice, occ, sz.w, sz.h, seed, ctr->t, won)
-                        : vote_one(rec_id[i], 0, g, xy, choice, occ, seed, ctr->t, won, gid);
+  const int regs = vote_one(rec_id[i], 0, g, xy, choice, occ, seed, ctr->t, won, gid);
+  if (regs > 2) atomicMax(&ctr->max_registrants, regs);
+  if (regs > 8) atomicOr(&ctr->err, kErrEnroll);
+}
+
+__global__ void __launch_bounds__(256, 2)
+    k_vote_sized(int n, const int32_t* __restrict__ rec_id, const int32_t* __restrict__ bin_start,
+                 int nbins, const int2* __restrict__ xy, const uint8_t* __restrict__ alive,
+                 uint8_t* __restrict__ choice, const int32_t* __restrict__ occ, Geo g, uint64_t seed,
+                 Counters* ctr, uint8_t* __restrict__ won, Sizes sz) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kQuad, sub = threadIdx.x % kQuad;
+  if (sub == 0 && i < n && !alive[i]) {
+    choice[i] = 0;
+    won[i] = 0;
+  }
+  const int p = i < bin_start[nbins] ? rec_id[i] : -1;
+  bool win = false;
+  int regs = 0;
+  if (p >= 0)
+    regs = vote_one_sized<kQuad>(p, g, xy, choice, occ, sz.w, sz.h, seed, ctr->t, sub, win);
+#pragma unroll
+  for (int o = 1; o < kQuad; o <<= 1) {
+    regs = max(regs, __shfl_xor_sync(0xffffffffu, regs, o));
+    win = win & __shfl_xor_sync(0xffffffffu, win, o);
+  }
+  if (p < 0 || sub) return;
+  won[p] = win ? 1 : 0;
   if (regs > 2) atomicMax(&ctr->max_registrants, regs);
   if (regs > 8) atomicOr(&ctr->err, kErrEnroll);
 }
@@ -1211,8 +1289,13 @@ void launch_vote(int n, const int32_t* rec_id, const int32_t* bin_start, const i
                  uint64_t seed, Counters* ctr, uint8_t* won, cudaStream_t s, const Sizes& sz,
                  const int32_t* gid) {
   if (n <= 0) return;
-  k_vote<<<cdiv(n, 256), 256, 0, s>>>(n, rec_id, bin_start, g.nbx * g.nby, xy, alive, choice, occ, g,
-                                      seed, ctr, won, sz, gid);
+  const int nbins = g.nbx * g.nby;
+  if (sz.w)
+    k_vote_sized<<<cdiv(n, 256 / kQuad), 256, 0, s>>>(n, rec_id, bin_start, nbins, xy, alive, choice, occ,
+                                                      g, seed, ctr, won, sz);
+  else
+    k_vote<<<cdiv(n, 256), 256, 0, s>>>(n, rec_id, bin_start, nbins, xy, alive, choice, occ, g, seed, ctr,
+                                        won, gid);
 }
 
 // ---------------------------------------------------------- S5: commit
@@ -1255,6 +1338,7 @@ void launch_commit(int n, const int32_t* rec_id, const int32_t* bin_start, int2*
 // dependent reads (record, position, neighbourhood, rivals), which the stages
 // have as well; with two launches less, the shorter binning and the early
 // starts a tick of the 100 x 100 room with 200 pedestrians went from 32 to 25 us.
+template <bool SIZED>
 __global__ void __launch_bounds__(kMoveMaxPeds)
     k_move(int n, const int32_t* rec_id, const int32_t* bin_start, int nbins, int2* xy,
            uint8_t* alive, uint8_t* heading, const uint8_t* __restrict__ goal,
@@ -1274,19 +1358,30 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
   bool decided = false, tie = false;
   if (p >= 0) {
     decided = !(wp.period && t % wp.period[p] != wp.phase[p]);
-    choice[p] = decided ? decide_one<true>(p, g, xy, heading, goal, cell, ocls, D, F, 0, -1, -1, 0, 0,
-                                           g.H, beta, own, dirdot, sz.w, sz.h, occ, &tie)
+    uint32_t blocked = 0;
+    if (SIZED && decided) {
+      const int2 q = xy[p];
+      blocked = blocked_moves<1>(g, cell, occ, q.x, q.y, sz.w[p] >> 1, sz.h[p] >> 1, 0);
+    }
+    choice[p] = decided ? decide_one<true, SIZED>(p, g, xy, heading, goal, cell, ocls, D, F, 0, -1, -1,
+                                                  0, 0, g.H, beta, own, dirdot, &tie, 0, blocked)
                         : (uint8_t)0;
   }
   __syncthreads();
   int regs = 0;
-  if (p >= 0)
-    regs = sz.w ? vote_one_sized(p, g, xy, choice, occ, sz.w, sz.h, seed, t, won)
-                : vote_one(p, 0, g, xy, choice, occ, seed, t, won, gid);
+  if (p >= 0) {
+    if (SIZED) {
+      bool win;
+      regs = vote_one_sized<1>(p, g, xy, choice, occ, sz.w, sz.h, seed, t, 0, win);
+      won[p] = win ? 1 : 0;
+    } else {
+      regs = vote_one(p, 0, g, xy, choice, occ, seed, t, won, gid);
+    }
+  }
   __syncthreads();
   bool moved = false, left = false;
   if (p >= 0) {
-    if (sz.w)
+    if (SIZED)
       commit_one_sized(p, g, xy, alive, heading, choice, won, cell, occ, ocls, sz.w, sz.h, moved, left);
     else
       commit_one(p, g, xy, alive, heading, choice, won, cell, occ, ocls, moved, left);
@@ -1313,7 +1408,7 @@ void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* x
                  uint64_t seed, const Tables& tb, uint8_t* choice, uint8_t* won, Counters* ctr,
                  cudaStream_t s, const WalkPeriods& wp, const Sizes& sz, const int32_t* gid,
                  bool early) {
-  launch_tick_kernel(k_move, 1, 32 * cdiv(n, 32), 0, s, early, n, rec_id, bin_start, g.nbx * g.nby, xy,
+  launch_tick_kernel(sz.w ? k_move<true> : k_move<false>, 1, 32 * cdiv(n, 32), 0, s, early, n, rec_id, bin_start, g.nbx * g.nby, xy,
                      alive, heading, goal, cell, occ, ocls, D, F, g, beta, seed, tb.own, tb.dirdot,
                      choice, won, ctr, wp, sz, gid);
 }

@@ -8,7 +8,9 @@ import numpy as np
 import pytest
 
 import paper_1803_04782_gb300 as sfm
+import scenegen as SG
 from paper_1803_04782_gb300 import build as B
+from parity import OracleRun, compare_choices, rect_cells
 
 pytestmark = pytest.mark.gpu
 
@@ -120,3 +122,41 @@ def test_footprints_agree_on_either_side_of_the_few(W, H, rho, r, periodic):
             fields.append(s.field())
     for f in fields[1:]:
         np.testing.assert_array_equal(f, fields[0])
+
+
+# Rectangles, also long ones (a side is shared by four lanes, or by a lane that
+# reads three su at a time), for one block's slots and for more.
+@pytest.mark.parametrize("W,H,n,periodic", [(90, 70, 700, 0), (200, 190, 3500, 1)])
+def test_rectangles_follow_the_oracle(W, H, n, periodic):
+    sc = SG.random_scene(W, H, n, r=5, seed=7, obstacles=0 if periodic else 2, periodic_x=periodic,
+                         periodic_y=periodic, ring=not periodic, exits=() if periodic else ("east",),
+                         exit_len=12, heading_mode="random")
+    rng = np.random.default_rng(3)
+    kinds = np.array([(1, 1), (1, 5), (7, 3), (9, 1), (3, 3)], np.uint8)
+    size = kinds[rng.choice(len(kinds), n, p=[0.5, 0.15, 0.1, 0.1, 0.15])]
+    keep, taken = [], set()
+    for p in range(n):
+        rc = rect_cells(W, H, periodic, periodic, *sc.xy[p], *size[p])
+        if rc is None or rc & taken or any(sc.cell[v, u] != SG.FREE for u, v in rc):
+            continue
+        keep.append(p)
+        taken |= rc
+    assert (len(keep) > 1024) == (W == 200)
+    sub = SG.Scene("rectangles", W, H, periodic, periodic, sc.cell, sc.xy[keep].copy(),
+                   sc.heading[keep].copy(), sc.goal[keep].copy(), sc.params)
+    w, h = (np.ascontiguousarray(size[keep, i]) for i in (0, 1))
+    orc = OracleRun(sub)
+    orc.st.w, orc.st.h = w, h
+    with sfm.Sim(sub, place=False) as sim:
+        sim.place_sized(sub.xy, sub.heading, sub.goal, np.ones(sub.n, np.uint8), w, h)
+        for _ in range(8):
+            sim.step(1)
+            Fo, So = orc.field()
+            ch_o, E, T, adm = orc.decide(Ffull=Fo.ravel(), Sfull=So.ravel())
+            ch_g, won_g = sim.decisions()
+            flips = compare_choices(ch_g, ch_o, E, T, adm)  # ties only
+            won_o, most = orc.advance(np.asarray(ch_g, np.uint8) if flips else ch_o)
+            np.testing.assert_array_equal(won_g, won_o)
+            for x, y in zip(sim.peds(), (orc.st.xy, orc.st.heading, orc.st.alive)):
+                np.testing.assert_array_equal(x, y)
+        assert sim.stats()["max_registrants"] >= 2 and sim.stats()["error_flags"] == 0
