@@ -11,6 +11,8 @@
 
 namespace sfm {
 
+constexpr int kFieldPad = kFieldPadRows;
+
 // Head of a kernel launched by launch_tick_kernel: the kernel after it may
 // start, and everything before this one is complete and visible.  Arrays that
 // change from tick to tick are no `const __restrict__` parameters of such
@@ -56,27 +58,38 @@ static __constant__ int c_csx[9] = SFM_CLASS_ROW(class_sx);
 static __constant__ int c_csy[9] = SFM_CLASS_ROW(class_sy);
 #undef SFM_CLASS_ROW
 
-constexpr int kFieldPad = kFieldPadRows;
 
-// Entry (dx, dy) of stored heading-class table t (0 none, 1 E, 2 N, 3 NE):
-// K_P((dx, dy); h_t) = kP d^aP (1 + gamma h_t . (dx, dy) / d) for 0 <
-// max(|dx|, |dy|) <= r, else 0; evaluated in FP64 (and rounded to FP32 by
-// the caller) so that every table layout holds the same values.  taper_in <
-// r: weighted by 1 up to Euclidean distance taper_in and a raised cosine
-// down to 0 at r (the surrogate's near part).
-__device__ __forceinline__ double class_kernel_value(int t, int dx, int dy, int r, double kP,
-                                                     double aP, double gamma, double taper_in) {
+// Entry i of the stored heading-class tables (0 none, 1 E, 2 N, 3 NE): K_P((dx,
+// dy); h_t) = kP d^aP (1 + gamma h_t . (dx, dy) / d) for 0 < max(|dx|, |dy|) <=
+// r, else 0; evaluated in FP64 and rounded to FP32, the same in every layout:
+// 2 r + 1 window rows of stride SP between kFieldPad zero rows, table after
+// table.  taper_in < r: weighted by 1 up to Euclidean distance taper_in and a
+// raised cosine down to 0 at r (the surrogate's near part).  A thread writes an
+// entry of all four tables: FP64 powers bound it (one for each table, 11 us at
+// r = 20; now 5).
+__device__ __forceinline__ void class_table_entry(int i, int r, int SP, double kP, double aP,
+                                                  double gamma, double taper_in,
+                                                  float* __restrict__ T) {
+  const int TS = (2 * r + 1 + 2 * kFieldPad) * SP;
+  const int dy = i / SP - (r + kFieldPad), dx = i % SP - r;
   const int adx = dx < 0 ? -dx : dx, ady = dy < 0 ? -dy : dy;
-  double v = 0.0;
-  if (adx <= r && ady <= r && (adx | ady) != 0) {
+  const bool in = adx <= r && ady <= r && (adx | ady) != 0;
+  double d = 1.0, radial = 0.0, w = 1.0;
+  if (in) {
+    d = sqrt((double)(dx * dx + dy * dy));
+    radial = kP * pow(d, aP);
+    if (taper_in < r && d > taper_in)
+      w = d >= r ? 0.0 : 0.5 * (1.0 + cos(3.14159265358979323846 * (d - taper_in) / (r - taper_in)));
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
     const double hx = (t == 1) ? 1.0 : (t == 3 ? 0.70710678118654752440 : 0.0);
     const double hy = (t == 2) ? 1.0 : (t == 3 ? 0.70710678118654752440 : 0.0);
-    const double d = sqrt((double)(dx * dx + dy * dy));
-    v = kP * pow(d, aP) * (1.0 + gamma * (hx * dx + hy * dy) / d);
-    if (taper_in < r && d > taper_in)
-      v *= d >= r ? 0.0 : 0.5 * (1.0 + cos(3.14159265358979323846 * (d - taper_in) / (r - taper_in)));
+    T[t * TS + i] = in ? (float)(radial * (1.0 + gamma * (hx * dx + hy * dy) / d) * w) : 0.f;
   }
-  return v;
+}
+__host__ __device__ constexpr int class_table_entries(int r, int SP) {
+  return (2 * r + 1 + 2 * kFieldPad) * SP;
 }
 
 // the same move offsets as compile-time functions, so unrolled loops index

@@ -213,19 +213,6 @@ void launch_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec, cons
                      out, out_row0, fy0, fy1, store_lo, store_hi, tickets, sorted, ring);
 }
 
-// the class tables in the layout of the row-trimmed gather: [4][2r+3][SP],
-// window row dy at table row dy + r + 1, column dx at dx + r
-__global__ void k_class_tables3(int r, int SP, double kP, double aP, double gamma,
-                                float* __restrict__ T) {
-  const int TR = 2 * r + 1 + 2 * kField3PadRows;
-  const int n = 4 * TR * SP;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int t = i / (TR * SP), rem = i % (TR * SP);
-  const int dy = rem / SP - (r + kField3PadRows), dx = rem % SP - r;
-  T[i] = (float)class_kernel_value(t, dx, dy, r, kP, aP, gamma, (double)r);
-}
-
 }  // namespace
 
 bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
@@ -245,13 +232,6 @@ bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec
   }
 #undef SFM_V3
   return true;
-}
-
-void launch_class_tables3(int r, const sfm_params& p, float* T, cudaStream_t s) {
-  const int sp = field3_stride(r);
-  if (!sp) return;
-  const int n = (int)field3_table_floats(r);
-  k_class_tables3<<<(n + 255) / 256, 256, 0, s>>>(r, sp, p.kP, p.aP, p.gamma, T);
 }
 
 }  // namespace sfm

@@ -77,6 +77,7 @@ static_assert((kTableGuard + max_class_table_floats(kMaxTableRadius)) * 4 +
 // (a visit reads whole blocks) and at least 15 zero columns after each row; the
 // row stride is one of a few compile-time classes.  Radius 1..40.
 constexpr int kField3PadRows = 15;
+static_assert(kField3PadRows == kFieldPadRows, "one table kernel writes both layouts");
 constexpr int kField3Threads = 896;
 constexpr int kShape16x16 = 0, kShape32x16 = 1, kShape32x32 = 2;
 constexpr int field3_stride(int r) {

@@ -1093,27 +1093,29 @@ void launch_field_v1(const Geo& g, const int32_t* bin_start, const uint32_t* rec
                                             store_lo, store_hi, cap, ctr);
 }
 
-
 __global__ void k_class_tables(int r, int SP, double kP, double aP, double gamma, double taper_in,
                                float* __restrict__ T) {
-  const int TR = 2 * r + 1 + 2 * kFieldPad;
-  const int n = 4 * TR * SP;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int t = i / (TR * SP), rem = i % (TR * SP);
-  const int dy = rem / SP - (r + kFieldPad), dx = rem % SP - r;
-  T[i] = (float)class_kernel_value(t, dx, dy, r, kP, aP, gamma, taper_in);
+  if (i < class_table_entries(r, SP)) class_table_entry(i, r, SP, kP, aP, gamma, taper_in, T);
 }
 
 int class_table_stride(int r) { return class_table_stride_of(r); }
 
 size_t class_table_floats(int r) { return class_table_floats_of(r); }
 
-void launch_class_tables(int r, const sfm_params& p, float* T, cudaStream_t s, double taper_in) {
-  const int sp = class_table_stride(r);
+static void class_tables(int r, int sp, const sfm_params& p, float* T, cudaStream_t s, double taper_in) {
   if (!sp) return;
-  const int n = (int)class_table_floats(r);
-  k_class_tables<<<cdiv(n, 256), 256, 0, s>>>(r, sp, p.kP, p.aP, p.gamma, taper_in, T);
+  k_class_tables<<<cdiv(class_table_entries(r, sp), 128), 128, 0, s>>>(r, sp, p.kP, p.aP, p.gamma, taper_in,
+                                                                       T);
+}
+
+void launch_class_tables(int r, const sfm_params& p, float* T, cudaStream_t s, double taper_in) {
+  class_tables(r, class_table_stride(r), p, T, s, taper_in);
+}
+
+// in the layout of the row-trimmed gather
+void launch_class_tables3(int r, const sfm_params& p, float* T, cudaStream_t s) {
+  class_tables(r, field3_stride(r), p, T, s, 1e30);
 }
 
 // --------------------------------------------------------- S3: decide

@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "sfm_device.cuh"
 #include "sfm_internal.h"
 
 using namespace sfm;
@@ -26,12 +27,11 @@ namespace {
 // Layout of the scratch array, in 32-bit words.
 constexpr int kNaBins = SFM_NOALLOC_MAX_BINS;
 constexpr int kNaPeds = SFM_NOALLOC_MAX_PEDS;
-constexpr size_t kNaCount = 0;                          // per-bin counts
-constexpr size_t kNaCursor = kNaCount + kNaBins;        // per-bin fill cursors
-constexpr size_t kNaStart = kNaCursor + kNaBins;        // bin starts (kNaBins + 1)
+constexpr size_t kNaErr = 0;                            // error word
+constexpr size_t kNaCount = kNaErr + 64;                // a call's bins: counts, then fill cursors
+constexpr size_t kNaStart = kNaCount + 2 * kNaBins;     // bin starts (kNaBins + 1)
 constexpr size_t kNaScanTmp = kNaStart + kNaBins + 64;  // scan block totals
-constexpr size_t kNaErr = kNaScanTmp + 64;              // error word
-constexpr size_t kNaRec = kNaErr + 64;                  // bin records
+constexpr size_t kNaRec = kNaScanTmp + 64;              // bin records
 constexpr size_t kNaTables = kNaRec + kNaPeds;          // heading-class tables
 constexpr size_t kNaTableFloats =
     std::max(max_class_table_floats(SFM_NOALLOC_MAX_RADIUS), max_field3_table_floats());
@@ -67,9 +67,17 @@ __device__ __forceinline__ bool na_valid(const int2 q, const Geo& g, const uint8
   return ok;
 }
 
+// Counts in the first `nblocks` blocks, the kernel tables in the others: they
+// take each other's time (10 us of a call).
 __global__ void k_na_count(int n, const int2* __restrict__ xy, const uint8_t* __restrict__ heading,
                            const uint8_t* __restrict__ alive, Geo g, int32_t* __restrict__ count,
-                           uint32_t* __restrict__ err) {
+                           uint32_t* __restrict__ err, int nblocks, int SP, double kP, double aP,
+                           double gamma, float* __restrict__ tables) {
+  if ((int)blockIdx.x >= nblocks) {
+    const int i = (blockIdx.x - nblocks) * blockDim.x + threadIdx.x;
+    if (i < class_table_entries(g.r, SP)) class_table_entry(i, g.r, SP, kP, aP, gamma, 1e30, tables);
+    return;
+  }
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n || (alive && !alive[p])) return;
   const int2 q = xy[p];
@@ -124,31 +132,29 @@ extern "C" sfm_status sfm_field_noalloc(const sfm_lattice* lat, const sfm_params
   if (st != SFM_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int32_t* count = reinterpret_cast<int32_t*>(S + kNaCount);
-  int32_t* cursor = reinterpret_cast<int32_t*>(S + kNaCursor);
+  int32_t* cursor = count + nbins;
   int32_t* start = reinterpret_cast<int32_t*>(S + kNaStart);
   int32_t* scan_tmp = reinterpret_cast<int32_t*>(S + kNaScanTmp);
   uint32_t* err = S + kNaErr;
   uint32_t* rec = S + kNaRec;
   float* tables = reinterpret_cast<float*>(S + kNaTables);
 
-  // what must start at zero: counts, cursors and the error word
-  if (cudaMemsetAsync(count, 0, sizeof(int32_t) * 2 * (size_t)kNaBins, s) != cudaSuccess ||
-      cudaMemsetAsync(err, 0, sizeof(uint32_t), s) != cudaSuccess)
+  // what must start at zero: the error word, this call's counts and cursors
+  if (cudaMemsetAsync(err, 0, sizeof(int32_t) * (kNaCount - kNaErr + 2 * (size_t)nbins), s) != cudaSuccess)
     return SFM_ECUDA;
   const int2* pxy = reinterpret_cast<const int2*>(xy);
-  if (n > 0) k_na_count<<<(n + 255) / 256, 256, 0, s>>>(n, pxy, heading, alive, g, count, err);
-  launch_scan(count, start, nbins, scan_tmp, s);
-  if (n > 0)
-    k_na_fill<<<(n + 255) / 256, 256, 0, s>>>(n, pxy, heading, alive, g, start, cursor, rec, err);
+  // the tables in the layout of the gather that runs
   Tables tb{};
   tb.CT = tables;
   tb.shape = default_field_shape(g.r, g.W, g.H);
-  if (field3_shape_ok(tb.shape, g.r)) {  // in the layout of the gather that runs
-    tb.CT3 = tables;
-    launch_class_tables3(g.r, *prm, tables, s);
-  } else {
-    launch_class_tables(g.r, *prm, tables, s);
-  }
+  if (field3_shape_ok(tb.shape, g.r)) tb.CT3 = tables;
+  const int sp = tb.CT3 ? field3_stride(g.r) : class_table_stride(g.r);
+  const int nblocks = (n + 127) / 128, tblocks = (class_table_entries(g.r, sp) + 127) / 128;
+  k_na_count<<<nblocks + tblocks, 128, 0, s>>>(n, pxy, heading, alive, g, count, err, nblocks, sp, prm->kP,
+                                               prm->aP, prm->gamma, tables);
+  launch_scan(count, start, nbins, scan_tmp, s);
+  if (n > 0)
+    k_na_fill<<<(n + 255) / 256, 256, 0, s>>>(n, pxy, heading, alive, g, start, cursor, rec, err);
   launch_field(g, start, rec, tb, base, field, 0, 0, g.H, nullptr, s);
 
   uint32_t h_err = 0;

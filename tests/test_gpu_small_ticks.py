@@ -160,3 +160,28 @@ def test_rectangles_follow_the_oracle(W, H, n, periodic):
             for x, y in zip(sim.peds(), (orc.st.xy, orc.st.heading, orc.st.alive)):
                 np.testing.assert_array_equal(x, y)
         assert sim.stats()["max_registrants"] >= 2 and sim.stats()["error_flags"] == 0
+
+
+# The allocation-free field on either side of 18 footprints of 32 x 32 su an SM
+# (2736 on 152 SMs): each gather with its own table layout, several sizes in a
+# row over the same scratch.  Its bins are in order of arrival: equal up to the
+# rounding of an FP32 sum of at most a window's terms (1e-5 of it).
+def test_allocation_free_field_takes_the_contexts_gather():
+    torch = pytest.importorskip("torch")
+    for W, H, n, r in [(1700, 1650, 9000, 3), (1700, 1620, 30000, 20), (40, 50, 300, 8), (1700, 1650, 0, 40),
+                       (1700, 1650, 30000, 40), (1700, 1650, 30000, 45)]:
+        rng = np.random.default_rng(r)
+        at = rng.choice(W * H, n, replace=False)
+        xy = np.stack([at % W, at // W], 1).astype(np.int32)
+        heading = rng.integers(0, 9, n).astype(np.uint8)
+        with sfm.Sim(W=W, H=H, cell=np.zeros((H, W), np.uint8), r=r) as s:
+            s.place(xy, heading, np.zeros(n, np.uint8))
+            s.compute_field()
+            want = s.field()
+        base = torch.zeros((H, W), dtype=torch.float32, device="cuda")
+        out = torch.full_like(base, float("nan"))
+        assert sfm.sfm_field_noalloc(sfm.Lattice(W, H, 0, 0), sfm.make_params(r=r),
+                                     torch.from_numpy(xy).cuda(), torch.from_numpy(heading).cuda(), None,
+                                     base, out) == sfm.SFM_OK
+        got = out.cpu().numpy()
+        assert np.abs(got - want).max() <= 1e-5 * max(np.abs(want).max(), 1e-30)
