@@ -696,8 +696,8 @@ __global__ void k_bin_count(Geo g, const uint8_t* ocls, int32_t* count) {
   if (lane == 0) count[b] = c;
 }
 
-// launches of launch_scan: three passes, or one when a block covers all n
-static int scan_launches(int n) { return scan_tmp_elems(n) == 1 ? 1 : 3; }
+// launches of launch_scan: two passes, or one when a block covers all n
+static int scan_launches(int n) { return scan_tmp_elems(n) == 1 ? 1 : 2; }
 
 // SCANNED: a scan has put the bins' first slots into `start`; else a block adds
 // up the counts of the bins before its own and writes its part of `start`.
@@ -818,9 +818,10 @@ int launch_bins_from_peds(const Geo& g, int n, const int2* xy, const uint8_t* al
 }
 
 // ------------------------------------------------------------------ scan
-// Exclusive prefix sum of n int32 into out[0..n] (out[n] = total), three
-// passes: per-block totals, a single-block scan of the totals, final; one
-// pass (the final one, from offset 0) when a block covers all n.
+// Exclusive prefix sum of n int32 into out[0..n] (out[n] = total), two passes:
+// per-block totals, and the final one, in which a block adds up the totals
+// before it (a pass of its own for them took 2.5 us); only the final one when a
+// block covers all n.
 constexpr int kScanThreads = 1024, kScanItems = 4, kScanChunk = kScanThreads * kScanItems;
 
 __device__ int block_exclusive_scan(int v, int* sWarp, int& total) {
@@ -862,30 +863,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_totals(const int32_t* __r
   if (threadIdx.x == 0) totals[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_top(int32_t* __restrict__ totals, int nb) {
-  __shared__ int sWarp[32];
-  int carry = 0;
-  for (int base = 0; base < nb; base += kScanChunk) {
-    int v[kScanItems], s = 0;
-    const int i0 = base + threadIdx.x * kScanItems;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-      v[k] = (i0 + k < nb) ? totals[i0 + k] : 0;
-      s += v[k];
-    }
-    int total;
-    int e = block_exclusive_scan(s, sWarp, total) + carry;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-      if (i0 + k < nb) totals[i0 + k] = e;
-      e += v[k];
-    }
-    carry += total;
-  }
-}
-
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(const int32_t* __restrict__ in, int n,
-                                                             const int32_t* __restrict__ offs,
+                                                             const int32_t* __restrict__ totals,
                                                              int32_t* __restrict__ out) {
   __shared__ int sWarp[32];
   const int i0 = blockIdx.x * kScanChunk + threadIdx.x * kScanItems;
@@ -895,8 +874,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(const int32_t* __re
     v[k] = (i0 + k < n) ? in[i0 + k] : 0;
     s += v[k];
   }
-  int total;
-  int e = block_exclusive_scan(s, sWarp, total) + (offs ? offs[blockIdx.x] : 0);
+  int total, before = 0;
+  if (totals) {  // of the blocks before this one
+    int t = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) t += totals[b];
+    block_exclusive_scan(t, sWarp, before);
+  }
+  int e = block_exclusive_scan(s, sWarp, total) + before;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
     if (i0 + k < n) out[i0 + k] = e;
@@ -909,13 +893,8 @@ int scan_tmp_elems(int n) { return cdiv(n > 0 ? n : 1, kScanChunk); }
 
 void launch_scan(const int32_t* in, int32_t* out, int n, int32_t* block_tmp, cudaStream_t s) {
   const int nb = scan_tmp_elems(n);
-  if (nb == 1) {  // small lattices: one launch instead of three
-    k_scan_final<<<1, kScanThreads, 0, s>>>(in, n, nullptr, out);
-    return;
-  }
-  k_scan_totals<<<nb, kScanThreads, 0, s>>>(in, n, block_tmp);
-  k_scan_top<<<1, kScanThreads, 0, s>>>(block_tmp, nb);
-  k_scan_final<<<nb, kScanThreads, 0, s>>>(in, n, block_tmp, out);
+  if (nb > 1) k_scan_totals<<<nb, kScanThreads, 0, s>>>(in, n, block_tmp);
+  k_scan_final<<<nb, kScanThreads, 0, s>>>(in, n, nb > 1 ? block_tmp : nullptr, out);
 }
 
 // ------------------------------------ S2: field gather for radius > 50
