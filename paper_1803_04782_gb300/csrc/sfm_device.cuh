@@ -1,6 +1,6 @@
 // sfm_device.cuh -- device building blocks of one tick, shared by the
-// single-lattice kernels (sfm_kernels.cu) and the batched persistent tick
-// (sfm_batch.cu).  Every function works on one lattice given by its Geo and
+// single-lattice kernels (sfm_kernels.cu, sfm_move.cu), the batch
+// (sfm_batch.cu) and the surrogate (sfm_surrogate.cu).  Every function works on one lattice given by its Geo and
 // pointers already offset to that lattice's arrays; pedestrian indices are
 // indices into the (possibly concatenated) pedestrian arrays.
 #pragma once
@@ -363,8 +363,8 @@ __device__ __forceinline__ void candidate_loads(const Geo& g, const uint8_t* __r
 template <bool TIE = false, bool SIZED = false>
 __device__ __forceinline__ uint8_t decide_one(
     int p, const Geo& g, const int2* __restrict__ xy, const uint8_t* __restrict__ heading,
-    const uint8_t* __restrict__ goal, const uint8_t* __restrict__ cell,
-    const uint8_t* __restrict__ ocls, const int32_t* __restrict__ D, const float* __restrict__ F,
+    const uint8_t* __restrict__ goal, const uint8_t* __restrict__ ocls,
+    const int32_t* __restrict__ D, const float* __restrict__ F,
     int main_off, int lo_row, int hi_row, int hi_off, int y_lo, int y_hi, float beta,
     const float* __restrict__ own, const float* __restrict__ dirdot,
     bool* tie = nullptr, int ring = 0, uint32_t blocked = 0) {

@@ -1105,8 +1105,8 @@ void launch_class_tables3(int r, const sfm_params& p, float* T, cudaStream_t s) 
 __global__ void __launch_bounds__(256, 4) k_decide(const int32_t* __restrict__ rec_id, const int32_t* __restrict__ bin_start,
                          int b_lo, int b_hi, const int2* __restrict__ xy,
                          const uint8_t* __restrict__ heading, const uint8_t* __restrict__ goal,
-                         const uint8_t* __restrict__ cell, const uint8_t* __restrict__ ocls,
-                         const int32_t* __restrict__ D, const float* __restrict__ F, int main_off,
+                         const uint8_t* __restrict__ ocls, const int32_t* __restrict__ D,
+                         const float* __restrict__ F, int main_off,
                          int lo_row, int hi_row, int hi_off, int y_lo, int y_hi, Geo g,
                          float beta, const float* __restrict__ own,
                          const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
@@ -1127,7 +1127,7 @@ __global__ void __launch_bounds__(256, 4) k_decide(const int32_t* __restrict__ r
       continue;
     }
     bool tie = false;
-    choice[p] = decide_one<true>(p, g, xy, heading, goal, cell, ocls, D, F, main_off, lo_row,
+    choice[p] = decide_one<true>(p, g, xy, heading, goal, ocls, D, F, main_off, lo_row,
                                  hi_row, hi_off, y_lo, y_hi, beta, own, dirdot, &tie, ring);
     ++decided;
     ties += tie ? 1u : 0u;
@@ -1173,7 +1173,7 @@ __global__ void __launch_bounds__(256, 4)
     for (int o = 1; o < kQuad; o <<= 1) blocked |= __shfl_xor_sync(0xffffffffu, blocked, o);
     if (p < 0 || sub) continue;
     bool tie = false;
-    choice[p] = walks ? decide_one<true, true>(p, g, xy, heading, goal, cell, nullptr, D, F, main_off,
+    choice[p] = walks ? decide_one<true, true>(p, g, xy, heading, goal, nullptr, D, F, main_off,
                                                lo_row, hi_row, hi_off, y_lo, y_hi, beta, own, dirdot,
                                                &tie, ring, blocked)
                       : (uint8_t)0;
@@ -1212,9 +1212,9 @@ void launch_decide(int n, const int32_t* rec_id, const int32_t* bin_start, int b
     return;
   }
   const int blocks = cdiv(n, 256) < max_blocks ? cdiv(n, 256) : max_blocks;
-  k_decide<<<blocks, 256, 0, s>>>(rec_id, bin_start, b_lo, b_hi, xy, heading, goal, cell,
-                                        ocls, D, F, main_off, lo_row, hi_row, hi_off, y_lo, y_hi,
-                                        g, beta, tb.own, tb.dirdot, choice, wp, ctr, ring);
+  k_decide<<<blocks, 256, 0, s>>>(rec_id, bin_start, b_lo, b_hi, xy, heading, goal, ocls, D, F, main_off,
+                                  lo_row, hi_row, hi_off, y_lo, y_hi, g, beta, tb.own, tb.dirdot, choice,
+                                  wp, ctr, ring);
 }
 
 // ------------------------------------------------------------ S4: vote
@@ -1344,7 +1344,7 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
       const int2 q = xy[p];
       blocked = blocked_moves<1>(g, cell, occ, q.x, q.y, sz.w[p] >> 1, sz.h[p] >> 1, 0);
     }
-    choice[p] = decided ? decide_one<true, SIZED>(p, g, xy, heading, goal, cell, ocls, D, F, 0, -1, -1,
+    choice[p] = decided ? decide_one<true, SIZED>(p, g, xy, heading, goal, ocls, D, F, 0, -1, -1,
                                                   0, 0, g.H, beta, own, dirdot, &tie, 0, blocked)
                         : (uint8_t)0;
   }
