@@ -209,7 +209,8 @@ void run_bins(sfm_ctx* c, bool early = false) {
 // One tick.  The kernels of the grid's binning, the gather and k_move start
 // while their predecessor ends (`early`): their launch, and the gather's table
 // copy, hide behind it; 26.8 -> 24.7 us a tick of a 100 x 100 lattice, 67.7 ->
-// 65.5 of 1000 x 200.  Decide, vote and commit, and the list's binning, do not:
+// 65.5 of 1000 x 200.  So do the ring bands' gathers, behind the decisions of the
+// band before (7338 -> 7285 us for four ticks of 16384 x 16384).  Decide, vote and commit, and the list's binning, do not:
 // blocks that start early pile up on the SMs that are free first (163 -> 186
 // us a tick of 4096 x 4096 at r = 40 with all of them early).
 void run_tick(sfm_ctx* c) {
@@ -270,7 +271,7 @@ void run_tick(sfm_ctx* c) {
       const int s_hi = yb + kTile < g.H ? yb + kTile : g.H;
       if (s_hi > s_lo) {
         StageScope sc(c, SFM_STAGE_FIELD);
-        launch_field_of(c, c->band_buf, s_lo - s_lo % R, s_lo, s_hi, R);
+        launch_field_of(c, c->band_buf, s_lo - s_lo % R, s_lo, s_hi, R, !c->timing);
       }
       const int y_lo = ya > 0 ? ya - 1 : 0, y_hi = yb + 1 < g.H ? yb + 1 : g.H;
       StageScope sc(c, SFM_STAGE_DECIDE);

@@ -17,8 +17,13 @@ constexpr int kFieldPad = kFieldPadRows;
 // start, and everything before this one is complete and visible.  Arrays that
 // change from tick to tick are no `const __restrict__` parameters of such
 // kernels, so that they are not read through the non-coherent path.
-__device__ __forceinline__ void tick_kernel_begin() {
+// (let_next_start alone: the kernel after it may start; for a kernel launched
+// plainly, which has everything before it behind it)
+__device__ __forceinline__ void let_next_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void tick_kernel_begin() {
+  let_next_start();
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 

@@ -1111,6 +1111,7 @@ __global__ void __launch_bounds__(256, 4) k_decide(const int32_t* __restrict__ r
                          float beta, const float* __restrict__ own,
                          const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
                          WalkPeriods wp, Counters* __restrict__ ctr, int ring) {
+  let_next_start();  // the next band's gather copies its tables on the SMs that are done
   // grid-stride over the records of bins [b_lo, b_hi): a band's launch needs
   // no more blocks than the GPU holds, whatever its share of the crowd.  The
   // records are taken from the last backwards: the gather wrote the band's
