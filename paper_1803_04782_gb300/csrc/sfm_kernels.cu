@@ -1329,6 +1329,9 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
            const float* __restrict__ own, const float* __restrict__ dirdot, uint8_t* choice,
            uint8_t* won, Counters* ctr, WalkPeriods wp, Sizes sz,
            const int32_t* __restrict__ gid) {
+  // by pedestrian: the choices and wins of the stages before, not read back
+  // from memory
+  __shared__ uint8_t s_choice[kMoveMaxPeds], s_won[kMoveMaxPeds];
   tick_kernel_begin();
   const int i = threadIdx.x;
   const long long t = ctr->t;
@@ -1345,28 +1348,31 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
       const int2 q = xy[p];
       blocked = blocked_moves<1>(g, cell, occ, q.x, q.y, sz.w[p] >> 1, sz.h[p] >> 1, 0);
     }
-    choice[p] = decided ? decide_one<true, SIZED>(p, g, xy, heading, goal, ocls, D, F, 0, -1, -1,
-                                                  0, 0, g.H, beta, own, dirdot, &tie, 0, blocked)
-                        : (uint8_t)0;
+    const uint8_t k = decided ? decide_one<true, SIZED>(p, g, xy, heading, goal, ocls, D, F, 0, -1, -1, 0,
+                                                        0, g.H, beta, own, dirdot, &tie, 0, blocked)
+                              : (uint8_t)0;
+    s_choice[p] = choice[p] = k;
   }
   __syncthreads();
   int regs = 0;
   if (p >= 0) {
     if (SIZED) {
       bool win;
-      regs = vote_one_sized<1>(p, g, xy, choice, occ, sz.w, sz.h, seed, t, 0, win);
-      won[p] = win ? 1 : 0;
+      regs = vote_one_sized<1>(p, g, xy, s_choice, occ, sz.w, sz.h, seed, t, 0, win);
+      s_won[p] = win ? 1 : 0;
     } else {
-      regs = vote_one(p, 0, g, xy, choice, occ, seed, t, won, gid);
+      regs = vote_one(p, 0, g, xy, s_choice, occ, seed, t, s_won, gid);
     }
+    won[p] = s_won[p];
   }
   __syncthreads();
   bool moved = false, left = false;
   if (p >= 0) {
     if (SIZED)
-      commit_one_sized(p, g, xy, alive, heading, choice, won, cell, occ, ocls, sz.w, sz.h, moved, left);
+      commit_one_sized(p, g, xy, alive, heading, s_choice, s_won, cell, occ, ocls, sz.w, sz.h, moved,
+                       left);
     else
-      commit_one(p, g, xy, alive, heading, choice, won, cell, occ, ocls, moved, left);
+      commit_one(p, g, xy, alive, heading, s_choice, s_won, cell, occ, ocls, moved, left);
   }
   const unsigned nd = __popc(__ballot_sync(0xffffffffu, decided));
   const unsigned nt = __popc(__ballot_sync(0xffffffffu, tie));
