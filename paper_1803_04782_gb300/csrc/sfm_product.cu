@@ -566,35 +566,43 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
 
 // Entry [plane][chunk][j][limb][half of the 16 window columns][su column]
 // [window column]: the kernel at dy = j - r - 15, dx = su column - window
-// column + r, evaluated in FP64, zero outside the window.  A thread a limb pair.
+// column + r, evaluated in FP64, zero outside the window.  A thread takes an
+// entry (dx, dy) of the kernel and writes it wherever it stands, for up to eight
+// su columns and all channels: FP64 powers bound it (a thread a limb pair, one
+// for each, took 33 us at r = 40; now 13).
 __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, double a1, double gamma,
                               double s0, double s1, __half* __restrict__ tab) {
-  const int C = chunks_of(r), J = 2 * r + 31;
+  const int C = chunks_of(r), J = 2 * r + 31, E = 16 * C + 7;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nch * C * J * 128) return;
-  const int kx = i & 7, nx = (i >> 3) & 7, h = (i >> 6) & 1;
-  const int j = (i >> 7) % J, c = (i >> 7) / J % C, ch = (i >> 7) / J / C;
-  const int dy = j - r - 15, dx = nx - (16 * c + 8 * h + kx) + r;
-  double v = 0.0;
-  if (dx >= -r && dx <= r && dy >= -r && dy <= r && (dx | dy) != 0) {
-    const double d = sqrt((double)(dx * dx + dy * dy));
+  if (i >= E * J) return;
+  const int e = i % E, j = i / E;
+  const int dy = j - r - 15, dx = r + 7 - e;  // = su column - window column + r
+  const bool in = dx >= -r && dx <= r && dy >= -r && dy <= r && (dx | dy) != 0;
+  const double d = in ? sqrt((double)(dx * dx + dy * dy)) : 1.0;
+  const double v0 = in ? k0 * pow(d, a0) : 0.0, v1 = in && nch == 2 ? k1 * pow(d, a1) : 0.0;
+  for (int ch = 0; ch < nch; ++ch) {
+    double v = v0;
     if (nch == 2) {
-      v = ch == 0 ? k0 * pow(d, a0) : k1 * pow(d, a1);
+      if (ch == 1) v = v1;
     } else {
-      v = k0 * pow(d, a0);
       const double q = 0.70710678118654752440;  // 1 / sqrt(2)
       if (ch == 1) v *= gamma * dx / d;
       if (ch == 2) v *= gamma * dy / d;
       if (ch == 3) v *= gamma * q * (dx + dy) / d;
       if (ch == 4) v *= gamma * q * (dy - dx) / d;
     }
+    // an integer of FP16: any up to 2048, the nearest even one above
+    const __half hi = __double2half(fabs(v * s0) > 2048.0 ? v * s0 : rint(v * s0));
+    const __half lo = __double2half(rint((v * s0 - (double)__half2float(hi)) * s1));
+#pragma unroll
+    for (int nx = 0; nx < 8; ++nx) {
+      const int w = nx - 7 + e;  // the window column
+      if (w < 0 || w >= 16 * C) continue;
+      __half* o = tab + ((size_t)(ch * C + w / 16) * J + j) * 256 + (w >> 3 & 1) * 64 + nx * 8 + (w & 7);
+      o[0] = hi;
+      o[128] = lo;
+    }
   }
-  // an integer of FP16: any up to 2048, the nearest even one above
-  const __half hi = __double2half(fabs(v * s0) > 2048.0 ? v * s0 : rint(v * s0));
-  const __half lo = __double2half(rint((v * s0 - (double)__half2float(hi)) * s1));
-  __half* o = tab + ((size_t)(ch * C + c) * J + j) * 256 + h * 64 + nx * 8 + kx;
-  o[0] = hi;
-  o[128] = lo;
 }
 
 // A law k d^a over the window of radius r: largest and smallest magnitude and
@@ -654,9 +662,9 @@ size_t product_table_bytes(int r, int nch) { return (size_t)nch * chunks_of(r) *
 
 void launch_limb_tables(int r, const sfm_params& p, const ProductScales& sc, int nch, uint8_t* tab,
                         cudaStream_t s) {
-  const int n = nch * chunks_of(r) * (2 * r + 31) * 128;
+  const int n = (16 * chunks_of(r) + 7) * (2 * r + 31);
   const bool crowd = nch == 5;
-  k_limb_tables<<<(n + 255) / 256, 256, 0, s>>>(r, nch, crowd ? p.kP : p.kO, crowd ? p.aP : p.aO, p.kE,
+  k_limb_tables<<<(n + 63) / 64, 64, 0, s>>>(r, nch, crowd ? p.kP : p.kO, crowd ? p.aP : p.aO, p.kE,
                                                 p.aE, p.gamma, sc.s0, sc.s1, reinterpret_cast<__half*>(tab));
 }
 
