@@ -82,6 +82,10 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src));
 }
+// 16 bytes, or zeros
+__device__ __forceinline__ void cp_async16_if(uint32_t dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 16 : 0));
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::); }
@@ -697,18 +701,18 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // pixels x 8 inputs, so 34 16-byte shared reads feed 768 packed FMAs (even
 // and odd outputs o side by side).  Shared 16-byte groups are swizzled by the
 // pixel's eight (dZ) and the input's eight (weights): no bank conflicts.
-// 131 us a layer on a 512 x 512 image (695 with a thread a pixel, which
-// read a scalar weight from shared memory per FMA).
+// 122 us a layer on a 512 x 512 image (695 with a thread a pixel, which
+// read a scalar weight from shared memory per FMA; 131 without the second
+// buffer).
 constexpr int kDxW = 64, kDxH = 8, kDxThreads = 32 * kDxH;
 constexpr int kDxPx = (kDxH + 2) * (kDxW + 2);
-constexpr size_t kDxSmem = (size_t)(kDxPx * 32 + 9 * 32 * 32) * sizeof(float);
+constexpr size_t kDxSmem = (size_t)(2 * kDxPx * 32 + 9 * 32 * 32) * sizeof(float);
 
 __global__ void __launch_bounds__(kDxThreads, 1)
     k_conv3_dx(const float* __restrict__ dZ, int Hout, int Wout, const float* __restrict__ Wt,
                const bf16* __restrict__ Ain, float* __restrict__ dZin) {
   extern __shared__ __align__(16) float smf[];
-  float4* sD = reinterpret_cast<float4*>(smf);
-  float4* sW = sD + kDxPx * 8;
+  float4* sW = reinterpret_cast<float4*>(smf) + 2 * kDxPx * 8;
   const int Hin = Hout + 2, Win = Wout + 2;
   const int ntx = (Win + kDxW - 1) / kDxW, ntiles = ntx * ((Hin + kDxH - 1) / kDxH);
   const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
@@ -717,18 +721,27 @@ __global__ void __launch_bounds__(kDxThreads, 1)
     sW[(i & ~7) | (q ^ (c >> 3))] = reinterpret_cast<const float4*>(Wt)[i];
   }
   const int cg = lane & 3, pg = lane >> 2;  // inputs 8 cg .., pixels 8 pg ..
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+  // a tile's dZ into one of two buffers, the next one's while it is used
+  auto fetch = [&](int t, int buf) {
     const int x0 = t % ntx * kDxW, y0 = t / ntx * kDxH;
-    __syncthreads();
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(smf) + buf * kDxPx * 128;
     for (int i = tid; i < kDxPx * 8; i += kDxThreads) {
       const int q = i & 7, p = i >> 3, px = p % (kDxW + 2), py = p / (kDxW + 2);
       const int gy = y0 - 2 + py, gx = x0 - 2 + px;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (gy >= 0 && gy < Hout && gx >= 0 && gx < Wout)
-        v = __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q);
-      sD[p * 8 + (q ^ ((px >> 3) & 7))] = v;
+      const bool in = gy >= 0 && gy < Hout && gx >= 0 && gx < Wout;
+      cp_async16_if(at + (p * 8 + (q ^ ((px >> 3) & 7))) * 16,
+                    dZ + (in ? ((size_t)gy * Wout + gx) * 32 + q * 4 : 0), in);
     }
-    __syncthreads();
+    cp_async_commit();
+  };
+  int buf = 0;
+  if ((int)blockIdx.x < ntiles) fetch(blockIdx.x, 0);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
+    const int x0 = t % ntx * kDxW, y0 = t / ntx * kDxH;
+    const float4* sD = reinterpret_cast<const float4*>(smf) + buf * kDxPx * 8;
+    cp_async_wait_all();
+    __syncthreads();  // the tile is there, and the last one's buffer is free
+    if (t + (int)gridDim.x < ntiles) fetch(t + gridDim.x, buf ^ 1);
     float2 acc[8][8];
 #pragma unroll
     for (int p = 0; p < 8; ++p)
@@ -815,8 +828,9 @@ __global__ void __launch_bounds__(256)
 // like the data gradient.  Twelve warps: a kernel row ky and a tile row each;
 // lane = 4 inputs x 8 outputs of the three kx, whose inputs slide along the
 // row, so a pixel is 48 packed FMAs on three 16-byte shared reads:
-// 130 us a layer on a 512 x 512 image (620 with a thread a weight, two
-// scalar shared reads per FMA and a partial sum for every 16 x 16 tile).
+// 99 us a layer on a 512 x 512 image (620 with a thread a weight, two scalar
+// shared reads per FMA and a partial sum for every 16 x 16 tile; 130 with a
+// tile's reads one after the other).
 constexpr int kDwW = 64, kDwH = 4, kDwThreads = 32 * 3 * kDwH;
 constexpr int kDwIn = (kDwH + 2) * (kDwW + 2) * 32, kDwD = kDwH * kDwW * 32;  // floats
 constexpr int kDwE = kNW2 + kLh;
@@ -842,12 +856,32 @@ __global__ void __launch_bounds__(kDwThreads, 1)
   float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);  // outputs 4 (tid mod 8) .. of the pixels this thread loads
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int x0 = t % ntx * kDwW, y0 = t / ntx * kDwH;
-    __syncthreads();
-    for (int i = tid; i < kDwIn / 8; i += kDwThreads) {
-      const int q = i & 3, p = i >> 2, px = p % (kDwW + 2), py = p / (kDwW + 2);
+    // all of a thread's reads in flight, and while the other warps finish
+    constexpr int KI = (kDwIn / 8 + kDwThreads - 1) / kDwThreads, KD = (kDwD / 4 + kDwThreads - 1) / kDwThreads;
+    uint4 vi[KI];
+    float4 vd[KD];
+#pragma unroll
+    for (int k = 0; k < KI; ++k) {
+      const int i = tid + k * kDwThreads, q = i & 3, p = i >> 2, px = p % (kDwW + 2), py = p / (kDwW + 2);
       const int gy = y0 + py, gx = x0 + px;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (gy < Hin && gx < Win) v = __ldg(reinterpret_cast<const uint4*>(in) + ((size_t)gy * Win + gx) * 4 + q);
+      vi[k] = make_uint4(0u, 0u, 0u, 0u);
+      if (i < kDwIn / 8 && gy < Hin && gx < Win)
+        vi[k] = __ldg(reinterpret_cast<const uint4*>(in) + ((size_t)gy * Win + gx) * 4 + q);
+    }
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      const int i = tid + k * kDwThreads, q = i & 7, p = i >> 3, px = p % kDwW, py = p / kDwW;
+      const int gy = y0 + py, gx = x0 + px;
+      vd[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < kDwD / 4 && gy < Hout && gx < Wout)
+        vd[k] = __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < KI; ++k) {
+      const int i = tid + k * kDwThreads;
+      if (i >= kDwIn / 8) continue;
+      const uint4 v = vi[k];
       // BF16 to FP32: the upper half of the word
       float4* dst = reinterpret_cast<float4*>(sI) + i * 2;
       dst[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
@@ -855,12 +889,11 @@ __global__ void __launch_bounds__(kDwThreads, 1)
       dst[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u),
                            __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
     }
-    for (int i = tid; i < kDwD / 4; i += kDwThreads) {
-      const int q = i & 7, p = i >> 3, px = p % kDwW, py = p / kDwW;
-      const int gy = y0 + py, gx = x0 + px;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (gy < Hout && gx < Wout)
-        v = __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q);
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      const int i = tid + k * kDwThreads;
+      if (i >= kDwD / 4) continue;
+      const float4 v = vd[k];
       reinterpret_cast<float4*>(sD)[i] = v;
       bias.x += v.x;
       bias.y += v.y;
