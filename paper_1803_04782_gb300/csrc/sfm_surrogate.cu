@@ -1018,16 +1018,35 @@ __global__ void __launch_bounds__(kDw1Threads)
   for (int k = 0; k < 15; ++k) acc[k] = 0.f;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int x0 = t % ntx * kDw1W, y0 = t / ntx * kDw1H;
-    __syncthreads();
-    for (int i = tid; i < (kDw1H + 4) * kDw1Row; i += kDw1Threads) {
-      const int e = i % kDw1Row, py = i / kDw1Row, gy = y0 + py;
-      sX[py][e] = gy < Hin && x0 * 3 + e < Win * 3 ? __bfloat162float(in[((size_t)gy * Win + x0) * 3 + e]) : 0.f;
+    // all of a thread's reads in flight, and while the other warps finish
+    constexpr int NX = (kDw1H + 4) * kDw1Row, ND = kDw1H * kDw1W * 8;
+    constexpr int KX = (NX + kDw1Threads - 1) / kDw1Threads, KD = (ND + kDw1Threads - 1) / kDw1Threads;
+    float vx[KX];
+    float4 vd[KD];
+#pragma unroll
+    for (int k = 0; k < KX; ++k) {
+      const int i = tid + k * kDw1Threads, e = i % kDw1Row, gy = y0 + i / kDw1Row;
+      vx[k] = i < NX && gy < Hin && x0 * 3 + e < Win * 3
+                  ? __bfloat162float(in[((size_t)gy * Win + x0) * 3 + e])
+                  : 0.f;
     }
-    for (int i = tid; i < kDw1H * kDw1W * 8; i += kDw1Threads) {
-      const int q = i & 7, p = i >> 3, gy = y0 + p / kDw1W, gx = x0 + p % kDw1W;
-      reinterpret_cast<float4*>(sD)[i] =
-          gy < Hout && gx < Wout ? __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      const int i = tid + k * kDw1Threads, q = i & 7, p = i >> 3, gy = y0 + p / kDw1W, gx = x0 + p % kDw1W;
+      vd[k] = i < ND && gy < Hout && gx < Wout
+                  ? __ldg(reinterpret_cast<const float4*>(dZ) + ((size_t)gy * Wout + gx) * 8 + q)
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < KX; ++k) {
+      const int i = tid + k * kDw1Threads;
+      if (i < NX) sX[i / kDw1Row][i % kDw1Row] = vx[k];
+    }
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      const int i = tid + k * kDw1Threads;
+      if (i < ND) reinterpret_cast<float4*>(sD)[i] = vd[k];
     }
     __syncthreads();
     const float4* xr = reinterpret_cast<const float4*>(sX[row + ky]);
