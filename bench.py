@@ -43,14 +43,21 @@ TIMING_EVERY = 9
 # 16384^2 floor with 4 bands, from a one-pass ncu capture of this benchmark
 # (dram__bytes_read.sum + dram__bytes_write.sum); valid only while the
 # gather's sources hash to the value they had when it was taken.
-GATHER_TRAFFIC = {"sha1": "448dec8a766d3e7d1ab154ddb47feea4c66ca156", "bands": 4,
-                  "footprint": "32x32r", "workload": "floor", "bytes_per_launch": 492707968}
+GATHER_TRAFFIC = {"sha1": "9e2697147b7c692cd9322e530fd3a65a70542373", "bands": 4,
+                  "footprint": "32x32r", "workload": "floor", "bytes_per_launch": 495307648}
 GATHER_SOURCES = ("paper_1803_04782_gb300/csrc/sfm_gather.cuh",
                   "paper_1803_04782_gb300/csrc/sfm_field3.cu",
                   "paper_1803_04782_gb300/csrc/sfm_internal.h",
                   "paper_1803_04782_gb300/csrc/sfm_api.cu")  # the bands' row ranges
 # the gather kernel of each footprint
 GATHER_KERNEL = {"16x16": "k_field_v2", "32x16": "k_field_v2", "32x32r": "k_field_v3"}
+
+
+def gather_kernel(footprint, W, H, nsm) -> str:
+    """16 x 16 footprints have a kernel of their own up to 16 an SM."""
+    if footprint == "16x16" and -(-W // 16) * -(-H // 16) <= 16 * nsm:
+        return "k_field_few"
+    return GATHER_KERNEL.get(footprint, "k_field")
 
 
 def gather_sources_sha1() -> str:
@@ -430,7 +437,7 @@ def secondary_measurements(torch, sfm, stream, nsm, mhz, mhz_src, ticks=20):
     """The other configurations, measured in the same run as the headline so
     that their numbers come from the same box and clock: the 1000x200
     corridor and the 100x100 room (autotuned, unbanded), the batch of 256
-    rooms (one persistent launch per tick, autotuned), and the floor's exact
+    rooms (stepped together, autotuned), and the floor's exact
     tick with the field at each pedestrian's 9 candidates only (unbanded; the
     surrogate entry point with delta = +inf, which runs no network) beside
     its lattice tick."""
@@ -448,7 +455,7 @@ def secondary_measurements(torch, sfm, stream, nsm, mhz, mhz_src, ticks=20):
             out[name] = {"workload": desc, "ped_steps_per_s": int(a0.sum()) / (ms / 1e3),
                          "ms_per_tick": ms, "field_ms": fms, "footprint": fp,
                          "roofline": gather_roofline(pairs, fms / 1e3, nsm, mhz, mhz_src,
-                                                     GATHER_KERNEL.get(fp, "k_field"))}
+                                                     gather_kernel(fp, sc.W, sc.H, nsm))}
     scenes = SG.batch(nscenes=256)
     with sfm.Batch(scenes, stream=stream) as bt:
         bt.autotune()
@@ -604,7 +611,7 @@ def run_gpu(args):
     field_s = stage_ms["field"] / 1e3  # over the `ticks` timed ticks
     pairs = 0.5 * (pairs0 + pairs1)
     roofline = gather_roofline(pairs, field_s / ticks, nsm, mhz, mhz_src,
-                               GATHER_KERNEL.get(footprint, "k_field"),
+                               gather_kernel(footprint, sc.W, sc.H, nsm),
                                gather_traffic(args.workload, st1["bands"], footprint))
     roofline["timed_ticks"] = ticks
 
