@@ -1343,6 +1343,11 @@ __global__ void k_field_err(const float* __restrict__ Fa, const float* __restric
 // stays strictly above the surrogate's choice, so the choice is the exact
 // one (ties included).  ref / raw_flips (optional): count decisions that differ from
 // ref before the fallback.
+// Place of slot i's candidate k in fb_dd: 32 slots (a warp's) side by side.
+__host__ __device__ __forceinline__ size_t fb_at(int i, int k) {
+  return (size_t)(i >> 5) * (9 * 32) + k * 32 + (i & 31);
+}
+
 __device__ __forceinline__ float margin_allowance(float delta, float emag, float fmag) {
   return delta * 1.0001f + 1e-6f * (emag + fmag);
 }
@@ -1465,7 +1470,7 @@ __global__ void k_sur_decide(const int32_t* __restrict__ rec_id, const int32_t* 
       uint32_t mask = 0;
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        fb_dd[(size_t)i * 9 + k] = dd[k];
+        fb_dd[fb_at(i, k)] = dd[k];
         const int xi = move_dx(k) + 1, yi = move_dy(k) + 1;
         if (k == 0 || (okx[xi] && oky[yi] && dd[k] != kDWall && oc[k] == 0)) mask |= 1u << k;
       }
@@ -1525,7 +1530,7 @@ __device__ __forceinline__ uint8_t decide_listed(int i, int2 q, const Geo& g,
     int tx, ty;
     const bool ok = wrap_coord(q.x + move_dx(k), g.W, g.px, tx) & wrap_coord(q.y + move_dy(k), g.H, g.py, ty);
     f[k] = ok ? at(k, (size_t)ty * g.W + tx) : 0.f;
-    dd[k] = fb_dd[(size_t)i * 9 + k];
+    dd[k] = fb_dd[fb_at(i, k)];
     oc[k] = (info >> k) & 1u ? 0 : 1;  // admissible iff its mask bit is set
   }
   const bool ok3[3] = {true, true, true};
@@ -1661,7 +1666,7 @@ __global__ void k_list_all(const int32_t* __restrict__ rec_id, const int32_t* __
       uint32_t mask = 0;
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        fb_dd[(size_t)i * 9 + k] = dd[k];
+        fb_dd[fb_at(i, k)] = dd[k];
         const int xi = move_dx(k) + 1, yi = move_dy(k) + 1;
         if (k == 0 || (okx[xi] && oky[yi] && dd[k] != kDWall && oc[k] == 0)) mask |= 1u << k;
       }
@@ -2080,7 +2085,7 @@ sfm_status ensure_lattice(sfm_surrogate* S, sfm_ctx* ctx) {
     sfree(S, S->flag_list);
     sfree(S, S->fb_flag);
     sfree(S, S->perr);
-    STRY(salloc(S, &S->fb_dd, (size_t)ctx->cap * 9));
+    STRY(salloc(S, &S->fb_dd, fb_at((ctx->cap + 31) / 32 * 32, 0)));
     STRY(salloc(S, &S->fb_info, (size_t)ctx->cap));
     STRY(salloc(S, &S->flag_list, (size_t)ctx->cap));
     STRY(salloc(S, &S->fb_flag, (size_t)ctx->cap));
