@@ -1538,6 +1538,14 @@ __device__ __forceinline__ uint8_t decide_listed(int i, int2 q, const Geo& g,
                                    beta, own, dirdot, nullptr);
 }
 
+// running totals of listed and decided pedestrians over surrogate ticks
+__device__ __forceinline__ void add_fallbacks(const int32_t* __restrict__ nflag,
+                                              const int32_t* __restrict__ nrec,
+                                              unsigned long long* __restrict__ tot) {
+  tot[0] += (unsigned long long)*nflag;
+  tot[1] += (unsigned long long)*nrec;
+}
+
 constexpr int kFbRunBins = 8;  // widest run of bins whose pedestrians share one walk
 
 template <int SP>
@@ -1547,16 +1555,22 @@ __global__ void __launch_bounds__(kFbThreads, 1)
                    const uint32_t* __restrict__ rec, const float* __restrict__ CT, int TS,
                    const float* __restrict__ Fs, const int32_t* __restrict__ fb_dd,
                    const uint32_t* __restrict__ fb_info, float beta, const float* __restrict__ own,
-                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice) {
+                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
+                   const int32_t* __restrict__ nflag, unsigned long long* __restrict__ tot) {
   extern __shared__ __align__(16) float sm[];
+  if (tot && blockIdx.x == 0 && threadIdx.x == 0) add_fallbacks(nflag, bin_start + nbins, tot);
   float* sT = sm + kTableGuard;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int2* scr = reinterpret_cast<int2*>(sT + 4 * TS) + w * 32;
   copy_to_shared<8>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
   __syncthreads();
   const int nrec = bin_start[nbins], r = g.r;
-  const int nchunks = (nrec + 31) / 32;
-  for (int c = blockIdx.x * nw + w; c < nchunks; c += gridDim.x * nw) {
+  // every CTA an equal run of chunks (its warps share records through L1): the
+  // SMs' shared memory bounds this kernel (250 000 pedestrians at r = 40: 131 ->
+  // 121 us against rounds of a chunk a warp, the last of which filled 92 SMs)
+  const long long nchunks = (nrec + 31) / 32;
+  const int c1 = (int)(nchunks * (blockIdx.x + 1) / gridDim.x);
+  for (int c = (int)(nchunks * blockIdx.x / gridDim.x) + w; c < c1; c += nw) {
     const int i = c * 32 + lane;
     const bool fl = i < nrec && fb_flag[i] != 0;
     unsigned todo = __ballot_sync(0xffffffffu, fl);
@@ -1679,11 +1693,9 @@ __global__ void k_list_all(const int32_t* __restrict__ rec_id, const int32_t* __
   if ((threadIdx.x & 31) == 0 && nl) atomicAdd(nflag, (int32_t)nl);
 }
 
-// running totals of listed and decided pedestrians over surrogate ticks
 __global__ void k_count_fallbacks(const int32_t* __restrict__ nflag, const int32_t* __restrict__ nrec,
                                   unsigned long long* __restrict__ tot) {
-  tot[0] += (unsigned long long)*nflag;
-  tot[1] += (unsigned long long)*nrec;
+  add_fallbacks(nflag, nrec, tot);
 }
 
 // per pedestrian (bin order): the spread max - min of Fa - Fb over its
@@ -2169,10 +2181,11 @@ void surrogate_field(sfm_surrogate* S, sfm_ctx* ctx) {
 // from Fsur (surrogate_field).  ref/raw_flips as k_sur_decide.
 // The exact candidate field and decision of every listed pedestrian
 // (k_sur_fallback on the context's class tables).
-void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice);
+// `tot`: the totals of listed and decided pedestrians to add to, or none.
+void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigned long long* tot);
 
 void surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uint8_t* ref,
-                      unsigned long long* raw_flips, bool cand) {
+                      unsigned long long* raw_flips, bool cand, unsigned long long* tot = nullptr) {
   const Geo& g = ctx->geo;
   const Tables tb = ctx->tables();
   const int nbins = g.nbx * g.nby;
@@ -2187,7 +2200,7 @@ void surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uin
                                                   ctx->heading, ctx->goal, ctx->ocls, ctx->D, choice,
                                                   S->nflag, S->fb_flag, S->fb_dd, S->fb_info,
                                                   ctx->walk());
-    surrogate_fallback(S, ctx, choice);
+    surrogate_fallback(S, ctx, choice, tot);
     return;
   }
   NearPart np;
@@ -2201,10 +2214,10 @@ void surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uin
       ctx->D, S->Fsur, ctx->rec, ctx->Fs, np, far_part(S), ctx->prm.beta, tb.own, tb.dirdot,
       S->delta, choice, S->flag_list, S->nflag, S->fb_flag, S->fb_dd, S->fb_info, ref, raw_flips,
       ctx->walk());
-  surrogate_fallback(S, ctx, choice);
+  surrogate_fallback(S, ctx, choice, tot);
 }
 
-void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
+void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigned long long* tot) {
   const Geo& g = ctx->geo;
   const Tables tb = ctx->tables();
   const int nbins = g.nbx * g.nby;
@@ -2216,6 +2229,7 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
     k_sur_listed<<<cdiv(ctx->n, 256), 256, 0, st>>>(S->fb_flag, ctx->rec_id, ctx->bin_start, nbins, g, ctx->xy,
                                                     S->Fnear, S->fb_dd, S->fb_info, ctx->prm.beta, tb.own,
                                                     tb.dirdot, choice);
+    if (tot) k_count_fallbacks<<<1, 1, 0, st>>>(S->nflag, ctx->bin_start + nbins, tot);
     return;
   }
   const int SP = class_table_stride(g.r);
@@ -2224,7 +2238,7 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
                       (size_t)kFbThreads / 32 * 32 * sizeof(int2);
   void (*fb)(const uint8_t*, const int32_t*, int, Geo, const int2*, const int32_t*, const uint32_t*,
              const float*, int, const float*, const int32_t*, const uint32_t*, float, const float*,
-             const float*, uint8_t*);
+             const float*, uint8_t*, const int32_t*, unsigned long long*);
   switch (SP) {
     case 34: fb = k_sur_fallback<34>; break;
     case 50: fb = k_sur_fallback<50>; break;
@@ -2240,7 +2254,7 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   fb<<<nsm > 0 ? nsm : 1, kFbThreads, smem, st>>>(
       S->fb_flag, ctx->rec_id, nbins, g, ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs,
-      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice);
+      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice, S->nflag, tot);
 }
 
 void round_params(sfm_surrogate* S) {
@@ -2502,8 +2516,7 @@ sfm_status sfm_surrogate_step(sfm_surrogate* S, sfm_ctx* ctx, int32_t nsteps) {
   for (int i = 0; i < nsteps; ++i) {
     ctx_run_bins(ctx);
     if (!std::isinf(S->delta)) surrogate_far(S, ctx);  // delta = +inf: no network (exact tick)
-    surrogate_decide(S, ctx, ctx->choice, nullptr, nullptr, true);
-    k_count_fallbacks<<<1, 1, 0, st>>>(S->nflag, ctx->bin_start + g.nbx * g.nby, S->fb_dev);
+    surrogate_decide(S, ctx, ctx->choice, nullptr, nullptr, true, S->fb_dev);
     launch_vote(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->alive, ctx->choice, ctx->occ, g,
                 ctx->prm.seed, ctx->ctr, ctx->won, st, Sizes(), ctx->ids());
     launch_commit(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->alive, ctx->heading,
