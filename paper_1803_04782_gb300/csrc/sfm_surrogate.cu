@@ -1428,6 +1428,7 @@ __global__ void k_sur_decide(const int32_t* __restrict__ rec_id, const int32_t* 
                              int32_t* __restrict__ fb_dd, uint32_t* __restrict__ fb_info,
                              const uint8_t* __restrict__ ref,
                              unsigned long long* __restrict__ raw_flips, WalkPeriods wp) {
+  let_next_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   bool differs = false;
   const long long t = wp.period ? wp.ctr->t : 0;
@@ -1550,19 +1551,20 @@ constexpr int kFbRunBins = 8;  // widest run of bins whose pedestrians share one
 
 template <int SP>
 __global__ void __launch_bounds__(kFbThreads, 1)
-    k_sur_fallback(const uint8_t* __restrict__ fb_flag, const int32_t* __restrict__ rec_id, int nbins,
+    k_sur_fallback(const uint8_t* fb_flag, const int32_t* __restrict__ rec_id, int nbins,
                    Geo g, const int2* __restrict__ xy, const int32_t* __restrict__ bin_start,
                    const uint32_t* __restrict__ rec, const float* __restrict__ CT, int TS,
-                   const float* __restrict__ Fs, const int32_t* __restrict__ fb_dd,
-                   const uint32_t* __restrict__ fb_info, float beta, const float* __restrict__ own,
-                   const float* __restrict__ dirdot, uint8_t* __restrict__ choice,
-                   const int32_t* __restrict__ nflag, unsigned long long* __restrict__ tot) {
+                   const float* __restrict__ Fs, const int32_t* fb_dd,
+                   const uint32_t* fb_info, float beta, const float* __restrict__ own,
+                   const float* __restrict__ dirdot, uint8_t* choice,
+                   const int32_t* nflag, unsigned long long* __restrict__ tot) {
   extern __shared__ __align__(16) float sm[];
-  if (tot && blockIdx.x == 0 && threadIdx.x == 0) add_fallbacks(nflag, bin_start + nbins, tot);
   float* sT = sm + kTableGuard;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int2* scr = reinterpret_cast<int2*>(sT + 4 * TS) + w * 32;
   copy_to_shared<8>(reinterpret_cast<float2*>(sT), reinterpret_cast<const float2*>(CT), 2 * TS);
+  tick_kernel_begin();  // the tables never change: copied while the listing still runs
+  if (tot && blockIdx.x == 0 && threadIdx.x == 0) add_fallbacks(nflag, bin_start + nbins, tot);
   __syncthreads();
   const int nrec = bin_start[nbins], r = g.r;
   // every CTA an equal run of chunks (its warps share records through L1): the
@@ -1663,6 +1665,7 @@ __global__ void k_list_all(const int32_t* __restrict__ rec_id, const int32_t* __
                            uint8_t* __restrict__ choice, int32_t* __restrict__ nflag,
                            uint8_t* __restrict__ fb_flag, int32_t* __restrict__ fb_dd,
                            uint32_t* __restrict__ fb_info, WalkPeriods wp) {
+  let_next_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   bool listed = false;
   if (i < bin_start[nbins]) {
@@ -2252,9 +2255,11 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigne
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  fb<<<nsm > 0 ? nsm : 1, kFbThreads, smem, st>>>(
-      S->fb_flag, ctx->rec_id, nbins, g, ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs,
-      S->fb_dd, S->fb_info, ctx->prm.beta, tb.own, tb.dirdot, choice, S->nflag, tot);
+  // early, behind the plain launch that listed the pedestrians (four ticks of
+  // the 8192^2 floor 1078 -> 1062 us)
+  launch_tick_kernel(fb, nsm > 0 ? nsm : 1, kFbThreads, smem, st, true, S->fb_flag, ctx->rec_id, nbins, g,
+                     ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs, S->fb_dd, S->fb_info,
+                     ctx->prm.beta, tb.own, tb.dirdot, choice, S->nflag, tot);
 }
 
 void round_params(sfm_surrogate* S) {
