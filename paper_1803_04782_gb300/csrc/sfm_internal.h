@@ -192,9 +192,9 @@ inline int default_field_shape(int r, int W, int H) {
 constexpr int kProductMaxRadius = 44;
 // A lattice is crowded, and its field summed by the product and not by a
 // gather, from 9 pedestrians on 20 su.  The product is the faster way from
-// far fewer (its time does not depend on the crowd: at radius 38 a 1000 x
-// 1000 lattice half full takes 1298 us by the gather, 168 by the product, and
-// at radius 3 70 and 30, one-pass ncu), but the two round differently,
+// far fewer (its time does not depend on the crowd: bins and field of a 1000 x
+// 1000 lattice half full take 599 us by the gather at radius 38, 173 by the
+// product, and at radius 3 66 and 39), but the two round differently,
 // and in a run of many ticks one decision in 10^5 that falls the other way
 // moves its neighbours: the line lies above the room, corridor and batch
 // workloads (at most 2 su in 5), whose runs stay bit for bit what they were.
