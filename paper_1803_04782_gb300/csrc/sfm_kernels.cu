@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "sfm_gather.cuh"
+#include "sfm_guide_queue.h"
 #include "sfm_internal.h"
 
 namespace sfm {
@@ -192,48 +193,29 @@ void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, co
 constexpr int kGuideThreads = kTile * kTile;
 constexpr int kGuideSpins = 1 << 23;  // naps of an idle CTA, each 100 ns and more: about a second
 
-// Queue of tiles: entry pos of the run sits in ring[pos mod ntiles] with its
-// position, so nothing is cleared.  A tile is in it at most once (`queued`), so
-// an entry is never overwritten before it is taken.  `work` holds the entries
-// made so far (low half) and the tiles queued or being relaxed (high half), so
-// that one atomic makes an entry's place and keeps the run alive.
-struct GuideQueue {
-  unsigned long long work;
-  int head, pad;
-};
-struct GuideTiles {
-  GuideQueue* q;
-  unsigned long long* ring;  // (pos + 1) << 32 | tile
-  int* queued;
-};
-__host__ __device__ __forceinline__ GuideTiles guide_tiles(int* scratch, int ntiles) {
-  GuideTiles t;
-  t.q = reinterpret_cast<GuideQueue*>(scratch);
-  t.ring = reinterpret_cast<unsigned long long*>(t.q + 1);
-  t.queued = reinterpret_cast<int*>(t.ring + ntiles);
-  return t;
-}
-
-__device__ __forceinline__ void guide_push(const GuideTiles& gt, int ntiles, int t) {
-  if (atomicExch(&gt.queued[t], 1) != 0) return;
-  const unsigned pos = (unsigned)atomicAdd(&gt.q->work, (1ull << 32) + 1ull);
-  *reinterpret_cast<volatile unsigned long long*>(&gt.ring[pos % (unsigned)ntiles]) =
-      (unsigned long long)(pos + 1u) << 32 | (unsigned)t;
+__device__ __forceinline__ void guide_push(const GuideTiles& gt, int t, Counters* ctr) {
+  if (!guide_mark(gt, t)) return;
+  const unsigned pos = guide_position(gt);
+  for (int i = 0; !guide_publish(gt, pos, t); ++i) {
+    if (i == kGuideSpins) {
+      atomicOr(&ctr->err, kErrTimeout);
+      return;
+    }
+    __nanosleep(100);
+  }
 }
 
 // the next tile of the queue, -1 when no tile is left (or the wait ran out)
-__device__ int guide_pop(const GuideTiles& gt, int ntiles, Counters* ctr) {
-  const unsigned pos = (unsigned)atomicAdd(&gt.q->head, 1);
-  volatile unsigned long long* slot = &gt.ring[pos % (unsigned)ntiles];
+__device__ int guide_pop(const GuideTiles& gt, Counters* ctr) {
+  const unsigned pos = guide_claim(gt);
   for (int i = 0; i < kGuideSpins; ++i) {
-    const unsigned long long v = *slot;
-    if ((unsigned)(v >> 32) == pos + 1u) {
-      const int t = (int)(unsigned)v;
-      atomicExch(&gt.queued[t], 0);  // from here on a neighbour may queue it again
-      __threadfence();               // and its values are read after that
+    const int t = guide_take(gt, pos);
+    if (t >= 0) {
+      guide_unmark(gt, t);
+      __threadfence();  // its values are read after that
       return t;
     }
-    if ((*reinterpret_cast<volatile unsigned long long*>(&gt.q->work) >> 32) == 0) return -1;
+    if (guide_over(guide_work(gt))) return -1;
     __nanosleep(100);
   }
   atomicOr(&ctr->err, kErrTimeout);
@@ -250,7 +232,8 @@ __device__ __forceinline__ int guide_neighbour(const Geo& g, int ntx, int nty, i
 
 // start values, and the tiles that see an exit into the queue
 __global__ void __launch_bounds__(1024)
-    k_guidance_init(Geo g, const uint8_t* __restrict__ cell, int32_t* __restrict__ D, GuideTiles gt) {
+    k_guidance_init(Geo g, const uint8_t* __restrict__ cell, int32_t* __restrict__ D, GuideTiles gt,
+                    Counters* ctr) {
   const int ntx = (g.W + kTile - 1) / kTile, nty = (g.H + kTile - 1) / kTile;
   const int tx = blockIdx.x % ntx, ty = blockIdx.x / ntx;
   const int x = tx * kTile + (threadIdx.x & 31), y = ty * kTile + (threadIdx.x >> 5);
@@ -263,7 +246,7 @@ __global__ void __launch_bounds__(1024)
   }
   if (__syncthreads_or(source) && threadIdx.x < 9) {
     const int t = guide_neighbour(g, ntx, nty, tx, ty, (int)threadIdx.x % 3 - 1, (int)threadIdx.x / 3 - 1);
-    if (t >= 0) guide_push(gt, ntx * nty, t);
+    if (t >= 0) guide_push(gt, t, ctr);
   }
 }
 
@@ -317,7 +300,7 @@ __global__ void __launch_bounds__(kGuideThreads, 2)
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;  // lane: column, w: row (and column w of a scan)
   for (;;) {
     if (tid == 0) {
-      s_tile = guide_pop(gt, ntx * nty, ctr);
+      s_tile = guide_pop(gt, ctr);
       s_edge = 0u;
     }
     __syncthreads();
@@ -405,10 +388,10 @@ __global__ void __launch_bounds__(kGuideThreads, 2)
     if (tid < 32) {
       if (tid < 9 && ((s_edge >> tid) & 1u)) {
         const int t = guide_neighbour(g, ntx, nty, tx, ty, tid % 3 - 1, tid / 3 - 1);
-        if (t >= 0) guide_push(gt, ntx * nty, t);
+        if (t >= 0) guide_push(gt, t, ctr);
       }
       __syncwarp();
-      if (tid == 0) atomicAdd(&gt.q->work, ~0ull << 32);  // one open tile less
+      if (tid == 0) guide_done(gt);
     }
     __syncthreads();
   }
@@ -428,7 +411,7 @@ int device_sm_count() {
 
 size_t guidance_scratch_ints(const Geo& g) {
   const size_t ntiles = (size_t)cdiv(g.W, kTile) * cdiv(g.H, kTile);
-  return sizeof(GuideQueue) / sizeof(int) + 3 * ntiles;
+  return kGuideQueueInts + kGuideTileInts * ntiles;
 }
 
 void launch_guidance(const Geo& g, const uint8_t* cell, int32_t* D, int* scratch, Counters* ctr,
@@ -436,8 +419,8 @@ void launch_guidance(const Geo& g, const uint8_t* cell, int32_t* D, int* scratch
   const int ntiles = cdiv(g.W, kTile) * cdiv(g.H, kTile);
   const GuideTiles gt = guide_tiles(scratch, ntiles);
   cudaMemsetAsync(scratch, 0, guidance_scratch_ints(g) * sizeof(int), s);
-  k_guidance_init<<<ntiles, 1024, 0, s>>>(g, cell, D, gt);
-  // idle CTAs wait for work that running ones make, never for one another
+  k_guidance_init<<<ntiles, 1024, 0, s>>>(g, cell, D, gt, ctr);
+  // CTAs wait for what running ones put into the queue or take out of it
   const int fit = 2 * device_sm_count();
   const int blocks = ntiles < fit ? ntiles : fit;
   k_guidance<<<blocks, kGuideThreads, 0, s>>>(g, D, gt, ctr);
