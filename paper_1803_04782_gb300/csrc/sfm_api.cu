@@ -150,8 +150,9 @@ sfm_status check_flags(sfm_ctx* ctx) {
 // ya-1 and yb (wrapped in periodic y) at out rows 0 and yb-ya+1.  Uses whole
 // tiles so every su is summed in the same order in every mode.  A crowded
 // lattice's rows come from the product, whose sums are exact.
-void launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int ring = 0,
-                     bool early = false) {
+cudaError_t launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int ring = 0,
+                            bool early = false) {
+  ++c->launches;
   if (c->use_product()) {
     ProductArgs a = c->prod;
     a.out = out;
@@ -159,28 +160,24 @@ void launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int r
     a.store_lo = lo;
     a.store_hi = hi;
     a.ring = ring;
-    launch_product(a, c->stream);
-  } else {
-    launch_field(c->geo, c->bin_start, c->rec, c->tables(), c->Fs, out, out_row0, lo, hi, c->ctr,
-                 c->stream, FarPart(), ring, early);
+    return launch_product(a, c->stream);
   }
-  ++c->launches;
+  return launch_field(c->geo, c->bin_start, c->rec, c->tables(), c->Fs, out, out_row0, lo, hi, c->ctr,
+                      c->stream, FarPart(), ring, early);
 }
 
-void field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos,
-                bool early = false) {
+cudaError_t field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos,
+                       bool early = false) {
   const Geo& g = c->geo;
-  if (!halos) {
-    launch_field_of(c, out, ya - main_off, ya, yb, 0, early);
-    return;
-  }
+  if (!halos) return launch_field_of(c, out, ya - main_off, ya, yb, 0, early);
   // one launch for the band and its in-lattice halo rows ya-1 and yb (out rows
   // 0 and yb-ya+1 follow from the same row mapping, main_off == 1)
   const int lo = ya - 1 >= 0 ? ya - 1 : 0, hi = yb + 1 <= g.H ? yb + 1 : g.H;
-  launch_field_of(c, out, ya - main_off, lo, hi);
+  cudaError_t e = launch_field_of(c, out, ya - main_off, lo, hi);
   // halo rows that wrap around a periodic y boundary
-  if (g.py && ya == 0) launch_field_of(c, out, g.H - 1, g.H - 1, g.H);
-  if (g.py && yb == g.H) launch_field_of(c, out, -(yb - ya + 1), 0, 1);
+  if (e == cudaSuccess && g.py && ya == 0) e = launch_field_of(c, out, g.H - 1, g.H - 1, g.H);
+  if (e == cudaSuccess && g.py && yb == g.H) e = launch_field_of(c, out, -(yb - ya + 1), 0, 1);
+  return e;
 }
 
 // Pedestrian-list binning when the crowd is sparse: its cost follows the
@@ -213,24 +210,27 @@ void run_bins(sfm_ctx* c, bool early = false) {
 // band before (7338 -> 7285 us for four ticks of 16384 x 16384).  Decide, vote and commit, and the list's binning, do not:
 // blocks that start early pile up on the SMs that are free first (163 -> 186
 // us a tick of 4096 x 4096 at r = 40 with all of them early).
-void run_tick(sfm_ctx* c) {
+// A field whose launch is refused ends the tick: nobody decides on an old one.
+cudaError_t run_tick(sfm_ctx* c) {
   StageScope whole(c, SFM_STAGE_STEP);
   const Geo& g = c->geo;
   const Tables tb = c->tables();
   const int nbins = g.nbx * g.nby;
   const bool early = !c->timing && nbins <= kBinsPrefix && !bins_from_peds(c);
   run_bins(c, early);
+  cudaError_t e = cudaSuccess;
   if (c->bands <= 1) {
     {
       StageScope sc(c, SFM_STAGE_FIELD);
-      field_rows(c, c->F, 0, g.H, 0, false, early);
+      e = field_rows(c, c->F, 0, g.H, 0, false, early);
     }
+    if (e != cudaSuccess) return e;
     if (!c->timing && c->n > 0 && c->n <= kMoveMaxPeds) {
       launch_move(c->n, c->rec_id, c->bin_start, c->xy, c->alive, c->heading, c->goal, c->cell, c->occ,
                   c->ocls, c->D, c->F, g, c->prm.beta, c->prm.seed, tb, c->choice, c->won, c->ctr,
                   c->stream, c->walk(), c->sizes(), c->ids(), early);
       ++c->launches;
-      return;
+      return cudaSuccess;
     }
     if (c->n > 0 && !c->sized && move_by_bins(g.W, g.H, c->n)) {
       {
@@ -247,7 +247,7 @@ void run_tick(sfm_ctx* c) {
       launch_commit_bins(g, c->bin_start, c->rec, c->rec_id, c->xy, c->alive, c->heading, c->cell, c->occ,
                          c->ocls, c->ctr, c->stream);
       c->launches += 3;
-      return;
+      return cudaSuccess;
     }
     StageScope sc(c, SFM_STAGE_DECIDE);
     launch_decide(c->n, c->rec_id, c->bin_start, 0, nbins, c->xy, c->heading, c->goal, c->cell,
@@ -271,8 +271,9 @@ void run_tick(sfm_ctx* c) {
       const int s_hi = yb + kTile < g.H ? yb + kTile : g.H;
       if (s_hi > s_lo) {
         StageScope sc(c, SFM_STAGE_FIELD);
-        launch_field_of(c, c->band_buf, s_lo - s_lo % R, s_lo, s_hi, R, !c->timing);
+        e = launch_field_of(c, c->band_buf, s_lo - s_lo % R, s_lo, s_hi, R, !c->timing);
       }
+      if (e != cudaSuccess) return e;
       const int y_lo = ya > 0 ? ya - 1 : 0, y_hi = yb + 1 < g.H ? yb + 1 : g.H;
       StageScope sc(c, SFM_STAGE_DECIDE);
       launch_decide(c->n, c->rec_id, c->bin_start, (ya / kBin) * g.nbx,
@@ -287,8 +288,9 @@ void run_tick(sfm_ctx* c) {
       const int yb = ya + c->band_rows < g.H ? ya + c->band_rows : g.H;
       {
         StageScope sc(c, SFM_STAGE_FIELD);
-        field_rows(c, c->band_buf, ya, yb, 1, true);
+        e = field_rows(c, c->band_buf, ya, yb, 1, true);
       }
+      if (e != cudaSuccess) return e;
       int lo = ya - 1, hi = yb;
       if (lo < 0) lo = g.py ? lo + g.H : -1;
       if (hi >= g.H) hi = g.py ? hi - g.H : -1;
@@ -310,6 +312,7 @@ void run_tick(sfm_ctx* c) {
   launch_commit(c->n, c->rec_id, c->bin_start, c->xy, c->alive, c->heading, c->choice, c->won,
                 c->cell, c->occ, c->ocls, g, c->ctr, c->stream, c->sizes());
   ++c->launches;
+  return cudaSuccess;
 }
 
 void drop_graph(sfm_ctx* c) {
@@ -343,9 +346,9 @@ cudaError_t build_tick_graph(sfm_ctx* c, int ticks, cudaGraphExec_t* exec, int64
   c->stream = cs;
   e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    for (int i = 0; i < ticks; ++i) run_tick(c);
+    for (int i = 0; i < ticks && e == cudaSuccess; ++i) e = run_tick(c);
     const cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
-    e = e2;
+    if (e == cudaSuccess) e = e2;
   }
   c->stream = saved;
   *launches = c->launches - l0;
@@ -371,8 +374,9 @@ cudaError_t build_timed_graph(sfm_ctx* c) {
   c->capturing_timed = true;
   e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    run_tick(c);
-    e = cudaStreamEndCapture(cs, &graph);
+    e = run_tick(c);
+    const cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
+    if (e == cudaSuccess) e = e2;
   }
   c->capturing_timed = false;
   c->stream = saved;
@@ -532,8 +536,8 @@ sfm_status copy_out(sfm_ctx* ctx, void* dst, const void* src, size_t bytes, int 
 
 void sfm::set_create_error(const std::string& msg) { g_create_err = msg; }
 void sfm::ctx_run_bins(sfm_ctx* c) { run_bins(c); }
-void sfm::ctx_field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos) {
-  field_rows(c, out, ya, yb, main_off, halos);
+cudaError_t sfm::ctx_field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos) {
+  return field_rows(c, out, ya, yb, main_off, halos);
 }
 
 extern "C" {
@@ -868,7 +872,7 @@ sfm_status sfm_step(sfm_ctx* ctx, int32_t nsteps) {
     const bool timed = every > 0 && ctx->timing_phase == 0;
     ctx->timing = timed;
     if (ctx->direct_ticks < 1) {
-      run_tick(ctx);
+      CU(run_tick(ctx));
       ++ctx->direct_ticks;
       ++ctx->t;
       ++i;
@@ -912,7 +916,7 @@ sfm_status sfm_compute_field(sfm_ctx* ctx) {
   run_bins(ctx);
   {
     StageScope sc(ctx, SFM_STAGE_FIELD);
-    field_rows(ctx, ctx->F, 0, ctx->geo.H, 0, false);
+    CU(field_rows(ctx, ctx->F, 0, ctx->geo.H, 0, false));
   }
   CU(cudaGetLastError());
   return SFM_OK;
@@ -925,7 +929,7 @@ sfm_status sfm_compute_field_into(sfm_ctx* ctx, float* dst, int32_t on_device) {
   const Geo& g = ctx->geo;
   run_bins(ctx);
   if (on_device) {
-    field_rows(ctx, dst, 0, g.H, 0, false);
+    CU(field_rows(ctx, dst, 0, g.H, 0, false));
     CU(cudaGetLastError());
     return check_flags(ctx);
   }
@@ -933,7 +937,7 @@ sfm_status sfm_compute_field_into(sfm_ctx* ctx, float* dst, int32_t on_device) {
   const int rows = ctx->bands > 1 ? ctx->band_rows : g.H;
   for (int ya = 0; ya < g.H; ya += rows) {
     const int yb = ya + rows < g.H ? ya + rows : g.H;
-    field_rows(ctx, buf, ya, yb, 0, false);
+    CU(field_rows(ctx, buf, ya, yb, 0, false));
     CU(cudaMemcpyAsync(dst + (size_t)ya * g.W, buf, (size_t)(yb - ya) * g.W * sizeof(float),
                        cudaMemcpyDeviceToHost, ctx->stream));
   }
@@ -964,7 +968,7 @@ sfm_status sfm_autotune(sfm_ctx* ctx, int32_t* shape_out) {
     float tot = 0.f;
     for (int rep = 0; rep < 3; ++rep) {
       CU(cudaEventRecord(e0, ctx->stream));
-      field_rows(ctx, out, 0, rows, 0, false);
+      CU(field_rows(ctx, out, 0, rows, 0, false));
       CU(cudaEventRecord(e1, ctx->stream));
       CU(cudaEventSynchronize(e1));
       float ms = 0.f;

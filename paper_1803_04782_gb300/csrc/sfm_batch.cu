@@ -651,7 +651,10 @@ sfm_status setup_product(sfm_ctx* ctx) {
 
 cudaError_t launch_tick(sfm_ctx* ctx, int field_only, cudaStream_t s) {
   BatchState* B = ctx->batch;
-  if (B->prod.ntiles) launch_product(B->prod, s);
+  if (B->prod.ntiles) {
+    const cudaError_t e = launch_product(B->prod, s);
+    if (e != cudaSuccess) return e;
+  }
   BatchArgs a = make_args(ctx);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(B->grid);
@@ -908,7 +911,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = batch_smem(B);
-    cudaFuncSetAttribute(k_tick_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(k_tick_batch, max_gather_shared(kBatchThreads));
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tick_batch, kBatchThreads, smem);
     if (per_sm < 1) {
       ctx->err = "batched tick does not fit an SM";

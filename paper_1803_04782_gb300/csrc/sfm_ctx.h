@@ -15,7 +15,7 @@ struct BatchState;  // sfm_batch.cu
 void set_create_error(const std::string& msg);
 // bins of the context's current state (S1), field rows (S2) into `out`
 void ctx_run_bins(sfm_ctx* c);
-void ctx_field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos);
+cudaError_t ctx_field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, bool halos);
 // batched lattices (sfm_batch.cu)
 sfm_status batch_tick(sfm_ctx* ctx, int nsteps, int field_only);
 sfm_status batch_sync(sfm_ctx* ctx);

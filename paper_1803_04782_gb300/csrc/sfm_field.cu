@@ -369,13 +369,14 @@ __global__ void __launch_bounds__(kFewThreads, 1)
 static int g_num_sms = 0;
 
 template <int SP, int SHAPE, int FAR>
-static void launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const float* CT,
-                      const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-                      cudaStream_t s, const FarPart& far, unsigned int* tickets, bool sorted, bool early) {
+static cudaError_t launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
+                             const float* CT, const float* Fs, float* out, int out_row0, int store_lo,
+                             int store_hi, cudaStream_t s, const FarPart& far, unsigned int* tickets,
+                             bool sorted, bool early) {
   constexpr int FW = SHAPE ? 32 : 16, FH = 16;
   const size_t smem = (kTableGuard + class_table_floats(g.r)) * sizeof(float) +
                       kV2Threads / 32 * 32 * sizeof(int2);
-  cudaFuncSetAttribute(k_field_v2<SP, SHAPE, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(k_field_v2<SP, SHAPE, FAR>, max_gather_shared(kV2Threads));
   if (!g_num_sms) {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -393,47 +394,42 @@ static void launch_v2(const Geo& g, const int32_t* bin_start, const uint32_t* re
   if constexpr (SHAPE == 0 && FAR == 0 && SP != kNarrowStride) {
     if (nf <= kFewPerSm * g_num_sms) {
       const size_t few = (kTableGuard + class_table_floats(g.r)) * sizeof(float) + kFewThreads * sizeof(int2);
-      cudaFuncSetAttribute(k_field_few<SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)few);
-      launch_tick_kernel(k_field_few<SP>, blocks, kFewThreads, few, s, early, g, bin_start, rec, CT, Fs, out,
-                         out_row0, fy0, fy1, store_lo, store_hi, sorted);
-      return;
+      allow_shared(k_field_few<SP>, max_gather_shared(kFewThreads));
+      return launch_tick_kernel(k_field_few<SP>, blocks, kFewThreads, few, s, early, g, bin_start, rec, CT,
+                                Fs, out, out_row0, fy0, fy1, store_lo, store_hi, sorted);
     }
   }
   // tickets only where there are whole rounds to rebalance (4 footprints per
   // warp or more); a small lattice keeps the static deal, without the
   // counter's atomics at the start and end of the launch
   if (nf < 4 * wpb * blocks) tickets = nullptr;
-  launch_tick_kernel(k_field_v2<SP, SHAPE, FAR>, blocks, kV2Threads, smem, s, early, g, bin_start, rec,
-                     CT, Fs, out, out_row0, fy0, fy1, store_lo, store_hi, far, tickets, sorted);
+  return launch_tick_kernel(k_field_v2<SP, SHAPE, FAR>, blocks, kV2Threads, smem, s, early, g, bin_start,
+                            rec, CT, Fs, out, out_row0, fy0, fy1, store_lo, store_hi, far, tickets, sorted);
 }
 
 template <int SP>
-static void launch_v2_shape(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
-                            const Tables& tb, const float* Fs, float* out, int out_row0,
-                            int store_lo, int store_hi, cudaStream_t s, const FarPart& far,
-                            unsigned int* tickets, bool sorted, bool early) {
+static cudaError_t launch_v2_shape(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
+                                   const Tables& tb, const float* Fs, float* out, int out_row0,
+                                   int store_lo, int store_hi, cudaStream_t s, const FarPart& far,
+                                   unsigned int* tickets, bool sorted, bool early) {
   // the far part (surrogate) has its own instantiations, 32 x 16 footprint
   // only (one for coarsening 8, one for any), so the exact gather carries no
   // code for it
   if (far.Y && far.s == 8)
-    launch_v2<SP, 1, 8>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
-  else if (far.Y)
-    launch_v2<SP, 1, 1>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
-  else if (tb.shape != kShape16x16)  // the row-trimmed shape where that gather is off
-    launch_v2<SP, 1, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
-  else
-    launch_v2<SP, 0, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    return launch_v2<SP, 1, 8>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+  if (far.Y)
+    return launch_v2<SP, 1, 1>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+  if (tb.shape != kShape16x16)  // the row-trimmed shape where that gather is off
+    return launch_v2<SP, 1, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+  return launch_v2<SP, 0, 0>(g, bin_start, rec, tb.CT, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
 }
 
-void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
-                  const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
-                  Counters* ctr, cudaStream_t s, const FarPart& far, int ring, bool early) {
-  if (store_hi <= store_lo) return;
+cudaError_t launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
+                         const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
+                         Counters* ctr, cudaStream_t s, const FarPart& far, int ring, bool early) {
+  if (store_hi <= store_lo) return cudaSuccess;
   const int sp = tb.CT ? class_table_stride(g.r) : 0;
-  if (!sp) {
-    launch_field_v1(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, ctr, s);
-    return;
-  }
+  if (!sp) return launch_field_v1(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, ctr, s);
   // the context's footprint ticket counter (no counter: a static schedule).
   // The far-part gather keeps the static one: its footprints cost about the
   // same everywhere (a 7 x 7 window and the epilogue), and they are so short
@@ -443,18 +439,19 @@ void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, c
   // a context's bins are sorted by row; those of the allocation-free field,
   // which has none, are in order of arrival
   const bool sorted = ctr != nullptr;
+  cudaError_t e = cudaSuccess;
   if (!far.Y && launch_field_v3(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi,
-                                tickets, sorted, s, ring, early))
-    return;
-  if (ring) return;  // the caller checked that the row-trimmed gather is in use
+                                tickets, sorted, s, ring, early, &e))
+    return e;
+  if (ring) return cudaErrorInvalidValue;  // the caller checked that the row-trimmed gather is in use
   switch (sp) {
-    case 34: launch_v2_shape<34>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
-    case 50: launch_v2_shape<50>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
-    case 66: launch_v2_shape<66>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
-    case 82: launch_v2_shape<82>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
-    case 98: launch_v2_shape<98>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
-    case 114: launch_v2_shape<114>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
-    default: launch_v2_shape<kNarrowStride>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early); break;
+    case 34: return launch_v2_shape<34>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    case 50: return launch_v2_shape<50>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    case 66: return launch_v2_shape<66>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    case 82: return launch_v2_shape<82>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    case 98: return launch_v2_shape<98>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    case 114: return launch_v2_shape<114>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
+    default: return launch_v2_shape<kNarrowStride>(g, bin_start, rec, tb, Fs, out, out_row0, store_lo, store_hi, s, far, tickets, sorted, early);
   }
 }
 

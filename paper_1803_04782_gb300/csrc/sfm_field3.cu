@@ -192,13 +192,14 @@ __global__ void __launch_bounds__(kField3Threads, 1)
 }
 
 template <int SP, int FH>
-void launch_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const float* CT3,
+cudaError_t launch_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const float* CT3,
                const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
                cudaStream_t s, unsigned int* tickets, bool sorted, int ring, bool early) {
   constexpr int FW = 32;
   const size_t smem = (kTableGuard + field3_table_floats(g.r)) * sizeof(float) +
                       kField3Threads / 32 * 32 * sizeof(int2);
-  cudaFuncSetAttribute(k_field_v3<SP, FH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(k_field_v3<SP, FH>, (kTableGuard + max_field3_table_floats()) * sizeof(float) +
+                                       kField3Threads * sizeof(int2));
   const int nsm = device_sm_count();
   const int fy0 = store_lo / FH, fy1 = (store_hi + FH - 1) / FH;
   const int nf = ((g.W + FW - 1) / FW) * (fy1 - fy0);
@@ -209,18 +210,19 @@ void launch_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec, cons
   if (blocks > nsm) blocks = nsm;
   if (blocks < 1) blocks = 1;
   if (nf < 4 * wpb * blocks) tickets = nullptr;
-  launch_tick_kernel(k_field_v3<SP, FH>, blocks, kField3Threads, smem, s, early, g, bin_start, rec, CT3, Fs,
-                     out, out_row0, fy0, fy1, store_lo, store_hi, tickets, sorted, ring);
+  return launch_tick_kernel(k_field_v3<SP, FH>, blocks, kField3Threads, smem, s, early, g, bin_start, rec,
+                            CT3, Fs, out, out_row0, fy0, fy1, store_lo, store_hi, tickets, sorted, ring);
 }
 
 }  // namespace
 
 bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                      const Tables& tb, const float* Fs, float* out, int out_row0, int store_lo,
-                     int store_hi, unsigned int* tickets, bool sorted, cudaStream_t s, int ring, bool early) {
+                     int store_hi, unsigned int* tickets, bool sorted, cudaStream_t s, int ring, bool early,
+                     cudaError_t* launched) {
   if (!tb.CT3 || !field3_shape_ok(tb.shape, g.r)) return false;
 #define SFM_V3(SP) \
-  case SP: launch_v3<SP, 32>(g, bin_start, rec, tb.CT3, Fs, out, out_row0, store_lo, store_hi, s, tickets, sorted, ring, early); break;
+  case SP: *launched = launch_v3<SP, 32>(g, bin_start, rec, tb.CT3, Fs, out, out_row0, store_lo, store_hi, s, tickets, sorted, ring, early); break;
   // one footprint: 32 x 32 su (measured against 32 x 16 and 16 x 32 row-
   // trimmed footprints, it was the fastest on the 16384^2 floor at r = 40)
   switch (field3_stride(g.r)) {

@@ -99,6 +99,20 @@ constexpr size_t max_field3_table_floats() {
 static_assert((kTableGuard + max_field3_table_floats()) * 4 + kField3Threads / 32 * 32 * 8 <=
                   227 * 1024,
               "row-trimmed gather tables exceed shared memory");
+// Dynamic shared memory that `k` may be launched with: a limit of the whole
+// device context, so it is always the most that any launch of k asks for, never
+// what one launch needs (which another host thread's launch, or another
+// context's captured one, may exceed).
+template <class K>
+inline cudaError_t allow_shared(K* k, size_t most) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+// ... of a gather's CTA of `threads` at any radius up to kMaxTableRadius
+constexpr size_t max_gather_shared(int threads) {
+  return (kTableGuard + max_class_table_floats(kMaxTableRadius)) * sizeof(float) +
+         (size_t)threads * sizeof(int2);
+}
+
 // the row-trimmed footprint `shape` can run at radius r
 constexpr bool field3_shape_ok(int shape, int r) {
   return field3_stride(r) != 0 && shape == kShape32x32;
@@ -241,7 +255,7 @@ void product_layout(int rmax, ProductArgs* a);  // shared-memory split for radii
 int product_tiles_x(int W);
 int product_tiles_y(int H);
 size_t product_scratch_floats();
-void launch_product(ProductArgs a, cudaStream_t s);
+cudaError_t launch_product(ProductArgs a, cudaStream_t s);
 
 // ---- launchers (sfm_kernels.cu) ----
 void launch_tables(int r, const sfm_params& p, float* T0, float* TX, float* TY, float* KO,
@@ -302,13 +316,14 @@ void launch_reset_counters(Counters* ctr, cudaStream_t s);
 // out[(y - out_row0) * W + x].  Every su is summed in the same order whatever
 // the row range, so banded and unbanded passes agree bit for bit.
 // the three-component gather (radius > 50), called by launch_field
-void launch_field_v1(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
+cudaError_t launch_field_v1(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
                      const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
                      Counters* ctr, cudaStream_t s);
 // ring > 0: out is a ring of `ring` rows, row y stored at (y - out_row0) mod
 // ring (y - out_row0 < 2 ring); only the row-trimmed gather takes one
 // (launch_field_v3 returns false otherwise)
-void launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
+// returns the launch's status: a tick stops where its field was refused
+cudaError_t launch_field(const Geo& g, const int32_t* bin_start, const uint32_t* rec, const Tables& tb,
                   const float* Fs, float* out, int out_row0, int store_lo, int store_hi,
                   Counters* ctr, cudaStream_t s, const FarPart& far = FarPart(), int ring = 0,
                   bool early = false);
@@ -322,8 +337,8 @@ void launch_class_tables(int r, const sfm_params& p, float* T, cudaStream_t s,
 // radius, the tables or the footprint do not select it
 bool launch_field_v3(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                      const Tables& tb, const float* Fs, float* out, int out_row0, int store_lo,
-                     int store_hi, unsigned int* tickets, bool sorted, cudaStream_t s, int ring = 0,
-                     bool early = false);
+                     int store_hi, unsigned int* tickets, bool sorted, cudaStream_t s, int ring,
+                     bool early, cudaError_t* launched);
 void launch_class_tables3(int r, const sfm_params& p, float* T, cudaStream_t s);
 
 // The per-pedestrian stages visit the live pedestrians of bins [b_lo, b_hi)

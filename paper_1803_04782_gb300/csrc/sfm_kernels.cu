@@ -167,7 +167,8 @@ void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, co
   }
   const int S = 2 * g.r + 1, HW = kTile + 2 * g.r;
   const size_t smem = (size_t)2 * S * S * sizeof(float) + (size_t)HW * HW;
-  cudaFuncSetAttribute(k_static_field, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int kMaxS = 2 * SFM_MAX_RADIUS + 1, kMaxHW = kTile + 2 * SFM_MAX_RADIUS;
+  allow_shared(k_static_field, (size_t)2 * kMaxS * kMaxS * sizeof(float) + (size_t)kMaxHW * kMaxHW);
   dim3 grid(cdiv(g.W, kTile), cdiv(g.H, kTile));
   k_static_field<<<grid, kFieldThreads, smem, s>>>(g, cell, tb.KO, tb.KE, Fs);
 }
@@ -1036,27 +1037,30 @@ __global__ void __launch_bounds__(kFieldThreads)
   }
 }
 
+constexpr size_t kFieldBudget = 200 * 1024;
+static_assert((size_t)3 * (2 * SFM_MAX_RADIUS + 1) * (2 * SFM_MAX_RADIUS + 1) * sizeof(float) +
+                      256 * sizeof(int4) <= kFieldBudget, "tables and a chunk fit at any radius");
 static int field_cap(int r, size_t* smem_out) {
   const int S = 2 * r + 1;
   const size_t tables = (size_t)3 * S * S * sizeof(float);
-  const size_t budget = 200 * 1024;
   int cap = kStageCap;
-  while (cap > 256 && tables + (size_t)cap * sizeof(int4) > budget) cap >>= 1;
+  while (cap > 256 && tables + (size_t)cap * sizeof(int4) > kFieldBudget) cap >>= 1;
   *smem_out = tables + (size_t)cap * sizeof(int4);
   return cap;
 }
 
-void launch_field_v1(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
+cudaError_t launch_field_v1(const Geo& g, const int32_t* bin_start, const uint32_t* rec,
                             const Tables& tb, const float* Fs, float* out, int out_row0,
                             int store_lo, int store_hi, Counters* ctr, cudaStream_t s) {
   const int ty0 = store_lo / kTile, ty1 = (store_hi + kTile - 1) / kTile;
-  if (ty1 <= ty0) return;
+  if (ty1 <= ty0) return cudaSuccess;
   size_t smem;
   const int cap = field_cap(g.r, &smem);
-  cudaFuncSetAttribute(k_field, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(k_field, kFieldBudget);
   dim3 grid(cdiv(g.W, kTile), ty1 - ty0);
   k_field<<<grid, kFieldThreads, smem, s>>>(g, bin_start, rec, tb, Fs, out, out_row0, ty0,
                                             store_lo, store_hi, cap, ctr);
+  return cudaPeekAtLastError();
 }
 
 __global__ void k_class_tables(int r, int SP, double kP, double aP, double gamma, double taper_in,

@@ -684,16 +684,17 @@ int product_tiles_x(int W) { return (W + kTW - 1) / kTW; }
 int product_tiles_y(int H) { return (H + kTH - 1) / kTH; }
 size_t product_scratch_floats() { return kScratchFloats; }
 
-void launch_product(ProductArgs a, cudaStream_t s) {
+cudaError_t launch_product(ProductArgs a, cudaStream_t s) {
   if (!a.lattices) {
     // the tile rows that hold rows [store_lo, store_hi)
     const int ty0 = a.store_lo / kTH, ty1 = (a.store_hi + kTH - 1) / kTH;
     a.tile0 = ty0 * a.one.ntx;
     a.ntiles = (ty1 - ty0) * a.one.ntx;
   }
-  if (a.ntiles <= 0) return;
-  cudaFuncSetAttribute(k_product, cudaFuncAttributeMaxDynamicSharedMemorySize, a.smem_bytes);
-  k_product<<<device_sm_count(), kProdThreads, a.smem_bytes, s>>>(a);
+  if (a.ntiles <= 0) return cudaSuccess;
+  const cudaError_t e = allow_shared(k_product, kSmem);
+  if (e != cudaSuccess) return e;
+  return launch_tick_kernel(k_product, device_sm_count(), kProdThreads, a.smem_bytes, s, false, a);
 }
 
 }  // namespace sfm

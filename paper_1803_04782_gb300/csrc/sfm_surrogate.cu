@@ -2185,16 +2185,17 @@ void surrogate_field(sfm_surrogate* S, sfm_ctx* ctx) {
 // The exact candidate field and decision of every listed pedestrian
 // (k_sur_fallback on the context's class tables).
 // `tot`: the totals of listed and decided pedestrians to add to, or none.
-void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigned long long* tot);
+cudaError_t surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigned long long* tot);
 
-void surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uint8_t* ref,
-                      unsigned long long* raw_flips, bool cand, unsigned long long* tot = nullptr) {
+cudaError_t surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uint8_t* ref,
+                             unsigned long long* raw_flips, bool cand,
+                             unsigned long long* tot = nullptr) {
   const Geo& g = ctx->geo;
   const Tables tb = ctx->tables();
   const int nbins = g.nbx * g.nby;
   cudaStream_t st = ctx->stream;
   cudaMemsetAsync(S->nflag, 0, sizeof(int32_t), st);
-  if (ctx->n <= 0) return;
+  if (ctx->n <= 0) return cudaSuccess;
   if (cand && std::isinf(S->delta) && !ref) {
     // delta = +inf: every pedestrian falls back, so neither the network's
     // output nor the surrogate composition is needed -- the exact tick with
@@ -2203,8 +2204,7 @@ void surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uin
                                                   ctx->heading, ctx->goal, ctx->ocls, ctx->D, choice,
                                                   S->nflag, S->fb_flag, S->fb_dd, S->fb_info,
                                                   ctx->walk());
-    surrogate_fallback(S, ctx, choice, tot);
-    return;
+    return surrogate_fallback(S, ctx, choice, tot);
   }
   NearPart np;
   np.CT = S->CTnear;
@@ -2217,10 +2217,10 @@ void surrogate_decide(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, const uin
       ctx->D, S->Fsur, ctx->rec, ctx->Fs, np, far_part(S), ctx->prm.beta, tb.own, tb.dirdot,
       S->delta, choice, S->flag_list, S->nflag, S->fb_flag, S->fb_dd, S->fb_info, ref, raw_flips,
       ctx->walk());
-  surrogate_fallback(S, ctx, choice, tot);
+  return surrogate_fallback(S, ctx, choice, tot);
 }
 
-void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigned long long* tot) {
+cudaError_t surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigned long long* tot) {
   const Geo& g = ctx->geo;
   const Tables tb = ctx->tables();
   const int nbins = g.nbx * g.nby;
@@ -2228,12 +2228,13 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigne
   if (ctx->use_product()) {
     // a crowded lattice's exact field is the product's, on the whole lattice
     // (Fnear is free outside training)
-    ctx_field_rows(ctx, S->Fnear, 0, g.H, 0, false);
+    const cudaError_t e = ctx_field_rows(ctx, S->Fnear, 0, g.H, 0, false);
+    if (e != cudaSuccess) return e;
     k_sur_listed<<<cdiv(ctx->n, 256), 256, 0, st>>>(S->fb_flag, ctx->rec_id, ctx->bin_start, nbins, g, ctx->xy,
                                                     S->Fnear, S->fb_dd, S->fb_info, ctx->prm.beta, tb.own,
                                                     tb.dirdot, choice);
     if (tot) k_count_fallbacks<<<1, 1, 0, st>>>(S->nflag, ctx->bin_start + nbins, tot);
-    return;
+    return cudaPeekAtLastError();
   }
   const int SP = class_table_stride(g.r);
   const int TS = (2 * g.r + 1 + 2 * kFieldPadRows) * SP;
@@ -2251,15 +2252,15 @@ void surrogate_fallback(sfm_surrogate* S, sfm_ctx* ctx, uint8_t* choice, unsigne
     case 114: fb = k_sur_fallback<114>; break;
     default: fb = k_sur_fallback<kNarrowStride>; break;
   }
-  cudaFuncSetAttribute(fb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_shared(fb, max_gather_shared(kFbThreads));
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   // early, behind the plain launch that listed the pedestrians (four ticks of
   // the 8192^2 floor 1078 -> 1062 us)
-  launch_tick_kernel(fb, nsm > 0 ? nsm : 1, kFbThreads, smem, st, true, S->fb_flag, ctx->rec_id, nbins, g,
-                     ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs, S->fb_dd, S->fb_info,
-                     ctx->prm.beta, tb.own, tb.dirdot, choice, S->nflag, tot);
+  return launch_tick_kernel(fb, nsm > 0 ? nsm : 1, kFbThreads, smem, st, true, S->fb_flag, ctx->rec_id, nbins,
+                            g, ctx->xy, ctx->bin_start, ctx->rec, ctx->CT, TS, ctx->Fs, S->fb_dd, S->fb_info,
+                            ctx->prm.beta, tb.own, tb.dirdot, choice, S->nflag, tot);
 }
 
 void round_params(sfm_surrogate* S) {
@@ -2427,7 +2428,7 @@ sfm_status sfm_surrogate_train(sfm_surrogate* S, sfm_ctx* ctx, int32_t iters, fl
   for (int it = 0; it < iters; ++it) {
     // exact field of the current state, its near part, inputs and targets
     ctx_run_bins(ctx);
-    ctx_field_rows(ctx, ctx->F, 0, ctx->geo.H, 0, false);
+    SCU(ctx_field_rows(ctx, ctx->F, 0, ctx->geo.H, 0, false));
     near_field(S, ctx);
     coarse_inputs(S, ctx);
     k_targets<<<cdiv(S->Hc * S->Wc, 256), 256, 0, st>>>(ctx->F, S->Fnear, ctx->geo.W, s, S->Hc,
@@ -2487,7 +2488,7 @@ sfm_status sfm_surrogate_calibrate(sfm_surrogate* S, sfm_ctx* ctx, double quanti
   const Geo& g = ctx->geo;
   const int nbins = g.nbx * g.nby;
   ctx_run_bins(ctx);
-  ctx_field_rows(ctx, ctx->F, 0, g.H, 0, false);
+  SCU(ctx_field_rows(ctx, ctx->F, 0, g.H, 0, false));
   surrogate_field(S, ctx);
   if (ctx->n > 0)
     k_sur_err<<<cdiv(ctx->n, 256), 256, 0, st>>>(ctx->rec_id, ctx->bin_start, nbins, g, ctx->xy,
@@ -2521,7 +2522,7 @@ sfm_status sfm_surrogate_step(sfm_surrogate* S, sfm_ctx* ctx, int32_t nsteps) {
   for (int i = 0; i < nsteps; ++i) {
     ctx_run_bins(ctx);
     if (!std::isinf(S->delta)) surrogate_far(S, ctx);  // delta = +inf: no network (exact tick)
-    surrogate_decide(S, ctx, ctx->choice, nullptr, nullptr, true, S->fb_dev);
+    SCU(surrogate_decide(S, ctx, ctx->choice, nullptr, nullptr, true, S->fb_dev));
     launch_vote(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->alive, ctx->choice, ctx->occ, g,
                 ctx->prm.seed, ctx->ctr, ctx->won, st, Sizes(), ctx->ids());
     launch_commit(ctx->n, ctx->rec_id, ctx->bin_start, ctx->xy, ctx->alive, ctx->heading,
@@ -2563,7 +2564,7 @@ sfm_status sfm_surrogate_eval(sfm_surrogate* S, sfm_ctx* ctx, sfm_surrogate_repo
   // exact: bins, field, decisions (into ctx->choice)
   SCU(cudaEventRecord(e0, st));
   ctx_run_bins(ctx);
-  ctx_field_rows(ctx, ctx->F, 0, g.H, 0, false);
+  SCU(ctx_field_rows(ctx, ctx->F, 0, g.H, 0, false));
   launch_decide(ctx->n, ctx->rec_id, ctx->bin_start, 0, nbins, ctx->xy, ctx->heading, ctx->goal,
                 ctx->cell, ctx->ocls, ctx->D, ctx->F, 0, -1, -1, 0, 0, g.H, g, ctx->prm.beta, tb,
                 ctx->choice, st, ctx->walk());
@@ -2574,7 +2575,7 @@ sfm_status sfm_surrogate_eval(sfm_surrogate* S, sfm_ctx* ctx, sfm_surrogate_repo
   SCU(cudaEventRecord(e1, st));
   ctx_run_bins(ctx);
   surrogate_far(S, ctx);
-  surrogate_decide(S, ctx, S->choice2, ctx->choice, S->cnt + 1, true);
+  SCU(surrogate_decide(S, ctx, S->choice2, ctx->choice, S->cnt + 1, true));
   SCU(cudaEventRecord(e2, st));
   // the surrogate field over the whole lattice (network and lattice pass)
   surrogate_field(S, ctx);

@@ -1,0 +1,67 @@
+"""Contexts side by side: launches that need different amounts of shared memory
+of one kernel do not take each other's limit away, whether they come from
+several host threads or from contexts made one after the other."""
+import threading
+
+import numpy as np
+import pytest
+
+import paper_1803_04782_gb300 as sfm
+import scenegen as SG
+from paper_1803_04782_gb300 import build as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+    sfm.lib()
+
+
+def _scene(r, rho, seed):
+    return SG.random_scene(96, 96, int(rho * 96 * 96), r=r, seed=seed, periodic_x=1, periodic_y=1, ring=False,
+                           exits=(), goal_mode="fixed", heading_mode="random")
+
+
+# the product of crowded lattices, the 16 x 16 gather (two radii of one table
+# stride), the scene's own static field
+@pytest.mark.parametrize("rho,radii", [(0.5, (3, 40)), (0.2, (33, 40)), (0.2, (42, 47))])
+def test_host_threads_with_contexts_of_their_own(rho, radii):
+    want, errors = {}, []
+    scenes = {r: _scene(r, rho, 40 + r) for r in radii}
+    for r, sc in scenes.items():
+        with sfm.Sim(sc) as s:
+            s.compute_field()
+            want[r] = s.field()
+    go = threading.Barrier(len(radii))
+
+    def work(r):
+        try:
+            with sfm.Sim(scenes[r]) as s:
+                go.wait()
+                for k in range(400):
+                    s.compute_field()
+                    if k % 100 == 0:
+                        np.testing.assert_array_equal(s.field(), want[r])
+                s.sync()
+        except BaseException as e:  # noqa: BLE001 - reported below
+            errors.append(f"r = {r}: {e}")
+    threads = [threading.Thread(target=work, args=(r,)) for r in radii]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+
+
+def test_a_batch_steps_after_a_smaller_one_was_made():
+    big, small = [_scene(45, 0.2, 1)], [_scene(3, 0.2, 2)]
+    with sfm.Batch(big) as alone:
+        alone.step(2)
+        want = [np.asarray(a[0]).copy() for a in alone.peds()]
+    with sfm.Batch(big) as a, sfm.Batch(small) as b:
+        a.step(2)
+        b.step(2)
+        for x, y in zip(want, a.peds()):
+            np.testing.assert_array_equal(x, y[0])
