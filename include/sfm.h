@@ -284,8 +284,18 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);
  * whole does.  Kept across placements.  Anything else is SFM_EINVAL. */
 sfm_status sfm_set_field_rule(sfm_ctx* ctx, int32_t mode);
 
-/* Wait for the context's stream and report device-side errors. */
+/* Wait for the context's stream and report device-side errors.  After
+ * SFM_ETIMEOUT the crowd stays where it was before the tick whose field is
+ * not whole, and the tick counter with it, until the next placement. */
 sfm_status sfm_sync(sfm_ctx* ctx);
+
+/* Test hook of two bounded device waits (single lattices).  which 0: the
+ * product of the next tick (SFM_ESTATE without a crowd whose field is one)
+ * waits for a builder of planes that does not exist.  1: solves the
+ * lattice's guidance once more, in memory of its own, with a tile that is
+ * never finished, and returns SFM_ETIMEOUT after about a second.  Anything
+ * else is SFM_EINVAL. */
+sfm_status sfm_test_wait_out(sfm_ctx* ctx, int32_t which);
 
 /* The superposed field that k-5 of Alg. 1 (Sec. 3.1) maintains: the sum of
  * the five field kinds of Sec. 2 (here static openings and obstacles plus

@@ -34,6 +34,7 @@ EXPORTS = [
     "sfm_compute_field_into", "sfm_read_static_field", "sfm_read_guidance", "sfm_read_peds",
     "sfm_read_decisions", "sfm_stats", "sfm_set_timing", "sfm_stage_times",
     "sfm_autotune", "sfm_set_field_footprint", "sfm_set_field_rule", "sfm_set_binning", "sfm_set_walk_periods",
+    "sfm_test_wait_out",
     "sfm_place_sized", "sfm_snapshot", "sfm_restore", "sfm_set_ids", "sfm_set_guidance", "sfm_field_noalloc", "sfm_batch_create", "sfm_batch_place", "sfm_batch_offsets",
     "sfm_batch_autotune", "sfm_batch_test_missing_ctas", "sfm_surrogate_nparams",
     "sfm_surrogate_create", "sfm_surrogate_destroy", "sfm_surrogate_last_error",
@@ -120,6 +121,7 @@ def lib():
             "sfm_set_field_footprint": (C.c_int, [P, I32]),
             "sfm_set_field_rule": (C.c_int, [P, I32]),
             "sfm_set_binning": (C.c_int, [P, I32]),
+            "sfm_test_wait_out": (C.c_int, [P, I32]),
             "sfm_set_walk_periods": (C.c_int, [P, P, P, I32]),
             "sfm_set_ids": (C.c_int, [P, P, I32]),
             "sfm_set_guidance": (C.c_int, [P, P, I32]),
@@ -353,6 +355,10 @@ def sfm_batch_autotune(ctx):
     shp = np.zeros(len(TABLE_STRIDES), np.int32)
     _check(ctx, lib().sfm_batch_autotune(ctx, shp.ctypes.data_as(C.c_void_p)))
     return {sp: ("32x16" if v else "16x16") for sp, v in zip(TABLE_STRIDES, shp)}
+
+
+def sfm_test_wait_out(ctx, which: int) -> None:
+    _check(ctx, lib().sfm_test_wait_out(ctx, int(which)))
 
 
 def sfm_batch_test_missing_ctas(ctx, missing: int) -> None:

@@ -872,7 +872,9 @@ sfm_status sfm_step(sfm_ctx* ctx, int32_t nsteps) {
     const bool timed = every > 0 && ctx->timing_phase == 0;
     ctx->timing = timed;
     if (ctx->direct_ticks < 1) {
-      CU(run_tick(ctx));
+      const cudaError_t re = run_tick(ctx);
+      ctx->prod.missing = 0;
+      CU(re);
       ++ctx->direct_ticks;
       ++ctx->t;
       ++i;
@@ -1101,6 +1103,34 @@ sfm_status sfm_set_field_rule(sfm_ctx* ctx, int32_t mode) {
     drop_graph(ctx);
   }
   return SFM_OK;
+}
+
+sfm_status sfm_test_wait_out(sfm_ctx* ctx, int32_t which) {
+  if (!ctx || which < 0 || which > 1) return SFM_EINVAL;
+  if (ctx->batch) return fail(ctx, SFM_EINVAL, "waits are tested on a single lattice");
+  if (which == 0) {
+    if (!ctx->placed || !ctx->use_product())
+      return fail(ctx, SFM_ESTATE, "no crowd whose field is a product");
+    drop_graph(ctx);  // so that the next tick is launched by itself
+    ctx->prod.missing = 1;
+    return SFM_OK;
+  }
+  const Geo& g = ctx->geo;
+  int32_t *D = nullptr, *scratch = nullptr;
+  Counters* ctr = nullptr;
+  const int64_t held = ctx->device_bytes;
+  sfm_status st = dalloc_block(ctx, {array_of(D, (size_t)g.W * g.H), array_of(scratch, guidance_scratch_ints(g)),
+                                     array_of(ctr, 1)});
+  if (st != SFM_OK) return st;
+  cudaMemsetAsync(ctr, 0, sizeof(Counters), ctx->stream);
+  launch_guidance(g, ctx->cell, D, scratch, ctr, ctx->stream, true);
+  Counters h{};
+  cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (e == cudaSuccess) e = cudaMemcpy(&h, ctr, sizeof(h), cudaMemcpyDeviceToHost);
+  dfree(ctx, D);
+  ctx->device_bytes = held;
+  CU(e);
+  return h.err & kErrTimeout ? fail(ctx, SFM_ETIMEOUT, "a bounded device wait gave up") : SFM_OK;
 }
 
 sfm_status sfm_sync(sfm_ctx* ctx) {

@@ -679,12 +679,12 @@ sfm_status check_batch(sfm_ctx* ctx) {
   Counters h;
   BCU(cudaMemcpy(&h, ctx->ctr, sizeof(h), cudaMemcpyDeviceToHost));
   if (h.err & kErrTimeout) {
-    // the barrier word is left mid-count: clear it and the flag so the
+    // the barrier word may be left mid-count: clear it and the flag so the
     // context can tick again
     h.err &= ~kErrTimeout;
     BCU(cudaMemcpy(ctx->ctr, &h, sizeof(h), cudaMemcpyHostToDevice));
     BCU(cudaMemset(ctx->batch->bar, 0, sizeof(unsigned int)));
-    return bfail(ctx, SFM_ETIMEOUT, "a grid barrier of the batched tick timed out");
+    return bfail(ctx, SFM_ETIMEOUT, "a bounded device wait of the batch gave up");
   }
   return SFM_OK;
 }

@@ -27,6 +27,16 @@ __device__ __forceinline__ void tick_kernel_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// For a wait's try `it`: a second of the global timer, looked at every 256 tries,
+// is over (t0: 0 at first).
+__device__ __forceinline__ bool second_is_over(int it, unsigned long long& t0) {
+  if ((it & 255) != 255) return false;
+  unsigned long long now;
+  asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(now));
+  if (t0 == 0) t0 = now;
+  return now - t0 > 1000000000ull;
+}
+
 // move offsets of the direction classes 0..8 and the class of the opposite move
 static __constant__ int c_dx[9] = {0, 1, 1, 0, -1, -1, -1, 0, 1};
 static __constant__ int c_dy[9] = {0, 0, 1, 1, 1, 0, -1, -1, -1};

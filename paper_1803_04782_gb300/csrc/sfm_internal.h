@@ -124,7 +124,7 @@ enum : uint32_t {
   kErrPlaceRange = 2u,     // off-lattice position or class > 8
   kErrEnroll = 4u,         // more than 8 registrants for one su (impossible by construction)
   kErrHalo = 8u,           // a tile's halo touched more bins than kMaxHaloBins
-  kErrTimeout = 16u,       // a bounded device wait gave up
+  kErrTimeout = 16u,       // a bounded device wait gave up; the crowd stays where it is
 };
 
 struct Counters {
@@ -240,6 +240,7 @@ struct ProductArgs {
   int out_row0 = 0, store_lo = 0, store_hi = 0, ring = 0;  // as launch_field's
   int plane_bytes = 0, stage_bytes = 0, nplanes = 0, nstages = 0, smem_bytes = 0;
   Counters* ctr = nullptr;
+  int missing = 0;  // a test's: builders of planes that are waited for and do not exist
 };
 // Fixed-point scales of the limb tables: T = L0 / s0 + L1 / (s0 s1).  false:
 // the law's range over the window is too wide for them.
@@ -268,8 +269,9 @@ void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, co
 // Guidance distances; scratch: guidance_scratch_ints() ints of device memory,
 // overwritten.  A bounded wait that runs out sets kErrTimeout in ctr.
 size_t guidance_scratch_ints(const Geo& g);
+// unfinished: a test's, with a tile that is never taken.
 void launch_guidance(const Geo& g, const uint8_t* cell, int32_t* D, int* scratch, Counters* ctr,
-                     cudaStream_t s);
+                     cudaStream_t s, bool unfinished = false);
 void launch_guidance_export(int32_t* D, size_t n, cudaStream_t s);
 void launch_guidance_import(const uint8_t* cell, int32_t* D, size_t n, cudaStream_t s);
 

@@ -192,13 +192,19 @@ void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, co
 // (scene set-up 2.90 against 1.61 ms).  256 threads a tile, eight CTAs an SM:
 // 878 us; without the scan down the columns 642.
 constexpr int kGuideThreads = kTile * kTile;
-constexpr int kGuideSpins = 1 << 23;  // naps of an idle CTA, each 100 ns and more: about a second
+// A wait lasts for a second at most, or this many looks.  It is one for one
+// position: an idle CTA's comes nearer with every tile that is queued, each
+// well under a millisecond after the last, so the wait covers a few hundred
+// tiles however long the chain is (52 000 tiles in a row, the most before the
+// distances end at 2^23: 0.28 s).
+constexpr int kGuideSpins = 1 << 23;
 
 __device__ __forceinline__ void guide_push(const GuideTiles& gt, int t, Counters* ctr) {
   if (!guide_mark(gt, t)) return;
   const unsigned pos = guide_position(gt);
+  unsigned long long t0 = 0;
   for (int i = 0; !guide_publish(gt, pos, t); ++i) {
-    if (i == kGuideSpins) {
+    if (i == kGuideSpins || second_is_over(i, t0)) {
       atomicOr(&ctr->err, kErrTimeout);
       return;
     }
@@ -209,7 +215,8 @@ __device__ __forceinline__ void guide_push(const GuideTiles& gt, int t, Counters
 // the next tile of the queue, -1 when no tile is left (or the wait ran out)
 __device__ int guide_pop(const GuideTiles& gt, Counters* ctr) {
   const unsigned pos = guide_claim(gt);
-  for (int i = 0; i < kGuideSpins; ++i) {
+  unsigned long long t0 = 0;
+  for (int i = 0; i < kGuideSpins && !second_is_over(i, t0); ++i) {
     const int t = guide_take(gt, pos);
     if (t >= 0) {
       guide_unmark(gt, t);
@@ -231,10 +238,11 @@ __device__ __forceinline__ int guide_neighbour(const Geo& g, int ntx, int nty, i
   return nx >= 0 && nx < ntx && ny >= 0 && ny < nty ? ny * ntx + nx : -1;
 }
 
-// start values, and the tiles that see an exit into the queue
+// start values, and the tiles that see an exit into the queue (test: and one
+// that no CTA will ever finish)
 __global__ void __launch_bounds__(1024)
     k_guidance_init(Geo g, const uint8_t* __restrict__ cell, int32_t* __restrict__ D, GuideTiles gt,
-                    Counters* ctr) {
+                    Counters* ctr, int unfinished) {
   const int ntx = (g.W + kTile - 1) / kTile, nty = (g.H + kTile - 1) / kTile;
   const int tx = blockIdx.x % ntx, ty = blockIdx.x / ntx;
   const int x = tx * kTile + (threadIdx.x & 31), y = ty * kTile + (threadIdx.x >> 5);
@@ -245,6 +253,7 @@ __global__ void __launch_bounds__(1024)
     source = v == kExit;
     D[c] = source ? 0 : (v == kWall ? kDWall : kDInf);
   }
+  if (unfinished && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&gt.q->work, 1ull << 32);
   if (__syncthreads_or(source) && threadIdx.x < 9) {
     const int t = guide_neighbour(g, ntx, nty, tx, ty, (int)threadIdx.x % 3 - 1, (int)threadIdx.x / 3 - 1);
     if (t >= 0) guide_push(gt, t, ctr);
@@ -416,11 +425,11 @@ size_t guidance_scratch_ints(const Geo& g) {
 }
 
 void launch_guidance(const Geo& g, const uint8_t* cell, int32_t* D, int* scratch, Counters* ctr,
-                     cudaStream_t s) {
+                     cudaStream_t s, bool unfinished) {
   const int ntiles = cdiv(g.W, kTile) * cdiv(g.H, kTile);
   const GuideTiles gt = guide_tiles(scratch, ntiles);
   cudaMemsetAsync(scratch, 0, guidance_scratch_ints(g) * sizeof(int), s);
-  k_guidance_init<<<ntiles, 1024, 0, s>>>(g, cell, D, gt, ctr);
+  k_guidance_init<<<ntiles, 1024, 0, s>>>(g, cell, D, gt, ctr, unfinished);
   // CTAs wait for what running ones put into the queue or take out of it
   const int fit = 2 * device_sm_count();
   const int blocks = ntiles < fit ? ntiles : fit;
@@ -1278,9 +1287,10 @@ __global__ void k_commit(const int32_t* __restrict__ rec_id, const int32_t* __re
                          const uint8_t* __restrict__ won, const uint8_t* __restrict__ cell,
                          int32_t* __restrict__ occ, uint8_t* __restrict__ ocls, Geo g,
                          Counters* ctr, Sizes sz) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, nrec = bin_start[nbins];
+  const bool whole = !(ctr->err & kErrTimeout);  // else nobody moves, on a field that is not
   bool moved = false, left = false;
-  if (i < bin_start[nbins]) {
+  if (i < nrec && whole) {
     if (sz.w)
       commit_one_sized(rec_id[i], g, xy, alive, heading, choice, won, cell, occ, ocls, sz.w, sz.h,
                        moved, left);
@@ -1293,7 +1303,7 @@ __global__ void k_commit(const int32_t* __restrict__ rec_id, const int32_t* __re
     if (nm) atomicAdd(&ctr->moved, (unsigned long long)nm);
     if (nl) atomicAdd(&ctr->exited, (unsigned long long)nl);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctr->t += 1;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && whole) ctr->t += 1;
 }
 
 void launch_commit(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy,
@@ -1326,6 +1336,7 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
   tick_kernel_begin();
   const int i = threadIdx.x;
   const long long t = ctr->t;
+  const bool whole = !(ctr->err & kErrTimeout);  // as in k_commit
   const int p = i < bin_start[nbins] ? rec_id[i] : -1;
   if (i < n && !alive[i]) {
     choice[i] = 0;
@@ -1358,7 +1369,7 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
   }
   __syncthreads();
   bool moved = false, left = false;
-  if (p >= 0) {
+  if (p >= 0 && whole) {
     if (SIZED)
       commit_one_sized(p, g, xy, alive, heading, s_choice, s_won, cell, occ, ocls, sz.w, sz.h, moved,
                        left);
@@ -1378,7 +1389,7 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
     if (regs > 2) atomicMax(&ctr->max_registrants, regs);
     if (regs > 8) atomicOr(&ctr->err, kErrEnroll);
   }
-  if (i == 0) ctr->t = t + 1;
+  if (i == 0 && whole) ctr->t = t + 1;
 }
 
 void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy, uint8_t* alive,

@@ -53,9 +53,11 @@ __global__ void __launch_bounds__(T)
     k_commit_bins(Geo g, const int32_t* bin_start, const uint32_t* rec, const int32_t* rec_id, int2* xy,
                   uint8_t* alive, uint8_t* heading, const uint8_t* cell, int32_t* occ, uint8_t* ocls,
                   Counters* ctr) {
-  const int b = blockIdx.x, end = bin_start[b + 1];
+  const int b = blockIdx.x, first = bin_start[b], last = bin_start[b + 1];
+  const bool whole = !(ctr->err & kErrTimeout);  // as in k_commit
+  const int end = whole ? last : first;
   unsigned nm = 0, nl = 0;
-  for (int i = bin_start[b] + threadIdx.x; i < end; i += T) {
+  for (int i = first + threadIdx.x; i < end; i += T) {
     const uint32_t rc = rec[i];
     if (!(rc >> kRecWon & 1u)) continue;
     bool left;
@@ -65,7 +67,7 @@ __global__ void __launch_bounds__(T)
   }
   __syncwarp();
   count_moves(ctr, nm, nl);
-  if (b == 0 && threadIdx.x == 0) ctr->t += 1;
+  if (b == 0 && threadIdx.x == 0 && whole) ctr->t += 1;
 }
 
 // few bins: at most two for each SM

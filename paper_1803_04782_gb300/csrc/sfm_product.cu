@@ -71,11 +71,11 @@ static_assert(kWorkers % 4 == 0, "the workers cover the four TMEM lane quarters 
 static_assert(kHeadBytes + plane_bytes_of(kProductMaxRadius) + 2 * stage_bytes_of(kProductMaxRadius) <= kSmem,
               "a plane and two table stages must fit");
 
-// bounded wait for an mbarrier phase, about a second of the global timer
-// (checked every 256 tries) with an iteration cap behind it; false: it ran out
+// bounded wait for an mbarrier phase, about a second with an iteration cap
+// behind it; false: it ran out
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  uint64_t t0 = 0;
-  for (int it = 0; it < (1 << 24); ++it) {
+  unsigned long long t0 = 0;
+  for (int it = 0; it < (1 << 26); ++it) {
     uint32_t done = 0;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -85,14 +85,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
-    if ((it & 255) == 255) {
-      uint64_t now;
-      asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(now));
-      if (t0 == 0)
-        t0 = now;
-      else if (now - t0 > 1000000000ull)
-        return false;
-    }
+    if (second_is_over(it, t0)) return false;
   }
   return false;
 }
@@ -191,7 +184,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(sempty(i)));
     }
     for (int i = 0; i < 2; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(pfull(i)), "r"(kWorkers));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(pfull(i)), "r"(kWorkers + a.missing));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(pempty(i)));
       // the issuer's own arrival (it publishes word[3 + i]) and its commit
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;\n" ::"r"(afull(i)));

@@ -1,6 +1,8 @@
 """Guidance distances of lattices of few tiles, set up again and again, against
 the oracle's Dijkstra: the kernel's CTAs then take every tile from the queue
 many times, in an order that differs from run to run."""
+import time
+
 import numpy as np
 import pytest
 
@@ -40,3 +42,15 @@ def test_few_tiles_again_and_again(W, H, px, py):
         for _ in range(12):
             with sfm.Sim(W=W, H=H, cell=sc.cell, periodic_x=px, periodic_y=py, r=1) as s:
                 np.testing.assert_array_equal(s.guidance(), want)
+
+
+def test_a_tile_that_is_never_finished_ends_the_wait():
+    sc = _maze(200, 150, 0, 0, 0)
+    with sfm.Sim(W=200, H=150, cell=sc.cell, r=1) as s:
+        before = s.guidance()
+        t0 = time.time()
+        with pytest.raises(sfm.SfmError) as e:
+            sfm.sfm_test_wait_out(s.ctx, 1)
+        assert e.value.status == sfm.SFM_ETIMEOUT and time.time() - t0 < 10
+        np.testing.assert_array_equal(s.guidance(), before)
+        s.sync()

@@ -2,6 +2,8 @@
 tensor-core product sums: against the FP64 oracle at the edges of its tiles,
 radii and alignments, closed and periodic; closer to it than the gather; and
 bit for bit the same in bands, in a batch and at the candidates only."""
+import time
+
 import numpy as np
 import pytest
 
@@ -90,6 +92,48 @@ def test_bands_batch_and_candidates_round_as_one_launch(px, py, r, rows):
             np.testing.assert_array_equal(d.decisions()[0], e.decisions()[0])
         for s in (a, b, c, d, e):
             assert s.stats()["error_flags"] == 0
+
+
+@pytest.mark.parametrize("n,sized,rows", [(900, False, 0), (0, False, 0), (0, False, 64), (0, True, 0)])
+def test_nobody_moves_on_a_field_whose_wait_ran_out(n, sized, rows):
+    """n: a crowd small enough for the stages in one block; rows: of a band."""
+    sc = _crowd(40 if n else 96, 40 if n else 256, 12, 0, 0, rho=0.7, seed=11)
+    n = n or sc.n
+    assert 20 * n >= 9 * sc.W * sc.H
+    xy, heading, goal = sc.xy[:n], sc.heading[:n], sc.goal[:n]
+    kw = dict(hbm_budget_bytes=sfm.band_budget(sc.W, sc.H, rows, 0, 0)) if rows else {}
+    sim = sfm.Sim(W=sc.W, H=sc.H, cell=sc.cell, r=12, **kw)
+    ones = np.ones(n, np.uint8)
+
+    def place():
+        if sized:
+            sim.place_sized(xy, heading, goal, ones, ones, ones)
+        else:
+            sim.place(xy, heading, goal)
+    with sim, sfm.Sim(W=sc.W, H=sc.H, cell=sc.cell, r=12) as ref:
+        place()
+        sfm.sfm_test_wait_out(sim.ctx, 0)
+        t0 = time.time()
+        sim.step(3)
+        with pytest.raises(sfm.SfmError) as e:
+            sim.sync()
+        assert e.value.status == sfm.SFM_ETIMEOUT and time.time() - t0 < 30
+        st = sim.stats()
+        assert (st["moved_total"], st["exited"], st["t"]) == (0, 0, 0)
+        where = np.zeros((n, 2), np.int32), np.zeros(n, np.uint8), np.zeros(n, np.uint8)
+        assert sfm.lib().sfm_read_peds(sim.ctx, *(a.ctypes.data for a in where), 0) == sfm.SFM_ETIMEOUT
+        for got, want in zip(where, (xy, heading, ones)):
+            np.testing.assert_array_equal(got, want)
+        # placed anew it goes on, the split tiles' sums and all
+        place()
+        ref.place(xy, heading, goal)
+        for s in (sim, ref):
+            s.set_time(0)
+            s.step(3)
+            s.sync()
+        for got, want in zip(sim.peds(), ref.peds()):
+            np.testing.assert_array_equal(got, want)
+        assert ref.stats()["moved_total"] > 0
 
 
 def test_two_row_bands_round_as_the_whole_lattice():
