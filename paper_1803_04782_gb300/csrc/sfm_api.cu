@@ -45,8 +45,10 @@ sfm_status dalloc(sfm_ctx* ctx, T** p, size_t count) {
   void* q = nullptr;
   const size_t bytes = count * sizeof(T) > 0 ? count * sizeof(T) : 16;
   cudaError_t e = cudaMalloc(&q, bytes);
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call as well
     return fail(ctx, SFM_ENOMEM, "cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
+  }
   ctx->allocs.push_back(q);
   ctx->device_bytes += (int64_t)bytes;
   *p = static_cast<T*>(q);
@@ -81,8 +83,10 @@ sfm_status dalloc_block(sfm_ctx* ctx, const std::vector<DeviceArray>& arrays) {
   for (const DeviceArray& a : arrays) total += padded(a.bytes);
   void* q = nullptr;
   const cudaError_t e = cudaMalloc(&q, total);
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
+    cudaGetLastError();
     return fail(ctx, SFM_ENOMEM, "cudaMalloc(%zu bytes): %s", total, cudaGetErrorString(e));
+  }
   ctx->allocs.push_back(q);
   char* at = static_cast<char*>(q);
   for (const DeviceArray& a : arrays) {
@@ -499,7 +503,6 @@ void ensure_product(sfm_ctx* c) {
   const std::string err = c->err;
   if (dalloc(c, &tab, product_table_bytes(g.r, 5)) != SFM_OK || dalloc(c, &a.tick, split) != SFM_OK ||
       dalloc(c, &a.scratch, product_scratch_floats() * split) != SFM_OK) {
-    cudaGetLastError();
     c->err = err;
     dfree(c, tab);
     dfree(c, a.tick);
@@ -768,7 +771,8 @@ static sfm_status place_impl(sfm_ctx* ctx, int32_t n, const int32_t* xy, const u
     CU(cudaStreamSynchronize(s));
     dfree(ctx, ctx->xy);  // the block of all of them
     ctx->xy = nullptr;
-    ctx->cap = 0;
+    ctx->cap = ctx->n = 0;  // nobody is placed, should the new block not fit
+    ctx->placed = ctx->walk_periods = ctx->has_ids = ctx->sized = false;
     const size_t m = n > 0 ? (size_t)n : 1;
     TRY(dalloc_block(ctx, {array_of(ctx->xy, m), array_of(ctx->heading, m), array_of(ctx->goal, m),
                            array_of(ctx->alive, m), array_of(ctx->choice, m), array_of(ctx->won, m),

@@ -473,12 +473,26 @@ sfm_status balloc(sfm_ctx* ctx, T** p, size_t count) {
   void* q = nullptr;
   const size_t bytes = count * sizeof(T) > 0 ? count * sizeof(T) : 16;
   const cudaError_t e = cudaMalloc(&q, bytes);
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call as well
     return bfail(ctx, SFM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   ctx->allocs.push_back(q);
   ctx->device_bytes += (int64_t)bytes;
   *p = static_cast<T*>(q);
   return SFM_OK;
+}
+
+template <class T>
+void bfree(sfm_ctx* ctx, T** p) {
+  if (!*p) return;
+  for (size_t i = 0; i < ctx->allocs.size(); ++i)
+    if (ctx->allocs[i] == *p) {
+      ctx->allocs.erase(ctx->allocs.begin() + (long)i);
+      break;
+    }
+  cudaFree(*p);
+  *p = nullptr;
 }
 
 #define BTRY(x)                  \
@@ -571,6 +585,7 @@ sfm_status setup_product(sfm_ctx* ctx) {
   std::vector<ProductLattice> pl(ns);
   std::vector<int> who;
   int rmax = 0, tiles = 0;
+  const std::string err = ctx->err;  // memory that cannot be had is no failure here
   for (int i = 0; i < ns; ++i) {
     const BatchScene& sc = B->hs[i];
     const Geo& g = sc.g;
@@ -584,7 +599,7 @@ sfm_status setup_product(sfm_ctx* ctx) {
     if (!B->tabs[i]) {
       uint8_t* t = nullptr;
       if (balloc(ctx, &t, product_table_bytes(g.r, 5)) != SFM_OK) {
-        cudaGetLastError();
+        ctx->err = err;
         continue;
       }
       launch_limb_tables(g.r, p, w, 5, t, s);
@@ -615,7 +630,9 @@ sfm_status setup_product(sfm_ctx* ctx) {
     ProductArgs a;
     if (balloc(ctx, &B->plat, (size_t)ns) != SFM_OK || balloc(ctx, &a.tick, split) != SFM_OK ||
         balloc(ctx, &a.scratch, product_scratch_floats() * split) != SFM_OK) {
-      cudaGetLastError();
+      bfree(ctx, &B->plat);
+      bfree(ctx, &a.tick);
+      ctx->err = err;
       return SFM_OK;
     }
     BCU(cudaMemsetAsync(a.tick, 0, split * sizeof(int), s));
@@ -623,8 +640,10 @@ sfm_status setup_product(sfm_ctx* ctx) {
     B->prod = a;
   }
   if (tiles > B->tiles_cap) {
+    bfree(ctx, &B->tiles);
+    B->tiles_cap = 0;
     if (balloc(ctx, &B->tiles, (size_t)tiles) != SFM_OK) {
-      cudaGetLastError();
+      ctx->err = err;
       return SFM_OK;
     }
     B->tiles_cap = tiles;
@@ -953,17 +972,17 @@ sfm_status sfm_batch_place(sfm_ctx* ctx, const int32_t* counts, const int32_t* x
   }
   BCU(cudaStreamSynchronize(s));
   if (n > ctx->cap || ctx->cap == 0) {
-    for (void* p : {(void*)ctx->xy, (void*)ctx->heading, (void*)ctx->goal, (void*)ctx->alive,
-                    (void*)ctx->choice, (void*)ctx->won, (void*)ctx->rec, (void*)ctx->rec_id,
-                    (void*)B->ped_scene}) {
-      if (!p) continue;
-      for (size_t i = 0; i < ctx->allocs.size(); ++i)
-        if (ctx->allocs[i] == p) {
-          ctx->allocs.erase(ctx->allocs.begin() + (long)i);
-          break;
-        }
-      cudaFree(p);
-    }
+    bfree(ctx, &ctx->xy);
+    bfree(ctx, &ctx->heading);
+    bfree(ctx, &ctx->goal);
+    bfree(ctx, &ctx->alive);
+    bfree(ctx, &ctx->choice);
+    bfree(ctx, &ctx->won);
+    bfree(ctx, &ctx->rec);
+    bfree(ctx, &ctx->rec_id);
+    bfree(ctx, &B->ped_scene);
+    ctx->cap = ctx->n = 0;  // nobody is placed, should the new arrays not fit
+    ctx->placed = false;
     const size_t cap = n > 0 ? (size_t)n : 1;
     BTRY(balloc(ctx, &ctx->xy, cap));
     BTRY(balloc(ctx, &ctx->heading, cap));

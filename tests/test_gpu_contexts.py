@@ -65,3 +65,38 @@ def test_a_batch_steps_after_a_smaller_one_was_made():
         b.step(2)
         for x, y in zip(want, a.peds()):
             np.testing.assert_array_equal(x, y[0])
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_a_placement_that_does_not_fit_leaves_nobody_placed(batch):
+    """The arrays of the crowd before are gone by then: a step must refuse, and
+    a smaller placement work as in a new context."""
+    torch = pytest.importorskip("torch")
+    sc, n = _scene(5, 0.2, 3), 40_000_000  # 44 bytes a pedestrian of a context, 23 of a batch's
+    big = np.zeros((n, 2), np.int32)
+    make = (lambda: sfm.Batch([sc])) if batch else (lambda: sfm.Sim(sc))
+    with make() as s, make() as ref:
+        s.step(2)
+        s.sync()
+        free, _ = torch.cuda.mem_get_info()
+        hold = torch.empty(free - (600 << 20), dtype=torch.uint8, device="cuda")
+        with pytest.raises(sfm.SfmError) as e:
+            if batch:
+                sfm.sfm_batch_place(s.ctx, [n], big, None, None)
+            else:
+                s.place(big)
+        assert e.value.status == sfm.SFM_ENOMEM
+        del hold
+        torch.cuda.empty_cache()
+        with pytest.raises(sfm.SfmError) as e:
+            s.step(1)
+        assert e.value.status == sfm.SFM_ESTATE and s.stats()["n"] == 0
+        for x in (s, ref):
+            if batch:
+                sfm.sfm_batch_place(x.ctx, [sc.n], sc.xy, sc.heading, sc.goal)
+            else:
+                x.place(sc.xy, sc.heading, sc.goal)
+            sfm.sfm_set_time(x.ctx, 0)
+            x.step(3)
+        for a, b in zip(s.peds(), ref.peds()):
+            np.testing.assert_array_equal(np.asarray(a), np.asarray(b))
