@@ -1796,13 +1796,18 @@ sfm_status sfail(sfm_surrogate* s, sfm_status st, const std::string& msg) {
 template <class T>
 sfm_status salloc(sfm_surrogate* S, T** p, size_t n) {
   void* q = nullptr;
-  SCU(cudaMalloc(&q, n * sizeof(T) > 0 ? n * sizeof(T) : 16));
+  const cudaError_t e = cudaMalloc(&q, n * sizeof(T) > 0 ? n * sizeof(T) : 16);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call as well
+    return sfail(S, SFM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   S->allocs.push_back(q);
   *p = static_cast<T*>(q);
   return SFM_OK;
 }
 
-void sfree(sfm_surrogate* S, void* p) {
+template <class T>
+void sfree(sfm_surrogate* S, T*& p) {
   if (!p) return;
   for (size_t i = 0; i < S->allocs.size(); ++i)
     if (S->allocs[i] == p) {
@@ -1810,6 +1815,7 @@ void sfree(sfm_surrogate* S, void* p) {
       break;
     }
   cudaFree(p);
+  p = nullptr;
 }
 
 #define STRY(x)                  \
@@ -1818,12 +1824,13 @@ void sfree(sfm_surrogate* S, void* p) {
     if (s_ != SFM_OK) return s_; \
   } while (0)
 
-// activation buffers for a padded input of (Hc + 2h) x (Wc + 2h) cells
+// activation buffers for a padded input of (Hc + 2h) x (Wc + 2h) cells (here and
+// below: the size that the buffers serve is set once all of them are there)
 sfm_status ensure_image(sfm_surrogate* S, int Hc, int Wc) {
   if (S->Hc == Hc && S->Wc == Wc && S->X) return SFM_OK;
-  for (void* q : {(void*)S->X, (void*)S->A1, (void*)S->A2, (void*)S->A3, (void*)S->Y, (void*)S->T,
-                  (void*)S->dY, (void*)S->dA3, (void*)S->dA2, (void*)S->dA1, (void*)S->Xf})
-    sfree(S, q);
+  S->Hc = S->Wc = 0;
+  for (bf16** q : {&S->X, &S->A1, &S->A2, &S->A3}) sfree(S, *q);
+  for (float** q : {&S->Xf, &S->Y, &S->T, &S->dY, &S->dA3, &S->dA2, &S->dA1}) sfree(S, *q);
   const size_t p0 = (size_t)(Hc + 2 * kHalo) * (Wc + 2 * kHalo);
   const size_t p1 = (size_t)(Hc + 6) * (Wc + 6), p2 = (size_t)(Hc + 4) * (Wc + 4),
                p3 = (size_t)(Hc + 2) * (Wc + 2), p4 = (size_t)Hc * Wc;
@@ -1849,7 +1856,6 @@ int sm_count() { return device_sm_count(); }
 sfm_status ensure_part(sfm_surrogate* S, size_t floats) {
   if (floats <= S->part_cap) return SFM_OK;
   sfree(S, S->part);
-  S->part = nullptr;
   S->part_cap = 0;
   STRY(salloc(S, &S->part, floats));
   S->part_cap = floats;
@@ -2006,7 +2012,6 @@ sfm_status backward(sfm_surrogate* S, float* loss_out, cudaStream_t s) {
   const int nb = cdiv(n, 256);
   if (nb > S->mse_cap) {
     sfree(S, S->mse);
-    S->mse = nullptr;
     S->mse_cap = 0;
     STRY(salloc(S, &S->mse, (size_t)nb));
     S->mse_cap = nb;
@@ -2084,13 +2089,14 @@ sfm_status ensure_lattice(sfm_surrogate* S, sfm_ctx* ctx) {
   if (nsu != S->nsu) {
     sfree(S, S->Fnear);
     sfree(S, S->Fsur);
-    S->Fnear = S->Fsur = nullptr;
+    S->nsu = 0;
     STRY(salloc(S, &S->Fnear, nsu));
     STRY(salloc(S, &S->Fsur, nsu));
     S->nsu = nsu;
   }
   if (ctx->cap > S->choice_cap) {
     sfree(S, S->choice2);
+    S->choice_cap = 0;
     STRY(salloc(S, &S->choice2, (size_t)ctx->cap));
     S->choice_cap = ctx->cap;
   }
@@ -2100,6 +2106,7 @@ sfm_status ensure_lattice(sfm_surrogate* S, sfm_ctx* ctx) {
     sfree(S, S->flag_list);
     sfree(S, S->fb_flag);
     sfree(S, S->perr);
+    S->fb_cap = 0;
     STRY(salloc(S, &S->fb_dd, fb_at((ctx->cap + 31) / 32 * 32, 0)));
     STRY(salloc(S, &S->fb_info, (size_t)ctx->cap));
     STRY(salloc(S, &S->flag_list, (size_t)ctx->cap));
@@ -2110,7 +2117,6 @@ sfm_status ensure_lattice(sfm_surrogate* S, sfm_ctx* ctx) {
   const int rn = S->cfg.near_radius;
   if (S->near_r_built != rn || !S->CTnear) {
     sfree(S, S->CTnear);
-    S->CTnear = nullptr;
     const size_t n = class_table_floats(rn);
     if (n) {
       STRY(salloc(S, &S->CTnear, n));

@@ -100,3 +100,24 @@ def test_a_placement_that_does_not_fit_leaves_nobody_placed(batch):
             x.step(3)
         for a, b in zip(s.peds(), ref.peds()):
             np.testing.assert_array_equal(np.asarray(a), np.asarray(b))
+
+
+def test_an_image_that_does_not_fit_leaves_none():
+    """A surrogate whose buffers could not be grown: the size before works again."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(5)
+    X, T = rng.random((3, 60, 70), np.float32), rng.random((50, 60), np.float32)
+    flat = rng.normal(0, 0.1, int(sfm.lib().sfm_surrogate_nparams())).astype(np.float32)
+    big = np.zeros((3, 2058, 2058), np.float32)  # activations of 2.4 GB
+    with sfm.Surrogate(params=flat) as sur:
+        loss, grads = sur.grad(X, T)
+        free, _ = torch.cuda.mem_get_info()
+        hold = torch.empty(free - (600 << 20), dtype=torch.uint8, device="cuda")
+        with pytest.raises(sfm.SfmError) as e:
+            sur.grad(big, np.zeros((2048, 2048), np.float32))
+        assert e.value.status == sfm.SFM_ENOMEM
+        del hold
+        torch.cuda.empty_cache()
+        again = sur.grad(X, T)
+        assert again[0] == loss
+        np.testing.assert_array_equal(again[1], grads)
