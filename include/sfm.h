@@ -188,8 +188,9 @@ sfm_status sfm_compute_field(sfm_ctx* ctx);
 
 /* Times the field gather of the current state with each of its warp
  * footprints (see sfm_set_field_footprint) and keeps the fastest for this
- * context (the choice survives later placements).  *shape_out (may be
- * NULL): 0..3.  The fields computed are identical either way.
+ * context (the choice survives later placements); a context whose crowd the
+ * product serves (sfm_set_field_rule) keeps the one it has.  *shape_out (may be
+ * NULL): 0..2.  The fields computed are identical either way.
  * Synchronising; moves nobody. */
 sfm_status sfm_autotune(sfm_ctx* ctx, int32_t* shape_out);
 
@@ -385,8 +386,9 @@ sfm_status sfm_stage_times(sfm_ctx* ctx, double* ms, int64_t* ticks);
  *   sharing a class-table row stride) with 16 x 16 and 32 x 16 su warp
  *   footprints and keeps the faster; shape_per_class[7] (may be NULL)
  *   receives 0 (16 x 16) or 1 (32 x 16) for the strides 34, 50, 66, 82, 98,
- *   114 (radius <= 1, 9, 17, 25, 33, 41) and 102 (radius 42..50).  Needs
- *   placed pedestrians; moves nobody.
+ *   114 (radius <= 1, 9, 17, 25, 33, 41) and 102 (radius 42..50); a class
+ *   whose lattices are all crowded keeps its footprint.  Needs placed
+ *   pedestrians; moves nobody.
  * sfm_batch_test_missing_ctas: test hook of the bounded barrier wait; the
  *   next tick's barriers wait for `missing` CTAs that are never launched, so
  *   the tick gives up after about a second and returns SFM_ETIMEOUT (the

@@ -955,9 +955,11 @@ sfm_status sfm_autotune(sfm_ctx* ctx, int32_t* shape_out) {
   if (!ctx) return SFM_EINVAL;
   if (ctx->batch) return fail(ctx, SFM_EINVAL, "use sfm_batch_autotune on a batch");
   if (!ctx->placed) return fail(ctx, SFM_ESTATE, "autotune needs placed pedestrians");
-  if (!ctx->CT) {
+  if (!ctx->CT || ctx->use_product()) {
+    // a radius beyond the class-table gathers, or a crowd that the product
+    // serves: nothing to choose (and a sparser crowd may come)
     if (shape_out) *shape_out = ctx->field_shape;
-    return SFM_OK;  // radius beyond the class-table gather: nothing to choose
+    return SFM_OK;
   }
   const Geo& g = ctx->geo;
   float* out = ctx->bands > 1 ? ctx->band_buf : ctx->F;

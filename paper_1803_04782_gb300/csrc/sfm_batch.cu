@@ -1096,10 +1096,18 @@ sfm_status sfm_batch_autotune(sfm_ctx* ctx, int32_t* shape_per_class) {
   cudaEvent_t e0, e1;
   BCU(cudaEventCreate(&e0));
   BCU(cudaEventCreate(&e1));
+  // the gathers alone are timed: a class keeps its footprint where the product
+  // serves all its lattices (a sparser crowd may come)
+  struct Restore {
+    int& ntiles;
+    const int was;
+    ~Restore() { ntiles = was; }
+  } restore{B->prod.ntiles, B->prod.ntiles};
+  B->prod.ntiles = 0;
   for (int ci = 0; ci < kNumStrideClasses; ++ci) {
     const int sp = stride_of_class(ci);
     bool present = false;
-    for (const BatchScene& sc : B->hs) present |= sc.sp == sp;
+    for (int i = 0; i < B->nscenes; ++i) present |= B->hs[i].sp == sp && !B->crowded[i];
     if (!present) continue;
     float best = 1e30f;
     int best_shape = 0;

@@ -94,6 +94,25 @@ def test_bands_batch_and_candidates_round_as_one_launch(px, py, r, rows):
             assert s.stats()["error_flags"] == 0
 
 
+def test_autotuning_a_crowded_lattice_keeps_its_footprint():
+    sc = _crowd(150, 256, 20, 1, 1, rho=0.55, seed=12)
+    with sfm.Sim(sc) as s:
+        for shape in sfm.FOOTPRINTS * 3:
+            s.set_footprint(shape)
+            assert s.autotune() == shape
+    few = sc.copy()
+    few.xy, few.heading, few.goal = (a[:sc.n // 10].copy() for a in (sc.xy, sc.heading, sc.goal))
+    with sfm.Batch([few]) as b:
+        was = b.autotune()
+        b.place([sc.xy], [sc.heading], [sc.goal])
+        for _ in range(8):
+            assert b.autotune() == was
+        with sfm.Sim(sc) as s:
+            for x in (s, b):
+                x.step(2)
+            np.testing.assert_array_equal(s.peds()[0], b.peds()[0][0])
+
+
 @pytest.mark.parametrize("n,sized,rows", [(900, False, 0), (0, False, 0), (0, False, 64), (0, True, 0)])
 def test_nobody_moves_on_a_field_whose_wait_ran_out(n, sized, rows):
     """n: a crowd small enough for the stages in one block; rows: of a band."""
