@@ -36,7 +36,7 @@ carried.
 from __future__ import annotations
 
 from dataclasses import dataclass
-from typing import Callable, Dict, List, Tuple
+from typing import Callable, Dict, List, Optional, Tuple
 
 import numpy as np
 
@@ -89,7 +89,7 @@ class BandLayout:
             raise ValueError(f"a periodic lattice is split only when its height is a multiple of {BIN}")
         self.H, self.py, self.r, self.nranks = int(H), int(periodic_y), int(r), int(nranks)
         self.h = self.r + HALO_EXTRA
-        self.crowd = None  # pedestrians of the whole lattice, as own_of last saw them
+        self.crowd = None  # pedestrians of the whole lattice (set by the first own_of)
         units = -(-self.H // BIN)
         if units < nranks:
             raise ValueError(f"{H} rows give fewer than {nranks} bands of {BIN} rows")
@@ -152,9 +152,10 @@ class BandLayout:
 
 def own_of(layout: BandLayout, k: int, peds: Peds) -> Peds:
     """The pedestrians of a whole-lattice set that rank k owns.  The layout
-    keeps the set's size: it decides how the whole lattice's field is summed
-    (sfm_set_field_rule), and the bands must round alike."""
-    layout.crowd = peds.n
+    notes the first set's size, for the steppers made after that (sim_stepper's
+    `crowd`)."""
+    if layout.crowd is None:
+        layout.crowd = peds.n
     return peds.take(layout.owner(peds.xy[:, 1]) == k)
 
 
@@ -222,21 +223,32 @@ def band_tick(layout: BandLayout, k: int, comm, stepper: Stepper, own: Peds,
 
 
 def sim_stepper(layout: BandLayout, k: int, W: int, periodic_x: int, cell: np.ndarray,
-                D: np.ndarray, params: dict, stream=None) -> Tuple[Stepper, object]:
+                D: np.ndarray, params: dict, stream=None,
+                crowd: Optional[int] = None) -> Tuple[Stepper, object]:
     """A stepper on this library: one context over rank k's halo'd rows (its
     cells, the whole lattice's guidance distances for them), re-placed every
     tick with the whole lattice's pedestrian numbers and tick.  Returns
-    (stepper, the Sim, to be closed by the caller)."""
+    (stepper, the Sim, to be closed by the caller).
+
+    `crowd`: pedestrians of the whole lattice as it was placed, the same on
+    all ranks.  It decides, once for the stepper's life, how the bands' fields
+    are summed, as it does for one context over the whole lattice
+    (sfm_set_field_rule: a product of 9 pedestrians on 20 su and more).  Without
+    it the size that own_of noted on this layout holds; where there is none
+    either (ranks that load sets of their own), the bands gather, as a whole
+    lattice below that density does."""
     from . import Sim
     a, n = layout.rows(k)
     rows = np.arange(a, a + n) % layout.H
     sim = Sim(W=W, H=n, cell=np.ascontiguousarray(cell[rows]), periodic_x=periodic_x,
               periodic_y=0, stream=stream, **params)
     sim.set_guidance(np.ascontiguousarray(D[rows], np.int32))
+    if crowd is None:
+        crowd = layout.crowd
+    crowded = crowd is not None and 20 * crowd >= 9 * W * layout.H
+    sim.set_field_rule("product" if crowded else "gather")
 
     def step(xy, heading, goal, ids, t):
-        crowded = layout.crowd is not None and 20 * layout.crowd >= 9 * W * layout.H
-        sim.set_field_rule("product" if crowded else "gather")
         sim.place(xy, heading, goal)
         sim.set_ids(ids)
         sim.set_time(t)

@@ -190,3 +190,48 @@ def test_two_row_bands_round_as_the_whole_lattice():
     np.testing.assert_array_equal(ids[order], live)
     np.testing.assert_array_equal(np.concatenate([o.xy for o in owned])[order], xy[live])
     np.testing.assert_array_equal(np.concatenate([o.heading for o in owned])[order], hd[live])
+
+
+def test_the_rule_of_row_bands_is_the_whole_lattices_throughout():
+    """Bands resumed from per-rank sets (no own_of), with the whole lattice's
+    crowd given; and a look at a part of the crowd changes no stepper's rule."""
+    from paper_1803_04782_gb300 import bands as BD
+    sc = _crowd(96, 320, 12, 1, 0, rho=0.5, seed=10)
+    assert 20 * sc.n >= 9 * sc.W * sc.H
+    peds = BD.Peds(np.arange(sc.n, dtype=np.int32), sc.xy, sc.heading, sc.goal)
+    with sfm.Sim(sc) as whole:
+        D = whole.guidance()
+        whole.compute_field()
+        F = whole.field()
+        whole.step(2)
+        xy, hd, al = whole.peds()
+    for given in (True, False):
+        L = BD.BandLayout(sc.H, 0, 12, 2)
+        who = L.owner(peds.xy[:, 1])
+        owned = [peds.take(who == k) for k in range(2)]
+        if not given:
+            owned = [BD.own_of(L, k, peds) for k in range(2)]
+        steps = [BD.sim_stepper(L, k, sc.W, 1, sc.cell, D, sc.params, crowd=sc.n if given else None)
+                 for k in range(2)]
+        try:
+            for t in range(2):
+                BD.own_of(L, 0, owned[0].take(np.arange(owned[0].n) < 10))
+                sends = [BD.sends_of(L, k, owned[k]) for k in range(2)]
+
+                class Comm:
+                    def __init__(self, k):
+                        self.k = k
+
+                    def exchange(self, mine):
+                        return {j: sends[j][self.k].pack() for j in mine}
+                owned = [BD.band_tick(L, k, Comm(k), steps[k][0], owned[k], t)[0] for k in range(2)]
+                for k in range(2 if t == 0 else 0):  # the product's bits, not the gather's
+                    y = np.arange(L.y0[k], L.y1[k])
+                    np.testing.assert_array_equal(steps[k][1].field()[L.local_row(k, y)], F[y])
+        finally:
+            for _, sim in steps:
+                sim.close()
+        ids = np.concatenate([o.ids for o in owned])
+        order, live = np.argsort(ids), np.flatnonzero(al)
+        np.testing.assert_array_equal(ids[order], live)
+        np.testing.assert_array_equal(np.concatenate([o.xy for o in owned])[order], xy[live])
