@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/sfm.h"
+#include "sfm_limbs.h"
 
 namespace sfm {
 
@@ -242,11 +243,8 @@ struct ProductArgs {
   Counters* ctr = nullptr;
   int missing = 0;  // a test's: builders of planes that are waited for and do not exist
 };
-// Fixed-point scales of the limb tables: T = L0 / s0 + L1 / (s0 s1).  false:
-// the law's range over the window is too wide for them.
-struct ProductScales {
-  double s0 = 0.0, s1 = 0.0;
-};
+// Fixed-point scales of the limb tables (sfm_limbs.h).  false: the radius or the
+// law's range over the window is beyond them.
 bool product_crowd_scales(int r, const sfm_params& p, ProductScales* out);
 bool product_cell_scales(int r, const sfm_params& p, ProductScales* out);
 size_t product_table_bytes(int r, int nch);

@@ -574,19 +574,9 @@ __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, d
   const double d = in ? sqrt((double)(dx * dx + dy * dy)) : 1.0;
   const double v0 = in ? k0 * pow(d, a0) : 0.0, v1 = in && nch == 2 ? k1 * pow(d, a1) : 0.0;
   for (int ch = 0; ch < nch; ++ch) {
-    double v = v0;
-    if (nch == 2) {
-      if (ch == 1) v = v1;
-    } else {
-      const double q = 0.70710678118654752440;  // 1 / sqrt(2)
-      if (ch == 1) v *= gamma * dx / d;
-      if (ch == 2) v *= gamma * dy / d;
-      if (ch == 3) v *= gamma * q * (dx + dy) / d;
-      if (ch == 4) v *= gamma * q * (dy - dx) / d;
-    }
-    // an integer of FP16: any up to 2048, the nearest even one above
-    const __half hi = __double2half(fabs(v * s0) > 2048.0 ? v * s0 : rint(v * s0));
-    const __half lo = __double2half(rint((v * s0 - (double)__half2float(hi)) * s1));
+    const double v = nch == 2 ? (ch == 1 ? v1 : v0) : crowd_entry(v0, gamma, dx, dy, d, ch);
+    const double first = limb16(v * s0);
+    const __half hi = __double2half(first), lo = __double2half(limb16((v * s0 - first) * s1));
 #pragma unroll
     for (int nx = 0; nx < 8; ++nx) {
       const int w = nx - 7 + e;  // the window column
@@ -598,57 +588,14 @@ __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, d
   }
 }
 
-// A law k d^a over the window of radius r: largest and smallest magnitude and
-// the sum of the magnitudes.
-struct LawRange {
-  double big = 0.0, least = 0.0, sum = 0.0;
-};
-LawRange law_range(int r, double k, double a) {
-  LawRange l;
-  const double u = fabs(k), v = fabs(k) * pow(r * sqrt(2.0), a);
-  l.big = u > v ? u : v;
-  l.least = u > v ? v : u;
-  for (int x = 1; x <= r; ++x)  // an octant: (x, 0) and (x, x) stand for 4 su, the others for 8
-    for (int y = 0; y <= x; ++y)
-      l.sum += (y == 0 || y == x ? 4.0 : 8.0) * fabs(k) * pow((double)(x * x + y * y), 0.5 * a);
-  return l;
-}
-
-// Largest powers of two whose limbs are FP16 integers (up to 2048 any, up to
-// 4096 even ones) and whose sums over a full window stay below 2^24 (exact in
-// FP32).  `big` bounds an entry, `sum` what a full window adds to a first
-// limb, `entries` the tables a su is in; the second limbs are at most s1 / 2,
-// but for the few entries above half of `big`.  What their rounding leaves
-// must stay 5e-6 below `least`, the law's smallest magnitude in the window.
-bool product_scales(int r, double big, double sum, int entries, double least, ProductScales* out) {
-  if (r < 1 || r > kProductMaxRadius || !(big > 0.0) || !isfinite(big) || !isfinite(sum)) return false;
-  const double n = (2.0 * r + 1) * (2.0 * r + 1) + 60.0, top = 16777215.0;
-  double s0 = ldexp(1.0, (int)floor(log2(4096.0 / big)));
-  while (sum * s0 + n * entries > top) s0 *= 0.5;
-  double s1 = 4096.0;
-  while (n * entries * s1 * 0.5 > top) s1 *= 0.5;
-  if (!(entries * 1.0 / (s0 * s1) <= 5e-6 * least)) return false;
-  if (!(s0 > 1e-30 && s0 * s1 < 1e30)) return false;  // the limbs' weights are FP32
-  out->s0 = s0;
-  out->s1 = s1;
-  return true;
-}
-
 }  // namespace
 
 bool product_crowd_scales(int r, const sfm_params& p, ProductScales* out) {
-  const LawRange l = law_range(r, p.kP, p.aP);
-  const double g = fabs((double)p.gamma);
-  return product_scales(r, g > 1.0 ? l.big * g : l.big, l.sum * (1.0 + g), 2, l.least, out);
+  return r >= 1 && r <= kProductMaxRadius && crowd_limb_scales(r, p.kP, p.aP, p.gamma, out);
 }
 
-// a su is a wall, an exit or neither, so it adds one entry
 bool product_cell_scales(int r, const sfm_params& p, ProductScales* out) {
-  LawRange o = law_range(r, p.kO, p.aO), e = law_range(r, p.kE, p.aE);
-  if (p.kO == 0.f) o.least = e.least;
-  if (p.kE == 0.f) e.least = o.least;
-  return product_scales(r, o.big > e.big ? o.big : e.big, o.sum + e.sum, 1,
-                        o.least < e.least ? o.least : e.least, out);
+  return r >= 1 && r <= kProductMaxRadius && cell_limb_scales(r, p.kO, p.aO, p.kE, p.aE, out);
 }
 
 size_t product_table_bytes(int r, int nch) { return (size_t)nch * chunks_of(r) * stage_bytes_of(r); }

@@ -3,9 +3,14 @@ addresses and sums, restated in NumPy from their description (sfm_product.cu),
 give the window sums of the class-table law for every radius class, and no
 entry, sum or address leaves its range."""
 import math
+import os
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 TW, TH, MAXR, SMEM = 64, 256, 44, 227 * 1024
 
@@ -18,21 +23,30 @@ def pitch(r):
     return (TW - 8 + 16 * chunks(r)) * 2
 
 
-def scales(r, k=1.0, a=-0.5, g=0.5):
-    v = np.abs(law(r, 0, k, a, g))
-    n = (2 * r + 1) ** 2 + 60
-    s0 = 2.0 ** math.floor(math.log2(4096.0 / (v.max() * max(1.0, abs(g)))))
-    while v.sum() * (1 + abs(g)) * s0 + 2 * n > 2 ** 24 - 1:
-        s0 /= 2
-    s1 = 4096.0
-    while n * 2 * s1 / 2 > 2 ** 24 - 1:
-        s1 /= 2
-    return s0, s1
+@pytest.fixture(scope="module")
+def chosen(tmp_path_factory):
+    """The library's own choice of scales (None: refused)."""
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no C++ compiler")
+    exe = str(tmp_path_factory.mktemp("limbs") / "scales")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-Werror", "-I",
+                    os.path.join(ROOT, "paper_1803_04782_gb300", "csrc"),
+                    os.path.join(ROOT, "tests", "limb_scales_host.cpp"), "-o", exe], check=True)
+
+    def run(*args):
+        out = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, check=True).stdout
+        return None if out.startswith("refused") else tuple(float(v) for v in out.split())
+    return run
+
+
+def limb16(v):
+    return np.where(np.abs(v) > 2048, v.astype(np.float16).astype(np.float64), np.rint(v))
 
 
 def split(v, s0, s1):
-    hi = np.where(np.abs(v * s0) > 2048, (v * s0).astype(np.float16).astype(np.float64), np.rint(v * s0))
-    return hi, np.rint((v * s0 - hi) * s1).astype(np.float16).astype(np.float64)
+    hi = limb16(v * s0)
+    return hi, limb16((v * s0 - hi) * s1)
 
 
 def law(r, ch, k=1.0, a=-0.5, g=0.5):
@@ -46,26 +60,66 @@ def law(r, ch, k=1.0, a=-0.5, g=0.5):
     return v
 
 
+def partial_sums(first, axes):
+    """Largest magnitude that a sum of a limb can reach over full windows: the
+    planes one after the other, presence first, a su with one heading at most."""
+    m = np.max(np.abs(axes), axis=0)
+    return max(np.maximum(0, first + m).sum(), np.maximum(0, m - first).sum(), m.sum())
+
+
+def crowd_limbs(r, s, k, a, g):
+    limbs = [split(law(r, ch, k, a, g), *s) for ch in range(5)]
+    for hi, lo in limbs:
+        for limb in (hi, lo):  # integers that FP16 holds
+            assert (limb == limb.astype(np.float16).astype(np.float64)).all() and (limb == np.rint(limb)).all()
+    return limbs
+
+
 @pytest.mark.parametrize("r", [1, 2, 3, 7, 12, 20, 31, 32, 36, 37, 40, 44])
-def test_limbs_are_exact_and_their_sums_fit(r):
-    s0, s1 = scales(r)
-    hi_all = lo_all = np.zeros((2 * r + 1, 2 * r + 1))
-    for ch in range(5):
-        v = law(r, ch)
-        hi, lo = split(v, s0, s1)
-        for limb in (hi, lo):
-            assert np.abs(limb).max() <= 4096 and (limb == np.rint(limb)).all()
-        # a su is in the occupancy plane and at most one heading plane
-        if ch == 0:
-            hi0, lo0 = np.abs(hi), np.abs(lo)
-        else:
-            hi_all = np.maximum(hi_all, np.abs(hi))
-            lo_all = np.maximum(lo_all, np.abs(lo))
-        # what the second limb's rounding leaves: 2^-23 of the law's largest
-        # entry and less, and far below its smallest
-        err = np.abs(hi / s0 + lo / (s0 * s1) - v).max()
-        assert err <= 2.0 ** -23 and 2 * err <= 5.0e-6 * np.abs(law(r, 0))[0, 0]
-    assert (hi0 + hi_all).sum() < 2 ** 24 and (lo0 + lo_all).sum() < 2 ** 24   # exact in FP32
+def test_limbs_are_exact_and_their_sums_fit(chosen, r):
+    s = chosen("crowd", r, 1.0, -0.5, 0.5)
+    limbs = crowd_limbs(r, s, 1.0, -0.5, 0.5)
+    for i in range(2):
+        assert partial_sums(limbs[0][i], [l[i] for l in limbs[1:]]) < 2 ** 24   # exact in FP32
+    # what the second limb's rounding leaves, far below the law's smallest
+    err = [np.abs(hi / s[0] + lo / (s[0] * s[1]) - law(r, ch)) for ch, (hi, lo) in enumerate(limbs)]
+    assert (err[0] + np.max(err[1:], axis=0)).max() <= 5.0e-6 * np.abs(law(r, 0))[0, 0]
+
+
+def test_sums_fit_for_flat_rising_and_steep_laws(chosen):
+    """Every law that the library takes, over exponents, heading weights and
+    magnitudes: flat ones just above a power of two have large second limbs
+    all over the window."""
+    taken = 0
+    for r in (3, 17, 28, 31, 44):
+        for a in (-2.0, -1.0, -0.3, -0.05, 0.0, 0.05, 0.5, 1.0):
+            for g in (0.0, 0.5, 1.0, 1.7, 2.0):
+                for k in (1.0, 0.51, 2049.0 / 2048.0, 4095.5 / 4096.0, -3.3e4):
+                    s = chosen("crowd", r, k, a, g)
+                    if s is None:
+                        continue
+                    taken += 1
+                    limbs = crowd_limbs(r, s, k, a, g)
+                    for i in range(2):
+                        assert partial_sums(limbs[0][i], [l[i] for l in limbs[1:]]) < 2 ** 24, (r, a, g, k)
+    assert taken > 300
+
+
+def test_sums_of_walls_and_exits_fit(chosen):
+    taken = 0
+    for r in (12, 28, 40, 44):
+        for k0, a0, k1, a1 in ((1.0, -0.5, -1.0, -0.5), (1.0, 0.0, -1.0, 0.0), (0.51, 0.0, 0.0, 0.0),
+                               (2049.0 / 2048.0, 0.01, -0.75, -0.01), (1.0, -0.2, -1.5, -0.4), (0.0, 0.0, 0.3, 0.1)):
+            s = chosen("cells", r, k0, a0, k1, a1)
+            if s is None:
+                continue
+            taken += 1
+            two = [split(law(r, 0, k, a), *s) for k, a in ((k0, a0), (k1, a1))]
+            for i in range(2):
+                up = np.maximum(np.maximum(two[0][i], two[1][i]), 0).sum()
+                down = np.maximum(np.maximum(-two[0][i], -two[1][i]), 0).sum()
+                assert max(up, down) < 2 ** 24, (r, k0, a0, k1, a1)
+    assert taken > 10
 
 
 @pytest.mark.parametrize("r", range(1, MAXR + 1))
@@ -82,12 +136,12 @@ def test_operand_addresses_stay_in_their_buffers(r):
 
 
 @pytest.mark.parametrize("r", [1, 3, 5, 9])
-def test_tile_product_equals_the_window_sums(r):
+def test_tile_product_equals_the_window_sums(chosen, r):
     """One tile through the tables and addresses, in integers, against the
     direct window sum of the same fixed-point law."""
     rng = np.random.default_rng(r)
     C, K, J = chunks(r), 2 * r + 16, 2 * r + 31
-    s0, s1 = scales(r)
+    s0, s1 = chosen("crowd", r, 1.0, -0.5, 0.5)
     width = TW - 8 + 16 * C
     for ch in (0, 3):
         v = law(r, ch)
