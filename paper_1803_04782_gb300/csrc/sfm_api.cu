@@ -501,7 +501,7 @@ void ensure_product(sfm_ctx* c) {
   const size_t split = (size_t)std::min(product_tiles_x(g.W) * product_tiles_y(g.H), device_sm_count());
   uint8_t* tab = nullptr;
   const std::string err = c->err;
-  if (dalloc(c, &tab, product_table_bytes(g.r, 5)) != SFM_OK || dalloc(c, &a.tick, split) != SFM_OK ||
+  if (dalloc(c, &tab, product_table_bytes(g.r, kCrowdPlanes)) != SFM_OK || dalloc(c, &a.tick, split) != SFM_OK ||
       dalloc(c, &a.scratch, product_scratch_floats() * split) != SFM_OK) {
     c->err = err;
     dfree(c, tab);
@@ -510,7 +510,7 @@ void ensure_product(sfm_ctx* c) {
   }
   cudaMemsetAsync(a.tick, 0, split * sizeof(int), c->stream);
   cudaMemsetAsync(a.scratch, 0, product_scratch_floats() * split * sizeof(float), c->stream);
-  launch_limb_tables(g.r, c->prm, sc, 5, tab, c->stream);
+  launch_limb_tables(g.r, c->prm, sc, kCrowdPlanes, tab, c->stream);
   ++c->launches;
   a.ctr = c->ctr;
   a.one.src = c->ocls;
@@ -620,7 +620,7 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
       array_of(ctx->cell, nsu),
       array_of(ctx->Fs, nsu),
       array_of(ctx->D, nsu),
-      array_of(ctx->occ, std::max({nsu, static_tmp_bytes(g.r, ctx->prm) / sizeof(int32_t), guidance_scratch_ints(g)})),
+      array_of(ctx->occ, std::max({nsu, static_tmp_bytes(g.r) / sizeof(int32_t), guidance_scratch_ints(g)})),
       array_of(ctx->ocls, (size_t)g.opitch * g.H),
       array_of(ctx->T0, (size_t)S * S),
       array_of(ctx->TX, (size_t)S * S),

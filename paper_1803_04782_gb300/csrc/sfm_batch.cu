@@ -598,11 +598,11 @@ sfm_status setup_product(sfm_ctx* ctx) {
     }
     if (!B->tabs[i]) {
       uint8_t* t = nullptr;
-      if (balloc(ctx, &t, product_table_bytes(g.r, 5)) != SFM_OK) {
+      if (balloc(ctx, &t, product_table_bytes(g.r, kCrowdPlanes)) != SFM_OK) {
         ctx->err = err;
         continue;
       }
-      launch_limb_tables(g.r, p, w, 5, t, s);
+      launch_limb_tables(g.r, p, w, kCrowdPlanes, t, s);
       ctx->launches += 1;
       B->tabs[i] = t;
     }
@@ -860,7 +860,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
     // the occupancy grids are the static fields' scratch until they are cleared
     size_t tmp = 0;
     for (int i = 0; i < nscenes; ++i)
-      tmp = std::max({tmp, static_tmp_bytes(B->hs[i].g.r, prms[i]),
+      tmp = std::max({tmp, static_tmp_bytes(B->hs[i].g.r),
                       guidance_scratch_ints(B->hs[i].g) * sizeof(int32_t)});
     BALLOC(ctx->occ, std::max((size_t)su, tmp / sizeof(int32_t)));
   }

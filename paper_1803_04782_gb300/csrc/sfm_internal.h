@@ -215,6 +215,10 @@ constexpr int kProductMaxRadius = 44;
 // workloads (at most 2 su in 5), whose runs stay bit for bit what they were.
 inline bool lattice_crowded(int W, int H, int64_t n) { return 20 * n >= 9 * (int64_t)W * H; }
 
+// Planes (and their tables): a crowd's presence and four heading axes; a cell
+// grid's walls and exits, twice each (sfm_limbs.h)
+constexpr int kCrowdPlanes = 5, kCellPlanes = 4;
+
 // One lattice of a product launch: the source bytes (class grid or cell
 // grid), the limb tables of its radius, and where the sums go.
 struct ProductLattice {
@@ -232,7 +236,7 @@ struct ProductArgs {
   const ProductLattice* lattices = nullptr;  // a batch's
   const int2* tiles = nullptr;               // a batch's tiles (lattice, tile), costly ones first
   int tile0 = 0, ntiles = 0;  // of `one`: set by launch_product from the rows to store
-  int nch = 5;                // planes: 5 of a crowd, 2 of a cell grid
+  int nch = kCrowdPlanes;     // or kCellPlanes
   // sums of split tiles, product_scratch_floats() a tile, zero between
   // launches (NULL: no tile is split)
   float* scratch = nullptr;
@@ -261,7 +265,7 @@ void launch_tables(int r, const sfm_params& p, float* T0, float* TX, float* TY, 
                    float* KE, float* own, float* dirdot, float2* hvec, cudaStream_t s);
 // tmp: static_tmp_bytes() of device memory, 16-byte aligned, overwritten (limb
 // tables).  ctr: error flags of a bounded wait.
-size_t static_tmp_bytes(int r, const sfm_params& prm);
+size_t static_tmp_bytes(int r);
 void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, const sfm_params& prm,
                          float* Fs, void* tmp, Counters* ctr, cudaStream_t s);
 // Guidance distances; scratch: guidance_scratch_ints() ints of device memory,

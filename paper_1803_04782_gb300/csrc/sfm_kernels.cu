@@ -123,31 +123,34 @@ __global__ void __launch_bounds__(kFieldThreads)
 }
 
 // From radius 12 on, the product of the wall and exit planes with the two
-// laws' tables (sfm_product.cu; rounded once, like the compensated sum above).
-// The dense gather reads (2r + 1)^2 cells a su: a 2048 x 2048 floor's field at
-// radius 40 took 7719 us, the product 162 and its tables 32 (one-pass ncu),
-// the whole set-up 10.5 ms against 2.9.  A 100 x 100 lattice is set up in the
-// same time either way at radius 12 (360 us; 372 against 347 at radius 8,
-// where a tile's start costs more than the gather), a 4096 x 4096 one in 6.3
-// ms against 9.2.  The rule looks at the radius and the laws alone, so a
-// lattice, its row bands and a batch round alike.
+// laws' tables (sfm_product.cu; every entry as close to its law as FP32, the sum
+// rounded once, like the compensated sum above).  The dense gather reads
+// (2r + 1)^2 cells a su.  Set-up by the host's clock, product against gather: a
+// 2048 x 2048 lattice 2.10 ms against 2.76 at radius 12 and 2.32 against 9.73 at
+// 40; a 512 x 512 one 596 us against 591 and 753 against 1137; a 100 x 100 one,
+// where the tables and a tile's start show, 309 against 277 and 464 against 574
+// (320 both at 18).  The rule looks at the radius and the laws alone, so a
+// lattice, its row bands and a batch round alike; the line lies where large
+// lattices gain more than small ones lose.  (The cells' second limbs take a
+// second table, for their precision: set-up of a 2048 x 2048 floor at radius 40
+// 1350 -> 1481 us.)
+constexpr int kStaticProductRadius = 12;
 static bool static_product(int r, const sfm_params& prm, ProductScales* sc) {
-  return r >= 12 && product_cell_scales(r, prm, sc);
+  return r >= kStaticProductRadius && product_cell_scales(r, prm, sc);
 }
 
-size_t static_tmp_bytes(int r, const sfm_params& prm) {
-  ProductScales sc;
-  return static_product(r, prm, &sc) ? product_table_bytes(r, 2) : 0;
+size_t static_tmp_bytes(int r) {
+  return r >= kStaticProductRadius && r <= kProductMaxRadius ? product_table_bytes(r, kCellPlanes) : 0;
 }
 
 void launch_static_field(const Geo& g, const uint8_t* cell, const Tables& tb, const sfm_params& prm,
                          float* Fs, void* tmp, Counters* ctr, cudaStream_t s) {
   ProductScales sc;
   if (static_product(g.r, prm, &sc)) {
-    launch_limb_tables(g.r, prm, sc, 2, static_cast<uint8_t*>(tmp), s);
+    launch_limb_tables(g.r, prm, sc, kCellPlanes, static_cast<uint8_t*>(tmp), s);
     ProductArgs a;
     product_layout(g.r, &a);
-    a.nch = 2;
+    a.nch = kCellPlanes;
     a.ctr = ctr;
     a.store_hi = g.H;
     a.one.src = cell;

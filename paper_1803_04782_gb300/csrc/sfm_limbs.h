@@ -1,5 +1,7 @@
 // sfm_limbs.h -- the fixed-point form of the product's tables (sfm_product.cu):
-// T = L0 / s0 + L1 / (s0 s1), the limbs L0 and L1 integers that FP16 holds.
+// T = L0 / s0 + L1 / (s0 s1), the limbs L0 and L1 integers that FP16 holds.  The
+// cells' L1 is any integer up to 65504 and takes two tables, what FP16 holds of
+// it and what that leaves.
 // Plain functions, compiled for the device and for the host.
 //
 // The tensor cores add limbs in FP32, so a sum is exact, whatever the order, as
@@ -61,7 +63,7 @@ struct LimbOffset {
 inline bool limb_scales(const std::vector<LimbOffset>& w, double big, bool either, double most0,
                         double most1, ProductScales* out) {
   if (!(big > 0.0) || !isfinite(big)) return false;
-  const double top = 16777215.0, grow = 1.0 + ldexp(1.0, -10);  // FP16's rounding of large limbs
+  const double top = 16777215.0, grow = 1.0 + ldexp(1.0, -9);  // FP16's rounding of large limbs
   double n = 0.0, mag = 0.0;
   for (const LimbOffset& o : w) {
     double m = 0.0;
@@ -105,10 +107,10 @@ inline bool limb_scales(const std::vector<LimbOffset>& w, double big, bool eithe
   return true;
 }
 
-// what the limbs of v leave of it
-inline double limb_error(double v, const ProductScales& s) {
+// what the limbs of v leave of it; whole: a second limb of two tables
+inline double limb_error(double v, const ProductScales& s, bool whole) {
   const double x = v * s.s0, rest = (x - limb16(x)) * s.s1;
-  return fabs(limb16(rest) - rest) / (s.s0 * s.s1);
+  return fabs((whole ? rint(rest) : limb16(rest)) - rest) / (s.s0 * s.s1);
 }
 
 // the window's offsets (x, y), 0 <= y <= x <= r, and how many each stands for
@@ -136,28 +138,31 @@ inline bool crowd_limb_scales(int r, double k, double a, double gamma, ProductSc
   if (!limb_scales(w, big, true, 4096.0, 4096.0, out)) return false;
   for (const LimbOffset& o : w) {
     double e = 0.0;
-    for (double v : o.others) e = std::max(e, limb_error(v, *out));
-    if (!(limb_error(o.first, *out) + e <= 5e-6 * least)) return false;
+    for (double v : o.others) e = std::max(e, limb_error(v, *out, false));
+    if (!(limb_error(o.first, *out, false) + e <= 5e-6 * least)) return false;
   }
   return true;
 }
 
 // Walls (k0 d^a0) and exits (k1 d^a1): a su is one or the other, or neither.
+// false: an entry would be further from its law than FP32's rounding puts it
+// (2^-24 of itself), which a su that sees a single wall far away would show.
+// Two FP16 limbs are 22 bits and up, so the second one has two tables: the
+// defaults' entries at radius 40 are off by 5.6e-8 at most (2.1e-7 with one).
 inline bool cell_limb_scales(int r, double k0, double a0, double k1, double a1, ProductScales* out) {
   std::vector<LimbOffset> w;
-  double big = 0.0, least = INFINITY;
+  double big = 0.0;
   for_octant(r, [&](int x, int y, double count) {
-    const double d = sqrt((double)(x * x + y * y)), v0 = k0 * pow(d, a0), v1 = k1 * pow(d, a1);
+    const double d = sqrt((double)(x * x + y * y)), p = pow(d, a0);
+    const double v0 = k0 * p, v1 = k1 * (a1 == a0 ? p : pow(d, a1));
     w.push_back(LimbOffset{count, 0.0, {v0, v1, 0.0, 0.0}});
     big = std::max(big, std::max(fabs(v0), fabs(v1)));
     if (!isfinite(v0) || !isfinite(v1)) big = INFINITY;
-    if (k0 != 0.0) least = std::min(least, fabs(v0));
-    if (k1 != 0.0) least = std::min(least, fabs(v1));
   });
-  if (!limb_scales(w, big, false, 4096.0, 4096.0, out)) return false;
+  if (!limb_scales(w, big, false, 8192.0, 16384.0, out)) return false;
   for (const LimbOffset& o : w)
     for (double v : {o.others[0], o.others[1]})
-      if (!(limb_error(v, *out) <= 5e-6 * least)) return false;
+      if (!(limb_error(v, *out, true) <= ldexp(fabs(v), -24))) return false;
   return true;
 }
 

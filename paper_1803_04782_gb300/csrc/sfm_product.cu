@@ -365,10 +365,11 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
       const int pb = nplanes == 2 ? n_plane & 1 : 0;
       wait(pempty(pb), ((uint32_t)(n_plane / nplanes) & 1u) ^ 1u);
       // class values 1 + heading: E 2, NE 3, N 4, NW 5, then W 6, SW 7, S 8,
-      // SE 9; a cell grid's 1 (wall) and 2 (exit) are planes of their own
-      const int v = nch == 2 ? 1 + ch : (ch == 0 ? 0 : (ch == 1 ? 2 : (ch == 2 ? 4 : (ch == 3 ? 3 : 5))));
+      // SE 9; a cell grid's 1 (wall) and 2 (exit) are two planes each
+      const bool cells = nch == kCellPlanes;
+      const int v = cells ? 1 + (ch >> 1) : (ch == 0 ? 0 : (ch == 1 ? 2 : (ch == 2 ? 4 : (ch == 3 ? 3 : 5))));
       const uint32_t pos = (uint32_t)v * 0x01010101u;
-      const uint32_t neg = nch == 2 || ch == 0 ? 0u : (uint32_t)(v + 4) * 0x01010101u;
+      const uint32_t neg = cells || ch == 0 ? 0u : (uint32_t)(v + 4) * 0x01010101u;
       const uint32_t dst = plane0 + (uint32_t)pb * plane_bytes + (uint32_t)(w * 32 + lane) * 16;
       uint32_t any = 0;
 #pragma unroll
@@ -572,11 +573,15 @@ __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, d
   const int dy = j - r - 15, dx = r + 7 - e;  // = su column - window column + r
   const bool in = dx >= -r && dx <= r && dy >= -r && dy <= r && (dx | dy) != 0;
   const double d = in ? sqrt((double)(dx * dx + dy * dy)) : 1.0;
-  const double v0 = in ? k0 * pow(d, a0) : 0.0, v1 = in && nch == 2 ? k1 * pow(d, a1) : 0.0;
+  const bool cells = nch == kCellPlanes;
+  const double v0 = in ? k0 * pow(d, a0) : 0.0, v1 = in && cells ? k1 * pow(d, a1) : 0.0;
   for (int ch = 0; ch < nch; ++ch) {
-    const double v = nch == 2 ? (ch == 1 ? v1 : v0) : crowd_entry(v0, gamma, dx, dy, d, ch);
-    const double first = limb16(v * s0);
-    const __half hi = __double2half(first), lo = __double2half(limb16((v * s0 - first) * s1));
+    const double v = cells ? (ch < 2 ? v0 : v1) : crowd_entry(v0, gamma, dx, dy, d, ch);
+    const double first = limb16(v * s0), rest = (v * s0 - first) * s1, whole = rint(rest);
+    // a cell plane's second table: what FP16 leaves of the second limb
+    const bool second = cells && (ch & 1);
+    const __half hi = __double2half(second ? 0.0 : first);
+    const __half lo = __double2half(!cells ? limb16(rest) : second ? whole - limb16(whole) : limb16(whole));
 #pragma unroll
     for (int nx = 0; nx < 8; ++nx) {
       const int w = nx - 7 + e;  // the window column
@@ -603,7 +608,7 @@ size_t product_table_bytes(int r, int nch) { return (size_t)nch * chunks_of(r) *
 void launch_limb_tables(int r, const sfm_params& p, const ProductScales& sc, int nch, uint8_t* tab,
                         cudaStream_t s) {
   const int n = (16 * chunks_of(r) + 7) * (2 * r + 31);
-  const bool crowd = nch == 5;
+  const bool crowd = nch == kCrowdPlanes;
   k_limb_tables<<<(n + 63) / 64, 64, 0, s>>>(r, nch, crowd ? p.kP : p.kO, crowd ? p.aP : p.aO, p.kE,
                                                 p.aE, p.gamma, sc.s0, sc.s1, reinterpret_cast<__half*>(tab));
 }

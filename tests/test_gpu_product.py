@@ -94,6 +94,34 @@ def test_bands_batch_and_candidates_round_as_one_launch(px, py, r, rows):
             assert s.stats()["error_flags"] == 0
 
 
+@pytest.mark.parametrize("r,law", [(12, {}), (25, {}), (40, {}), (44, {}), (30, dict(aO=-1.0, aE=-0.7)),
+                                   (16, dict(kO=3.7e4, aO=-0.25, kE=0.0))])
+def test_a_wall_far_away_is_as_exact_as_fp32(r, law):
+    """One WALL and one EXIT su, in reach of different su: an entry rounded to
+    FP32 (2^-24 of itself) and the rounding of the sum."""
+    W = H = 4 * r + 9
+    cell = np.zeros((H, W), np.uint8)
+    at = {1: (r + 2, r + 1), 2: (W - r - 3, H - r - 2)}  # (x, y)
+    for kind, (x, y) in at.items():
+        cell[y, x] = kind
+    p = dict(kO=1.0, aO=-0.5, kE=-1.0, aE=-0.5)
+    p.update(law)
+    want, terms = np.zeros((H, W)), np.zeros((H, W))
+    yy, xx = np.mgrid[:H, :W]
+    for kind, (x, y) in at.items():
+        dx, dy = xx - x, yy - y
+        near = (np.maximum(abs(dx), abs(dy)) <= r) & ((dx != 0) | (dy != 0))
+        k, a = (np.float32(p["kO"]), np.float32(p["aO"])) if kind == 1 else (np.float32(p["kE"]), np.float32(p["aE"]))
+        d = np.hypot(dx, dy)
+        d[y, x] = 1.0
+        v = np.where(near, float(k) * d ** float(a), 0.0)
+        want += v
+        terms += abs(v)
+    with sfm.Sim(W=W, H=H, cell=cell, r=r, **p) as s:
+        got = s.static_field().astype(np.float64)
+    assert (np.abs(got - want) <= 2.0 ** -24 * (terms + np.abs(want)) * 1.0001).all()
+
+
 def test_autotuning_a_crowded_lattice_keeps_its_footprint():
     sc = _crowd(150, 256, 20, 1, 1, rho=0.55, seed=12)
     with sfm.Sim(sc) as s:

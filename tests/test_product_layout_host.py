@@ -105,8 +105,10 @@ def test_sums_fit_for_flat_rising_and_steep_laws(chosen):
     assert taken > 300
 
 
-def test_sums_of_walls_and_exits_fit(chosen):
+def test_sums_of_walls_and_exits_fit_and_no_entry_is_further_off_than_fp32s(chosen):
+    """The second limb is any integer up to 65504, in two tables."""
     taken = 0
+    assert all(chosen("cells", r, 1.0, -0.5, -1.0, -0.5) for r in range(12, 41))  # the default laws
     for r in (12, 28, 40, 44):
         for k0, a0, k1, a1 in ((1.0, -0.5, -1.0, -0.5), (1.0, 0.0, -1.0, 0.0), (0.51, 0.0, 0.0, 0.0),
                                (2049.0 / 2048.0, 0.01, -0.75, -0.01), (1.0, -0.2, -1.5, -0.4), (0.0, 0.0, 0.3, 0.1)):
@@ -114,10 +116,20 @@ def test_sums_of_walls_and_exits_fit(chosen):
             if s is None:
                 continue
             taken += 1
-            two = [split(law(r, 0, k, a), *s) for k, a in ((k0, a0), (k1, a1))]
-            for i in range(2):
-                up = np.maximum(np.maximum(two[0][i], two[1][i]), 0).sum()
-                down = np.maximum(np.maximum(-two[0][i], -two[1][i]), 0).sum()
+            two = []
+            for k, a in ((k0, a0), (k1, a1)):
+                v = law(r, 0, k, a)
+                hi = limb16(v * s[0])
+                lo = np.rint((v * s[0] - hi) * s[1])
+                most = limb16(lo)
+                for limb in (hi, most, lo - most):
+                    assert (limb == limb.astype(np.float16).astype(np.float64)).all()
+                assert (np.abs(hi / s[0] + lo / (s[0] * s[1]) - v) <= 2.0 ** -24 * np.abs(v)).all()
+                two.append((hi, most, np.abs(lo - most)))
+            for i in range(2):  # a partial sum has some of the small tables' entries
+                extra = i * np.maximum(two[0][2], two[1][2])
+                up = (np.maximum(np.maximum(two[0][i], two[1][i]), 0) + extra).sum()
+                down = (np.maximum(np.maximum(-two[0][i], -two[1][i]), 0) + extra).sum()
                 assert max(up, down) < 2 ** 24, (r, k0, a0, k1, a1)
     assert taken > 10
 
