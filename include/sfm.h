@@ -279,7 +279,10 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);
  * the field is a matrix product whose sums are exact (radius 1..44; laws
  * whose range over the window fits its fixed-point tables), rounded once;
  * below that, a gather of FP32 sums.  Both lie within the field's error
- * bound, the product closer, so they may differ in the last bits.  1: always
+ * bound and may differ in the last bits: the product is closer where many
+ * pedestrians are in reach (3e-8 of the field against 3e-7 to 9e-7), the gather
+ * where a single one is (2^-24 of its term; the product's entries are held to
+ * 2^-21, with the default law to 2.1e-7 up to radius 40).  1: always
  * the gather, 2: the product at any density where it can serve the radius.
  * For a context that is one band of a larger lattice and has to round as the
  * whole does.  Kept across placements.  Anything else is SFM_EINVAL. */

@@ -102,6 +102,7 @@ struct BatchState {
   // launch ahead of the tick's (they have no chunks then); their limb tables
   std::vector<uint8_t> crowded;
   std::vector<uint8_t*> tabs;
+  std::vector<ProductScales> scales;  // of the lattice's law (s0 0: not looked at, < 0: refused)
   std::vector<sfm_params> prms;
   ProductLattice* plat = nullptr;
   int2* tiles = nullptr;
@@ -590,8 +591,10 @@ sfm_status setup_product(sfm_ctx* ctx) {
     const BatchScene& sc = B->hs[i];
     const Geo& g = sc.g;
     const sfm_params& p = B->prms[i];
-    ProductScales w;
-    if (!lattice_crowded(g.W, g.H, sc.n) || !product_crowd_scales(g.r, p, &w)) continue;
+    if (!lattice_crowded(g.W, g.H, sc.n)) continue;
+    ProductScales& w = B->scales[i];
+    if (w.s0 == 0.0 && !product_crowd_scales(g.r, p, &w)) w.s0 = -1.0;
+    if (w.s0 < 0.0) continue;
     for (int k = 0; k < ns && !B->tabs[i]; ++k) {
       const sfm_params& q = B->prms[k];
       if (B->tabs[k] && q.r == p.r && q.kP == p.kP && q.aP == p.aP && q.gamma == p.gamma) B->tabs[i] = B->tabs[k];
@@ -802,6 +805,7 @@ sfm_status sfm_batch_create(int32_t nscenes, const sfm_lattice* lats, const uint
   B->nscenes = nscenes;
   B->prms.assign(prms, prms + nscenes);
   B->tabs.assign(nscenes, nullptr);
+  B->scales.assign(nscenes, ProductScales());
   B->crowded.assign(nscenes, 0);
   ctx->stream = static_cast<cudaStream_t>(stream);
   ctx->lat = lats[0];

@@ -121,25 +121,28 @@ inline void for_octant(int r, F f) {
 }
 
 // A crowd's law k d^a (1 + gamma h . u).  false: its range over the window is
-// too wide for the two limbs (their rounding must stay 5e-6 below the law's
-// smallest magnitude).
+// too wide for the two limbs: what a pedestrian adds to a su would be off by
+// more than 2^-21 of k d^a there.  The gathers' FP32 sums of a crowd are off by
+// that and more (3e-7 to 9e-7), but a lone pedestrian's entry, which they hold
+// to 2^-24, is not: the exact sums leave no room for a third limb in FP32.  The
+// default law's entries are off by 2.1e-7 at most up to radius 40 (a
+// pedestrian without heading 1.1e-7), by 4.2e-7 at 44.
 inline bool crowd_limb_scales(int r, double k, double a, double gamma, ProductScales* out) {
   std::vector<LimbOffset> w;
-  double big = 0.0, least = INFINITY;
+  double big = 0.0;
   for_octant(r, [&](int x, int y, double count) {
     const double d = sqrt((double)(x * x + y * y)), v = k * pow(d, a);
     LimbOffset o{count, v, {}};
     for (int j = 0; j < 4; ++j) o.others[j] = crowd_entry(v, gamma, x, y, d, 1 + j);
     for (double e : {o.first, o.others[0], o.others[1], o.others[2], o.others[3]})
       big = isfinite(e) ? std::max(big, fabs(e)) : INFINITY;
-    least = std::min(least, fabs(v));
     w.push_back(o);
   });
-  if (!limb_scales(w, big, true, 4096.0, 4096.0, out)) return false;
+  if (!limb_scales(w, big, true, 16384.0, 8192.0, out)) return false;
   for (const LimbOffset& o : w) {
     double e = 0.0;
     for (double v : o.others) e = std::max(e, limb_error(v, *out, false));
-    if (!(limb_error(o.first, *out, false) + e <= 5e-6 * least)) return false;
+    if (!(limb_error(o.first, *out, false) + e <= ldexp(fabs(o.first), -21))) return false;
   }
   return true;
 }

@@ -122,6 +122,28 @@ def test_a_wall_far_away_is_as_exact_as_fp32(r, law):
     assert (np.abs(got - want) <= 2.0 ** -24 * (terms + np.abs(want)) * 1.0001).all()
 
 
+@pytest.mark.parametrize("r,law", [(3, {}), (12, {}), (40, {}), (44, {}), (20, dict(aP=-1.0)), (40, dict(aP=-1.0))])
+def test_a_pedestrian_far_away_keeps_its_digits(r, law):
+    """One pedestrian by the product, or by the gather where the law is refused."""
+    aP = np.float64(law.get("aP", -0.5))
+    S = 2 * r + 3
+    yy, xx = np.mgrid[:S, :S]
+    dx, dy = xx - r - 1.0, yy - r - 1.0
+    d = np.hypot(dx, dy)
+    d[r + 1, r + 1] = 1.0
+    with sfm.Sim(W=S, H=S, cell=np.zeros((S, S), np.uint8), r=r, **law) as s:
+        s.set_field_rule("product")
+        for h, (ux, uy) in enumerate([(0, 0), (1, 0), (1, 1), (0, 1), (-1, 1), (-1, 0), (-1, -1), (0, -1), (1, -1)]):
+            s.place(np.array([[r + 1, r + 1]], np.int32), np.array([h], np.uint8))
+            s.compute_field()
+            u = max(1.0, np.hypot(ux, uy))
+            base = np.where(np.maximum(abs(dx), abs(dy)) <= r, d ** aP, 0.0)
+            base[r + 1, r + 1] = 0.0
+            want = base * (1 + 0.5 * (ux * dx + uy * dy) / (u * d))
+            off = np.abs(s.field() - want)
+            assert (off <= (2.2e-7 if r <= 40 and not law else 2.0 ** -21) * base + 2.0 ** -24 * np.abs(want) * 1.001).all()
+
+
 def test_autotuning_a_crowded_lattice_keeps_its_footprint():
     sc = _crowd(150, 256, 20, 1, 1, rho=0.55, seed=12)
     with sfm.Sim(sc) as s:
