@@ -95,6 +95,7 @@ struct BatchState {
   int* work = nullptr;
   int max_ts = 0;
   int shape_of_sp[kNumStrideClasses] = {};  // footprint shape per class-table stride
+  bool by_bins = true;  // S3-S5 a block a bin (by the placement's density), else by pedestrian
   int missing = 0;  // test hook: CTAs the barrier expects beyond those launched
   int grid = 0;
   std::vector<int> order;  // lattices by decreasing field cost
@@ -397,6 +398,55 @@ __global__ void __launch_bounds__(kMoveThreads) k_batch_commit(BatchArgs a) {
   count_moves(a.ctr, nm, nl);
 }
 
+// The same by pedestrian (a thread each, in bin order), for sparse batches, whose
+// bins hold too few for their su to be read whole: below a pedestrian on every
+// tenth su of all lattices, as in a single lattice (move_by_bins).  A tick of 8
+// lattices of 1024^2 to 2048^2 at r = 5, by pedestrian and by bins: 235 and 309
+// us at a density of 0.001, 358 and 418 at 0.02, 646 both at 0.08, 822 and 783
+// at 0.12, 1833 and 1481 at 0.4; of 256 lattices of 200^2 163 and 208, 214 and
+// 284, 366 and 404, 464 and 477, 1058 and 884.  (A line for each lattice, with
+// both forms launched, took 4 % of a batch of 32 uneven rooms.)
+__device__ __forceinline__ int batch_ped(const BatchArgs& a, const BatchScene*& sc) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t err = a.ctr->err;
+  if (i >= a.bin_start[a.total_bins] || err & kErrTimeout) return -1;
+  const int p = a.rec_id[i];
+  sc = a.scenes + a.ped_scene[p];
+  return p;
+}
+
+__global__ void __launch_bounds__(256) k_batch_decide_peds(BatchArgs a) {
+  const BatchScene* sc;
+  const int p = batch_ped(a, sc);
+  if (p < 0) return;
+  const int at = a.ped_scene[p];
+  a.choice[p] = decide_one(p, sc->g, a.xy, a.heading, a.goal, a.ocls + sc->ocls_off, a.D + sc->su_off,
+                           a.F + sc->su_off, 0, -1, -1, 0, 0, sc->g.H, sc->beta, a.own + 81 * at,
+                           a.dirdot + 81 * at);
+}
+
+__global__ void __launch_bounds__(256) k_batch_vote_peds(BatchArgs a) {
+  const BatchScene* sc;
+  const int p = batch_ped(a, sc);
+  int most = 0;
+  if (p >= 0)
+    most = vote_one(p, sc->ped_off, sc->g, a.xy, a.choice, a.occ + sc->su_off, sc->seed, a.ctr->t, a.won);
+  __syncwarp();
+  count_votes(a.ctr, most);
+}
+
+__global__ void __launch_bounds__(256) k_batch_commit_peds(BatchArgs a) {
+  const BatchScene* sc;
+  const int p = batch_ped(a, sc);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && !(a.ctr->err & kErrTimeout)) a.ctr->t += 1;
+  bool moved = false, left = false;
+  if (p >= 0)
+    commit_one(p, sc->g, a.xy, a.alive, a.heading, a.choice, a.won, a.cell + sc->su_off,
+               a.occ + sc->su_off, a.ocls + sc->ocls_off, moved, left);
+  __syncwarp();
+  count_moves(a.ctr, moved, left);
+}
+
 // The lattice of each pedestrian: the last one whose pedestrians start at or
 // before it.  (Filled by the host and copied, 2.8 million took 500 us a placement.)
 __global__ void k_batch_owner(int n, int nscenes, const BatchScene* __restrict__ scenes,
@@ -690,10 +740,21 @@ cudaError_t launch_tick(sfm_ctx* ctx, int field_only, cudaStream_t s) {
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k_tick_batch, a);
   if (e != cudaSuccess || field_only) return e;
-  k_batch_decide<<<B->total_bins, kMoveThreads, 0, s>>>(a);
-  k_batch_vote<<<B->total_bins, kMoveThreads, 0, s>>>(a);
-  k_batch_commit<<<B->total_bins, kMoveThreads, 0, s>>>(a);
+  if (B->by_bins) {
+    k_batch_decide<<<B->total_bins, kMoveThreads, 0, s>>>(a);
+    k_batch_vote<<<B->total_bins, kMoveThreads, 0, s>>>(a);
+    k_batch_commit<<<B->total_bins, kMoveThreads, 0, s>>>(a);
+  } else {
+    const int blocks = (ctx->n + 255) / 256;
+    k_batch_decide_peds<<<blocks, 256, 0, s>>>(a);
+    k_batch_vote_peds<<<blocks, 256, 0, s>>>(a);
+    k_batch_commit_peds<<<blocks, 256, 0, s>>>(a);
+  }
   return cudaGetLastError();
+}
+
+int tick_launches(const BatchState* B, int field_only) {
+  return (B->prod.ntiles ? 2 : 1) + (field_only ? 0 : 3);
 }
 
 sfm_status check_batch(sfm_ctx* ctx) {
@@ -729,7 +790,7 @@ sfm_status batch_tick(sfm_ctx* ctx, int nsteps, int field_only) {
     // test hook: one direct tick whose barrier waits for CTAs that do not
     // exist; the bounded wait gives up and the tick reports SFM_ETIMEOUT
     BCU(launch_tick(ctx, field_only, ctx->stream));
-    ctx->launches += field_only ? 1 : 4;
+    ctx->launches += tick_launches(B, field_only);
     B->missing = 0;
     return check_batch(ctx);
   }
@@ -767,7 +828,7 @@ sfm_status batch_tick(sfm_ctx* ctx, int nsteps, int field_only) {
     } else {
       BCU(cudaGraphLaunch(B->graph, ctx->stream));
     }
-    ctx->launches += (B->prod.ntiles ? 2 : 1) + (field_only ? 0 : 3);
+    ctx->launches += tick_launches(B, field_only);
     if (!field_only) ++ctx->t;
   }
   if (ctx->timing && !field_only) ctx->timed_ticks += nsteps;
@@ -1012,6 +1073,7 @@ sfm_status sfm_batch_place(sfm_ctx* ctx, const int32_t* counts, const int32_t* x
       B->hs[i].n = counts[i];
       off += counts[i];
     }
+    B->by_bins = n == 0 || (int64_t)n * 10 >= ctx->nsu_total;
   }
   BCU(cudaMemcpyAsync(B->scenes, B->hs.data(), B->hs.size() * sizeof(BatchScene),
                       cudaMemcpyHostToDevice, s));

@@ -157,3 +157,42 @@ def test_batch_placement_errors():
         b.place([s.xy for s in scenes], [s.heading for s in scenes], [s.goal for s in scenes])
         b.step(1)
         assert b.stats()["error_flags"] == 0
+
+
+def test_sparse_and_dense_lattices_in_one_batch():
+    """Decide, vote and commit go by pedestrian below a pedestrian on every tenth
+    su of the batch, by bins from there on: batches of sparse and dense lattices
+    on either side of the line, against single contexts."""
+    def scene(W, H, n, seed, px):
+        return SG.random_scene(W, H, n, r=4, seed=seed, periodic_x=px, periodic_y=px, ring=not px,
+                               exits=() if px else ("east",), goal_mode="fixed" if px else "mixed",
+                               heading_mode="random")
+    sparse = [scene(90, 70, 629, 1, 1), scene(33, 65, 3, 2, 0), scene(300, 200, 900, 3, 0)]
+    dense = [scene(90, 70, 630, 4, 1), scene(64, 64, 1200, 5, 0), scene(31, 37, 1147 // 2, 6, 1)]
+    for scenes in (sparse, dense, sparse[:2] + dense + sparse[2:]):
+        with sfm.Batch(scenes) as b:
+            singles = [sfm.Sim(s) for s in scenes]
+            try:
+                for _ in range(2):
+                    for x in singles + [b]:
+                        x.step(3)
+                    for got, want in zip(zip(*b.peds()), (s.peds() for s in singles)):
+                        for x, y in zip(got, want):
+                            np.testing.assert_array_equal(x, y)
+                    for got, want in zip(zip(*b.decisions()), (s.decisions() for s in singles)):
+                        for x, y in zip(got, want):
+                            np.testing.assert_array_equal(x, y)
+                st, of = b.stats(), [s.stats() for s in singles]
+                assert st["t"] == 6 and st["error_flags"] == 0
+                for key in ("moved_total", "exited"):
+                    assert st[key] == sum(s[key] for s in of)
+                assert st["max_registrants"] == max(s["max_registrants"] for s in of)
+                # the same lattices with everybody but one gone, then nobody
+                sfm.sfm_batch_place(b.ctx, [1] + [0] * (len(scenes) - 1), scenes[0].xy[:1].copy())
+                b.step(2)
+                sfm.sfm_batch_place(b.ctx, [0] * len(scenes), np.zeros((0, 2), np.int32))
+                b.step(2)
+                assert b.stats()["t"] == 10
+            finally:
+                for s in singles:
+                    s.close()
