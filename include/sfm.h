@@ -276,7 +276,8 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);
 
 /* How the field of a crowded lattice is summed.  0 (the default): by the
  * context's own crowd -- from 9 pedestrians of the last placement on 20 su
- * the field is a matrix product whose sums are exact (radius 1..44; laws
+ * (in a lattice no larger than the window either way: where it is also the
+ * faster way; sfm_crowded) the field is a matrix product whose sums are exact (radius 1..44; laws
  * whose range over the window fits its fixed-point tables), rounded once;
  * below that, a gather of FP32 sums.  Both lie within the field's error
  * bound and may differ in the last bits: the product is closer where many
@@ -287,6 +288,10 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);
  * For a context that is one band of a larger lattice and has to round as the
  * whole does.  Kept across placements.  Anything else is SFM_EINVAL. */
 sfm_status sfm_set_field_rule(sfm_ctx* ctx, int32_t mode);
+
+/* Whether rule 0 takes a crowd of n pedestrians on the lattice at radius r
+ * for crowded (1) or not (0, also for arguments that make no lattice). */
+int32_t sfm_crowded(const sfm_lattice* lat, int32_t r, int64_t n);
 
 /* Wait for the context's stream and report device-side errors.  After
  * SFM_ETIMEOUT the crowd stays where it was before the tick whose field is

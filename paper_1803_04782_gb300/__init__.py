@@ -33,7 +33,7 @@ EXPORTS = [
     "sfm_set_time", "sfm_step", "sfm_compute_field", "sfm_sync", "sfm_read_field",
     "sfm_compute_field_into", "sfm_read_static_field", "sfm_read_guidance", "sfm_read_peds",
     "sfm_read_decisions", "sfm_stats", "sfm_set_timing", "sfm_stage_times",
-    "sfm_autotune", "sfm_set_field_footprint", "sfm_set_field_rule", "sfm_set_binning", "sfm_set_walk_periods",
+    "sfm_autotune", "sfm_set_field_footprint", "sfm_set_field_rule", "sfm_crowded", "sfm_set_binning", "sfm_set_walk_periods",
     "sfm_test_wait_out",
     "sfm_place_sized", "sfm_snapshot", "sfm_restore", "sfm_set_ids", "sfm_set_guidance", "sfm_field_noalloc", "sfm_batch_create", "sfm_batch_place", "sfm_batch_offsets",
     "sfm_batch_autotune", "sfm_batch_test_missing_ctas", "sfm_surrogate_nparams",
@@ -120,6 +120,7 @@ def lib():
             "sfm_autotune": (C.c_int, [P, P]),
             "sfm_set_field_footprint": (C.c_int, [P, I32]),
             "sfm_set_field_rule": (C.c_int, [P, I32]),
+            "sfm_crowded": (I32, [C.POINTER(Lattice), I32, C.c_int64]),
             "sfm_set_binning": (C.c_int, [P, I32]),
             "sfm_test_wait_out": (C.c_int, [P, I32]),
             "sfm_set_walk_periods": (C.c_int, [P, P, P, I32]),
@@ -198,6 +199,10 @@ def sfm_abi_version() -> int:
 
 def sfm_resident_bytes(lat: Lattice) -> int:
     return int(lib().sfm_resident_bytes(C.byref(lat)))
+
+
+def sfm_crowded(lat: Lattice, r: int, n: int) -> bool:
+    return bool(lib().sfm_crowded(C.byref(lat), int(r), int(n)))
 
 
 # rows of the band buffer beyond a band's own (sfm_resident_bytes in sfm.h)

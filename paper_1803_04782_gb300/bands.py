@@ -233,11 +233,11 @@ def sim_stepper(layout: BandLayout, k: int, W: int, periodic_x: int, cell: np.nd
     `crowd`: pedestrians of the whole lattice as it was placed, the same on
     all ranks.  It decides, once for the stepper's life, how the bands' fields
     are summed, as it does for one context over the whole lattice
-    (sfm_set_field_rule: a product of 9 pedestrians on 20 su and more).  Without
+    (sfm_set_field_rule, sfm_crowded).  Without
     it the size that own_of noted on this layout holds; where there is none
     either (ranks that load sets of their own), the bands gather, as a whole
     lattice below that density does."""
-    from . import Sim
+    from . import Lattice, Sim, sfm_crowded
     a, n = layout.rows(k)
     rows = np.arange(a, a + n) % layout.H
     sim = Sim(W=W, H=n, cell=np.ascontiguousarray(cell[rows]), periodic_x=periodic_x,
@@ -245,7 +245,7 @@ def sim_stepper(layout: BandLayout, k: int, W: int, periodic_x: int, cell: np.nd
     sim.set_guidance(np.ascontiguousarray(D[rows], np.int32))
     if crowd is None:
         crowd = layout.crowd
-    crowded = crowd is not None and 20 * crowd >= 9 * W * layout.H
+    crowded = crowd is not None and sfm_crowded(Lattice(W, layout.H, periodic_x, layout.py), layout.r, crowd)
     sim.set_field_rule("product" if crowded else "gather")
 
     def step(xy, heading, goal, ids, t):

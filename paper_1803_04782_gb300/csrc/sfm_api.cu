@@ -1099,6 +1099,10 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape) {
   return SFM_OK;
 }
 
+int32_t sfm_crowded(const sfm_lattice* lat, int32_t r, int64_t n) {
+  return lat && lat->W > 0 && lat->H > 0 && r >= 0 && n >= 0 && lattice_crowded(lat->W, lat->H, r, n);
+}
+
 sfm_status sfm_set_field_rule(sfm_ctx* ctx, int32_t mode) {
   if (!ctx) return SFM_EINVAL;
   if (ctx->batch) return fail(ctx, SFM_EINVAL, "a batch judges each lattice by its own crowd");

@@ -641,7 +641,7 @@ sfm_status setup_product(sfm_ctx* ctx) {
     const BatchScene& sc = B->hs[i];
     const Geo& g = sc.g;
     const sfm_params& p = B->prms[i];
-    if (!lattice_crowded(g.W, g.H, sc.n)) continue;
+    if (!lattice_crowded(g.W, g.H, g.r, sc.n)) continue;
     ProductScales& w = B->scales[i];
     if (w.s0 == 0.0 && !product_crowd_scales(g.r, p, &w)) w.s0 = -1.0;
     if (w.s0 < 0.0) continue;

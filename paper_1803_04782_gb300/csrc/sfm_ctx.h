@@ -137,7 +137,7 @@ struct sfm_ctx {
     return sz;
   }
   bool wants_product() const {
-    return field_rule == 2 || (field_rule == 0 && sfm::lattice_crowded(geo.W, geo.H, n));
+    return field_rule == 2 || (field_rule == 0 && sfm::lattice_crowded(geo.W, geo.H, geo.r, n));
   }
   bool use_product() const { return prod.smem_bytes && wants_product(); }
   const int32_t* ids() const { return has_ids ? gid : nullptr; }

@@ -94,6 +94,24 @@ def test_bands_batch_and_candidates_round_as_one_launch(px, py, r, rows):
             assert s.stats()["error_flags"] == 0
 
 
+@pytest.mark.parametrize("W,H,r,product", [(20, 20, 38, False), (24, 26, 20, False), (300, 8, 20, False),
+                                           (40, 40, 44, True), (64, 64, 38, True), (41, 45, 20, True)])
+def test_lattices_smaller_than_the_window_take_the_faster_way(W, H, r, product):
+    sc = _crowd(W, H, r, 0, 0, rho=0.95, seed=13)
+    assert 20 * sc.n >= 9 * W * H
+    assert sfm.sfm_crowded(sfm.Lattice(W, H, 0, 0), r, sc.n) == product
+    fields = []
+    with sfm.Sim(sc) as s, sfm.Batch([sc]) as b:
+        for rule in ("auto", "gather", "product"):
+            s.set_field_rule(rule)
+            s.compute_field()
+            fields.append(s.field())
+        b.compute_field()
+        np.testing.assert_array_equal(b.fields()[0], fields[0])
+    np.testing.assert_array_equal(fields[0], fields[2 if product else 1])
+    assert not np.array_equal(fields[1], fields[2])
+
+
 @pytest.mark.parametrize("r,law", [(12, {}), (25, {}), (40, {}), (44, {}), (30, dict(aO=-1.0, aE=-0.7)),
                                    (16, dict(kO=3.7e4, aO=-0.25, kE=0.0))])
 def test_a_wall_far_away_is_as_exact_as_fp32(r, law):
