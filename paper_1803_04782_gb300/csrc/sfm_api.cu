@@ -229,10 +229,10 @@ cudaError_t run_tick(sfm_ctx* c) {
       e = field_rows(c, c->F, 0, g.H, 0, false, early);
     }
     if (e != cudaSuccess) return e;
-    if (!c->timing && c->n > 0 && c->n <= kMoveMaxPeds) {
+    if (!c->timing && move_in_one(g.W, g.H, g.r, c->n, c->sized)) {
       launch_move(c->n, c->rec_id, c->bin_start, c->xy, c->alive, c->heading, c->goal, c->cell, c->occ,
                   c->ocls, c->D, c->F, g, c->prm.beta, c->prm.seed, tb, c->choice, c->won, c->ctr,
-                  c->stream, c->walk(), c->sizes(), c->ids(), early);
+                  c->stream, c->walk(), c->ids(), early);
       ++c->launches;
       return cudaSuccess;
     }

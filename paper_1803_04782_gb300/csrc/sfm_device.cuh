@@ -248,14 +248,14 @@ __device__ __forceinline__ uint32_t blocked_moves(const Geo& g, const uint8_t* _
     return !in || cell[s] == kWall || occ[s] >= 0;
   };
   uint32_t m = 0;
-#pragma unroll LANES == 1 ? 3 : 1
+#pragma unroll 1
   for (int j = sub - b; j <= b; j += LANES) {
     const uint32_t up = j > -b, down = j < b;
     const bool e = blocked(a + 1, j), w = blocked(-a - 1, j);
     m |= e ? 1u << 1 | up << 2 | down << 8 : 0u;
     m |= w ? 1u << 5 | up << 4 | down << 6 : 0u;
   }
-#pragma unroll LANES == 1 ? 3 : 1
+#pragma unroll 1
   for (int i = sub - a; i <= a; i += LANES) {
     const uint32_t right = i > -a, left = i < a;
     const bool n = blocked(i, b + 1), s = blocked(i, -b - 1);

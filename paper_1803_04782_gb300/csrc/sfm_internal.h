@@ -390,14 +390,24 @@ void launch_commit(int n, const int32_t* rec_id, const int32_t* bin_start, int2*
                    const uint8_t* cell, int32_t* occ, uint8_t* ocls, const Geo& g, Counters* ctr,
                    cudaStream_t s, const Sizes& sz = Sizes());
 // Decide, vote and commit of a whole lattice (F: its rows) of n <=
-// kMoveMaxPeds pedestrian slots in one launch.
+// kMoveMaxPeds pedestrian slots of 1 x 1 su in one launch.
 constexpr int kMoveMaxPeds = 1024;
+// One block saves two launches, but its reads are those of one SM.  A tick by it
+// and by three launches: 256 pedestrians on 300 x 300 19.8 and 22.6 us, 512 23.3
+// both, 1024 31.1 and 23.5; 384 on 2000 x 2000 32.0 and 31.9; where many share a
+// su's surroundings later: 768 on 100 x 100 27.8 and 28.6, 1024 29.6 and 27.4, on
+// 40 x 40 45.7 and 49.0.  Beside a gather of large tables the block has little
+// L1: 617 x 477 at r = 40, 128 pedestrians 24.5 and 24.9, 256 30.8 and 26.4 (at r =
+// 30 22.5 and 25.5).  Rectangles read their whole rings: always slower.
+inline bool move_in_one(int W, int H, int r, int n, bool sized) {
+  const int64_t su = (int64_t)W * H;
+  return !sized && n > 0 && n <= (r > 33 ? 128 : su > 128 * 128 ? 384 : su > 64 * 64 ? 768 : kMoveMaxPeds);
+}
 void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy, uint8_t* alive,
                  uint8_t* heading, const uint8_t* goal, const uint8_t* cell, int32_t* occ,
                  uint8_t* ocls, const int32_t* D, const float* F, const Geo& g, float beta,
                  uint64_t seed, const Tables& tb, uint8_t* choice, uint8_t* won, Counters* ctr,
-                 cudaStream_t s, const WalkPeriods& wp, const Sizes& sz, const int32_t* gid,
-                 bool early);
+                 cudaStream_t s, const WalkPeriods& wp, const int32_t* gid, bool early);
 
 // The same stages of a whole lattice of 1 x 1 pedestrians, a block a bin
 // (sfm_move.cu): the choice and the win are kept in the records as well.

@@ -1323,16 +1323,14 @@ void launch_commit(int n, const int32_t* rec_id, const int32_t* bin_start, int2*
 // a block barrier where the single stages have a launch.  Bound by the chain of
 // dependent reads (record, position, neighbourhood, rivals), which the stages
 // have as well; with two launches less, the shorter binning and the early
-// starts a tick of the 100 x 100 room with 200 pedestrians went from 32 to 25 us.
-template <bool SIZED>
+// starts a tick of the 100 x 100 room with 200 pedestrians went from 32 to 21 us.
 __global__ void __launch_bounds__(kMoveMaxPeds)
     k_move(int n, const int32_t* rec_id, const int32_t* bin_start, int nbins, int2* xy,
            uint8_t* alive, uint8_t* heading, const uint8_t* __restrict__ goal,
            const uint8_t* __restrict__ cell, int32_t* occ, uint8_t* ocls,
            const int32_t* __restrict__ D, const float* F, Geo g, float beta, uint64_t seed,
            const float* __restrict__ own, const float* __restrict__ dirdot, uint8_t* choice,
-           uint8_t* won, Counters* ctr, WalkPeriods wp, Sizes sz,
-           const int32_t* __restrict__ gid) {
+           uint8_t* won, Counters* ctr, WalkPeriods wp, const int32_t* __restrict__ gid) {
   // by pedestrian: the choices and wins of the stages before, not read back
   // from memory
   __shared__ uint8_t s_choice[kMoveMaxPeds], s_won[kMoveMaxPeds];
@@ -1348,37 +1346,20 @@ __global__ void __launch_bounds__(kMoveMaxPeds)
   bool decided = false, tie = false;
   if (p >= 0) {
     decided = !(wp.period && t % wp.period[p] != wp.phase[p]);
-    uint32_t blocked = 0;
-    if (SIZED && decided) {
-      const int2 q = xy[p];
-      blocked = blocked_moves<1>(g, cell, occ, q.x, q.y, sz.w[p] >> 1, sz.h[p] >> 1, 0);
-    }
-    const uint8_t k = decided ? decide_one<true, SIZED>(p, g, xy, heading, goal, ocls, D, F, 0, -1, -1, 0,
-                                                        0, g.H, beta, own, dirdot, &tie, 0, blocked)
+    const uint8_t k = decided ? decide_one<true>(p, g, xy, heading, goal, ocls, D, F, 0, -1, -1, 0, 0, g.H,
+                                                 beta, own, dirdot, &tie)
                               : (uint8_t)0;
     s_choice[p] = choice[p] = k;
   }
   __syncthreads();
   int regs = 0;
   if (p >= 0) {
-    if (SIZED) {
-      bool win;
-      regs = vote_one_sized<1>(p, g, xy, s_choice, occ, sz.w, sz.h, seed, t, 0, win);
-      s_won[p] = win ? 1 : 0;
-    } else {
-      regs = vote_one(p, 0, g, xy, s_choice, occ, seed, t, s_won, gid);
-    }
+    regs = vote_one(p, 0, g, xy, s_choice, occ, seed, t, s_won, gid);
     won[p] = s_won[p];
   }
   __syncthreads();
   bool moved = false, left = false;
-  if (p >= 0 && whole) {
-    if (SIZED)
-      commit_one_sized(p, g, xy, alive, heading, s_choice, s_won, cell, occ, ocls, sz.w, sz.h, moved,
-                       left);
-    else
-      commit_one(p, g, xy, alive, heading, s_choice, s_won, cell, occ, ocls, moved, left);
-  }
+  if (p >= 0 && whole) commit_one(p, g, xy, alive, heading, s_choice, s_won, cell, occ, ocls, moved, left);
   const unsigned nd = __popc(__ballot_sync(0xffffffffu, decided));
   const unsigned nt = __popc(__ballot_sync(0xffffffffu, tie));
   const unsigned nm = __popc(__ballot_sync(0xffffffffu, moved));
@@ -1399,11 +1380,10 @@ void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* x
                  uint8_t* heading, const uint8_t* goal, const uint8_t* cell, int32_t* occ,
                  uint8_t* ocls, const int32_t* D, const float* F, const Geo& g, float beta,
                  uint64_t seed, const Tables& tb, uint8_t* choice, uint8_t* won, Counters* ctr,
-                 cudaStream_t s, const WalkPeriods& wp, const Sizes& sz, const int32_t* gid,
-                 bool early) {
-  launch_tick_kernel(sz.w ? k_move<true> : k_move<false>, 1, 32 * cdiv(n, 32), 0, s, early, n, rec_id, bin_start, g.nbx * g.nby, xy,
-                     alive, heading, goal, cell, occ, ocls, D, F, g, beta, seed, tb.own, tb.dirdot,
-                     choice, won, ctr, wp, sz, gid);
+                 cudaStream_t s, const WalkPeriods& wp, const int32_t* gid, bool early) {
+  launch_tick_kernel(k_move, 1, 32 * cdiv(n, 32), 0, s, early, n, rec_id, bin_start, g.nbx * g.nby, xy, alive,
+                     heading, goal, cell, occ, ocls, D, F, g, beta, seed, tb.own, tb.dirdot, choice, won, ctr,
+                     wp, gid);
 }
 
 }  // namespace sfm

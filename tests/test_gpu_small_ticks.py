@@ -1,7 +1,7 @@
 """The short launch sequences of small lattices against the long ones: bins
 from the class grid in one launch (64 bins), two (4096) or three and more, the
-pedestrian list's bins, and decide, vote and commit in one block (1024
-pedestrian slots) or three launches; and those stages bin by bin against
+pedestrian list's bins, and decide, vote and commit in one block or three
+launches; and those stages bin by bin against
 pedestrian by pedestrian; and the gather of few footprints against the
 others.  All leave the same bits."""
 import numpy as np
@@ -21,13 +21,13 @@ def _built():
     sfm.lib()
 
 
-def _sim(W, H, n, periodic, walk):
+def _sim(W, H, n, periodic, walk, r=5):
     rng = np.random.default_rng(W + H + n)
     cell = np.zeros((H, W), np.uint8)
     cell[:, W // 2] = 1
     cell[H // 3:H // 2, W // 2] = 0
     cell[0, W // 4:W // 2] = 2
-    s = sfm.Sim(W=W, H=H, cell=cell, periodic_x=periodic, periodic_y=periodic, r=5)
+    s = sfm.Sim(W=W, H=H, cell=cell, periodic_x=periodic, periodic_y=periodic, r=r)
     at = rng.choice(np.flatnonzero(cell.ravel() == 0), n, replace=False)
     s.place(np.stack([at % W, at // W], 1).astype(np.int32), rng.integers(0, 9, n).astype(np.uint8),
             rng.integers(0, 9, n).astype(np.uint8), (rng.random(n) < 0.9).astype(np.uint8))
@@ -61,6 +61,25 @@ def test_short_and_long_launch_sequences_agree(W, H, n, periodic, walk):
         assert stats == got[0][1]
         for a, b in zip(arrays, got[0][0]):
             np.testing.assert_array_equal(a, b)
+
+
+# decide, vote and commit in one block up to 384 pedestrians, 768 on at most
+# 128 x 128 su, 1024 on 64 x 64, 128 beyond radius 33
+@pytest.mark.parametrize("W,H,r,n", [(64, 64, 5, 1024), (64, 64, 5, 1025), (65, 64, 5, 768), (128, 128, 33, 769),
+                                     (129, 128, 33, 384), (300, 300, 5, 385), (90, 80, 34, 128), (90, 80, 34, 129)])
+def test_one_block_or_three_launches(W, H, r, n):
+    got = []
+    for timing in (False, True):  # a timed tick runs stage by stage
+        with _sim(W, H, n, 1, True, r) as s:
+            s.set_timing(timing)
+            before = s.stats()["kernel_launches"]
+            got.append(_run(s, 1))
+            got[-1][1]["launches"] = s.stats()["kernel_launches"] - before
+    one = n <= (128 if r > 33 else 384 if W * H > 128 * 128 else 768 if W * H > 64 * 64 else 1024)
+    assert got[1][1].pop("launches") - got[0][1].pop("launches") == (2 if one else 0)
+    assert got[0][1] == got[1][1]
+    for a, b in zip(got[0][0], got[1][0]):
+        np.testing.assert_array_equal(a, b)
 
 
 # Lattices whose last bins are ragged; 512 threads a bin up to twice the SMs in
