@@ -1091,23 +1091,18 @@ sfm_status sfm_batch_place(sfm_ctx* ctx, const int32_t* counts, const int32_t* x
     BCU(cudaMemsetAsync(ctx->choice, 0, n, s));
     BCU(cudaMemsetAsync(ctx->won, 0, n, s));
   }
-  BCU(cudaStreamSynchronize(s));
-  Counters h;
-  BCU(cudaMemcpy(&h, ctx->ctr, sizeof(h), cudaMemcpyDeviceToHost));
-  h.moved = 0;
-  h.exited = 0;
-  h.max_registrants = 0;
-  h.err = 0;
-  BCU(cudaMemcpy(ctx->ctr, &h, sizeof(h), cudaMemcpyHostToDevice));
+  launch_reset_counters(ctx->ctr, s);
+  ctx->launches += 1;
   if (n > 0) {
     k_batch_scatter<<<(n + 255) / 256, 256, 0, s>>>(n, ctx->xy, ctx->heading, ctx->goal, ctx->alive,
                                                     B->ped_scene, B->scenes, ctx->cell, ctx->occ,
                                                     ctx->ocls, ctx->ctr);
     ctx->launches += 1;
   }
+  Counters h;
+  BCU(cudaMemcpyAsync(&h, ctx->ctr, sizeof(h), cudaMemcpyDeviceToHost, s));
   BCU(cudaStreamSynchronize(s));
   BCU(cudaGetLastError());
-  BCU(cudaMemcpy(&h, ctx->ctr, sizeof(h), cudaMemcpyDeviceToHost));
   if (h.err) {
     const uint32_t flags = h.err;
     cudaMemsetAsync(ctx->occ, 0xff, (size_t)ctx->nsu_total * sizeof(int32_t), s);
