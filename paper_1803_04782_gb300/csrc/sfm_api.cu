@@ -155,7 +155,7 @@ sfm_status check_flags(sfm_ctx* ctx) {
 // tiles so every su is summed in the same order in every mode.  A crowded
 // lattice's rows come from the product, whose sums are exact.
 cudaError_t launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi, int ring = 0,
-                            bool early = false) {
+                            bool early = false, bool one_row = false) {
   ++c->launches;
   if (c->use_product()) {
     ProductArgs a = c->prod;
@@ -166,7 +166,10 @@ cudaError_t launch_field_of(sfm_ctx* c, float* out, int out_row0, int lo, int hi
     a.ring = ring;
     return launch_product(a, c->stream);
   }
-  return launch_field(c->geo, c->bin_start, c->rec, c->tables(), c->Fs, out, out_row0, lo, hi, c->ctr,
+  Tables tb = c->tables();
+  // a launch of one row lasts as long as a footprint's chain of visits: the smallest footprint
+  if (one_row) tb.shape = kShape16x16;
+  return launch_field(c->geo, c->bin_start, c->rec, tb, c->Fs, out, out_row0, lo, hi, c->ctr,
                       c->stream, FarPart(), ring, early);
 }
 
@@ -179,8 +182,8 @@ cudaError_t field_rows(sfm_ctx* c, float* out, int ya, int yb, int main_off, boo
   const int lo = ya - 1 >= 0 ? ya - 1 : 0, hi = yb + 1 <= g.H ? yb + 1 : g.H;
   cudaError_t e = launch_field_of(c, out, ya - main_off, lo, hi);
   // halo rows that wrap around a periodic y boundary
-  if (e == cudaSuccess && g.py && ya == 0) e = launch_field_of(c, out, g.H - 1, g.H - 1, g.H);
-  if (e == cudaSuccess && g.py && yb == g.H) e = launch_field_of(c, out, -(yb - ya + 1), 0, 1);
+  if (e == cudaSuccess && g.py && ya == 0) e = launch_field_of(c, out, g.H - 1, g.H - 1, g.H, 0, false, true);
+  if (e == cudaSuccess && g.py && yb == g.H) e = launch_field_of(c, out, -(yb - ya + 1), 0, 1, 0, false, true);
   return e;
 }
 
@@ -575,7 +578,6 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
   sfm_ctx* ctx = new sfm_ctx;
   ctx->lat = *lat;
   ctx->nsu_total = (int64_t)lat->W * lat->H;
-  ctx->field_shape = default_field_shape(prm->r, lat->W, lat->H);
   ctx->prm = *prm;
   ctx->prm.bin = kBin;
   ctx->stream = static_cast<cudaStream_t>(stream);
@@ -616,6 +618,7 @@ sfm_status sfm_create(const sfm_lattice* lat, const uint8_t* cell, int32_t cell_
     ctx->band_rows = (int)rows;
     ctx->bands = (int)((g.H + rows - 1) / rows);
   }
+  ctx->field_shape = default_field_shape(g.r, g.W, ctx->bands > 1 ? ctx->band_rows : g.H);
   std::vector<DeviceArray> arrays = {
       array_of(ctx->cell, nsu),
       array_of(ctx->Fs, nsu),

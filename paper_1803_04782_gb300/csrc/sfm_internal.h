@@ -187,15 +187,17 @@ struct Tables {
   int shape = 0;        // class-table gather footprint: kShape16x16 .. kShape32x32
 };
 
-// Footprint of the class-table gather used when none has been tuned: the
-// largest of which a lattice has enough to occupy the warps (18 of an SM's 28;
-// 2736 on 152 SMs).  32 x 32 against 16 x 16, bins and field, a pedestrian on
-// every 40th su: 2048^2 68 us against 81 at r = 20 and 146 against 169 at r =
-// 40, 1750^2 (3025 footprints) 59 and 66, 118 and 128; but 1500^2 (2209) 54 and
-// 50, 105 and 97, 1000^2 49 and 34, 92 and 55.  Beyond the 32 x 32's radii, 32 x
-// 16 at r = 45: 1250^2 (3160) 89 against 112, but 1000^2 (2016) 78 and 68.
+// Footprint of the class-table gather used when none has been tuned; W x H: the
+// su of a launch (a band's rows).  32 x 32 from 16 an SM on (2432 on 152 SMs):
+// up to there the 16 x 16 ones' four times as many make two rounds of the warps,
+// then three.  16 x 16 over 32 x 32, a tick, at a pedestrian on every 50th su and
+// at three on ten: r = 7 2401 footprints 0.95 and 0.83, 2500 1.02 and 0.96; r = 20
+// 0.96 and 0.90, 1.06 and 1.04; r = 36 0.95 and 0.92, 1.03 and 1.05 (in bands of
+// 2048 columns 2304 0.93 and 0.91, 2560 1.10 and 1.08 at r = 20; 1024 0.65 and
+// 0.55).  Beyond the 32 x 32's radii, 32 x 16 at r = 45: 1250^2 (3160) 89 us
+// against 112, but 1000^2 (2016) 78 and 68.
 inline int default_field_shape(int r, int W, int H) {
-  const int64_t nx = (W + 31) / 32, enough = 18 * (int64_t)device_sm_count();
+  const int64_t nx = (W + 31) / 32, enough = 16 * (int64_t)device_sm_count() + 1;
   if (field3_stride(r)) return nx * ((H + 31) / 32) >= enough ? kShape32x32 : kShape16x16;
   return r > 30 && nx * ((H + 15) / 16) >= enough ? kShape32x16 : kShape16x16;
 }

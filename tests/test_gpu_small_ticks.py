@@ -204,3 +204,27 @@ def test_allocation_free_field_takes_the_contexts_gather():
                                      base, out) == sfm.SFM_OK
         got = out.cpu().numpy()
         assert np.abs(got - want).max() <= 1e-5 * max(np.abs(want).max(), 1e-30)
+
+
+@pytest.mark.parametrize("W,H,rows,r,periodic", [(2100, 2400, 1216, 5, 0), (2100, 2400, 1120, 5, 0),
+                                                 (520, 640, 160, 33, 1), (520, 640, 160, 33, 0)])
+def test_bands_take_the_footprint_of_their_own_rows(W, H, rows, r, periodic):
+    """The default footprint goes by the footprints of one launch; whatever it
+    is, the bands' fields and moves are the whole lattice's."""
+    rng = np.random.default_rng(W + rows)
+    n = W * H // 30
+    at = rng.choice(W * H, n, replace=False)
+    xy = np.stack([at % W, at // W], 1).astype(np.int32)
+    heading, goal = (rng.integers(0, 9, n).astype(np.uint8) for _ in range(2))
+    budget = sfm.band_budget(W, H, rows, periodic, periodic)
+    kw = dict(W=W, H=H, cell=np.zeros((H, W), np.uint8), periodic_x=periodic, periodic_y=periodic, r=r)
+    with sfm.Sim(**kw) as whole, sfm.Sim(hbm_budget_bytes=budget, **kw) as bands:
+        assert bands.stats()["bands"] == -(-H // rows)
+        for s in (whole, bands):
+            s.place(xy, heading, goal)
+            s.compute_field() if s is whole else None
+        np.testing.assert_array_equal(bands.field_banded(), whole.field())
+        for s in (whole, bands):
+            s.step(3)
+        for a, b in zip(whole.peds(), bands.peds()):
+            np.testing.assert_array_equal(a, b)
