@@ -207,11 +207,12 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
   // CTAs that would idle, the integer sums added up in `scratch` and joined
   // by the last CTA of the tile.
   const int nch = a.nch, T = a.ntiles, whole = T / G, rest = T - whole * G;
-  // the clocks of a plane of the list's last tile (the rest is at its end):
-  // 128 a product, and its plane to build
+  // the clocks of a plane of the rest's first tile, the largest radius in it:
+  // 128 a product, and its plane to build (by the last one's, a batch's few
+  // tiles of radius 44 beside others of 3 were not split and took 190 us)
   int S;
   {
-    const int r = a.lattices ? a.lattices[a.tiles[T - 1].x].r : a.one.r;
+    const int r = a.lattices ? a.lattices[a.tiles[rest ? whole * G : 0].x].r : a.one.r;
     S = a.scratch ? slices_of(rest, nch, G, (2 * r + 16) * chunks_of(r) * 128 + 2000) : 1;
   }
   const int units = whole + (rest * S) / G + (me < rest * S % G ? 1 : 0);
