@@ -276,8 +276,8 @@ sfm_status sfm_set_field_footprint(sfm_ctx* ctx, int32_t shape);
 
 /* How the field of a crowded lattice is summed.  0 (the default): by the
  * context's own crowd -- from 9 pedestrians of the last placement on 20 su
- * (in a lattice no larger than the window either way, or of under 1024 su:
- * where it is also the faster way; sfm_crowded) the field is a matrix product whose sums are exact (radius 1..44; laws
+ * (in a lattice no larger than the window either way: where it is also the
+ * faster way; sfm_crowded) the field is a matrix product whose sums are exact (radius 1..44; laws
  * whose range over the window fits its fixed-point tables), rounded once;
  * below that, a gather of FP32 sums.  Both lie within the field's error
  * bound and may differ in the last bits: the product is closer where many

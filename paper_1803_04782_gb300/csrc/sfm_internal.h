@@ -216,16 +216,16 @@ constexpr int kProductMaxRadius = 44;
 // moves its neighbours: the line lies above the room, corridor and batch
 // workloads (at most 2 su in 5), whose runs stay bit for bit what they were.
 //
-// A lattice no larger than the window either way, or of under 1024 su, is summed
-// by whichever takes less.  There the gather's launch lasts as long as one footprint's chain of
+// A lattice no larger than the window either way is summed by whichever takes
+// less.  There the gather's launch lasts as long as one footprint's chain of
 // visits, 45 ns each (107 beyond the wide strides' radii), the product's as
 // long as its start and a plane's products.  Ticks by product and gather at a
 // density of 0.46: 20 x 20 at r = 38 62 and 20 us, 3000 x 10 at r = 30 82 and
-// 33, 28 x 28 at r = 20 37 and 27, 20 x 20 at r = 1 36 and 26, but 40 x 40 at r = 20 39 and 43, 64 x 64 at r =
+// 33, 28 x 28 at r = 20 37 and 27, but 40 x 40 at r = 20 39 and 43, 64 x 64 at r =
 // 38 69 and 84, at r = 44 73 and 211.
 inline bool lattice_crowded(int W, int H, int r, int64_t n) {
   if (20 * n < 9 * (int64_t)W * H) return false;
-  if (W > 2 * r && H > 2 * r && (int64_t)W * H >= 1024) return true;
+  if (W > 2 * r && H > 2 * r) return true;
   const double seen = 2.0 * r + 16;  // su a side that a 16 x 16 footprint's window spans
   const double visits = (double)n / ((double)W * H) * (W < seen ? W : seen) * (H < seen ? H : seen);
   const double products = seen * ((2 * r + 8 + 15) / 16);  // a plane's, 128 clocks each
