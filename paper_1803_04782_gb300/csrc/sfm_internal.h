@@ -216,20 +216,21 @@ constexpr int kProductMaxRadius = 44;
 // moves its neighbours: the line lies above the room, corridor and batch
 // workloads (at most 2 su in 5), whose runs stay bit for bit what they were.
 //
-// A lattice no larger than the window either way is summed by whichever takes
-// less.  There the gather's launch lasts as long as one footprint's chain of
-// visits, 45 ns each (107 beyond the wide strides' radii), the product's as
-// long as its start and a plane's products.  Ticks by product and gather at a
-// density of 0.46: 20 x 20 at r = 38 62 and 20 us, 3000 x 10 at r = 30 82 and
-// 33, 28 x 28 at r = 20 37 and 27, but 40 x 40 at r = 20 39 and 43, 64 x 64 at r =
-// 38 69 and 84, at r = 44 73 and 211.
+// A lattice no larger than the window either way is summed by the gather where
+// that is clearly the faster way: its launch lasts as long as one footprint's
+// chain of visits, 45 ns each in a context (107 beyond the wide strides' radii)
+// and about twice that in a batch, which has to decide alike; the product's
+// lasts as long as its start and a plane's products.  Ticks by product and
+// gather at a density of 0.46: 20 x 20 at r = 38 62 and 20 us, 300 x 7 at r = 30
+// 54 and 27, 3000 x 10 at r = 30 82 and 33; but 40 x 40 at r = 20 39 and 43, 64 x
+// 64 at r = 38 69 and 84, at r = 44 73 and 211.
 inline bool lattice_crowded(int W, int H, int r, int64_t n) {
   if (20 * n < 9 * (int64_t)W * H) return false;
   if (W > 2 * r && H > 2 * r) return true;
   const double seen = 2.0 * r + 16;  // su a side that a 16 x 16 footprint's window spans
   const double visits = (double)n / ((double)W * H) * (W < seen ? W : seen) * (H < seen ? H : seen);
   const double products = seen * ((2 * r + 8 + 15) / 16);  // a plane's, 128 clocks each
-  return 25.0 + products * 128.0 / 2070.0 < 12.0 + visits * (r > 41 ? 0.107 : 0.045);
+  return 25.0 + products * 128.0 / 2070.0 < 12.0 + visits * (r > 41 ? 0.2 : 0.1);
 }
 
 // Planes (and their tables): a crowd's presence and four heading axes; a cell
@@ -399,11 +400,11 @@ constexpr int kMoveMaxPeds = 1024;
 // both, 1024 31.1 and 23.5; 384 on 2000 x 2000 32.0 and 31.9; where many share a
 // su's surroundings later: 768 on 100 x 100 27.8 and 28.6, 1024 29.6 and 27.4, on
 // 40 x 40 45.7 and 49.0.  Beside a gather of large tables the block has little
-// L1: 617 x 477 at r = 40, 128 pedestrians 24.5 and 24.9, 256 30.8 and 26.4 (at r =
-// 30 22.5 and 25.5).  Rectangles read their whole rings: always slower.
+// L1: 617 x 477 at r = 45, 128 pedestrians 24.1 and 25.3, 200 27.8 and 26.3, 256 31.0
+// and 27.2 (at r = 30 22.5 and 25.5).  Rectangles read their whole rings: always slower.
 inline bool move_in_one(int W, int H, int r, int n, bool sized) {
   const int64_t su = (int64_t)W * H;
-  return !sized && n > 0 && n <= (r > 33 ? 128 : su > 128 * 128 ? 384 : su > 64 * 64 ? 768 : kMoveMaxPeds);
+  return !sized && n > 0 && n <= (r > 33 ? 192 : su > 128 * 128 ? 384 : su > 64 * 64 ? 768 : kMoveMaxPeds);
 }
 void launch_move(int n, const int32_t* rec_id, const int32_t* bin_start, int2* xy, uint8_t* alive,
                  uint8_t* heading, const uint8_t* goal, const uint8_t* cell, int32_t* occ,

@@ -94,7 +94,7 @@ def test_bands_batch_and_candidates_round_as_one_launch(px, py, r, rows):
             assert s.stats()["error_flags"] == 0
 
 
-@pytest.mark.parametrize("W,H,r,product", [(20, 20, 38, False), (24, 26, 20, False), (300, 8, 20, False),
+@pytest.mark.parametrize("W,H,r,product", [(20, 20, 38, False), (12, 16, 20, False), (300, 4, 20, False),
                                            (40, 40, 44, True), (64, 64, 38, True), (41, 45, 20, True)])
 def test_lattices_smaller_than_the_window_take_the_faster_way(W, H, r, product):
     sc = _crowd(W, H, r, 0, 0, rho=0.95, seed=13)

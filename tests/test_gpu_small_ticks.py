@@ -64,9 +64,9 @@ def test_short_and_long_launch_sequences_agree(W, H, n, periodic, walk):
 
 
 # decide, vote and commit in one block up to 384 pedestrians, 768 on at most
-# 128 x 128 su, 1024 on 64 x 64, 128 beyond radius 33
+# 128 x 128 su, 1024 on 64 x 64, 192 beyond radius 33
 @pytest.mark.parametrize("W,H,r,n", [(64, 64, 5, 1024), (64, 64, 5, 1025), (65, 64, 5, 768), (128, 128, 33, 769),
-                                     (129, 128, 33, 384), (300, 300, 5, 385), (90, 80, 34, 128), (90, 80, 34, 129)])
+                                     (129, 128, 33, 384), (300, 300, 5, 385), (90, 80, 34, 192), (90, 80, 34, 193)])
 def test_one_block_or_three_launches(W, H, r, n):
     got = []
     for timing in (False, True):  # a timed tick runs stage by stage
@@ -75,7 +75,7 @@ def test_one_block_or_three_launches(W, H, r, n):
             before = s.stats()["kernel_launches"]
             got.append(_run(s, 1))
             got[-1][1]["launches"] = s.stats()["kernel_launches"] - before
-    one = n <= (128 if r > 33 else 384 if W * H > 128 * 128 else 768 if W * H > 64 * 64 else 1024)
+    one = n <= (192 if r > 33 else 384 if W * H > 128 * 128 else 768 if W * H > 64 * 64 else 1024)
     assert got[1][1].pop("launches") - got[0][1].pop("launches") == (2 if one else 0)
     assert got[0][1] == got[1][1]
     for a, b in zip(got[0][0], got[1][0]):
