@@ -43,7 +43,7 @@
 #include <math.h>
 #include <stdint.h>
 
-#include "sfm_device.cuh"
+#include "sfm_umma.cuh"
 
 namespace sfm {
 
@@ -70,41 +70,6 @@ static_assert(kTW * 2 == 128, "8 blocks side by side are one core matrix");
 static_assert(kWorkers % 4 == 0, "the workers cover the four TMEM lane quarters alike");
 static_assert(kHeadBytes + plane_bytes_of(kProductMaxRadius) + 2 * stage_bytes_of(kProductMaxRadius) <= kSmem,
               "a plane and two table stages must fit");
-
-// bounded wait for an mbarrier phase, about a second with an iteration cap
-// behind it; false: it ran out
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  unsigned long long t0 = 0;
-  for (int it = 0; it < (1 << 26); ++it) {
-    uint32_t done = 0;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (second_is_over(it, t0)) return false;
-  }
-  return false;
-}
-
-__device__ __forceinline__ void arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
-               : "memory");
-}
-
-// no-swizzle K-major operand: start, offset between the two 8-column halves
-// of K, offset between groups of 8 rows
-__device__ __forceinline__ uint64_t operand(uint32_t saddr, uint32_t khalf, uint32_t group) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(khalf >> 4) << 16) |
-         ((uint64_t)(group >> 4) << 32) | (1ull << 46);
-}
 
 // kind::f16: FP32 accumulators, FP16 operands, M = 128, N = 256
 constexpr uint32_t kIdesc = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
@@ -298,36 +263,32 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
             if (failed) break;
             if (some) {
               asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-              uint64_t ad = operand(plane0 + (uint32_t)pb * plane_bytes + (uint32_t)(c * 32), 16,
+              uint64_t ad = umma_desc(plane0 + (uint32_t)pb * plane_bytes + (uint32_t)(c * 32), 16,
                                     (uint32_t)(16 * P));
-              uint64_t bd = operand(stage0 + (uint32_t)st * stage_bytes + (uint32_t)((K - 1) * 512), 128, 256);
+              uint64_t bd = umma_desc(stage0 + (uint32_t)st * stage_bytes + (uint32_t)((K - 1) * 512), 128, 256);
               for (int ky = 0; ky < K; ++ky) {
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "setp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-                    "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
+                umma_f16(d, ad, bd, kIdesc, acc);
                 acc = 1;
                 ad += (uint64_t)(P >> 4);
                 bd -= (uint64_t)(512 >> 4);
               }
-              commit(sempty(st));
+              umma_commit(sempty(st));
             } else {
-              arrive(sempty(st));
+              mbar_arrive(sempty(st));
             }
             word[6] = n_stage + 1;
           }
           if (some)
-            commit(pempty(pb));
+            umma_commit(pempty(pb));
           else
-            arrive(pempty(pb));
+            mbar_arrive(pempty(pb));
         }
         word[3 + set] = (int)acc;
-        arrive(afull(set));
+        mbar_arrive(afull(set));
         if (acc)
-          commit(afull(set));
+          umma_commit(afull(set));
         else
-          arrive(afull(set));
+          mbar_arrive(afull(set));
       }
     }
     __syncwarp();
@@ -386,7 +347,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
       if (__any_sync(0xffffffffu, any != 0) && lane == 0) word[1 + pb] = n_plane + 1;
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       __syncwarp();
-      if (lane == 0) arrive(pfull(pb));
+      if (lane == 0) mbar_arrive(pfull(pb));
       ++n_plane;
     };
     // this thread's block (bx, by): lane m of the accumulators
@@ -478,7 +439,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
       }
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
       __syncwarp();
-      if (lane == 0) arrive(aempty(set));
+      if (lane == 0) mbar_arrive(aempty(set));
       if (part) {
         // the last slice of the tile joins the limbs and leaves zeros
         __threadfence();

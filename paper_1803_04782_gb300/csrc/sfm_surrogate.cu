@@ -20,6 +20,7 @@
 
 #include "sfm_ctx.h"
 #include "sfm_gather.cuh"
+#include "sfm_umma.cuh"
 
 using namespace sfm;
 
@@ -260,60 +261,11 @@ static_assert(kUmRowBytes % 512 == 0 && kUmA % 512 == 0 && kUmB % 16 == 0,
 static_assert(2 * kUmRows * 32 <= kUmTmemCols, "accumulators exceed the TMEM allocation");
 static_assert(kUmSmem <= 227 * 1024, "shared memory of the tcgen05 convolution");
 
-// shared-memory matrix descriptor, no swizzle: start, K-direction (leading)
-// and M/N-direction (stride) byte offsets between core matrices
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
-         ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
-}
-
-// the same with the 64-byte swizzle (K-major rows of 64 bytes, 8-row groups
+// umma_desc with the 64-byte swizzle (K-major rows of 64 bytes, 8-row groups
 // 512 bytes apart; the leading offset is unused)
 __device__ __forceinline__ uint64_t umma_desc_sw64(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) |
          (1ull << 46) | (4ull << 61);
-}
-
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void umma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-               : "memory");
-}
-
-// bounded wait for the mbarrier phase `parity`; false on a timeout.  The
-// bound is about one second of the global timer (checked every 256 tries,
-// each of which may suspend the thread for a short, system-defined time),
-// with an iteration cap behind it.
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
-  uint64_t t0 = 0;
-  for (int it = 0; it < (1 << 24); ++it) {
-    uint32_t done = 0;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if ((it & 255) == 255) {
-      uint64_t now;
-      asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(now));
-      if (t0 == 0)
-        t0 = now;
-      else if (now - t0 > 1000000000ull)
-        return false;
-    }
-  }
-  return false;
 }
 
 __global__ void __launch_bounds__(kWsThreads, 1)
@@ -487,7 +439,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       }
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(acce(ac)) : "memory");
+      if (lane == 0) mbar_arrive(acce(ac));
     }
   }
   if (failed) atomicExch(err, 1);
