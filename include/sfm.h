@@ -365,17 +365,19 @@ sfm_status sfm_set_timing(sfm_ctx* ctx, int32_t every);
 sfm_status sfm_stage_times(sfm_ctx* ctx, double* ms, int64_t* ticks);
 
 /* ---- Batches of independent lattices -------------------------------------
- * Many small or uneven lattices stepped together: every tick is ONE
- * persistent (cooperative) kernel launch that runs bins, field, decisions,
- * vote and commit for all lattices, separated by grid-wide barriers whose
- * waits are bounded (a barrier that times out ends the launch and the next
- * synchronising call returns SFM_ETIMEOUT).  The field stage walks a work
- * list of (lattice, 32-footprint chunk) items sorted by decreasing cost; the
- * tick launch is captured once in a CUDA graph and replayed.  Each lattice
- * evolves exactly as it would in its own context (same bins, same summation
- * order, its own seed and pedestrian numbering), which the tests check bit
- * for bit.  This batches the paper's concurrency technique (several tasks in
- * flight, Sec. 4.2) across scenarios.
+ * Many small or uneven lattices stepped together.  A tick is one persistent
+ * (cooperative) launch that runs bins and field for all lattices, separated
+ * by grid-wide barriers whose waits are bounded (a barrier that times out
+ * ends the launch, nobody moves, and the next synchronising call returns
+ * SFM_ETIMEOUT), and three more for decisions, vote and commit; crowded
+ * lattices' fields (sfm_set_field_rule's rule 0, lattice by lattice) come from
+ * a launch ahead of it.  The field stage walks a work list of (lattice,
+ * 32-footprint chunk) items sorted by decreasing cost; the tick's launches are
+ * captured once in a CUDA graph and replayed.  Each lattice evolves exactly
+ * as it would in its own context (same bins, same summation order or the same
+ * exact sums, its own seed and pedestrian numbering), which the tests check
+ * bit for bit.  This batches the paper's concurrency technique (several tasks
+ * in flight, Sec. 4.2) across scenarios.
  *
  * sfm_batch_create: nscenes lattices (1..65535); lats[i], cells[i] (host,
  *   W*H bytes each), prms[i] (r <= 50).  The context then accepts

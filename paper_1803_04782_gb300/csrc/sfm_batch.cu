@@ -1,7 +1,8 @@
 // sfm_batch.cu -- a batch of independent lattices stepped together: one
 // persistent (cooperative) kernel per tick runs the binning and the field of
 // every lattice, separated by grid-wide barriers with bounded waits, and three
-// launches the decisions, votes and moves of every lattice's bins.  The
+// launches the decisions, votes and moves (by bins, or by pedestrian where the
+// batch is sparse); crowded lattices' fields come from the product ahead.  The
 // field stage walks a work list of (lattice, footprint chunk) items sorted by
 // cost; the footprint height of each radius class is chosen by timing
 // (sfm_batch_autotune).  A tick launch is captured once in a CUDA graph and

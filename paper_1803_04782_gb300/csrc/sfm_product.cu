@@ -7,13 +7,14 @@
 // Arithmetic.  A crowd is five planes of {-1, 0, +1}: occupancy and the four
 // heading axes (E-W, N-S, NE-SW, NW-SE), and K_P is the sum of five window
 // tables, one a plane.  Each table entry is held in fixed point as two
-// integers of FP16 ("limbs"): T = L0 / s0 + L1 / (s0 s1), |L0|, |L1| <= 4096.
+// integers of FP16 ("limbs"): T = L0 / s0 + L1 / (s0 s1) (sfm_limbs.h).
 // Products with {-1, 0, +1} and every partial sum are integers below 2^24 in
-// magnitude (product_scales), so the FP32 accumulators hold them exactly: a
-// sum is the same whatever the order, the tile or the split, and is rounded
-// once, when the limbs are joined.  Against 64 bits the field of a periodic
-// 1000 x 1000 lattice half full at radius 38 is off by 4.2e-8 (2-norm), the
-// gathers' FP32 sums by 8.6e-7.
+// magnitude, so the FP32 accumulators hold them exactly: a sum is the same
+// whatever the order, the tile or the split, and is rounded once, when the
+// limbs are joined.  Against 64 bits the field of a periodic 1000 x 1000
+// lattice half full at radius 38 is off by 3.0e-8 (2-norm), the gathers' FP32
+// sums by 8.6e-7.  A cell grid (the static field) is its walls and exits, two
+// planes each.
 //
 // The product.  A tile is 64 x 256 su = 8 x 16 blocks of 8 x 16 su.  D[m][n]
 // = sum_k A[m][k] B[n][k]: m a block, n a su of the block and a limb, k a su
@@ -24,14 +25,15 @@
 // halves of K), so no im2col copy exists.  B is Toeplitz in y: stored by the
 // difference j = (su row) - (window row), so a window row is a shift of the
 // start address.  Both limbs ride in one M = 128, N = 256 product, which
-// reads A once; one takes 126 clocks (128 at the unit's nominal rate), so the
-// tensor pipe bounds a launch with many tiles.  The 1000 x 1000 lattice has
-// 64 tiles for 152 SMs: at radius 38 their planes are split over two CTAs a
-// tile (212 000 clocks of products of 300 000, clock64), at radius 3 a tile
-// is one CTA's and latency bounds it (six windows' reads, 220 products).
-// Measured there (one-pass ncu): 168 us at radius 38 and 30 at radius 3,
-// where the gathers took 1298 and 70; a plane rebuilt from memory each time
-// took 233 and 63.
+// reads A once and keeps the pipe busy for 128 clocks, so the tensor pipe
+// bounds a launch with many tiles.  The 1000 x 1000 lattice has 64 tiles for
+// 152 SMs: at radius 38 their planes are split over two CTAs a tile (the pipe
+// is busy for 69 % of the SMs' active clocks; the longest CTA has three planes,
+// the mean 2.1), at radius 3 a tile is one CTA's and latency bounds it (21 %;
+// six windows' reads, 220 products).  Measured there (ncu, cold): 168 us at
+// radius 38 and 31 at radius 3; bins and field together took 599 and 66 us by
+// the gathers and take 173 and 39; a plane rebuilt from memory each time took
+// 233 and 63.
 //
 // Roles of a CTA, one an SM: warp 0 copies tables (one plane's 16 window
 // columns a stage), warp 1 issues the products, the others build planes from
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(kProdThreads, 1) k_product(const __grid_consta
 // column + r, evaluated in FP64, zero outside the window.  A thread takes an
 // entry (dx, dy) of the kernel and writes it wherever it stands, for up to eight
 // su columns and all channels: FP64 powers bound it (a thread a limb pair, one
-// for each, took 33 us at r = 40; now 13).
+// for each, took 33 us at r = 40; now 13, and 20 for the cells' two laws).
 __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, double a1, double gamma,
                               double s0, double s1, __half* __restrict__ tab) {
   const int C = chunks_of(r), J = 2 * r + 31, E = 16 * C + 7;
@@ -536,7 +538,8 @@ __global__ void k_limb_tables(int r, int nch, double k0, double a0, double k1, d
   const bool in = dx >= -r && dx <= r && dy >= -r && dy <= r && (dx | dy) != 0;
   const double d = in ? sqrt((double)(dx * dx + dy * dy)) : 1.0;
   const bool cells = nch == kCellPlanes;
-  const double v0 = in ? k0 * pow(d, a0) : 0.0, v1 = in && cells ? k1 * pow(d, a1) : 0.0;
+  const double p0 = in ? pow(d, a0) : 0.0, p1 = !cells ? 0.0 : a1 == a0 ? p0 : in ? pow(d, a1) : 0.0;
+  const double v0 = in ? k0 * p0 : 0.0, v1 = in ? k1 * p1 : 0.0;
   for (int ch = 0; ch < nch; ++ch) {
     const double v = cells ? (ch < 2 ? v0 : v1) : crowd_entry(v0, gamma, dx, dy, d, ch);
     const double first = limb16(v * s0), rest = (v * s0 - first) * s1, whole = rint(rest);
