@@ -181,14 +181,15 @@ def test_rectangles_follow_the_oracle(W, H, n, periodic):
         assert sim.stats()["max_registrants"] >= 2 and sim.stats()["error_flags"] == 0
 
 
-# The allocation-free field on either side of 18 footprints of 32 x 32 su an SM
-# (2736 on 152 SMs): each gather with its own table layout, several sizes in a
+# The allocation-free field on either side of 16 footprints of 32 x 32 su an SM
+# (2432 on 152 SMs; 1568 x 1600 has 2450, 1568 x 1568 2401): each gather with its own table layout, several sizes in a
 # row over the same scratch.  Its bins are in order of arrival: equal up to the
 # rounding of an FP32 sum of at most a window's terms (1e-5 of it).
 def test_allocation_free_field_takes_the_contexts_gather():
     torch = pytest.importorskip("torch")
     for W, H, n, r in [(1700, 1650, 9000, 3), (1700, 1620, 30000, 20), (40, 50, 300, 8), (1700, 1650, 0, 40),
-                       (1700, 1650, 30000, 40), (1700, 1650, 30000, 45)]:
+                       (1700, 1650, 30000, 40), (1700, 1650, 30000, 45), (1568, 1600, 30000, 20),
+                       (1568, 1568, 30000, 20)]:
         rng = np.random.default_rng(r)
         at = rng.choice(W * H, n, replace=False)
         xy = np.stack([at % W, at // W], 1).astype(np.int32)
